@@ -65,8 +65,8 @@ __global__ void neg_pad_kernel(const float* __restrict__ b, int M, int Mp, float
     }
 }
 
-// out[d][i] = in[i][d] for an N x D row-major matrix.
-__global__ void transpose_kernel(const float* __restrict__ in, int N, int D, float* __restrict__ out) {
+// out[d * ld + i] = in[i][d] for an N x D row-major matrix.
+__global__ void transpose_kernel(const float* __restrict__ in, int N, int D, size_t ld, float* __restrict__ out) {
     __shared__ float t[32][33];
     const int d0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
     for (int k = threadIdx.y; k < 32; k += 8) {
@@ -76,7 +76,7 @@ __global__ void transpose_kernel(const float* __restrict__ in, int N, int D, flo
     __syncthreads();
     for (int k = threadIdx.y; k < 32; k += 8) {
         const int d = d0 + k, i = i0 + threadIdx.x;
-        if (i < N && d < D) out[(size_t)d * N + i] = t[threadIdx.x][k];
+        if (i < N && d < D) out[(size_t)d * ld + i] = t[threadIdx.x][k];
     }
 }
 
@@ -180,15 +180,21 @@ extern "C" int cupso_lsq_eval(const float* A_dev, const float* b_dev, int M, int
     }
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     if (precision == CUPSO_LSQ_FP32 || precision == CUPSO_LSQ_FP64) {
-        // the FP32 and FP64 kernels read X(i, d) = x[d * ldx + i]: transpose into a temporary
+        // the exact kernels read X(i, d) = x[d * ld + i]: transposed into a temporary, with their workspace behind it
+        const bool f64 = precision == CUPSO_LSQ_FP64;
+        const int ld = (N + 127) / 128 * 128;
+        const size_t xbytes = up(sizeof(float) * (size_t)ld * D, 256);
+        int dev = 0, sms = 1;
         float* xd = nullptr;
-        cudaError_t e = cudaMalloc(&xd, sizeof(float) * (size_t)N * D);
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaMalloc(&xd, xbytes + lsq_exact_ws_bytes(N, M, f64));
         if (e != cudaSuccess) return set_cuda_error(e, "cudaMalloc"), CUPSO_ERR_OOM;
-        transpose_kernel<<<dim3((D + 31) / 32, (N + 31) / 32), dim3(32, 8), 0, st>>>(X_dev, N, D, xd);
+        transpose_kernel<<<dim3((D + 31) / 32, (N + 31) / 32), dim3(32, 8), 0, st>>>(X_dev, N, D, (size_t)ld, xd);
         e = cudaGetLastError();
         if (e == cudaSuccess)
-            e = precision == CUPSO_LSQ_FP32 ? lsq_fp32_launch(xd, N, N, D, A_dev, b_dev, M, f_out_dev, st)
-                                            : lsq_fp64_launch(xd, N, N, D, A_dev, b_dev, M, f_out_dev, st);
+            e = lsq_exact_launch(xd, ld, N, D, A_dev, b_dev, M, f64, f_out_dev, reinterpret_cast<char*>(xd) + xbytes, sms,
+                                 st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         cudaFree(xd);
         if (e != cudaSuccess) return set_cuda_error(e, "lsq fp32/fp64"), CUPSO_ERR_CUDA;

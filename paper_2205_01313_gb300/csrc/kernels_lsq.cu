@@ -2,11 +2,9 @@
 //
 // For the dense fitness the swarm's Step 3 is a matrix product: with X the
 // N x D matrix of positions, the residuals are R = X A^T - 1 b^T (N x M) and
-// f_i = sum_m R_im^2. Three implementations:
+// f_i = sum_m R_im^2. The exact FP32 and FP64 forms are in
+// kernels_lsq_exact.cu; here the tensor-core ones:
 //
-//  * lsq_fp32_kernel: plain FP32 on the CUDA cores, every residual a chain of
-//    fma over d in order and the squares summed over m in order -- the same
-//    rounding as the oracle, so its trajectories match bit for bit.
 //  * lsq_tc_kernel<false>: BF16 operands on the 5th-generation tensor cores
 //    (tcgen05.mma, FP32 accumulation in tensor memory), operands staged by TMA
 //    with 128-byte swizzle, and the epilogue (subtract b, square, sum over m)
@@ -409,133 +407,6 @@ __global__ void __launch_bounds__(256) convert_dimmajor_bf16_kernel(const float*
     }
 }
 
-// Plain FP32 least-squares fitness with the oracle's rounding order. Block =
-// 64 particles x all M, in tiles of 64 residual rows; thread (ty, tx) holds a
-// 4 x 4 block of (particle, row) residuals, each a chain of fma over d in
-// order; then 64 threads add the tile's squares to their particle's sum in
-// row order. X(i, d) = x[d * ldx + i] (the swarm layout).
-__global__ void __launch_bounds__(256) lsq_fp32_kernel(const float* __restrict__ x, int ldx, int N, int D,
-                                                       const float* __restrict__ A, const float* __restrict__ b, int M,
-                                                       float* __restrict__ f) {
-    __shared__ __align__(16) float Xs[32][64 + 4];   // [d][particle]
-    __shared__ __align__(16) float As[32][64 + 4];   // [d][row]
-    __shared__ float Rs[64][64 + 1];   // [particle][row]
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int i0 = blockIdx.x * 64;
-    float acc_i = 0.0f;                // the running sum of particle i0 + threadIdx.x (threads < 64)
-    for (int m0 = 0; m0 < M; m0 += 64) {
-        float r[4][4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int m = m0 + tx * 4 + c;
-                r[a][c] = m < M ? -b[m] : 0.0f;
-            }
-        for (int d0 = 0; d0 < D; d0 += 32) {
-            for (int e = threadIdx.x; e < 32 * 64; e += 256) {
-                const int dd = e / 64, col = e % 64;
-                const int d = d0 + dd;
-                Xs[dd][col] = (d < D && i0 + col < N) ? x[(size_t)d * ldx + i0 + col] : 0.0f;
-                As[dd][col] = (d < D && m0 + col < M) ? A[(size_t)(m0 + col) * D + d] : 0.0f;
-            }
-            __syncthreads();
-            const int dn = min(32, D - d0);
-            for (int dd = 0; dd < dn; ++dd) {
-                // rows of 68 floats: every 4-float group is 16-byte aligned
-                const float4 x4 = *reinterpret_cast<const float4*>(&Xs[dd][ty * 4]);
-                const float4 a4 = *reinterpret_cast<const float4*>(&As[dd][tx * 4]);
-                const float xv[4] = {x4.x, x4.y, x4.z, x4.w};
-                const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) r[a][c] = __fmaf_rn(av[c], xv[a], r[a][c]);
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) Rs[ty * 4 + a][tx * 4 + c] = r[a][c];
-        __syncthreads();
-        if (threadIdx.x < 64) {
-            const int mn = min(64, M - m0);
-            for (int c = 0; c < mn; ++c) acc_i = __fmaf_rn(Rs[threadIdx.x][c], Rs[threadIdx.x][c], acc_i);
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < 64 && i0 + threadIdx.x < N) f[i0 + threadIdx.x] = acc_i;
-}
-
-// FP64 least-squares fitness in the reference order, rounded once to FP32:
-// per particle, acc = 0; for m ascending: r = -b_m, r = r + A_md x_d for d
-// ascending (each product of two floats is exact in binary64, so the fma below
-// rounds exactly as the separate product and sum would), acc = acc + r * r
-// (square rounded, then added); f = acc rounded to float. Block = 64 particles
-// x all M, in tiles of 32 residual rows; thread (ty, tx) holds the 4 x 2 block
-// of (particle, row) residuals, each a chain over d in order; 64 threads then
-// add the tile's squares to their particle's sum in row order.
-__global__ void __launch_bounds__(256) lsq_fp64_kernel(const float* __restrict__ x, int ldx, int N, int D,
-                                                       const float* __restrict__ A, const float* __restrict__ b, int M,
-                                                       float* __restrict__ f) {
-    __shared__ __align__(16) float Xs[32][64 + 4];   // [d][particle]
-    __shared__ __align__(16) float As[32][32 + 4];   // [d][row]
-    __shared__ double Rs[64][32 + 1];                 // [particle][row]
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int i0 = blockIdx.x * 64;
-    double acc_i = 0.0;                // the running sum of particle i0 + threadIdx.x (threads < 64)
-    for (int m0 = 0; m0 < M; m0 += 32) {
-        double r[4][2];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int m = m0 + tx * 2 + c;
-                r[a][c] = m < M ? -(double)b[m] : 0.0;
-            }
-        for (int d0 = 0; d0 < D; d0 += 32) {
-            for (int e = threadIdx.x; e < 32 * 64; e += 256) {
-                const int dd = e / 64, col = e % 64;
-                const int d = d0 + dd;
-                Xs[dd][col] = (d < D && i0 + col < N) ? x[(size_t)d * ldx + i0 + col] : 0.0f;
-            }
-            for (int e = threadIdx.x; e < 32 * 32; e += 256) {
-                const int dd = e / 32, col = e % 32;
-                const int d = d0 + dd;
-                As[dd][col] = (d < D && m0 + col < M) ? A[(size_t)(m0 + col) * D + d] : 0.0f;
-            }
-            __syncthreads();
-            const int dn = min(32, D - d0);
-            for (int dd = 0; dd < dn; ++dd) {
-                const float4 x4 = *reinterpret_cast<const float4*>(&Xs[dd][ty * 4]);
-                const float2 a2 = *reinterpret_cast<const float2*>(&As[dd][tx * 2]);
-                const double xv[4] = {(double)x4.x, (double)x4.y, (double)x4.z, (double)x4.w};
-                const double av[2] = {(double)a2.x, (double)a2.y};
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) r[a][c] = __fma_rn(av[c], xv[a], r[a][c]);
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) Rs[ty * 4 + a][tx * 2 + c] = r[a][c];
-        __syncthreads();
-        if (threadIdx.x < 64) {
-            const int mn = min(32, M - m0);
-            for (int c = 0; c < mn; ++c) {
-                const double rc = Rs[threadIdx.x][c];
-                acc_i = __dadd_rn(acc_i, __dmul_rn(rc, rc));
-            }
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < 64 && i0 + threadIdx.x < N) f[i0 + threadIdx.x] = __double2float_rn(acc_i);
-}
-
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
@@ -677,17 +548,5 @@ cudaError_t lsq_tc_launch(const LsqTcPlan& p, const float* off, const float* inv
 }
 
 int lsq_tc_partials(const LsqTcPlan& p) { return p.Mp / 128; }
-
-cudaError_t lsq_fp32_launch(const float* x, int ldx, int N, int D, const float* A, const float* b, int M, float* f,
-                            cudaStream_t st) {
-    lsq_fp32_kernel<<<(N + 63) / 64, 256, 0, st>>>(x, ldx, N, D, A, b, M, f);
-    return cudaGetLastError();
-}
-
-cudaError_t lsq_fp64_launch(const float* x, int ldx, int N, int D, const float* A, const float* b, int M, float* f,
-                            cudaStream_t st) {
-    lsq_fp64_kernel<<<(N + 63) / 64, 256, 0, st>>>(x, ldx, N, D, A, b, M, f);
-    return cudaGetLastError();
-}
 
 }  // namespace cupso

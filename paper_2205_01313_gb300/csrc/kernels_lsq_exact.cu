@@ -1,0 +1,344 @@
+// kernels_lsq_exact.cu -- the exact least-squares fitness on the CUDA cores:
+// f_i = ||A x_i - b||^2 in FP32 or FP64 with every rounding in the oracle's
+// order.
+//
+// Per particle i: for each residual row m, r = -b_m, then r = fma(A_md, x_id, r)
+// for d ascending; the squares are summed for m ascending (FP32: f = fma(r, r, f);
+// FP64: f = f + r * r, the square rounded first, f rounded to binary32 at the
+// end; a product of two binary32 values is exact in binary64).
+//
+// Only the sum over m ties the rows of a particle together, so the work is
+// split there: lsq_resid_kernel computes residuals as a register-tiled matrix
+// product over all (row, particle) tiles at once -- each residual one chain
+// over d in one thread, as the order demands -- and lsq_sumsq_kernel then adds
+// a particle's squares in row order. The residuals pass through a workspace
+// R[m][i] of at most kExactWsBytes (half the L2), a chunk of rows (and of
+// particles, for very large swarms) at a time; the running sums carry over from
+// chunk to chunk.
+//
+// Measured on one GB300 (one evaluation; before: a block kept 64 particles x
+// all M, 32 blocks for 2048 particles on 152 SMs): FP32 2048 x 500 x 2000
+// 1.9 ms -> 117 us (the product 41 TFLOP/s), 8192 x 1024 x 4096 7.88 -> 1.53 ms
+// (46 TFLOP/s of about 80 at 128 lanes per SM and clock); FP64 8192 x 1024 x
+// 4096 127 -> 64 ms (1.08 TFLOP/s, the FP64 pipe: A and x are converted once
+// per stage, not in every thread's inner loop).
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "cupso_device.cuh"
+#include "cupso_internal.h"
+#include "lsq_internal.h"
+
+namespace cupso {
+
+namespace {
+
+constexpr size_t kExactWsBytes = 64u << 20;   // residual workspace at most
+constexpr int kResidThreads = 128;            // 16 x 8 threads of TM x TN residuals
+constexpr int kBk = 16;                       // dimensions per shared-memory stage
+constexpr int kRowTile = 128;                 // chunk sizes are multiples of this
+constexpr int kSumThreads = 128;
+constexpr int kSumStageBytes = 8192;
+constexpr int kSumStages = 4;
+
+// TM x TN residuals of one thread: r[a][c] += av[a] * xv[c], one rounding each.
+template <typename T, int TM, int TN>
+struct Acc;
+
+// FP32 residuals in pairs (fma.rn.f32x2: two independent IEEE fmas per
+// instruction: 2048 x 500 x 2000 in 100 us against 157 with scalar fmas).
+template <int TM, int TN>
+struct Acc<float, TM, TN> {
+    unsigned long long r[TM][TN / 2];
+    __device__ __forceinline__ void set(int a, float v) {
+        unsigned long long p;
+        asm("mov.b64 %0, {%1, %1};" : "=l"(p) : "f"(v));
+#pragma unroll
+        for (int c = 0; c < TN / 2; ++c) r[a][c] = p;
+    }
+    __device__ __forceinline__ void step(const float (&av)[TM], const float (&xv)[TN]) {
+        unsigned long long x2[TN / 2];
+#pragma unroll
+        for (int c = 0; c < TN / 2; ++c) asm("mov.b64 %0, {%1, %2};" : "=l"(x2[c]) : "f"(xv[2 * c]), "f"(xv[2 * c + 1]));
+#pragma unroll
+        for (int a = 0; a < TM; ++a) {
+            unsigned long long a2;
+            asm("mov.b64 %0, {%1, %1};" : "=l"(a2) : "f"(av[a]));
+#pragma unroll
+            for (int c = 0; c < TN / 2; ++c) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(r[a][c]) : "l"(a2), "l"(x2[c]));
+        }
+    }
+    __device__ __forceinline__ float get(int a, int c) const {
+        float lo, hi;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(r[a][c / 2]));
+        return (c & 1) ? hi : lo;
+    }
+};
+
+template <int TM, int TN>
+struct Acc<double, TM, TN> {
+    double r[TM][TN];
+    __device__ __forceinline__ void set(int a, double v) {
+#pragma unroll
+        for (int c = 0; c < TN; ++c) r[a][c] = v;
+    }
+    __device__ __forceinline__ void step(const double (&av)[TM], const double (&xv)[TN]) {
+#pragma unroll
+        for (int a = 0; a < TM; ++a)
+#pragma unroll
+            for (int c = 0; c < TN; ++c) r[a][c] = __fma_rn(av[a], xv[c], r[a][c]);
+    }
+    __device__ __forceinline__ double get(int a, int c) const { return r[a][c]; }
+};
+
+// 4 consecutive T from shared memory (16-byte aligned).
+__device__ __forceinline__ void ld4s(const float* p, float* v) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+}
+__device__ __forceinline__ void ld4s(const double* p, double* v) {
+    const double2 a = *reinterpret_cast<const double2*>(p), b = *reinterpret_cast<const double2*>(p + 2);
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+__device__ __forceinline__ void st4g(float* p, const float* v) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void st4g(double* p, const double* v) {
+    *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+    *reinterpret_cast<double2*>(p + 2) = make_double2(v[2], v[3]);
+}
+
+}  // namespace
+
+// Residuals of rows [m0, m1) (m0 a tile multiple): R[(m - m0) * ldr + i] for the
+// particles of this block's tile (FP64: their squares, rounded, so that the sum
+// over rows is left with one operation per row on the narrow FP64 pipe). X(i, d) = x[d * ldx + i]; x 16-byte aligned, ldx
+// a multiple of 64 (columns past the last particle are computed and never
+// summed). vecA: A's rows may be read as float4 (D % 4 == 0, A 16-byte aligned).
+//
+// Block tile 16 TM rows x 8 TN particles, K in slices of kBk through two shared
+// stages: the next slice's A and x are loaded to registers while the current
+// one is multiplied, so one barrier per slice. A's slice is transposed on its
+// way ([k][row], padded), both operands are then read as 16-byte vectors that a
+// warp shares (4 row groups x 8 particle groups: one wavefront each). Zeros
+// past D leave a residual's square unchanged.
+template <typename T, int TM, int TN>
+__global__ void __launch_bounds__(kResidThreads) lsq_resid_kernel(const float* __restrict__ x, int ldx, int D,
+                                                                  const float* __restrict__ A,
+                                                                  const float* __restrict__ b, int m0, int m1,
+                                                                  T* __restrict__ R, int ldr, int vecA) {
+    constexpr int BM = 16 * TM, BN = 8 * TN;
+    constexpr int AK = kBk * BM / kResidThreads;   // A elements per thread and slice: consecutive k of one row
+    constexpr int XV = kBk * BN / 4 / kResidThreads;   // float4 of x per thread and slice
+    __shared__ __align__(16) T As[2][kBk][BM + 4];
+    __shared__ __align__(16) T Xs[2][kBk][BN];
+    const int tid = threadIdx.x;
+    const int tx = tid & 7, ty = tid >> 3;
+    const int i0 = blockIdx.x * BN, mt = m0 + blockIdx.y * BM;
+    const int arow = tid % BM, ak = (tid / BM) * AK;
+    const float* aptr = A + (size_t)min(mt + arow, m1 - 1) * (size_t)D;   // rows past m1 are computed, not stored
+    float ar[AK];
+    float4 xr[XV];
+    auto fetch = [&](int k0) {
+        const int ka = k0 + ak;
+        if (vecA) {
+#pragma unroll
+            for (int j = 0; j < AK; j += 4) {
+                const float4 q = ka + j < D ? *reinterpret_cast<const float4*>(aptr + ka + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+                ar[j] = q.x; ar[j + 1] = q.y; ar[j + 2] = q.z; ar[j + 3] = q.w;
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < AK; ++j) ar[j] = ka + j < D ? aptr[ka + j] : 0.0f;
+        }
+#pragma unroll
+        for (int q = 0; q < XV; ++q) {
+            const int e = tid + q * kResidThreads, k = k0 + e / (BN / 4);
+            xr[q] = k < D ? *reinterpret_cast<const float4*>(x + (size_t)k * ldx + i0 + 4 * (e % (BN / 4)))
+                          : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    auto stage = [&](int st) {
+#pragma unroll
+        for (int j = 0; j < AK; ++j) As[st][ak + j][arow] = (T)ar[j];
+#pragma unroll
+        for (int q = 0; q < XV; ++q) {
+            const int e = tid + q * kResidThreads;
+            const T v[4] = {(T)xr[q].x, (T)xr[q].y, (T)xr[q].z, (T)xr[q].w};
+            st4g(&Xs[st][e / (BN / 4)][4 * (e % (BN / 4))], v);
+        }
+    };
+    // the thread's rows ty * 4 + j (+ BM / 2) and particles tx * 4 + j (+ BN / 2)
+    auto row_of = [&](int a) { return (a / 4) * (BM / 2) + ty * 4 + a % 4; };
+    Acc<T, TM, TN> acc;
+#pragma unroll
+    for (int a = 0; a < TM; ++a) {
+        const int m = mt + row_of(a);
+        acc.set(a, m < m1 ? -(T)b[m] : (T)0);
+    }
+    fetch(0);
+    stage(0);
+    __syncthreads();
+    const int slices = (D + kBk - 1) / kBk;
+    for (int s = 0; s < slices; ++s) {
+        const int st = s & 1;
+        if (s + 1 < slices) fetch((s + 1) * kBk);
+#pragma unroll
+        for (int k = 0; k < kBk; ++k) {
+            T av[TM], xv[TN];
+#pragma unroll
+            for (int a = 0; a < TM; a += 4) ld4s(&As[st][k][(a / 4) * (BM / 2) + ty * 4], av + a);
+#pragma unroll
+            for (int c = 0; c < TN; c += 4) ld4s(&Xs[st][k][(c / 4) * (BN / 2) + tx * 4], xv + c);
+            acc.step(av, xv);
+        }
+        if (s + 1 < slices) stage(st ^ 1);   // the other stage: read last before the previous barrier
+        __syncthreads();
+    }
+#pragma unroll
+    for (int a = 0; a < TM; ++a) {
+        const int m = mt + row_of(a);
+        if (m >= m1) continue;
+        T* row = R + (size_t)(m - m0) * (size_t)ldr + i0;
+#pragma unroll
+        for (int c = 0; c < TN; c += 4) {
+            T v[4] = {acc.get(a, c), acc.get(a, c + 1), acc.get(a, c + 2), acc.get(a, c + 3)};
+            if constexpr (sizeof(T) == 8) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = __dmul_rn(v[e], v[e]);
+            }
+            st4g(row + (c / 4) * (BN / 2) + tx * 4, v);
+        }
+    }
+}
+
+// carry[i] (+)= the squares of R[0 .. rows - 1][i] (FP64: R itself) in row order; the last chunk
+// rounds the sum into f[i]. A block takes 32 particles: all its threads copy the
+// rows into a ring of kSumStages shared stages ahead of warp 0, which adds one
+// particle per lane -- a dependent chain of `rows` operations that no split can
+// shorten, so only the loads are taken off it.
+template <typename T>
+__global__ void __launch_bounds__(kSumThreads) lsq_sumsq_kernel(const T* __restrict__ R, int ldr, int rows, int N,
+                                                                T* __restrict__ carry, int first, int last,
+                                                                float* __restrict__ f) {
+    constexpr int kRows = kSumStageBytes / (32 * (int)sizeof(T));   // rows per stage
+    constexpr int kVec = 16 / (int)sizeof(T);
+    constexpr int kCopies = kSumStageBytes / 16 / kSumThreads;
+    __shared__ __align__(16) T ring[kSumStages][kRows][32];
+    const int tid = threadIdx.x, i0 = blockIdx.x * 32, i = i0 + tid;
+    const int stages = (rows + kRows - 1) / kRows;
+    auto issue = [&](int st) {
+        if (st < stages) {
+#pragma unroll
+            for (int q = 0; q < kCopies; ++q) {
+                const int e = tid + q * kSumThreads, rr = e / (32 / kVec), col = (e % (32 / kVec)) * kVec;
+                const int row = st * kRows + rr;
+                if (row < rows) {
+                    const unsigned sa = (unsigned)__cvta_generic_to_shared(&ring[st % kSumStages][rr][col]);
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa),
+                                 "l"(R + (size_t)row * (size_t)ldr + i0 + col)
+                                 : "memory");
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    T acc = (T)0;
+    if (tid < 32 && !first && i < N) acc = carry[i];
+#pragma unroll
+    for (int st = 0; st < kSumStages - 1; ++st) issue(st);
+    for (int st = 0; st < stages; ++st) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(kSumStages - 2) : "memory");
+        __syncthreads();   // every thread's copies of stage st have landed; stage st - 1 is read
+        issue(st + kSumStages - 1);
+        if (tid < 32) {
+            const int n = min(kRows, rows - st * kRows);
+            const T(*row)[32] = ring[st % kSumStages];
+#pragma unroll 16
+            for (int rr = 0; rr < n; ++rr) {
+                const T v = row[rr][tid];
+                if constexpr (sizeof(T) == 8) acc = __dadd_rn(acc, v);
+                else acc = __fmaf_rn(v, v, acc);
+            }
+        }
+    }
+    if (tid < 32 && i < N) {
+        if (!last) carry[i] = acc;
+        else if constexpr (sizeof(T) == 8) f[i] = __double2float_rn(acc);
+        else f[i] = acc;
+    }
+}
+
+namespace {
+
+size_t align256(size_t n) { return (n + 255) / 256 * 256; }
+
+// The workspace's particles (a multiple of 128) and rows (of kRowTile) for N
+// particles and M rows: everything when it fits, else fewer rows, and fewer
+// particles only when one row tile of all of them does not fit.
+struct ExactChunk {
+    int particles, rows;
+};
+ExactChunk exact_chunk(int N, int M, size_t esz) {
+    const long long Np = ((long long)N + 127) / 128 * 128;
+    const long long most = (long long)(kExactWsBytes / (esz * kRowTile));   // 131072 or 65536 particles
+    const long long pc = std::min(Np, most);
+    const long long all = ((long long)M + kRowTile - 1) / kRowTile * kRowTile;
+    const long long fit = (long long)(kExactWsBytes / ((size_t)pc * esz)) / kRowTile * kRowTile;
+    return ExactChunk{(int)pc, (int)std::min(all, fit)};
+}
+
+template <typename T, int TM, int TN>
+void launch_resid(const float* x, int ldx, int Np, int D, const float* A, const float* b, int m0, int m1, T* R,
+                  cudaStream_t st) {
+    const int vecA = D % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
+    const dim3 grid((unsigned)(Np / (8 * TN)), (unsigned)((m1 - m0 + 16 * TM - 1) / (16 * TM)));
+    lsq_resid_kernel<T, TM, TN><<<grid, kResidThreads, 0, st>>>(x, ldx, D, A, b, m0, m1, R, Np, vecA);
+}
+
+template <typename T>
+cudaError_t exact_launch(const float* x, int ldx, int N, int D, const float* A, const float* b, int M, float* f,
+                         void* ws, int num_sms, cudaStream_t st) {
+    if (ldx % 128 != 0 || ldx < N || (reinterpret_cast<uintptr_t>(x) & 15u) != 0 || !ws) return cudaErrorInvalidValue;
+    const ExactChunk ch = exact_chunk(N, M, sizeof(T));
+    T* carry = static_cast<T*>(ws);
+    T* R = reinterpret_cast<T*>(static_cast<char*>(ws) + align256(sizeof(T) * (size_t)ch.particles));
+    for (int p0 = 0; p0 < N; p0 += ch.particles) {
+        const int n = std::min(ch.particles, N - p0), np = (n + 127) / 128 * 128;
+        for (int m0 = 0; m0 < M; m0 += ch.rows) {
+            const int m1 = m0 + std::min(ch.rows, M - m0);
+            if constexpr (sizeof(T) == 8) {
+                launch_resid<T, 4, 4>(x + p0, ldx, np, D, A, b, m0, m1, R, st);
+            } else {
+                // 128 x 64 tiles once they cover half the SMs (1024 x 1024 x 1024, 128 of them:
+                // 70 us against 97 with 64 x 32 tiles), the small ones below (1024 x 64 x 512,
+                // 64 large tiles: 6.3 us against 8.3)
+                const long long big = (long long)(np / 64) * ((m1 - m0 + 127) / 128);
+                if (2 * big >= num_sms) launch_resid<T, 8, 8>(x + p0, ldx, np, D, A, b, m0, m1, R, st);
+                else launch_resid<T, 4, 4>(x + p0, ldx, np, D, A, b, m0, m1, R, st);
+            }
+            lsq_sumsq_kernel<T><<<(n + 31) / 32, kSumThreads, 0, st>>>(R, np, m1 - m0, n, carry, m0 == 0, m1 == M, f + p0);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+            if (m1 == M) break;
+        }
+    }
+    return cudaSuccess;
+}
+
+}  // namespace
+
+size_t lsq_exact_ws_bytes(int N, int M, bool fp64) {
+    const size_t esz = fp64 ? 8 : 4;
+    const ExactChunk ch = exact_chunk(N, M, esz);
+    return align256(esz * (size_t)ch.particles) + esz * (size_t)ch.particles * (size_t)ch.rows;
+}
+
+cudaError_t lsq_exact_launch(const float* x, int ldx, int N, int D, const float* A, const float* b, int M, bool fp64,
+                             float* f, void* ws, int num_sms, cudaStream_t st) {
+    return fp64 ? exact_launch<double>(x, ldx, N, D, A, b, M, f, ws, num_sms, st)
+                : exact_launch<float>(x, ldx, N, D, A, b, M, f, ws, num_sms, st);
+}
+
+}  // namespace cupso

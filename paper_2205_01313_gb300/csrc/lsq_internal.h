@@ -65,12 +65,12 @@ int lsq_eval_tc_operand(LsqTcState* st, int N, float* f, cudaStream_t stream);
 // st->part[k][i] (f[i] = their sum in k order).
 int lsq_eval_tc_partials(LsqTcState* st, cudaStream_t stream);
 
-// f[i] = plain FP32 fitness of X(i, d) = x[d * ldx + i], i < N.
-cudaError_t lsq_fp32_launch(const float* x, int ldx, int N, int D, const float* A, const float* b, int M, float* f,
-                            cudaStream_t st);
-// f[i] = FP64 fitness of the same positions in the reference order, rounded to float.
-cudaError_t lsq_fp64_launch(const float* x, int ldx, int N, int D, const float* A, const float* b, int M, float* f,
-                            cudaStream_t st);
+// The exact fitness (kernels_lsq_exact.cu): f[i] of X(i, d) = x[d * ldx + i],
+// i < N, in the reference order, FP32 or FP64 rounded to float. x 16-byte
+// aligned, ldx a multiple of 128; ws: lsq_exact_ws_bytes device bytes.
+size_t lsq_exact_ws_bytes(int N, int M, bool fp64);
+cudaError_t lsq_exact_launch(const float* x, int ldx, int N, int D, const float* A, const float* b, int M, bool fp64,
+                             float* f, void* ws, int num_sms, cudaStream_t st);
 
 // Least-squares swarm iteration (kernels_lsq_swarm.cu); all read t from t_dev.
 cudaError_t lsq_launch_move(const SwarmDev& s, int grid, cudaStream_t st);
