@@ -1198,7 +1198,8 @@ int cupso_set_lsq(cupso_handle h, const float* A_dev, const float* b_dev, int M,
         // are at most max_pos - min_pos in magnitude
         const float span = h->dev.hi - h->dev.lo;
         const float sx = std::isfinite(span) && span > 0.0f ? 448.0f / span : 1.0f;
-        rc = lsq_setup_tc(&L->tc, A_dev, b_dev, M, h->D, h->Np, precision == CUPSO_LSQ_FP8, sx, h->stream);
+        rc = lsq_setup_tc(&L->tc, A_dev, b_dev, M, h->D, h->Np, precision == CUPSO_LSQ_FP8, sx, nullptr, 0,
+                          h->stream);
         if (rc) return rc;
         if (!lsq_make_move_maps(L->tc.tmMove, h->dev.x, h->dev.v, h->dev.pb, h->Np, h->D))
             return fail(CUPSO_ERR_UNSUPPORTED, "tensor maps of the move could not be encoded%s");

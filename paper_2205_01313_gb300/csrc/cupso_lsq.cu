@@ -1,10 +1,11 @@
 // cupso_lsq.cu -- host side of the least-squares fitness.
+#include <cuda_bf16.h>
+#include <cuda_fp8.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
-#include <vector>
 
 #include "../../include/cupso.h"
 #include "cupso_device.cuh"
@@ -17,51 +18,117 @@ namespace {
 
 size_t up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// A in the tensor-core operand format ([Mp][Kp], zero rows and columns past
-// M, D), per-row FP8 scales folded into inv_scale (m) = 1 / (sx * sa_m).
-__global__ void row_absmax_kernel(const float* __restrict__ A, int M, int D, float* __restrict__ amax) {
-    const int m = blockIdx.x;
+// Largest magnitude in x[0 .. n - 1] as the bits of a float (0 before the first
+// launch; non-negative floats order as their bits, NaN is skipped).
+__global__ void __launch_bounds__(256) absmax_kernel(const float* __restrict__ x, size_t n, int vec,
+                                                     unsigned int* __restrict__ out) {
     float v = 0.0f;
-    for (int d = threadIdx.x; d < D; d += blockDim.x) v = fmaxf(v, fabsf(A[(size_t)m * D + d]));
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
-    __shared__ float red[32];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float w = 0.0f;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) w = fmaxf(w, red[k]);
-        amax[m] = w;
+    const size_t stride = (size_t)gridDim.x * blockDim.x, t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    size_t done = 0;
+    if (vec) {
+        const float4* x4 = reinterpret_cast<const float4*>(x);
+        const size_t n4 = n / 4;
+#pragma unroll 4
+        for (size_t e = t; e < n4; e += stride) {
+            const float4 q = x4[e];
+            v = fmaxf(v, fmaxf(fmaxf(fabsf(q.x), fabsf(q.y)), fmaxf(fabsf(q.z), fabsf(q.w))));
+        }
+        done = 4 * n4;
     }
+    for (size_t e = done + t; e < n; e += stride) v = fmaxf(v, fabsf(x[e]));
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(v));
 }
 
-// Scale each row of A in place into a scratch copy: As[m][d] = A[m][d] * sa_m,
-// with sa_m = 448 / amax_m (1 for an all-zero row); inv[m] = 1 / (sx * sa_m).
-__global__ void scale_rows_kernel(const float* __restrict__ A, int M, int D, const float* __restrict__ amax, float sx,
-                                  float* __restrict__ As, float* __restrict__ inv, int Mp) {
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < (size_t)M * D; e += (size_t)gridDim.x * blockDim.x) {
-        const int m = (int)(e / D);
-        const float sa = amax[m] > 0.0f ? 448.0f / amax[m] : 1.0f;
-        As[e] = A[e] * sa;
-    }
-    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < Mp; m += gridDim.x * blockDim.x) {
-        if (m < M) {
-            const float sa = amax[m] > 0.0f ? 448.0f / amax[m] : 1.0f;
-            inv[m] = 1.0f / (sx * sa);
+// The FP8 scale that brings a largest magnitude to the e4m3 limit.
+__device__ __forceinline__ float fp8_scale(float amax) { return amax > 0.0f ? 448.0f / amax : 1.0f; }
+
+// Both operands of the product from row-major sources, one warp per row:
+//  * rows 0 .. Mp - 1 of A: as BF16, or scaled by the row's own factor and
+//    rounded to FP8 e4m3 (448 / its largest magnitude; the row is read twice, the
+//    second time from L1), with inv[m] = 1 / (sx * that factor), 0 past M; and
+//    negb[m] = roff[m] = -b[m], 0 past M (negation is exact, so y + negb[m]
+//    rounds exactly as y - b[m]; roff starts at reference point 0);
+//  * with X: rows 0 .. Np - 1 of X, as BF16 or X * sx in FP8.
+// Zero past the last row and past D. sx: from *xmax (absmax_kernel) when given.
+// One pass over either source in one launch; before, A took three (largest
+// magnitudes, a scaled FP32 copy, the conversion) and X one of its own: 4000 x
+// 1000 and 8192 x 1000 in FP8 46 us for the four, 48 us with the offsets.
+struct OperandArgs {
+    const float *A, *b, *X;
+    int M, Mp, N, Np, D, Kp, vecA, vecX;
+    float sx;
+    const unsigned int* xmax;
+    float *inv, *negb, *roff;
+    void *Aq, *Xq;
+};
+
+template <bool FP8>
+__device__ __forceinline__ void convert_row(const float* __restrict__ src, int D, int Kp, bool vec, float scale, int lane,
+                                            char* __restrict__ dst) {
+#pragma unroll 4
+    for (int k = 4 * lane; k < Kp; k += 128) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (src) {
+            if (vec) {
+                if (k < D) v = *reinterpret_cast<const float4*>(src + k);
+            } else {
+                if (k + 0 < D) v.x = src[k + 0];
+                if (k + 1 < D) v.y = src[k + 1];
+                if (k + 2 < D) v.z = src[k + 2];
+                if (k + 3 < D) v.w = src[k + 3];
+            }
+        }
+        if constexpr (FP8) {
+            const __nv_fp8x4_e4m3 q(make_float4(v.x * scale, v.y * scale, v.z * scale, v.w * scale));
+            *reinterpret_cast<uint32_t*>(dst + k) = q.__x;
         } else {
-            inv[m] = 0.0f;
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+            *reinterpret_cast<uint2*>(dst + 2 * (size_t)k) =
+                make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
         }
     }
 }
 
-// negb[m] = -b[m] for m < M, 0 up to Mp (negation is exact, so y + negb[m]
-// rounds exactly as y - b[m]); roff starts as the same offsets (reference
-// point 0) until the swarm sets its own.
-__global__ void neg_pad_kernel(const float* __restrict__ b, int M, int Mp, float* __restrict__ negb,
-                               float* __restrict__ roff) {
-    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < Mp; m += gridDim.x * blockDim.x) {
-        const float v = m < M ? -b[m] : 0.0f;
-        negb[m] = v;
-        roff[m] = v;
+template <bool FP8>
+__global__ void __launch_bounds__(256) operands_kernel(const OperandArgs p) {
+    constexpr size_t esz = FP8 ? 1 : 2;
+    const int lane = threadIdx.x & 31;
+    const long long rows = (long long)p.Mp + (p.X ? p.Np : 0);
+    const float sx = !FP8 ? 1.0f : (p.xmax ? fp8_scale(__uint_as_float(*p.xmax)) : p.sx);
+    for (long long r = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += (long long)gridDim.x * 8) {
+        if (r < p.Mp) {
+            const int m = (int)r;
+            const float* src = m < p.M ? p.A + (size_t)m * p.D : nullptr;
+            float sa = 1.0f;
+            if constexpr (FP8) {
+                float v = 0.0f;
+                if (src) {
+                    if (p.vecA) {
+#pragma unroll 4
+                        for (int k = 4 * lane; k < p.D; k += 128) {
+                            const float4 q = *reinterpret_cast<const float4*>(src + k);
+                            v = fmaxf(v, fmaxf(fmaxf(fabsf(q.x), fabsf(q.y)), fmaxf(fabsf(q.z), fabsf(q.w))));
+                        }
+                    } else {
+                        for (int k = lane; k < p.D; k += 32) v = fmaxf(v, fabsf(src[k]));
+                    }
+                }
+                for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
+                sa = fp8_scale(v);
+            }
+            if (lane == 0) {
+                const float nb = src ? -p.b[m] : 0.0f;
+                p.negb[m] = nb;
+                p.roff[m] = nb;
+                if constexpr (FP8) p.inv[m] = src ? 1.0f / (sx * sa) : 0.0f;
+            }
+            convert_row<FP8>(src, p.D, p.Kp, p.vecA, sa, lane, static_cast<char*>(p.Aq) + (size_t)m * p.Kp * esz);
+        } else {
+            const int i = (int)(r - p.Mp);
+            convert_row<FP8>(i < p.N ? p.X + (size_t)i * p.D : nullptr, p.D, p.Kp, p.vecX, sx, lane,
+                             static_cast<char*>(p.Xq) + (size_t)i * p.Kp * esz);
+        }
     }
 }
 
@@ -80,10 +147,18 @@ __global__ void transpose_kernel(const float* __restrict__ in, int N, int D, siz
     }
 }
 
+// f[i] = part[0][i] + part[1][i] + ... in that order, 16 loads in flight.
 __global__ void sum_parts_kernel(const float* __restrict__ part, int nparts, int Np, int N, float* __restrict__ f) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
         float s = 0.0f;
-        for (int k = 0; k < nparts; ++k) s = __fadd_rn(s, part[(size_t)k * Np + i]);
+        for (int k0 = 0; k0 < nparts; k0 += 16) {
+            float v[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] = k0 + e < nparts ? part[(size_t)(k0 + e) * Np + i] : 0.0f;
+#pragma unroll
+            for (int e = 0; e < 16; ++e)
+                if (k0 + e < nparts) s = __fadd_rn(s, v[e]);
+        }
         f[i] = s;
     }
 }
@@ -91,9 +166,11 @@ __global__ void sum_parts_kernel(const float* __restrict__ part, int nparts, int
 }  // namespace
 
 // Everything the tensor-core fitness needs for fixed A, b: operand copies,
-// scales, padded b, and the TMA descriptors (built for a given X buffer).
+// scales, padded b, and the TMA descriptors (built for a given X buffer). With
+// X (row-major [N][D]) its operand as well, for an evaluation of given
+// positions; the FP8 scale of X is then that of its largest magnitude.
 int cupso::lsq_setup_tc(LsqTcState* st, const float* A, const float* b, int M, int D, int Np, bool fp8, float sx,
-                        cudaStream_t stream) {
+                        const float* X, int N, cudaStream_t stream) {
     st->fp8 = fp8;
     st->M = M;
     st->D = D;
@@ -105,8 +182,7 @@ int cupso::lsq_setup_tc(LsqTcState* st, const float* A, const float* b, int M, i
     const size_t bytes_A = (size_t)st->Mp * st->Kp * esz, bytes_X = (size_t)Np * st->Kp * esz;
     const size_t nparts = (size_t)st->Mp / 128;   // one partial sum per 128 residual rows
     const size_t bytes = up(bytes_A, 256) + up(bytes_X, 256) + up(sizeof(float) * st->Mp, 256) * 3 +
-                         up(sizeof(float) * nparts * Np, 256) + up(sizeof(float) * (size_t)M * D, 256) +
-                         up(sizeof(float) * M, 256) + 512;
+                         up(sizeof(float) * nparts * Np, 256) + 512;
     cudaError_t e = cudaMalloc(&st->arena, bytes);
     if (e != cudaSuccess) return set_cuda_error(e, "cudaMalloc (lsq)"), e == cudaErrorMemoryAllocation ? CUPSO_ERR_OOM : CUPSO_ERR_CUDA;
     char* p = static_cast<char*>(st->arena);
@@ -116,27 +192,30 @@ int cupso::lsq_setup_tc(LsqTcState* st, const float* A, const float* b, int M, i
     st->roff = reinterpret_cast<float*>(p); p += up(sizeof(float) * st->Mp, 256);
     st->inv = reinterpret_cast<float*>(p); p += up(sizeof(float) * st->Mp, 256);
     st->part = reinterpret_cast<float*>(p); p += up(sizeof(float) * nparts * Np, 256);
-    float* Ascaled = reinterpret_cast<float*>(p); p += up(sizeof(float) * (size_t)M * D, 256);
-    float* amax = reinterpret_cast<float*>(p); p += up(sizeof(float) * M, 256);
     st->status = reinterpret_cast<unsigned int*>(p); p += 256;
     st->roff_stale = reinterpret_cast<int*>(p);
+    unsigned int* xmax = st->status + 1;
     e = cudaMemsetAsync(st->status, 0, 512, stream);
     if (e == cudaSuccess) e = lsq_prepare();
     if (e != cudaSuccess) return set_cuda_error(e, "lsq setup"), CUPSO_ERR_CUDA;
-    neg_pad_kernel<<<(st->Mp + 255) / 256, 256, 0, stream>>>(b, M, st->Mp, st->negb, st->roff);
-    const float* Asrc = A;
-    if (fp8) {
-        row_absmax_kernel<<<M, 256, 0, stream>>>(A, M, D, amax);
-        scale_rows_kernel<<<1024, 256, 0, stream>>>(A, M, D, amax, st->sx, Ascaled, st->inv, st->Mp);
-        Asrc = Ascaled;
-    }
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = lsq_convert(Asrc, (size_t)D, 1, M, D, st->Mp, st->Kp, fp8, 1.0f, st->Aq, stream);
-    if (e != cudaSuccess) return set_cuda_error(e, "lsq operand A"), CUPSO_ERR_CUDA;
     if (!lsq_tc_plan(&st->plan, st->Xq, st->Aq, fp8, Np, st->Mp, st->Kp)) {
         set_last_error("cuTensorMapEncodeTiled unavailable or rejected the operand layout");
         return CUPSO_ERR_UNSUPPORTED;
     }
+    auto vec = [&](const float* q) { return D % 4 == 0 && (reinterpret_cast<uintptr_t>(q) & 15u) == 0; };
+    if (fp8 && X) {
+        const size_t n = (size_t)N * D;
+        const int grid = (int)std::max<size_t>(1, std::min<size_t>((n + 4095) / 4096, 1216));
+        absmax_kernel<<<grid, 256, 0, stream>>>(X, n, (reinterpret_cast<uintptr_t>(X) & 15u) == 0, xmax);
+    }
+    const OperandArgs args{A, b, X, M, st->Mp, N, Np, D, st->Kp, vec(A), vec(X), st->sx, fp8 && X ? xmax : nullptr,
+                           st->inv, st->negb, st->roff, st->Aq, st->Xq};
+    const long long rows = (long long)st->Mp + (X ? Np : 0);
+    const int grid = (int)std::min<long long>((rows + 7) / 8, 1 << 16);
+    if (fp8) operands_kernel<true><<<grid, 256, 0, stream>>>(args);
+    else operands_kernel<false><<<grid, 256, 0, stream>>>(args);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return set_cuda_error(e, "lsq operands"), CUPSO_ERR_CUDA;
     return CUPSO_OK;
 }
 
@@ -206,22 +285,13 @@ extern "C" int cupso_lsq_eval(const float* A_dev, const float* b_dev, int M, int
     }
     LsqTcState s{};
     const int Np = (N + 127) / 128 * 128;
-    const bool fp8 = precision == CUPSO_LSQ_FP8;
-    float xmax = 0.0f;
-    {
-        // FP8 scale of X from its largest magnitude
-        std::vector<float> h((size_t)N * D);
-        cudaError_t e = cudaMemcpyAsync(h.data(), X_dev, sizeof(float) * h.size(), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return set_cuda_error(e, "cudaMemcpy"), CUPSO_ERR_CUDA;
-        for (float v : h) xmax = std::max(xmax, std::fabs(v));
-    }
-    const float sx = xmax > 0.0f ? 448.0f / xmax : 1.0f;
-    int rc = lsq_setup_tc(&s, A_dev, b_dev, M, D, Np, fp8, sx, st);
-    if (rc == CUPSO_OK) rc = lsq_eval_tc(&s, X_dev, (size_t)D, 1, N, f_out_dev, st);
-    cudaError_t e = cudaStreamSynchronize(st);
+    int rc = lsq_setup_tc(&s, A_dev, b_dev, M, D, Np, precision == CUPSO_LSQ_FP8, 1.0f, X_dev, N, st);
+    if (rc == CUPSO_OK) rc = lsq_eval_tc_operand(&s, N, f_out_dev, st);
     unsigned int status = 0;
-    if (e == cudaSuccess && s.status) e = cudaMemcpy(&status, s.status, sizeof(unsigned), cudaMemcpyDeviceToHost);
+    cudaError_t e = cudaSuccess;
+    if (rc == CUPSO_OK) e = cudaMemcpyAsync(&status, s.status, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
+    const cudaError_t es = cudaStreamSynchronize(st);
+    if (e == cudaSuccess) e = es;
     lsq_free_tc(&s);
     if (rc != CUPSO_OK) return rc;
     if (e != cudaSuccess) return set_cuda_error(e, "lsq eval"), CUPSO_ERR_CUDA;

@@ -53,8 +53,10 @@ struct LsqTcState {
     // 64 particles x 64 dimensions) for the TMA-fed move (lsq_make_move_maps)
     alignas(64) unsigned char tmMove[3][128];
 };
+// X (may be null): row-major [N][D] positions whose operand is formed too, with
+// the FP8 scale from their largest magnitude in place of sx.
 int lsq_setup_tc(LsqTcState* st, const float* A, const float* b, int M, int D, int Np, bool fp8, float sx,
-                 cudaStream_t stream);
+                 const float* X, int N, cudaStream_t stream);
 void lsq_free_tc(LsqTcState* st);
 // f[i] for positions X(i, k) = src[i * si + k * sk], i < N (asynchronous).
 int lsq_eval_tc(LsqTcState* st, const float* src, size_t si, size_t sk, int N, float* f, cudaStream_t stream);
