@@ -15,7 +15,7 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libcupso.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
-SOURCES = ["cupso_api.cu", "cupso_batch.cu", "cupso_lsq.cu", "kernels_stream.cu", "kernels_pipelined.cu",
+SOURCES = ["cupso_api.cu", "cupso_batch.cu", "cupso_lsq.cu", "kernels_state.cu", "kernels_stream.cu", "kernels_pipelined.cu",
            "kernels_batch.cu", "kernels_lsq.cu", "kernels_lsq_exact.cu", "kernels_lsq_swarm.cu", "kernels_onchip.cu",
            "kernels_paper.cu", "kernels_tiled.cu", "kernels_panel.cu", "cupso_noalloc.cu"]
 HEADERS = ["cupso_device.cuh", "cupso_internal.h", "stream_common.cuh", "paper_kernels.h", "tiled_kernels.h",

@@ -108,6 +108,10 @@ struct cupso_swarm {
         int fitness_timed = 0;
     };
     Lsq* lsq = nullptr;
+    // staged rows of get_state / set_state (allocated on first use, at most
+    // kStageBytes unless one particle's row is larger)
+    void* stage = nullptr;
+    size_t stage_bytes = 0;
     // pinned host staging of the gbest reads (allocated on first use)
     void* pinned = nullptr;
     size_t pinned_bytes = 0;
@@ -731,6 +735,78 @@ int ensure_pinned(cupso_swarm* h, size_t bytes) {
     return CUPSO_OK;
 }
 
+// The staging buffer for rows of `row` bytes, N of them: all at once, or chunks
+// of up to kStageBytes; fewer when memory is short, down to one row.
+constexpr size_t kStageBytes = 32u << 20;
+int ensure_stage(cupso_swarm* h, size_t row, size_t N) {
+    const size_t least = row;
+    if (h->stage_bytes >= std::min(row * N, std::max(least, kStageBytes))) return CUPSO_OK;
+    if (h->stage) cudaFree(h->stage);
+    h->stage = nullptr;
+    h->stage_bytes = 0;
+    size_t want = std::min(row * N, std::max(least, kStageBytes));
+    cudaError_t e;
+    while ((e = cudaMalloc(&h->stage, want)) == cudaErrorMemoryAllocation && want > least) {
+        cudaGetLastError();
+        want = std::max(least, want / 4);
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        h->stage = nullptr;
+        return cuda_fail(e, "cudaMalloc (state staging)");
+    }
+    h->stage_bytes = want;
+    return CUPSO_OK;
+}
+
+// out[i][d], i < N, from a device array in `panel` layout; queued on the
+// handle's stream (the caller waits).
+template <typename T>
+int download_rows(cupso_swarm* h, const T* src, int panel, T* out) {
+    const size_t D = (size_t)h->D, row = sizeof(T) * D;
+    if (D == 1) {   // one row either way
+        CUPSO_CUDA(cudaMemcpyAsync(out, src, sizeof(T) * (size_t)h->N, cudaMemcpyDeviceToHost, h->stream), "cudaMemcpyAsync");
+        return CUPSO_OK;
+    }
+    const int rc = ensure_stage(h, row, (size_t)h->N);
+    if (rc) return rc;
+    const int per = (int)std::min<size_t>((size_t)h->N, h->stage_bytes / row);
+    for (int i0 = 0; i0 < h->N; i0 += per) {
+        const int n = std::min(per, h->N - i0);
+        CUPSO_CUDA(launch_unpack_rows(src, static_cast<T*>(h->stage), h->D, h->Np, panel, i0, n, h->stream), "unpack launch");
+        CUPSO_CUDA(cudaMemcpyAsync(out + (size_t)i0 * D, h->stage, row * (size_t)n, cudaMemcpyDeviceToHost, h->stream),
+                   "cudaMemcpyAsync");
+        if (n == h->N - i0) break;
+    }
+    return CUPSO_OK;
+}
+
+// The reverse: a device array in `panel` layout from in[i][d], zeros in the padding.
+template <typename T>
+int upload_rows(cupso_swarm* h, const T* in, int panel, T* dst) {
+    const size_t D = (size_t)h->D, row = sizeof(T) * D;
+    const int pad = h->Np - h->N;
+    if (D == 1) {
+        CUPSO_CUDA(cudaMemcpyAsync(dst, in, sizeof(T) * (size_t)h->N, cudaMemcpyHostToDevice, h->stream), "cudaMemcpyAsync");
+        CUPSO_CUDA(cudaMemsetAsync(dst + h->N, 0, sizeof(T) * (size_t)pad, h->stream), "cudaMemsetAsync");
+        return CUPSO_OK;
+    }
+    const int rc = ensure_stage(h, row, (size_t)h->N);
+    if (rc) return rc;
+    const int per = (int)std::min<size_t>((size_t)h->N, h->stage_bytes / row);
+    for (int i0 = 0; i0 < h->N; i0 += per) {
+        const int n = std::min(per, h->N - i0);
+        const bool last = n == h->N - i0;
+        CUPSO_CUDA(cudaMemcpyAsync(h->stage, in + (size_t)i0 * D, row * (size_t)n, cudaMemcpyHostToDevice, h->stream),
+                   "cudaMemcpyAsync");
+        CUPSO_CUDA(launch_pack_rows(static_cast<const T*>(h->stage), dst, h->D, h->Np, panel, i0, n, last ? n + pad : n,
+                                    h->stream),
+                   "pack launch");
+        if (last) break;
+    }
+    return CUPSO_OK;
+}
+
 int status_code(unsigned st) {
     if (st & kStatusBadArg) return CUPSO_ERR_CUDA;   // a device-side bound check dropped work
     if (st & kStatusTimeout) return CUPSO_ERR_DEVICE_TIMEOUT;
@@ -1072,28 +1148,19 @@ int cupso_gbest_wait(cupso_handle h, int slot, float* fit_out, float* pos_out, i
 int cupso_get_state(cupso_handle h, float* pos, float* v, float* pbest_pos, float* pbest_fit, uint32_t* t_out) {
     if (!h) return fail(CUPSO_ERR_INVALID_ARG, "handle is NULL%s");
     if (h->fp64) return fail(CUPSO_ERR_UNSUPPORTED, "double-precision swarm: use the _fp64 functions%s");
-    const size_t N = (size_t)h->N, D = (size_t)h->D, Np = (size_t)h->Np;
-    std::vector<float> stage;
-    float* outs[3] = {pos, v, pbest_pos};
-    const float* srcs[3] = {h->dev.x, h->dev.v, h->dev.pb};
     const int mrc = ensure_materialized(h);
     if (mrc) return mrc;
-    CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    float* outs[3] = {pos, v, pbest_pos};
+    const float* srcs[3] = {h->dev.x, h->dev.v, h->dev.pb};
     for (int a = 0; a < 3; ++a) {
         if (!outs[a]) continue;
-        stage.resize(D * Np);
-        CUPSO_CUDA(cudaMemcpy(stage.data(), srcs[a], sizeof(float) * D * Np, cudaMemcpyDeviceToHost), "cudaMemcpy");
-        if (h->panel) {   // element (d, i) at ((d / W) Np + i) W + d % W
-            const size_t W = (size_t)h->panel;
-            for (size_t i = 0; i < N; ++i)
-                for (size_t d = 0; d < D; ++d) outs[a][i * D + d] = stage[((d / W) * Np + i) * W + (d % W)];
-        } else {
-            for (size_t i = 0; i < N; ++i)
-                for (size_t d = 0; d < D; ++d) outs[a][i * D + d] = stage[d * Np + i];
-        }
+        const int rc = download_rows(h, srcs[a], h->panel, outs[a]);
+        if (rc) return rc;
     }
     if (pbest_fit)
-        CUPSO_CUDA(cudaMemcpy(pbest_fit, h->dev.pf, sizeof(float) * N, cudaMemcpyDeviceToHost), "cudaMemcpy");
+        CUPSO_CUDA(cudaMemcpyAsync(pbest_fit, h->dev.pf, sizeof(float) * (size_t)h->N, cudaMemcpyDeviceToHost, h->stream),
+                   "cudaMemcpyAsync");
+    CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
     if (t_out) *t_out = h->t_host;
     return CUPSO_OK;
 }
@@ -1103,27 +1170,26 @@ int cupso_set_state(cupso_handle h, const float* pos, const float* v, const floa
     if (!h) return fail(CUPSO_ERR_INVALID_ARG, "handle is NULL%s");
     if (h->fp64) return fail(CUPSO_ERR_UNSUPPORTED, "double-precision swarm: use the _fp64 functions%s");
     if (!pos || !v || !pbest_pos || !pbest_fit) return fail(CUPSO_ERR_INVALID_ARG, "state array is NULL%s");
-    const size_t N = (size_t)h->N, D = (size_t)h->D, Np = (size_t)h->Np;
     CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
-    std::vector<float> stage(D * Np, 0.0f);
+    // straight into the layout that the next step reads
+    const int panel = resolved_mode(h) == CUPSO_MODE_SYNC ? panel_cfg(h).width : 0;
     const float* ins[3] = {pos, v, pbest_pos};
     float* dsts[3] = {h->dev.x, h->dev.v, h->dev.pb};
     for (int a = 0; a < 3; ++a) {
-        for (size_t i = 0; i < N; ++i)
-            for (size_t d = 0; d < D; ++d) stage[d * Np + i] = ins[a][i * D + d];
-        CUPSO_CUDA(cudaMemcpy(dsts[a], stage.data(), sizeof(float) * D * Np, cudaMemcpyHostToDevice), "cudaMemcpy");
+        const int rc = upload_rows(h, ins[a], panel, dsts[a]);
+        if (rc) return rc;
     }
-    std::vector<float> pf(Np, INFINITY);
-    std::memcpy(pf.data(), pbest_fit, sizeof(float) * N);
-    CUPSO_CUDA(cudaMemcpy(h->dev.pf, pf.data(), sizeof(float) * Np, cudaMemcpyHostToDevice), "cudaMemcpy");
-    CUPSO_CUDA(cudaMemset(h->dev.pflag, 0, Np), "cudaMemset");
+    CUPSO_CUDA(cudaMemcpyAsync(h->dev.pf, pbest_fit, sizeof(float) * (size_t)h->N, cudaMemcpyHostToDevice, h->stream),
+               "cudaMemcpyAsync");
+    CUPSO_CUDA(cudaMemsetAsync(h->dev.pflag, 0, (size_t)h->Np, h->stream), "cudaMemsetAsync");
     h->lazy_pending = false;
-    h->panel = 0;   // uploaded dimension-major
+    if (h->panel != panel) drop_graph(h);
+    h->panel = panel;
     if (h->lsq && lsq_approx(h->lsq->precision)) {
         // the given pbest_fit are approximate values: gbest only from the rescoring
         CUPSO_CUDA(lsq_reset_gbest(h, h->dev.pf, t, h->stream), "lsq gbest");
     } else {
-        CUPSO_CUDA(launch_recompute(h->dev, t, h->stream), "recompute launch");
+        CUPSO_CUDA(launch_recompute(h->dev, t, panel, true, h->stream), "recompute launch");
     }
     CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
     h->t_host = t;
@@ -1231,7 +1297,7 @@ int cupso_set_lsq(cupso_handle h, const float* A_dev, const float* b_dev, int M,
                                     h->num_sms, h->stream),
                    "lsq fitness");
         CUPSO_CUDA(lsq_launch_set_pf(h->dev, L->f, h->stream), "lsq pbest");
-        CUPSO_CUDA(launch_recompute(h->dev, h->t_host, h->stream), "recompute launch");
+        CUPSO_CUDA(launch_recompute(h->dev, h->t_host, 0, false, h->stream), "recompute launch");
     } else {
         // the positions' own fitness (reference point 0: offsets -b)
         rc = lsq_eval_tc(&L->tc, h->dev.pb, 1, (size_t)h->Np, h->N, L->f, h->stream);
@@ -1301,20 +1367,17 @@ int cupso_get_state_fp64(cupso_handle h, double* pos, double* v, double* pbest_p
                          uint32_t* t_out) {
     if (!h) return fail(CUPSO_ERR_INVALID_ARG, "handle is NULL%s");
     if (!h->fp64) return fail(CUPSO_ERR_UNSUPPORTED, "not a double-precision swarm%s");
-    const size_t N = (size_t)h->N, D = (size_t)h->D, Np = (size_t)h->Np;
-    std::vector<double> stage;
     double* outs[3] = {pos, v, pbest_pos};
     const double* srcs[3] = {h->dev64.x, h->dev64.v, h->dev64.pb};
-    CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
     for (int a = 0; a < 3; ++a) {
         if (!outs[a]) continue;
-        stage.resize(D * Np);
-        CUPSO_CUDA(cudaMemcpy(stage.data(), srcs[a], sizeof(double) * D * Np, cudaMemcpyDeviceToHost), "cudaMemcpy");
-        for (size_t i = 0; i < N; ++i)
-            for (size_t d = 0; d < D; ++d) outs[a][i * D + d] = stage[d * Np + i];
+        const int rc = download_rows(h, srcs[a], 0, outs[a]);
+        if (rc) return rc;
     }
     if (pbest_fit)
-        CUPSO_CUDA(cudaMemcpy(pbest_fit, h->dev64.pf, sizeof(double) * N, cudaMemcpyDeviceToHost), "cudaMemcpy");
+        CUPSO_CUDA(cudaMemcpyAsync(pbest_fit, h->dev64.pf, sizeof(double) * (size_t)h->N, cudaMemcpyDeviceToHost, h->stream),
+                   "cudaMemcpyAsync");
+    CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
     if (t_out) *t_out = h->t_host;
     return CUPSO_OK;
 }
@@ -1324,20 +1387,20 @@ int cupso_set_state_fp64(cupso_handle h, const double* pos, const double* v, con
     if (!h) return fail(CUPSO_ERR_INVALID_ARG, "handle is NULL%s");
     if (!h->fp64) return fail(CUPSO_ERR_UNSUPPORTED, "not a double-precision swarm%s");
     if (!pos || !v || !pbest_pos || !pbest_fit) return fail(CUPSO_ERR_INVALID_ARG, "state array is NULL%s");
-    const size_t N = (size_t)h->N, D = (size_t)h->D, Np = (size_t)h->Np;
+    const size_t N = (size_t)h->N;
     CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
-    std::vector<double> stage(D * Np, 0.0);
     const double* ins[3] = {pos, v, pbest_pos};
     double* dsts[3] = {h->dev64.x, h->dev64.v, h->dev64.pb};
     for (int a = 0; a < 3; ++a) {
-        for (size_t i = 0; i < N; ++i)
-            for (size_t d = 0; d < D; ++d) stage[d * Np + i] = ins[a][i * D + d];
-        CUPSO_CUDA(cudaMemcpy(dsts[a], stage.data(), sizeof(double) * D * Np, cudaMemcpyHostToDevice), "cudaMemcpy");
+        const int rc = upload_rows(h, ins[a], 0, dsts[a]);
+        if (rc) return rc;
     }
-    std::vector<double> pf(Np, INFINITY);
-    std::memcpy(pf.data(), pbest_fit, sizeof(double) * N);
-    CUPSO_CUDA(cudaMemcpy(h->dev64.pf, pf.data(), sizeof(double) * Np, cudaMemcpyHostToDevice), "cudaMemcpy");
-    CUPSO_CUDA(cudaMemcpy(h->dev64.t_dev, &t, sizeof(t), cudaMemcpyHostToDevice), "cudaMemcpy");
+    static const std::vector<double> inf((size_t)kPad, (double)INFINITY);   // pbest_fit of the padding
+    CUPSO_CUDA(cudaMemcpyAsync(h->dev64.pf, pbest_fit, sizeof(double) * N, cudaMemcpyHostToDevice, h->stream), "cudaMemcpyAsync");
+    CUPSO_CUDA(cudaMemcpyAsync(h->dev64.pf + N, inf.data(), sizeof(double) * (size_t)(h->Np - h->N), cudaMemcpyHostToDevice,
+                               h->stream),
+               "cudaMemcpyAsync");
+    CUPSO_CUDA(cudaMemcpyAsync(h->dev64.t_dev, &t, sizeof(t), cudaMemcpyHostToDevice, h->stream), "cudaMemcpyAsync");
     CUPSO_CUDA(launch_recompute64(h->dev64, h->pbufs, h->stream), "recompute launch");
     CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
     h->t_host = t;
@@ -1429,6 +1492,7 @@ int cupso_destroy(cupso_handle h) {
     if (h->rec_dev) cudaFree(h->rec_dev);
     if (h->rec_host) cudaFreeHost(h->rec_host);
     if (h->arena) cudaFree(h->arena);
+    if (h->stage) cudaFree(h->stage);
     if (h->pinned) cudaFreeHost(h->pinned);
     if (h->capture) cudaStreamDestroy(h->capture);
     if (h->own) cudaStreamDestroy(h->own);

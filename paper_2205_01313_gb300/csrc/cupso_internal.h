@@ -25,7 +25,18 @@ cudaError_t launch_tree_step(const SwarmDev& s, int fid, bool unrolled, cudaStre
 // tile of 4 * block particles per pass.
 cudaError_t launch_async(const SwarmDev& s, int fid, int grid, int block, uint32_t t_first, int iters,
                          int hold_lock, cudaStream_t st);
-cudaError_t launch_recompute(const SwarmDev& s, uint32_t t, cudaStream_t st);
+
+// The state between particle-major rows and the device layouts (kernels_state.cu).
+// rows: device, [n][D], the particles i0 .. i0 + n - 1 of an array in panels of
+// `panel` (8, 16) or dimension-major (0; doubles always). pack also zeroes
+// particles i0 + n .. i0 + np - 1.
+template <typename T>
+cudaError_t launch_pack_rows(const T* rows, T* dst, int D, int Np, int panel, int i0, int n, int np, cudaStream_t st);
+template <typename T>
+cudaError_t launch_unpack_rows(const T* src, T* rows, int D, int Np, int panel, int i0, int n, cudaStream_t st);
+// gbest from pbest after the host loads a state (pb in `panel` layout), at
+// iteration t; fill_pad: pbest_fit of the padding becomes infinity.
+cudaError_t launch_recompute(const SwarmDev& s, uint32_t t, int panel, bool fill_pad, cudaStream_t st);
 
 // Pipelined fused step (kernels_pipelined.cu): `stages`-deep cp.async ring.
 bool pipelined_supported(int stages, int D);

@@ -21,7 +21,6 @@
 //                       lock-protected global best read under a sequence lock
 //                       (async_common.cuh). Large swarms and D = 1; smaller
 //                       ones run the tiled form (kernels_tiled.cu).
-//  * recompute_kernel   gbest from pbest after the host loads a state.
 #include <cuda_runtime.h>
 
 #include "cupso_device.cuh"
@@ -321,32 +320,6 @@ __global__ void __launch_bounds__(kBlock) async_kernel(const __grid_constant__ S
 }
 
 // ---------------------------------------------------------------------------
-// gbest = lexicographic argmin over (pbest_fit, index), one block.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) recompute_kernel(const __grid_constant__ SwarmDev s, uint32_t t) {
-    __shared__ unsigned long long red[32];
-    unsigned long long k = kKeyNone;
-    bool nan = false;
-    for (int i = threadIdx.x; i < s.N; i += blockDim.x) {
-        const float f = s.pf[i];
-        const unsigned long long kk = pack_key(f, (uint32_t)i);
-        k = kk < k ? kk : k;
-        nan |= (f != f);
-    }
-    k = block_min(k, red);
-    if (__syncthreads_or(nan) && threadIdx.x == 0) atomicOr(s.status, kStatusNaN);
-    const int cur = (int)(t & 1u);
-    const uint32_t g = (uint32_t)(k & 0xFFFFFFFFull);
-    for (int d = threadIdx.x; d < s.D; d += blockDim.x) s.G[(size_t)cur * s.D + d] = s.pb[(size_t)d * s.Np + g];
-    if (threadIdx.x == 0) {
-        s.gkey[0] = k;
-        s.gkey[1] = k;
-        *s.t_dev = t;
-        *s.ticket = 0u;
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Launch wrappers
 // ---------------------------------------------------------------------------
 #define CUPSO_DISPATCH_FIT(fid, KERNEL_CALL)                       \
@@ -400,11 +373,6 @@ cudaError_t launch_async(const SwarmDev& s, int fid, int grid, int block, uint32
     if (e != cudaSuccess) return e;
     const size_t smem = sizeof(float) * (size_t)s.D;
     CUPSO_DISPATCH_FIT(fid, (async_kernel<F><<<grid, block, smem, st>>>(s, t_first, iters)));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_recompute(const SwarmDev& s, uint32_t t, cudaStream_t st) {
-    recompute_kernel<<<1, 1024, 0, st>>>(s, t);
     return cudaGetLastError();
 }
 
