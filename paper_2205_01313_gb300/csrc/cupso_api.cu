@@ -494,6 +494,18 @@ int cupso::check_problem_args(int D, int N, const cupso_bounds* b, float w, floa
     return CUPSO_OK;
 }
 
+// The fast arithmetic path's constants and whether it gives the same bits:
+// c * 2^-24 is exact unless it would be subnormal (checked by scaling back), and
+// the min/max clamps need bounds that are not zero.
+void cupso::set_fast_paths(SwarmDev* s) {
+    s->c1s = std::ldexp(s->c1, -24);
+    s->c2s = std::ldexp(s->c2, -24);
+    s->fast_cr = (std::ldexp(s->c1s, 24) == s->c1 && std::ldexp(s->c2s, 24) == s->c2 &&
+                  (s->c1 == 0.0f || std::fabs(s->c1s) >= FLT_MIN) && (s->c2 == 0.0f || std::fabs(s->c2s) >= FLT_MIN))
+                     ? 1 : 0;
+    s->fast_clamp = (s->lo != 0.0f && s->hi != 0.0f) ? 1 : 0;
+}
+
 namespace {
 
 int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c2, int fid, uint64_t seed,
@@ -578,13 +590,7 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
     s.swarm = swarm;
     s.wait_limit_ns = 2000000000ll;
     h->pbufs = paper_bufs_at(base + o_paper, h->Np, list_cap);
-    // c * 2^-24 is exact unless it would be subnormal; check by scaling back.
-    s.c1s = std::ldexp(c1, -24);
-    s.c2s = std::ldexp(c2, -24);
-    s.fast_cr = (std::ldexp(s.c1s, 24) == c1 && std::ldexp(s.c2s, 24) == c2 &&
-                 (c1 == 0.0f || std::fabs(s.c1s) >= FLT_MIN) && (c2 == 0.0f || std::fabs(s.c2s) >= FLT_MIN))
-                    ? 1 : 0;
-    s.fast_clamp = (b->min_pos != 0.0f && b->max_pos != 0.0f) ? 1 : 0;
+    set_fast_paths(&s);
 
     int cl = 0, per = 0;
     h->onchip_cluster = (fid != CUPSO_LSQ && onchip_fits(N, D, &cl, &per)) ? cl : 0;

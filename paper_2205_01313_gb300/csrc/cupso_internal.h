@@ -82,6 +82,9 @@ int async_blocks_per_sm(int fid, int D);
 void set_last_error(const char* msg);
 void set_cuda_error(cudaError_t e, const char* where);
 
+// c1s, c2s, fast_cr and fast_clamp of a swarm whose other parameters are set.
+void set_fast_paths(SwarmDev* s);
+
 // Host-side argument check of one problem (CUPSO_OK or CUPSO_ERR_INVALID_ARG).
 int check_problem_args(int D, int N, const cupso_bounds* b, float w, float c1, float c2, int fid);
 // Solve one problem through its own handle (create, iters steps, gbest, destroy).

@@ -8,16 +8,18 @@
 // allocator's accounting or fail against its reservation. Such a caller keeps
 // the swarm in its own device buffers and only needs the iteration.
 //
-// The iteration is the tree-reduction variant (first kernel: update, fitness,
-// pbest and a block tree reduction into one key per block; second kernel:
-// reduction of those keys and the gbest gather). Its working storage -- the
-// per-block keys, the double-buffered gbest position, the iteration counter
-// and status words -- lives in the file-scope device array below, of fixed
-// size. Every GPU that loads the library holds that array until the process
-// exits.
+// The iteration gives what the tree-reduction variant gives. Up to the sizes
+// of tiled_wins it is one kernel over tiles (noalloc_tiled_kernel); above them
+// the tree step's own two kernels (update, fitness, pbest and a block tree
+// reduction into one key per block; then the reduction of those keys and the
+// gbest gather). The working storage -- the per-block keys, the
+// double-buffered gbest position, the iteration counter, ticket and status
+// words -- lives in the file-scope device array below, of fixed size. Every GPU
+// that loads the library holds that array until the process exits.
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -25,6 +27,7 @@
 #include "../../include/cupso.h"
 #include "cupso_device.cuh"
 #include "cupso_internal.h"
+#include "tiled_kernels.h"
 
 namespace cupso {
 namespace {
@@ -41,6 +44,15 @@ struct NoAllocScratch {
     unsigned long long aux[kNoAllocMaxTiles];
     float G[2 * kNoAllocMaxD];
 };
+
+// The tiled kernel spreads a particle's dimensions over threads, the tree step
+// gives each thread four whole particles: measured against each other (sphere,
+// Rastrigin, Rosenbrock; N 500 .. 4 M, D 2 .. 1024), tiles win by 1.05-40x up
+// to 2^18 columns and about 52 M column-dimensions (500 x 2: 13 against 19 us,
+// 65536 x 128: 55 against 187, 50000 x 1024: 970 against 1440); beyond, the tree
+// step fills the GPU and its 16-byte accesses win (4 M x 10: 186 against 209 to
+// 272 us, 200000 x 512: 883 against 1459).
+bool tiled_wins(int ld, int D) { return ld <= (1 << 18) && (long long)ld * D <= (52ll << 20); }
 
 // The scratch. Host code must not use this name as an address: it is only a
 // host-side stand-in. The host obtains the device address with
@@ -84,6 +96,7 @@ __global__ void noalloc_epilogue(const NoAllocScratch* sc, float* gbest_pos, flo
 // and looks the address up again when the current context differs.
 constexpr int kMaxDevices = 64;
 NoAllocScratch* g_scratch_ptr[kMaxDevices] = {};
+int g_scratch_sms[kMaxDevices] = {};
 void* g_scratch_ctx[kMaxDevices] = {};
 std::mutex g_scratch_mutex;
 
@@ -104,7 +117,7 @@ CtxGetCurrentFn ctx_get_current_fn() {
     return fn;
 }
 
-int scratch_on_current_device(NoAllocScratch** out, char* err, size_t errlen) {
+int scratch_on_current_device(NoAllocScratch** out, int* sms, char* err, size_t errlen) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) {
@@ -130,10 +143,16 @@ int scratch_on_current_device(NoAllocScratch** out, char* err, size_t errlen) {
         }
         ctx = nullptr;
         if (get_ctx) get_ctx(&ctx);
+        e = cudaDeviceGetAttribute(&g_scratch_sms[dev], cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) {
+            std::snprintf(err, errlen, "cudaDeviceGetAttribute: %s", cudaGetErrorString(e));
+            return CUPSO_ERR_CUDA;
+        }
         g_scratch_ptr[dev] = static_cast<NoAllocScratch*>(p);
         g_scratch_ctx[dev] = ctx;
     }
     *out = g_scratch_ptr[dev];
+    *sms = g_scratch_sms[dev];
     return CUPSO_OK;
 }
 
@@ -180,7 +199,8 @@ int noalloc_step(int D, int N, const cupso_bounds* bounds, float w, float c1, fl
         return CUPSO_ERR_INVALID_ARG;
     }
     NoAllocScratch* sc = nullptr;
-    const int rc = scratch_on_current_device(&sc, err, errlen);
+    int sms = 1;
+    const int rc = scratch_on_current_device(&sc, &sms, err, errlen);
     if (rc != CUPSO_OK) return rc;
 
     SwarmDev s{};
@@ -207,15 +227,22 @@ int noalloc_step(int D, int N, const cupso_bounds* bounds, float w, float c1, fl
     s.key1 = (uint32_t)(seed >> 32);
     philox_round_keys(s.key0, s.key1, s.rk0, s.rk1);
     s.swarm = swarm_id;
-    s.wait_limit_ns = 2000000000ll;
+    set_fast_paths(&s);
 
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    noalloc_prologue<<<1, 256, 0, st>>>(sc, gbest_pos, D, t);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = launch_tree_step(s, fitness_id, false, st);
-    if (e == cudaSuccess) {
-        noalloc_epilogue<<<1, 256, 0, st>>>(sc, gbest_pos, gbest_fit, gbest_idx, status_out, D, t);
+    cudaError_t e = cudaSuccess;
+    if (tiled_wins(ld, D)) {
+        e = cudaMemsetAsync(sc, 0, offsetof(NoAllocScratch, aux), st);   // key, ticket and status start fresh
+        if (e == cudaSuccess)
+            e = launch_noalloc_tiled(s, fitness_id, t, NoAllocOut{gbest_pos, gbest_fit, gbest_idx, status_out}, sms, st);
+    } else {
+        noalloc_prologue<<<1, 256, 0, st>>>(sc, gbest_pos, D, t);
         e = cudaGetLastError();
+        if (e == cudaSuccess) e = launch_tree_step(s, fitness_id, false, st);
+        if (e == cudaSuccess) {
+            noalloc_epilogue<<<1, 256, 0, st>>>(sc, gbest_pos, gbest_fit, gbest_idx, status_out, D, t);
+            e = cudaGetLastError();
+        }
     }
     if (e != cudaSuccess) {
         std::snprintf(err, errlen, "launch: %s", cudaGetErrorString(e));

@@ -16,8 +16,12 @@
 //  * async_tiled_kernel  ASYNC: persistent CTAs own fixed tiles and iterate
 //                        with no grid barrier against the lock-protected
 //                        gbest record;
-//  * batch_tiled_kernel  a batch: (swarm, tile) units of all swarms per launch.
+//  * batch_tiled_kernel  a batch: (swarm, tile) units of all swarms per launch;
+//  * noalloc_tiled_kernel  one iteration on the caller's buffers, with the
+//                        unconditional argmin of the tree-reduction modes.
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "async_common.cuh"
 #include "cupso_device.cuh"
@@ -131,7 +135,8 @@ struct TileSwarm {
     float *x, *v, *pb, *pf;
     unsigned char* pflag;   // lazy-pbest flags left by the streaming kernels, or null
     const float* G;         // gbest_pos at the end of the previous iteration [D]
-    int N, D, Np;
+    int N, D, Np;           // N particles; columns N .. Nm - 1 (padding) are moved too
+    int Nm;
     float lo, hi, vmax, w, c1, c2, c1s, c2s;
     uint32_t key0, key1, swarm;
 };
@@ -159,9 +164,10 @@ __device__ __forceinline__ void move_tile(float& x, float& v, float pb, float g,
 
 // Steps 2-4 for the tile of P particles starting at `base` (all D dimensions)
 // at iteration t; the tile's Step-5 candidates (improved and below K) are
-// folded into `best`. Every thread of the block calls it; it ends with a
-// barrier, so X, H and imp can be reused at once.
-template <int FIT, bool FAST>
+// folded into `best` (ALL: the key of every particle's pbest_fit after Step 4).
+// Every thread of the block calls it; it ends with a barrier, so X, H and imp
+// can be reused at once.
+template <int FIT, bool FAST, bool ALL = false>
 __device__ __forceinline__ void process_tile(const TileSwarm& s, int fid, int P, int base, uint32_t t,
                                              unsigned long long K, float* X, float* H, int* imp,
                                              unsigned long long& best, bool& nan) {
@@ -171,8 +177,8 @@ __device__ __forceinline__ void process_tile(const TileSwarm& s, int fid, int P,
     // every thread keeps one particle lane p; P (a power of two) divides blockDim
     const int p = tid & (P - 1);
     const int row0 = tid / P, rows = blockDim.x / P;
-    const int n = min(P, s.N - base);
-    const bool live = p < n;
+    const int n = min(P, s.N - base);             // may be <= 0 in a tile of padding
+    const bool live = p < min(P, s.Nm - base);
     const uint32_t i = (uint32_t)(base + p);
     // a particle flagged by the lazy write-back has pbest_pos == pos: use and write it
     const bool lazy = live && s.pflag && s.pflag[i];
@@ -227,17 +233,21 @@ __device__ __forceinline__ void process_tile(const TileSwarm& s, int fid, int P,
         const float f = tile_sum<FIT>(fid, X, H, P, tid, D);
         const uint32_t ip = (uint32_t)(base + tid);
         nan |= (f != f);
-        const bool better = f < s.pf[ip];
+        const float pf = s.pf[ip];
+        const bool better = f < pf;
         imp[tid] = better ? 1 : 0;
-        if (better) {
-            s.pf[ip] = f;
+        if (better) s.pf[ip] = f;
+        if constexpr (ALL) {
+            const unsigned long long k = pack_key(better ? f : pf, ip);
+            if (k < best) best = k;
+        } else if (better) {
             const unsigned long long k = pack_key(f, ip);
             if (k < K && k < best) best = k;
         }
         if (s.pflag && s.pflag[ip]) s.pflag[ip] = 0;
     }
     __syncthreads();
-    if (live && imp[p])
+    if (p < n && imp[p])
         for (int d = row0; d < D; d += rows) s.pb[(size_t)d * Np + i] = X[d * P + p];
     __syncthreads();
 }
@@ -253,7 +263,7 @@ __global__ void __launch_bounds__(kTiledThreads) sync_tiled_kernel(const __grid_
     const uint32_t t = t_prev + 1u;
     const int cur = (int)(t_prev & 1u), nxt = cur ^ 1;
     const unsigned long long K = __ldcg(s.gkey + cur);   // gbest at the end of t-1
-    const TileSwarm ts{s.x, s.v, s.pb, s.pf, nullptr, s.G + (size_t)cur * s.D, s.N, s.D, s.Np, s.lo, s.hi, s.vmax,
+    const TileSwarm ts{s.x, s.v, s.pb, s.pf, nullptr, s.G + (size_t)cur * s.D, s.N, s.D, s.Np, s.N, s.lo, s.hi, s.vmax,
                        s.w, s.c1, s.c2, s.c1s, s.c2s, s.key0, s.key1, s.swarm};
     const int ntiles = (s.N + P - 1) / P;
     unsigned long long best = kKeyNone;
@@ -292,7 +302,7 @@ __global__ void __launch_bounds__(kTiledThreads, 4) async_tiled_kernel(const __g
     extern __shared__ float Gs[];   // [D] the gbest this CTA's iteration uses
     const int tid = threadIdx.x;
     const int ntiles = (s.N + P - 1) / P;
-    const TileSwarm ts{s.x, s.v, s.pb, s.pf, nullptr, Gs, s.N, s.D, s.Np, s.lo, s.hi, s.vmax,
+    const TileSwarm ts{s.x, s.v, s.pb, s.pf, nullptr, Gs, s.N, s.D, s.Np, s.N, s.lo, s.hi, s.vmax,
                        s.w, s.c1, s.c2, s.c1s, s.c2s, s.key0, s.key1, s.swarm};
     for (int k = 0; k < iters; ++k) {
         const uint32_t t = t_first + (uint32_t)k;
@@ -364,7 +374,7 @@ __global__ void __launch_bounds__(kTiledThreads, 3) batch_tiled_kernel(const __g
         const BatchSwarm& w = b.swarms[un.x];
         const int P = bt.P[un.x];
         const unsigned long long K = __ldcg(w.gkey + cur);
-        const TileSwarm ts{w.x, w.v, w.pb, w.pf, w.pflag, w.G + (size_t)cur * w.D, w.N, w.D, w.Np, w.lo, w.hi,
+        const TileSwarm ts{w.x, w.v, w.pb, w.pf, w.pflag, w.G + (size_t)cur * w.D, w.N, w.D, w.Np, w.N, w.lo, w.hi,
                            w.vmax, w.w, w.c1, w.c2, w.c1s, w.c2s, w.key0, w.key1, w.swarm};
         unsigned long long best = kKeyNone;
         bool nan = false;
@@ -406,6 +416,56 @@ __global__ void __launch_bounds__(kTiledThreads, 3) batch_tiled_kernel(const __g
         b.work[(t + 1u) & 1u] = 0u;
         *b.ticket = 0u;
         *b.t_dev = t;
+    }
+}
+
+// One synchronous iteration on the caller's buffers (cupso_noalloc.cu): tiles
+// over all columns of the stride, gbest = the argmin over every particle's
+// pbest as the tree reduction finds it, here by one atomic per block on the
+// complemented key (scratch zeroed before the launch, so 0 is "none yet"). The
+// last block gathers gbest_pos over the one that this iteration read (every
+// block is done with it) and writes the caller's outputs: one kernel where the
+// two of the tree step and a copy in and out made four (3000 x 20: 31 -> 12 us
+// a call).
+template <int FIT, bool FAST>
+__global__ void __launch_bounds__(kTiledThreads) noalloc_tiled_kernel(const __grid_constant__ SwarmDev s, int P, uint32_t t,
+                                                                     const NoAllocOut o) {
+    __shared__ float X[kTiledItems];
+    __shared__ float H[kTiledItems];
+    __shared__ unsigned long long red[kTiledThreads / 32];
+    __shared__ int imp[kTiledMaxP];
+    __shared__ int s_last;
+    const TileSwarm ts{s.x, s.v, s.pb, s.pf, nullptr, o.gbest_pos, s.N, s.D, s.Np, s.Np, s.lo, s.hi, s.vmax,
+                       s.w, s.c1, s.c2, s.c1s, s.c2s, s.key0, s.key1, s.swarm};
+    const int ntiles = (s.Np + P - 1) / P;
+    unsigned long long best = kKeyNone;
+    bool nan = false;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
+        process_tile<FIT, FAST, true>(ts, FIT, P, tile * P, t, kKeyNone, X, H, imp, best, nan);
+    best = block_min(best, red);
+    const bool any_nan = __syncthreads_or(nan);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (best != kKeyNone) atomicMax(s.gkey, ~best);
+        if (any_nan) atomicOr(s.status, kStatusNaN);
+        __threadfence();
+        s_last = atomicAdd(s.ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const unsigned long long key = ~__ldcg(s.gkey);
+    const uint32_t g = (uint32_t)(key & 0xFFFFFFFFull);
+    if (g < (uint32_t)s.N)
+        for (int d = threadIdx.x; d < s.D; d += blockDim.x) o.gbest_pos[d] = __ldcg(s.pb + (size_t)d * s.Np + g);
+    if (threadIdx.x == 0) {
+        const uint32_t k = (uint32_t)(key >> 32);
+        uint32_t bits = (k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k;
+        if (k == 0xFFFFFFFFu) bits = 0x7FC00000u;   // NaN ranks last
+        if (o.gbest_fit) *o.gbest_fit = __uint_as_float(bits);
+        if (o.gbest_idx) *o.gbest_idx = (int64_t)g;
+        if (o.status) *o.status = __ldcg(s.status);
     }
 }
 
@@ -456,6 +516,19 @@ cudaError_t launch_sync_tiled(const SwarmDev& s, int fid, int P, int grid, cudaS
         CUPSO_TILED_DISPATCH(fid, false, return launch_pdl(sync_tiled_kernel<F, false>, dim3(g), dim3(threads), 0, st, s, P));
     }
     return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_noalloc_tiled(const SwarmDev& s, int fid, uint32_t t, const NoAllocOut& o, int num_sms, cudaStream_t st) {
+    const int P = tiled_particles(s.Np, s.D, num_sms);
+    if (P < 1) return cudaErrorInvalidValue;
+    const int tiles = (s.Np + P - 1) / P, threads = tile_threads(P, s.D);
+    const int g = std::min(tiles, num_sms * tiled_blocks_per_sm(fid, P, s.D));
+    if (s.fast_cr && s.fast_clamp) {
+        CUPSO_TILED_DISPATCH(fid, true, (noalloc_tiled_kernel<F, true><<<g, threads, 0, st>>>(s, P, t, o)));
+    } else {
+        CUPSO_TILED_DISPATCH(fid, false, (noalloc_tiled_kernel<F, false><<<g, threads, 0, st>>>(s, P, t, o)));
+    }
+    return cudaGetLastError();
 }
 
 int tiled_blocks_per_sm(int fid, int P, int D) {

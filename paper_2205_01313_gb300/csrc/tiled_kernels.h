@@ -47,6 +47,17 @@ int batch_tiled_blocks_per_sm();
 // tiles (at most one block per tile).
 cudaError_t launch_sync_tiled(const SwarmDev& s, int fid, int P, int grid, cudaStream_t st);
 
+// One iteration on caller-owned buffers (cupso_noalloc.cu): s.x, v, pb, pf with
+// stride s.Np, s.gkey (complemented key), s.ticket and s.status zero; gbest_pos
+// [D] is read and replaced.
+struct NoAllocOut {
+    float* gbest_pos;
+    float* gbest_fit;      // these may be null
+    int64_t* gbest_idx;
+    unsigned int* status;
+};
+cudaError_t launch_noalloc_tiled(const SwarmDev& s, int fid, uint32_t t, const NoAllocOut& o, int num_sms, cudaStream_t st);
+
 // Resident blocks per SM of the tiled kernel for (fitness, P, D).
 int tiled_blocks_per_sm(int fid, int P, int D);
 
