@@ -95,8 +95,13 @@ typedef enum {
 
 /* How the global best is aggregated (cupso_set_option(CUPSO_OPT_MODE)). */
 typedef enum {
-    CUPSO_MODE_AUTO = 0,   /* ONCHIP when the swarm fits, else SYNC                        */
-    CUPSO_MODE_SYNC = 1,   /* fused kernel, conditional atomicMin + last-CTA gather (Sec. 3.1) */
+    CUPSO_MODE_AUTO = 0,   /* ONCHIP when the swarm fits, else SYNC; a long cupso_step call of an
+                              ONCHIP swarm may keep it in the registers of all SMs instead of one
+                              cluster's shared memory, as SYNC does (same results)           */
+    CUPSO_MODE_SYNC = 1,   /* fused kernel, conditional atomicMin + last-CTA gather (Sec. 3.1); a step
+                              of several iterations keeps a swarm of up to about a million
+                              particle-dimensions in the registers of all SMs, in one cooperative
+                              launch                                                         */
     CUPSO_MODE_TREE = 2,   /* parallel-reduction baseline: two kernels per iteration (Sec. 2.2) */
     CUPSO_MODE_TREE_UNROLLED = 3, /* the same with the unrolled reduction (Sec. 2.2)       */
     CUPSO_MODE_ASYNC = 4,  /* persistent CTAs, no grid barrier, lock-protected gbest (Sec. 3.2) */
@@ -126,12 +131,13 @@ typedef enum {
                                      BF16/FP8: the tensor-core product alone (the move kernel
                                      before it writes the operand; the selection after it adds the
                                      product's partial sums) */
-    CUPSO_OPT_ITERS_PER_LAUNCH = 9, /* SYNC step on the panel layout: iterations per launch of a
-                                       cupso_step call. 1: one kernel per iteration (graphs per
-                                       CUPSO_OPT_GRAPH_CHUNK); n > 1: up to n per cooperative launch,
-                                       all CTAs resident, a grid barrier between iterations (each
-                                       wait bounded by CUPSO_OPT_WAIT_LIMIT_NS); 0 (default): up to
-                                       4096. Same results either way. */
+    CUPSO_OPT_ITERS_PER_LAUNCH = 9, /* SYNC step on the panel layout or in registers: iterations per
+                                       launch of a cupso_step call. 1: one kernel per iteration
+                                       (graphs per CUPSO_OPT_GRAPH_CHUNK); n > 1: up to n per
+                                       cooperative launch, all CTAs resident, a grid barrier between
+                                       iterations (each wait bounded by CUPSO_OPT_WAIT_LIMIT_NS);
+                                       0 (default): up to 4096 (registers: 2^22). Same results either
+                                       way. */
     CUPSO_OPT_LSQ_RESCORE = 10,   /* BF16 / FP8 least-squares swarm with D <= M: arithmetic of
                                      the Gram-form rescoring of its gbest candidates. 0 (default):
                                      the off-diagonal part of x^T (A^T A) x in float-float (pairs

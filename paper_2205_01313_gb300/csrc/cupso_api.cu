@@ -55,6 +55,7 @@ struct cupso_swarm {
     bool fp64 = false;              // a double-precision swarm: dev64 instead of dev
     SwarmDev64 dev64{};
     PaperBufs pbufs{};              // one-particle-per-thread designs (QUEUE, QUEUE_LOCK, FP64 modes)
+    ResidentBufs rbufs{};           // the resident SYNC kernel's exchange (slots null: it does not fit)
     bool onchip64 = false;          // the FP64 swarm fits the on-chip kernel
     int N = 0, D = 0, Np = 0, fid = 0;
     uint64_t seed = 0;
@@ -258,6 +259,27 @@ int sync_grid(const cupso_swarm* h) {
 // cupso_step call up to kPanelMaxIters.
 int panel_iters_per_launch(const cupso_swarm* h) {
     return h->iters_per_launch > 0 ? h->iters_per_launch : kPanelMaxIters;
+}
+
+// Whether `iters` iterations run in the resident kernel (kernels_resident.cu):
+// synchronous swarm, AUTO kernel choice, default grid, several iterations per
+// launch allowed.
+//  * SYNC: loading and storing the registers costs as much as one or two iterations
+//    of the kernels that keep the state in memory; measured per iteration against
+//    them at 2, 3 and 4 iterations: 1024 x 32 6.4, 4.6, 4.2 us against 5.4, 5.3, 5.2;
+//    20000 x 48 11.2, 8.6, 7.2 against 11.3, 10.6, 10.2; one more where the state is
+//    in panels, whose loads are strided here.
+//  * AUTO, where the swarm also fits one cluster's shared memory: an iteration takes
+//    1.0 to 1.5 us (2.2 while gbest improves) whatever the swarm, against 1.1 us (32 x
+//    1) to 4.7 (2048 x 32) on the cluster, whose launch costs less: 2048 x 32 at 4
+//    iterations 4.0 against 6.7 us, 1000 x 2 3.1 against 2.8; 300 x 8 (Rosenbrock)
+//    at 100 1.95 against 1.68, at 1000 1.51 against 1.58.
+bool use_resident(const cupso_swarm* h, int mode, int iters) {
+    if (!h->rbufs.slots || h->sync_kernel != CUPSO_SYNC_KERNEL_AUTO || h->grid_override != 0 || h->iters_per_launch == 1)
+        return false;
+    if (mode == CUPSO_MODE_SYNC) return iters >= (h->panel ? 4 : 3);
+    if (mode != CUPSO_MODE_ONCHIP || h->mode != CUPSO_MODE_AUTO) return false;
+    return h->N >= 1000 ? iters >= 5 : ((long long)h->N * h->D >= 1000 && iters >= 300);
 }
 
 // CTAs of a multi-iteration panel launch: the SYNC grid, at most what the SMs
@@ -550,6 +572,8 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
     const size_t o_words = off; off = align_up(off + 128, A);
     const int list_cap = paper_blocks(h->Np);      // one candidate per block of the queue designs
     const size_t o_paper = off; off = align_up(off + paper_bufs_bytes(h->Np, list_cap), A);
+    const size_t res_bytes = fid == CUPSO_LSQ ? 0 : resident_bytes(N, D, h->num_sms);
+    const size_t o_res = off; off = align_up(off + res_bytes, A);
     h->arena_bytes = off;
     e = cudaMalloc(&h->arena, h->arena_bytes);
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
@@ -591,6 +615,7 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
     s.wait_limit_ns = 2000000000ll;
     h->pbufs = paper_bufs_at(base + o_paper, h->Np, list_cap);
     set_fast_paths(&s);
+    if (res_bytes && resident_fits(s, fid, h->num_sms)) h->rbufs = resident_bufs_at(base + o_res);
 
     int cl = 0, per = 0;
     h->onchip_cluster = (fid != CUPSO_LSQ && onchip_fits(N, D, &cl, &per)) ? cl : 0;
@@ -1018,6 +1043,20 @@ int cupso_step(cupso_handle h, int iters) {
     if (h->fp64 && mode == CUPSO_MODE_PERSISTENT) {
         cudaError_t e = launch_persist64(h->dev64, h->pbufs, h->fid, iters, h->num_sms, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "persistent launch");
+        h->t_host += (uint32_t)iters;
+        return CUPSO_OK;
+    }
+    if (!h->fp64 && use_resident(h, mode, iters)) {
+        // any layout, pending pbest rows included; a launch's iterations as for the panel step
+        const int most = h->iters_per_launch > 0 ? h->iters_per_launch : kResidentMaxIters;
+        for (int left = iters; left > 0;) {
+            const int n = std::min(left, most);
+            const cudaError_t e = launch_resident(h->dev, h->rbufs, h->fid, h->panel, n, h->stall_barrier != 0, h->num_sms,
+                                                  h->stream);
+            if (e != cudaSuccess) return cuda_fail(e, "resident launch");
+            left -= n;
+        }
+        h->lazy_pending = false;
         h->t_host += (uint32_t)iters;
         return CUPSO_OK;
     }

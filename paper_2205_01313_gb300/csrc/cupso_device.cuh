@@ -159,6 +159,25 @@ __device__ __forceinline__ float cos2pi(float x) {
     return cos2pi_poly(a);
 }
 
+// cos2pi for |x| <= 2^21 (kSmallX), the same bits with fewer and cheaper
+// instructions: k = rint(2 x) by adding 1.5 * 2^23 (round to nearest even; the
+// rounding instruction runs at an eighth of the rate), r = x - k / 2 exact with
+// |r| <= 1/4, cos(2 pi x) = (-1)^k cos(2 pi r). |r| is cos2pi's argument of the
+// polynomial (a, or 1/2 - a where k is odd, which is where a > 1/4), squared there.
+constexpr float kSmallX = 0x1p21f;
+__device__ __forceinline__ float cos2pi_small(float x) {
+    const float m = __fmaf_rn(2.0f, x, 0x1.8p23f);
+    const float r = __fmaf_rn(-0.5f, __fsub_rn(m, 0x1.8p23f), x);
+    return __uint_as_float(__float_as_uint(cos2pi_poly(r)) ^ (__float_as_uint(m) << 31));
+}
+
+// SMALL: every x lies within kSmallX.
+template <bool SMALL>
+__device__ __forceinline__ float cosine2pi(float x) {
+    if constexpr (SMALL) return cos2pi_small(x);
+    else return cos2pi(x);
+}
+
 __device__ __forceinline__ float exp_own(float y) {
     if (y != y) return y;
     if (y > 88.8f) return __int_as_float(0x7f800000);

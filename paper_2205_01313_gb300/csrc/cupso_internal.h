@@ -74,6 +74,22 @@ cudaError_t launch_materialize_panel(const SwarmDev& s, int width, int grid, cud
 cudaError_t launch_relayout(const float* src, float* dst, int D, int Np, int width, bool to_panel, int grid,
                             cudaStream_t st);
 
+// Several SYNC iterations in one cooperative launch with the swarm in registers
+// (kernels_resident.cu): swarms of up to about 4000 (dimension pair, particle)
+// items and at most 1024 particles per SM. `panel`: the state's layout (0: dimension-major);
+// pending pbest rows are taken over, and none are pending afterwards.
+struct ResidentBufs {
+    unsigned long long* key = nullptr;   // [2] lowest key of an iteration, by parity
+    unsigned long long* bar = nullptr;   // arrivals and candidate counts
+    float* slots = nullptr;              // [2][grid][D] candidates' positions
+};
+constexpr int kResidentMaxIters = 1 << 22;   // per launch: iterations x (SMs + 1) stays below 2^32
+bool resident_fits(const SwarmDev& s, int fid, int num_sms);
+size_t resident_bytes(int N, int D, int num_sms);   // 0: does not fit
+ResidentBufs resident_bufs_at(void* base);
+cudaError_t launch_resident(const SwarmDev& s, const ResidentBufs& rb, int fid, int panel, int iters, bool stall_barrier,
+                            int num_sms, cudaStream_t st);
+
 // Resident CTAs per SM of the persistent kernels (for grid sizing).
 int sync_blocks_per_sm(int fid, int D);
 int async_blocks_per_sm(int fid, int D);

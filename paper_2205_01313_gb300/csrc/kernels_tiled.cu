@@ -26,6 +26,7 @@
 #include "async_common.cuh"
 #include "cupso_device.cuh"
 #include "cupso_internal.h"
+#include "fit_terms.cuh"
 #include "pdl.cuh"
 #include "stream_common.cuh"
 #include "tiled_kernels.h"
@@ -36,53 +37,6 @@ namespace {
 
 constexpr int kTiledThreads = 256;
 constexpr int kChunk = 4;     // dimension pairs whose loads a thread issues together
-
-// Fitness from per-dimension terms; sum() equals FitAcc<FIT> over d in order.
-template <int FIT>
-struct FitTerms {
-    // Rosenbrock's term d pairs x_d with x_{d+1}
-    static constexpr bool kNeedsNext = (FIT == kRosenbrock);
-    // no term array: the sum fuses x * x itself
-    static constexpr bool kNoTerm = (FIT == kSphere);
-    __device__ static __forceinline__ float term(float x, float xn) {
-        if constexpr (FIT == kRastrigin) {
-            return __fmaf_rn(x, x, __fmaf_rn(-10.0f, cos2pi(x), 10.0f));
-        } else if constexpr (FIT == kAckley) {
-            return cos2pi(x);
-        } else if constexpr (FIT == kRosenbrock) {
-            const float p = __fmaf_rn(-x, x, xn);
-            const float q = __fsub_rn(1.0f, x);
-            return __fmaf_rn(__fmul_rn(100.0f, p), p, __fmul_rn(q, q));
-        } else if constexpr (FIT == kCubicMax) {
-            return __fmaf_rn(__fmaf_rn(__fsub_rn(x, 0.8f), x, -1000.0f), x, 8000.0f);
-        } else {
-            return 0.0f;
-        }
-    }
-    // particle column p (stride P) of X and H
-    __device__ static __forceinline__ float sum(const float* X, const float* H, int P, int p, int D) {
-        FitAcc<FIT> a;
-        if constexpr (FIT == kSphere) {
-#pragma unroll 8
-            for (int d = 0; d < D; ++d) {
-                const float x = X[d * P + p];
-                a.acc = __fmaf_rn(x, x, a.acc);
-            }
-        } else if constexpr (FIT == kAckley) {
-#pragma unroll 8
-            for (int d = 0; d < D; ++d) {
-                const float x = X[d * P + p];
-                a.acc = __fmaf_rn(x, x, a.acc);
-                a.acc2 = __fadd_rn(a.acc2, H[d * P + p]);
-            }
-        } else {
-            const int n = FIT == kRosenbrock ? D - 1 : D;
-#pragma unroll 8
-            for (int d = 0; d < n; ++d) a.acc = __fadd_rn(a.acc, H[d * P + p]);
-        }
-        return a.finish(D);
-    }
-};
 
 // Fitness chosen at run time (a batch mixes them): FIT = kAnyFit dispatches on
 // `fid`, uniformly for a whole tile; a fixed FIT compiles to its own code.
