@@ -19,7 +19,7 @@ def P():
 # M, D, N, floats by which A is shifted off its allocation
 @pytest.mark.parametrize("M,D,N,shift", [
     (1, 1, 1, 0), (520, 36, 1300, 0), (520, 36, 1300, 1), (521, 33, 1281, 0), (129, 16, 5000, 0), (127, 17, 63, 0),
-    (4000, 4, 4500, 0), (3, 2, 140000, 0),
+    (4000, 4, 4500, 0), (3, 2, 140000, 0), (66, 2, 140000, 0), (64, 17, 257, 0), (65, 17, 257, 0),
 ])
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 def test_exact_fitness_bits(P, precision, M, D, N, shift):
