@@ -113,9 +113,8 @@ struct cupso_swarm {
     // kStageBytes unless one particle's row is larger)
     void* stage = nullptr;
     size_t stage_bytes = 0;
-    // pinned host staging of the gbest reads (allocated on first use)
-    void* pinned = nullptr;
-    size_t pinned_bytes = 0;
+    char* rec_now = nullptr;        // device record of a gbest read, in the arena
+    std::vector<char> rec_copy;     // its host copy
     // result slots of cupso_gbest_post / _wait (allocated on first use): a
     // device record and a pinned host copy per slot, the copy stream, and per
     // slot the events of the snapshot and of its copy
@@ -516,6 +515,10 @@ int cupso::check_problem_args(int D, int N, const cupso_bounds* b, float w, floa
     return CUPSO_OK;
 }
 
+namespace {
+size_t rec_bytes(int D, bool fp64);   // of a gbest read's record, below
+}
+
 // The fast arithmetic path's constants and whether it gives the same bits:
 // c * 2^-24 is exact unless it would be subnormal (checked by scaling back), and
 // the min/max clamps need bounds that are not zero.
@@ -574,10 +577,12 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
     const size_t o_paper = off; off = align_up(off + paper_bufs_bytes(h->Np, list_cap), A);
     const size_t res_bytes = fid == CUPSO_LSQ ? 0 : resident_bytes(N, D, h->num_sms);
     const size_t o_res = off; off = align_up(off + res_bytes, A);
+    const size_t o_rec = off; off = align_up(off + rec_bytes(D, false), A);
     h->arena_bytes = off;
     e = cudaMalloc(&h->arena, h->arena_bytes);
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
     char* base = static_cast<char*>(h->arena);
+    h->rec_now = base + o_rec;
     SwarmDev& s = h->dev;
     s.x = reinterpret_cast<float*>(base + o_x);
     s.v = reinterpret_cast<float*>(base + o_v);
@@ -619,8 +624,9 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
 
     int cl = 0, per = 0;
     h->onchip_cluster = (fid != CUPSO_LSQ && onchip_fits(N, D, &cl, &per)) ? cl : 0;
-    h->pipelined_ok = prepare_pipelined(D) == cudaSuccess;
-    h->panel_ok = fid != CUPSO_LSQ && panel_supported(8, 3, D) && prepare_panel(D) == cudaSuccess;
+    const bool fast = s.fast_cr && s.fast_clamp;
+    h->pipelined_ok = prepare_pipelined(fid, fast) == cudaSuccess;
+    h->panel_ok = fid != CUPSO_LSQ && panel_supported(8, 3, D) && prepare_panel(fid, fast) == cudaSuccess;
     cudaGetLastError();
 
     e = cudaMemsetAsync(base + o_words, 0, 128, h->stream);
@@ -701,10 +707,12 @@ int create_swarm64(int D, int N, const cupso_bounds_f64* b, double w, double c1,
     const size_t o_words = off; off = align_up(off + 64, A);
     const int list_cap = h->Np;   // the tiled step may run up to one block per particle
     const size_t o_paper = off; off = align_up(off + paper_bufs_bytes(h->Np, list_cap), A);
+    const size_t o_rec = off; off = align_up(off + rec_bytes(D, true), A);
     h->arena_bytes = off;
     e = cudaMalloc(&h->arena, h->arena_bytes);
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
     char* base = static_cast<char*>(h->arena);
+    h->rec_now = base + o_rec;
     SwarmDev64& s = h->dev64;
     s.x = reinterpret_cast<double*>(base + o_x);
     s.v = reinterpret_cast<double*>(base + o_v);
@@ -751,18 +759,6 @@ int create_swarm64(int D, int N, const cupso_bounds_f64* b, double w, double c1,
     e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return bail(cuda_fail(e, "init"));
     *out = h;
-    return CUPSO_OK;
-}
-
-// Pinned staging for small reads: async copies into pinned memory need no
-// host-side staging and finish with one stream synchronisation.
-int ensure_pinned(cupso_swarm* h, size_t bytes) {
-    if (h->pinned_bytes >= bytes) return CUPSO_OK;
-    if (h->pinned) cudaFreeHost(h->pinned);
-    h->pinned = nullptr;
-    h->pinned_bytes = 0;
-    CUPSO_CUDA(cudaMallocHost(&h->pinned, bytes), "cudaMallocHost");
-    h->pinned_bytes = bytes;
     return CUPSO_OK;
 }
 
@@ -879,24 +875,52 @@ void cupso::set_cuda_error(cudaError_t e, const char* where) { cuda_fail(e, wher
 
 namespace {
 
-// Bytes of one result record: key at 0, status at 8, position from 32.
-size_t rec_bytes(int D) { return (32 + sizeof(float) * (size_t)D + 255) / 256 * 256; }
+// One result record: the gbest key at 0 (16 bytes, of which a single-precision
+// swarm uses 8), the sticky status at 16, gbest_pos from 32.
+constexpr size_t kRecStatus = 16, kRecPos = 32;
+size_t rec_bytes(int D, bool fp64) { return align_up(kRecPos + (fp64 ? 8 : 4) * (size_t)D, 256); }
 
-// gbest of one parity -- its key, the sticky status and its position -- into
-// a contiguous record.
-__global__ void gbest_record_kernel(const unsigned long long* __restrict__ key, const unsigned* __restrict__ status,
-                                    const float* __restrict__ G, int D, char* __restrict__ rec) {
-    float* pos = reinterpret_cast<float*>(rec + 32);
-    for (int d = threadIdx.x; d < D; d += blockDim.x) pos[d] = __ldcg(G + d);
-    if (threadIdx.x == 0) {
-        *reinterpret_cast<unsigned long long*>(rec) = __ldcg(key);
-        *reinterpret_cast<unsigned*>(rec + 8) = __ldcg(status);
+// The current gbest into a contiguous record, so that one copy brings it to the host.
+__global__ void gbest_record_kernel(const uint32_t* __restrict__ key, int key_words, const unsigned* __restrict__ status,
+                                    const uint32_t* __restrict__ G, int g_words, uint32_t* __restrict__ rec) {
+    for (int e = threadIdx.x; e < g_words; e += blockDim.x) rec[kRecPos / 4 + e] = __ldcg(G + e);
+    if ((int)threadIdx.x < key_words) rec[threadIdx.x] = __ldcg(key + threadIdx.x);
+    if (threadIdx.x == 32) rec[kRecStatus / 4] = __ldcg(status);
+}
+
+cudaError_t queue_record(const cupso_swarm* h, char* rec) {
+    const size_t cur = h->t_host & 1u, D = (size_t)h->D;
+    uint32_t* out = reinterpret_cast<uint32_t*>(rec);
+    if (h->fp64)
+        gbest_record_kernel<<<1, 256, 0, h->stream>>>(reinterpret_cast<const uint32_t*>(h->dev64.gkey + cur), 4,
+                                                      h->dev64.status, reinterpret_cast<const uint32_t*>(h->dev64.G + cur * D),
+                                                      (int)(2 * D), out);
+    else
+        gbest_record_kernel<<<1, 256, 0, h->stream>>>(reinterpret_cast<const uint32_t*>(h->dev.gkey + cur), 2, h->dev.status,
+                                                      reinterpret_cast<const uint32_t*>(h->dev.G + cur * D), (int)D, out);
+    return cudaGetLastError();
+}
+
+// The current gbest in h->rec_copy (its position only if asked for): one kernel, one
+// copy into ordinary memory and one wait (24 us with the wait for an idle stream, as
+// with a copy per field into pinned memory, which took 130 us to allocate with the
+// first read and 120 to free with the handle).
+int read_record(cupso_swarm* h, bool pos) {
+    const size_t bytes = pos ? kRecPos + (h->fp64 ? 8 : 4) * (size_t)h->D : kRecPos;
+    try {
+        h->rec_copy.resize(rec_bytes(h->D, h->fp64));
+    } catch (...) {
+        return fail(CUPSO_ERR_OOM, "host allocation failed%s");
     }
+    CUPSO_CUDA(queue_record(h, h->rec_now), "gbest record launch");
+    CUPSO_CUDA(cudaMemcpyAsync(h->rec_copy.data(), h->rec_now, bytes, cudaMemcpyDeviceToHost, h->stream), "cudaMemcpyAsync");
+    CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    return CUPSO_OK;
 }
 
 int ensure_records(cupso_swarm* h) {
     if (h->rec_dev) return CUPSO_OK;
-    const size_t bytes = 2 * rec_bytes(h->D);
+    const size_t bytes = 2 * rec_bytes(h->D, false);
     CUPSO_CUDA(cudaMalloc(&h->rec_dev, bytes), "cudaMalloc (gbest records)");
     CUPSO_CUDA(cudaMallocHost(&h->rec_host, bytes), "cudaMallocHost (gbest records)");
     CUPSO_CUDA(cudaStreamCreateWithFlags(&h->rec_stream, cudaStreamNonBlocking), "cudaStreamCreate");
@@ -1122,22 +1146,14 @@ int cupso_step(cupso_handle h, int iters) {
 int cupso_get_gbest(cupso_handle h, float* fit_out, float* pos_out, int64_t* idx_out) {
     if (!h) return fail(CUPSO_ERR_INVALID_ARG, "handle is NULL%s");
     if (h->fp64) return fail(CUPSO_ERR_UNSUPPORTED, "double-precision swarm: use the _fp64 functions%s");
-    const int cur = (int)(h->t_host & 1u);
-    int rc = ensure_pinned(h, 32 + sizeof(float) * (size_t)h->D);
+    int rc = read_record(h, pos_out != nullptr);
     if (rc) return rc;
-    char* pin = static_cast<char*>(h->pinned);
-    CUPSO_CUDA(cudaMemcpyAsync(pin, h->dev.gkey + cur, 8, cudaMemcpyDeviceToHost, h->stream), "cudaMemcpyAsync");
-    CUPSO_CUDA(cudaMemcpyAsync(pin + 8, h->dev.status, 4, cudaMemcpyDeviceToHost, h->stream), "cudaMemcpyAsync");
-    if (pos_out)
-        CUPSO_CUDA(cudaMemcpyAsync(pin + 32, h->dev.G + (size_t)cur * h->D, sizeof(float) * (size_t)h->D,
-                                   cudaMemcpyDeviceToHost, h->stream),
-                   "cudaMemcpyAsync");
-    CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    const char* rec = h->rec_copy.data();
     unsigned long long key = 0;
     unsigned st = 0;
-    std::memcpy(&key, pin, 8);
-    std::memcpy(&st, pin + 8, 4);
-    if (pos_out) std::memcpy(pos_out, pin + 32, sizeof(float) * (size_t)h->D);
+    std::memcpy(&key, rec, 8);
+    std::memcpy(&st, rec + kRecStatus, 4);
+    if (pos_out) std::memcpy(pos_out, rec + kRecPos, sizeof(float) * (size_t)h->D);
     if (fit_out) *fit_out = key_to_fit(key);
     if (idx_out) *idx_out = (int64_t)(key & 0xFFFFFFFFull);
     rc = status_code(st);
@@ -1152,16 +1168,13 @@ int cupso_gbest_post(cupso_handle h, int slot) {
     if (h->rec_posted[slot]) return fail(CUPSO_ERR_INVALID_ARG, "slot already holds a result; wait for it first%s");
     int rc = ensure_records(h);
     if (rc) return rc;
-    const size_t rb = rec_bytes(h->D);
+    const size_t rb = rec_bytes(h->D, false);
     char* dev = h->rec_dev + (size_t)slot * rb;
-    const int cur = (int)(h->t_host & 1u);
     // the snapshot follows the queued steps on the handle's stream; the next
     // step cannot change what it copies (a step rewrites these words only
     // after the stream reaches it). Its copy to the host runs on the second
     // stream, beside the next steps.
-    gbest_record_kernel<<<1, 256, 0, h->stream>>>(h->dev.gkey + cur, h->dev.status, h->dev.G + (size_t)cur * h->D,
-                                                  h->D, dev);
-    CUPSO_CUDA(cudaGetLastError(), "gbest record launch");
+    CUPSO_CUDA(queue_record(h, dev), "gbest record launch");
     CUPSO_CUDA(cudaEventRecord(h->rec_ev[slot], h->stream), "cudaEventRecord");
     CUPSO_CUDA(cudaStreamWaitEvent(h->rec_stream, h->rec_ev[slot], 0), "cudaStreamWaitEvent");
     CUPSO_CUDA(cudaMemcpyAsync(h->rec_host + (size_t)slot * rb, dev, rb, cudaMemcpyDeviceToHost, h->rec_stream),
@@ -1177,12 +1190,12 @@ int cupso_gbest_wait(cupso_handle h, int slot, float* fit_out, float* pos_out, i
     if (!h->rec_posted[slot]) return fail(CUPSO_ERR_INVALID_ARG, "nothing posted to this slot%s");
     CUPSO_CUDA(cudaEventSynchronize(h->rec_done[slot]), "cudaEventSynchronize");
     h->rec_posted[slot] = false;
-    const char* rec = h->rec_host + (size_t)slot * rec_bytes(h->D);
+    const char* rec = h->rec_host + (size_t)slot * rec_bytes(h->D, false);
     unsigned long long key = 0;
     unsigned st = 0;
     std::memcpy(&key, rec, 8);
-    std::memcpy(&st, rec + 8, 4);
-    if (pos_out) std::memcpy(pos_out, rec + 32, sizeof(float) * (size_t)h->D);
+    std::memcpy(&st, rec + kRecStatus, 4);
+    if (pos_out) std::memcpy(pos_out, rec + kRecPos, sizeof(float) * (size_t)h->D);
     if (fit_out) *fit_out = key_to_fit(key);
     if (idx_out) *idx_out = (int64_t)(key & 0xFFFFFFFFull);
     const int rc = status_code(st);
@@ -1384,23 +1397,14 @@ int cupso_create_fp64(int D, int N, const cupso_bounds_f64* bounds, double w, do
 int cupso_get_gbest_fp64(cupso_handle h, double* fit_out, double* pos_out, int64_t* idx_out) {
     if (!h) return fail(CUPSO_ERR_INVALID_ARG, "handle is NULL%s");
     if (!h->fp64) return fail(CUPSO_ERR_UNSUPPORTED, "not a double-precision swarm%s");
-    const int cur = (int)(h->t_host & 1u);
-    int rc = ensure_pinned(h, 32 + sizeof(double) * (size_t)h->D);
+    int rc = read_record(h, pos_out != nullptr);
     if (rc) return rc;
-    char* pin = static_cast<char*>(h->pinned);
-    CUPSO_CUDA(cudaMemcpyAsync(pin, h->dev64.gkey + cur, sizeof(PKey), cudaMemcpyDeviceToHost, h->stream),
-               "cudaMemcpyAsync");
-    CUPSO_CUDA(cudaMemcpyAsync(pin + 16, h->dev64.status, 4, cudaMemcpyDeviceToHost, h->stream), "cudaMemcpyAsync");
-    if (pos_out)
-        CUPSO_CUDA(cudaMemcpyAsync(pin + 32, h->dev64.G + (size_t)cur * h->D, sizeof(double) * (size_t)h->D,
-                                   cudaMemcpyDeviceToHost, h->stream),
-                   "cudaMemcpyAsync");
-    CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    const char* rec = h->rec_copy.data();
     PKey key{};
     unsigned st = 0;
-    std::memcpy(&key, pin, sizeof(PKey));
-    std::memcpy(&st, pin + 16, 4);
-    if (pos_out) std::memcpy(pos_out, pin + 32, sizeof(double) * (size_t)h->D);
+    std::memcpy(&key, rec, sizeof(PKey));
+    std::memcpy(&st, rec + kRecStatus, 4);
+    if (pos_out) std::memcpy(pos_out, rec + kRecPos, sizeof(double) * (size_t)h->D);
     if (fit_out) *fit_out = key_to_fit64(key.k);
     if (idx_out) *idx_out = (int64_t)key.i;
     rc = status_code(st);
@@ -1538,7 +1542,6 @@ int cupso_destroy(cupso_handle h) {
     if (h->rec_host) cudaFreeHost(h->rec_host);
     if (h->arena) cudaFree(h->arena);
     if (h->stage) cudaFree(h->stage);
-    if (h->pinned) cudaFreeHost(h->pinned);
     if (h->capture) cudaStreamDestroy(h->capture);
     if (h->own) cudaStreamDestroy(h->own);
     delete h;

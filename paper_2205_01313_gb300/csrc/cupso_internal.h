@@ -40,7 +40,7 @@ cudaError_t launch_recompute(const SwarmDev& s, uint32_t t, int panel, bool fill
 
 // Pipelined fused step (kernels_pipelined.cu): `stages`-deep cp.async ring.
 bool pipelined_supported(int stages, int D);
-cudaError_t prepare_pipelined(int D);   // raise the dynamic shared-memory limit; call outside capture
+cudaError_t prepare_pipelined(int fid, bool fast);   // raise the dynamic shared-memory limit
 // ppt: particles per thread (4, 2 or 1); a warp takes units of 32 * ppt particles.
 int pipelined_blocks_per_sm(int stages, int fid, int D, int ppt);
 cudaError_t launch_sync_pipelined(const SwarmDev& s, int fid, int stages, int ppt, int grid, cudaStream_t st);
@@ -62,7 +62,7 @@ cudaError_t launch_batch_init(const BatchDev& b, int grid, cudaStream_t st);
 // x, v, pb at ((d / W) * Np + i) * W + d % W, panel width W = 8 or 16, ring
 // depth 3 or 5 panels.
 bool panel_supported(int width, int stages, int D);
-cudaError_t prepare_panel(int D);
+cudaError_t prepare_panel(int fid, bool fast);
 int panel_blocks_per_sm(int width, int stages, int fid, int D);
 // Iterations of one panel launch; more than one is a cooperative launch with a
 // grid barrier per iteration (every CTA resident; see kernels_panel.cu).

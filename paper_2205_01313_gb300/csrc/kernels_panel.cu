@@ -443,6 +443,8 @@ __global__ void __launch_bounds__(kBlock) relayout_kernel(const float* __restric
 
 namespace {
 
+constexpr int kPanelMaxD = 8192;
+
 size_t panel_smem(int stages, int D) {
     return sizeof(float4) * (size_t)stages * 3 * kBlock + sizeof(float) * (size_t)D;
 }
@@ -473,19 +475,21 @@ const void* panel_kernel(int width, int stages, bool fast, int fid) {
 
 bool panel_supported(int width, int stages, int D) {
     return (width == 8 || width == 16) && (stages == 3 || stages == 5) && D % width == 0 &&
-           D / width >= stages - 1 && D <= 8192;
+           D / width >= stages - 1 && D <= kPanelMaxD;
 }
 
-cudaError_t prepare_panel(int D) {
-    for (int width = 8; width <= 16; width += 8)
-        for (int stages = 3; stages <= 5; stages += 2)
-            for (int fast = 0; fast < 2; ++fast)
-                for (int fid = kSphere; fid <= kCubicMax; ++fid) {
-                    cudaError_t e = cudaFuncSetAttribute(panel_kernel(width, stages, fast != 0, fid),
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         (int)panel_smem(stages, D));
-                    if (e != cudaSuccess) return e;
-                }
+// Raises the shared-memory limit of this fitness's kernels to what the largest D
+// needs: the same value for every swarm, so no swarm lowers another's. The fast
+// form always: the grids are sized by its occupancy.
+cudaError_t prepare_panel(int fid, bool fast) {
+    for (int form = fast ? 1 : 0; form <= 1; ++form)
+        for (int width = 8; width <= 16; width += 8)
+            for (int stages = 3; stages <= 5; stages += 2) {
+                const cudaError_t e = cudaFuncSetAttribute(panel_kernel(width, stages, form != 0, fid),
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           (int)panel_smem(stages, kPanelMaxD));
+                if (e != cudaSuccess) return e;
+            }
     return cudaSuccess;
 }
 

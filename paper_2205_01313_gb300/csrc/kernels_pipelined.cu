@@ -264,6 +264,8 @@ __global__ void __launch_bounds__(kBlock) materialize_kernel(const __grid_consta
 
 namespace {
 
+constexpr int kPipelinedMaxD = 8192;
+
 size_t smem_of(int stages, int ppt, int D) {
     return sizeof(float) * (size_t)ppt * (size_t)stages * 6 * kBlock + sizeof(float) * (size_t)D;
 }
@@ -300,20 +302,22 @@ const void* kernel_of(int stages, bool fast, int fid, int ppt) {
 }  // namespace
 
 bool pipelined_supported(int stages, int D) {
-    return (stages == 3 || stages == 4) && (D + 1) / 2 >= stages - 1 && D <= 8192;
+    return (stages == 3 || stages == 4) && (D + 1) / 2 >= stages - 1 && D <= kPipelinedMaxD;
 }
 
-cudaError_t prepare_pipelined(int D) {
-    const int ppts[3] = {4, 2, 1};
-    for (int stages = 3; stages <= 4; ++stages)
-        for (int pi = 0; pi < 3; ++pi)
-            for (int fast = 0; fast < 2; ++fast)
-                for (int fid = kSphere; fid <= kCubicMax; ++fid) {
-                    cudaError_t e = cudaFuncSetAttribute(kernel_of(stages, fast != 0, fid, ppts[pi]),
-                                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         (int)smem_of(stages, ppts[pi], D));
-                    if (e != cudaSuccess) return e;
-                }
+// Raises the shared-memory limit of this fitness's kernels to what the largest D
+// needs: the same value for every swarm, so no swarm lowers another's. The fast
+// form always: the grids are sized by its occupancy.
+cudaError_t prepare_pipelined(int fid, bool fast) {
+    for (int form = fast ? 1 : 0; form <= 1; ++form)
+        for (int stages = 3; stages <= 4; ++stages)
+            for (int ppt : {4, 2, 1}) {
+                const void* k = kernel_of(stages, form != 0, fid, ppt);
+                if (!k) return cudaSuccess;   // the least-squares fitness has none
+                const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           (int)smem_of(stages, ppt, kPipelinedMaxD));
+                if (e != cudaSuccess) return e;
+            }
     return cudaSuccess;
 }
 
