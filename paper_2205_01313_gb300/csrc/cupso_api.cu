@@ -743,6 +743,8 @@ int create_swarm64(int D, int N, const cupso_bounds_f64* b, double w, double c1,
     s.k_hi = order_key64(b->max_pos);
     s.k_vlo = order_key64(-b->max_v);
     s.k_vhi = order_key64(b->max_v);
+    s.k_inf = order_key64((double)INFINITY);
+    s.vlo = -b->max_v;
     h->dev.wait_limit_ns = s.wait_limit_ns;
     h->dev.status = s.status;
     h->pbufs = paper_bufs_at(base + o_paper, h->Np, list_cap);

@@ -117,13 +117,16 @@ __device__ __forceinline__ double c_times_u53(double c, int cexp, uint32_t hi, u
 // Closed clamp to [lo, hi] with a NaN going to lo, as comparisons of the
 // values' order keys (klo, khi: keys of lo, hi). Equal to the floating-point
 // comparison form for every a (-0 and +0 compare equal in both), but it runs
-// on the integer pipes instead of the FP64 one.
-__device__ __forceinline__ double clamp64(double a, double lo, double hi, long long klo, long long khi) {
-    const long long b = __double_as_longlong(a);
-    const long long mag = b & 0x7FFFFFFFFFFFFFFFll;
-    if (mag > 0x7FF0000000000000ll) return lo;
-    const long long k = b >= 0 ? b : -mag;
-    return k < klo ? lo : (k > khi ? hi : a);
+// on the integer pipes instead of the FP64 one -- as long as neither step is
+// written in a way that the compiler turns back into an FP64 instruction: clearing
+// the sign bit becomes one (hence the exclusive or: k = -magnitude for a negative
+// a), and so does a test for NaN against constants (hence kinf, the key of infinity,
+// as a parameter; a NaN lies above it or, with the sign bit, below every other).
+__device__ __forceinline__ double clamp64(double a, double lo, double hi, long long klo, long long khi,
+                                          long long kinf) {
+    const long long b = __double_as_longlong(a), sign = b >> 63;
+    const long long k = (b ^ (sign & 0x7FFFFFFFFFFFFFFFll)) - sign;
+    return k < klo ? lo : (k > khi ? (k > kinf ? lo : hi) : a);
 }
 
 __device__ __forceinline__ unsigned long long fit_key64(double f) {
@@ -158,14 +161,22 @@ struct FitAcc64 {
 // Eq. 1 and Eq. 2 in binary64 with the clamps of Alg. 1 (same order as FP32),
 // from the dimension's Philox words. Products that are exact by construction
 // (w v with w = 1, c r with c a power of two) are formed without the FP64 pipe.
-__device__ __forceinline__ void move_one64(double& x, double& v, double pb, double g, uint4 r, const SwarmDev64& s) {
+template <bool W1>
+__device__ __forceinline__ void move_one64_t(double& x, double& v, double pb, double g, uint4 r, const SwarmDev64& s) {
     const double cognitive = __dsub_rn(pb, x);
     const double social = __dsub_rn(g, x);
-    double vel = s.w_one ? v : __dmul_rn(s.w, v);
+    double vel = W1 ? v : __dmul_rn(s.w, v);
     vel = __fma_rn(c_times_u53(s.c1, s.c1_exp, r.x, r.y), cognitive, vel);
     vel = __fma_rn(c_times_u53(s.c2, s.c2_exp, r.z, r.w), social, vel);
-    v = clamp64(vel, -s.vmax, s.vmax, s.k_vlo, s.k_vhi);
-    x = clamp64(__dadd_rn(x, v), s.lo, s.hi, s.k_lo, s.k_hi);
+    v = clamp64(vel, s.vlo, s.vmax, s.k_vlo, s.k_vhi, s.k_inf);
+    x = clamp64(__dadd_rn(x, v), s.lo, s.hi, s.k_lo, s.k_hi, s.k_inf);
+}
+
+// The two forms apart: as one, the product w v is formed (on the narrow FP64 pipe)
+// and then not used.
+__device__ __forceinline__ void move_one64(double& x, double& v, double pb, double g, uint4 r, const SwarmDev64& s) {
+    if (s.w_one) move_one64_t<true>(x, v, pb, g, r, s);
+    else move_one64_t<false>(x, v, pb, g, r, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -488,8 +499,8 @@ __global__ void __launch_bounds__(kPaperBlock) init64_kernel(const __grid_consta
         FitAcc64<FIT> acc;
         for (int d = 0; d < s.D; ++d) {
             const uint4 r = philox4x32_10(make_uint4((uint32_t)d, i, 0u, s.swarm), s.key0, s.key1);
-            const double x = clamp64(__fma_rn(u53(r.x, r.y), span, s.lo), s.lo, s.hi, s.k_lo, s.k_hi);
-            const double v = clamp64(__fma_rn(u53(r.z, r.w), vspan, -s.vmax), -s.vmax, s.vmax, s.k_vlo, s.k_vhi);
+            const double x = clamp64(__fma_rn(u53(r.x, r.y), span, s.lo), s.lo, s.hi, s.k_lo, s.k_hi, s.k_inf);
+            const double v = clamp64(__fma_rn(u53(r.z, r.w), vspan, -s.vmax), -s.vmax, s.vmax, s.k_vlo, s.k_vhi, s.k_inf);
             const size_t off = (size_t)d * Np + i;
             s.x[off] = x;
             s.v[off] = v;

@@ -56,6 +56,8 @@ struct SwarmDev64 {
     int c1_exp, c2_exp;          // c == 2^k: c r is r with k added to its exponent; else kNoExp
     long long k_lo, k_hi;        // order keys of min_pos, max_pos (clamps as integer compares)
     long long k_vlo, k_vhi;      // order keys of -max_v, max_v
+    long long k_inf;             // order key of infinity
+    double vlo;                  // -max_v
 };
 
 constexpr int kNoExp = 0x7FFF;
