@@ -114,7 +114,8 @@ typedef enum {
                               than one block (N > 256) the trajectory depends on timing. */
     CUPSO_MODE_PERSISTENT = 8 /* double-precision swarms: one cooperative launch runs all iterations of a
                               cupso_step call, a grid-wide barrier per iteration in place of the kernel
-                              boundary (synchronous PSO, one particle per thread) */
+                              boundary (synchronous PSO; SYNC does the same for a call of several
+                              iterations) */
 } cupso_mode;
 
 typedef enum {

@@ -56,6 +56,7 @@ struct cupso_swarm {
     SwarmDev64 dev64{};
     PaperBufs pbufs{};              // one-particle-per-thread designs (QUEUE, QUEUE_LOCK, FP64 modes)
     ResidentBufs rbufs{};           // the resident SYNC kernel's exchange (slots null: it does not fit)
+    Sync64Bufs s64bufs{};           // the FP64 one-launch steps' exchange (slots null: D too large)
     bool onchip64 = false;          // the FP64 swarm fits the on-chip kernel
     int N = 0, D = 0, Np = 0, fid = 0;
     uint64_t seed = 0;
@@ -279,6 +280,22 @@ bool use_resident(const cupso_swarm* h, int mode, int iters) {
     if (mode == CUPSO_MODE_SYNC) return iters >= (h->panel ? 4 : 3);
     if (mode != CUPSO_MODE_ONCHIP || h->mode != CUPSO_MODE_AUTO) return false;
     return h->N >= 1000 ? iters >= 5 : ((long long)h->N * h->D >= 1000 && iters >= 300);
+}
+
+// Whether `iters` iterations of an FP64 swarm run in one cooperative launch
+// (kernels_sync64.cu). Its start and end cost as much as two to five iterations of the
+// kernels with a launch per iteration (SYNC; us per iteration at 2 and 10: 32 x 1 5.6
+// and 2.3 against 4.6 and 4.5, 131072 x 1 10.7 and 6.3 against 9.2, 30000 x 10 at 10
+// 11.9 against 15.8), and more than those of the cluster (AUTO where the swarm
+// fits one: 512 x 1 at 10 and 200 2.4 and 1.55 against 2.3 and 1.8, 8192 x 1 2.6 and
+// 1.6 against 4.7 and 4.2).
+bool use_sync64(const cupso_swarm* h, int mode, int iters) {
+    if (!h->s64bufs.slots) return false;
+    if (mode == CUPSO_MODE_PERSISTENT) return true;
+    if (h->iters_per_launch == 1) return false;
+    const long long pd = (long long)h->N * h->D;
+    if (mode == CUPSO_MODE_SYNC) return iters >= (pd >= (1 << 18) ? 5 : 3);
+    return mode == CUPSO_MODE_ONCHIP && h->mode == CUPSO_MODE_AUTO && iters >= (pd >= 2000 ? 10 : 50);
 }
 
 // CTAs of a multi-iteration panel launch: the SYNC grid, at most what the SMs
@@ -708,11 +725,14 @@ int create_swarm64(int D, int N, const cupso_bounds_f64* b, double w, double c1,
     const int list_cap = h->Np;   // the tiled step may run up to one block per particle
     const size_t o_paper = off; off = align_up(off + paper_bufs_bytes(h->Np, list_cap), A);
     const size_t o_rec = off; off = align_up(off + rec_bytes(D, true), A);
+    const size_t s64_bytes = sync64_bytes(fid, N, D, h->num_sms);
+    const size_t o_s64 = off; off = align_up(off + s64_bytes, A);
     h->arena_bytes = off;
     e = cudaMalloc(&h->arena, h->arena_bytes);
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
     char* base = static_cast<char*>(h->arena);
     h->rec_now = base + o_rec;
+    if (s64_bytes) h->s64bufs = sync64_bufs_at(base + o_s64);
     SwarmDev64& s = h->dev64;
     s.x = reinterpret_cast<double*>(base + o_x);
     s.v = reinterpret_cast<double*>(base + o_v);
@@ -1060,15 +1080,15 @@ int cupso_step(cupso_handle h, int iters) {
         return CUPSO_OK;
     }
     const int mode = resolved_mode(h);
-    if (h->fp64 && mode == CUPSO_MODE_ONCHIP) {
-        cudaError_t e = launch_onchip64(h->dev64, h->fid, iters, h->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "on-chip launch");
+    if (h->fp64 && use_sync64(h, mode, iters)) {
+        cudaError_t e = launch_sync64(h->dev64, h->s64bufs, h->fid, iters, h->num_sms, h->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "one-launch step");
         h->t_host += (uint32_t)iters;
         return CUPSO_OK;
     }
-    if (h->fp64 && mode == CUPSO_MODE_PERSISTENT) {
-        cudaError_t e = launch_persist64(h->dev64, h->pbufs, h->fid, iters, h->num_sms, h->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "persistent launch");
+    if (h->fp64 && mode == CUPSO_MODE_ONCHIP) {
+        cudaError_t e = launch_onchip64(h->dev64, h->fid, iters, h->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "on-chip launch");
         h->t_host += (uint32_t)iters;
         return CUPSO_OK;
     }

@@ -304,6 +304,10 @@ __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long k)
     return k;
 }
 
+// Named barriers of a block: wait with, or count towards, `threads` threads.
+__device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int threads) { asm volatile("barrier.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+
 __device__ __forceinline__ long long global_ns() {
     long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

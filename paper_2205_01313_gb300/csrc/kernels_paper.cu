@@ -30,6 +30,7 @@
 
 #include "cupso_device.cuh"
 #include "cupso_internal.h"
+#include "fp64_common.cuh"
 #include "paper_kernels.h"
 #include "pdl.cuh"
 #include "stream_common.cuh"
@@ -39,44 +40,6 @@ namespace cg = cooperative_groups;
 namespace cupso {
 
 namespace {
-
-// ---------------------------------------------------------------------------
-// Candidate keys
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ PKey key_none() { return PKey{~0ull, kNoIdx, 0u}; }
-
-__device__ __forceinline__ bool key_less(const PKey& a, const PKey& b) {
-    return a.k < b.k || (a.k == b.k && a.i < b.i);
-}
-
-__device__ __forceinline__ PKey warp_min_key(PKey a) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        PKey b;
-        b.k = __shfl_xor_sync(0xFFFFFFFFu, a.k, o);
-        b.i = __shfl_xor_sync(0xFFFFFFFFu, a.i, o);
-        b.pad = 0u;
-        if (key_less(b, a)) a = b;
-    }
-    return a;
-}
-
-// Minimum over the block (every thread returns it). red: >= 32 entries.
-__device__ __forceinline__ PKey block_min_key(PKey k, PKey* red) {
-    k = warp_min_key(k);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = k;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        PKey m = threadIdx.x < (blockDim.x + 31) / 32 ? red[threadIdx.x] : key_none();
-        m = warp_min_key(m);
-        if (threadIdx.x == 0) red[0] = m;
-    }
-    __syncthreads();
-    const PKey r = red[0];
-    __syncthreads();
-    return r;
-}
 
 // Appends a block's candidate to the list; a push beyond the capacity is
 // dropped and reported (launchers never start more blocks than list_cap).
@@ -88,95 +51,6 @@ __device__ __forceinline__ void push_candidate(const PaperBufs& b, const PKey& k
 
 __device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned long long* p) {
     return *reinterpret_cast<const volatile unsigned long long*>(p);
-}
-
-// ---------------------------------------------------------------------------
-// Double precision building blocks
-// ---------------------------------------------------------------------------
-
-// Two words -> (m + 1) 2^-53 with m = hi 2^21 + (lo >> 11), in (0, 1], times
-// 2^k. The double is assembled from integer parts: exponent from the leading
-// bit of v = m + 1 (plus k), the bits below it as the fraction (v <= 2^53, so
-// it is exact; callers keep |k| <= 512, so the result stays normal).
-__device__ __forceinline__ double u53_pow2(uint32_t hi, uint32_t lo, int k) {
-    const unsigned long long v = (((unsigned long long)hi << 21) | (unsigned long long)(lo >> 11)) + 1ull;
-    const int lz = __clzll((long long)v);
-    const unsigned long long frac = ((v << lz) << 1) >> 12;
-    const unsigned long long e = (unsigned long long)(1033 - lz + k);
-    return __longlong_as_double((long long)((e << 52) | frac));
-}
-
-__device__ __forceinline__ double u53(uint32_t hi, uint32_t lo) { return u53_pow2(hi, lo, 0); }
-
-// c * u53(hi, lo), rounded once: an exponent shift when c = 2^k (exact).
-__device__ __forceinline__ double c_times_u53(double c, int cexp, uint32_t hi, uint32_t lo) {
-    if (cexp != kNoExp) return u53_pow2(hi, lo, cexp);
-    return __dmul_rn(c, u53(hi, lo));
-}
-
-// Closed clamp to [lo, hi] with a NaN going to lo, as comparisons of the
-// values' order keys (klo, khi: keys of lo, hi). Equal to the floating-point
-// comparison form for every a (-0 and +0 compare equal in both), but it runs
-// on the integer pipes instead of the FP64 one -- as long as neither step is
-// written in a way that the compiler turns back into an FP64 instruction: clearing
-// the sign bit becomes one (hence the exclusive or: k = -magnitude for a negative
-// a), and so does a test for NaN against constants (hence kinf, the key of infinity,
-// as a parameter; a NaN lies above it or, with the sign bit, below every other).
-__device__ __forceinline__ double clamp64(double a, double lo, double hi, long long klo, long long khi,
-                                          long long kinf) {
-    const long long b = __double_as_longlong(a), sign = b >> 63;
-    const long long k = (b ^ (sign & 0x7FFFFFFFFFFFFFFFll)) - sign;
-    return k < klo ? lo : (k > khi ? (k > kinf ? lo : hi) : a);
-}
-
-__device__ __forceinline__ unsigned long long fit_key64(double f) {
-    if (f != f) return ~0ull;
-    unsigned long long b = (unsigned long long)__double_as_longlong(f);
-    if ((b << 1) == 0ull) b = 0ull;  // -0 -> +0
-    return (b >> 63) ? ~b : (b | (1ull << 63));
-}
-
-template <int FIT>
-struct FitAcc64 {
-    double acc = 0.0;
-    double prev = 0.0;
-    __device__ __forceinline__ void add(int d, double x) {
-        if constexpr (FIT == kSphere) {
-            acc = __fma_rn(x, x, acc);
-        } else if constexpr (FIT == kRosenbrock) {
-            if (d > 0) {
-                const double p = __fma_rn(-prev, prev, x);
-                const double q = __dsub_rn(1.0, prev);
-                acc = __dadd_rn(acc, __fma_rn(__dmul_rn(100.0, p), p, __dmul_rn(q, q)));
-            }
-            prev = x;
-        } else if constexpr (FIT == kCubicMax) {
-            const double h = __fma_rn(__fma_rn(__dsub_rn(x, 0.8), x, -1000.0), x, 8000.0);
-            acc = __dadd_rn(acc, h);
-        }
-    }
-    __device__ __forceinline__ double finish() const { return FIT == kCubicMax ? -acc : acc; }
-};
-
-// Eq. 1 and Eq. 2 in binary64 with the clamps of Alg. 1 (same order as FP32),
-// from the dimension's Philox words. Products that are exact by construction
-// (w v with w = 1, c r with c a power of two) are formed without the FP64 pipe.
-template <bool W1>
-__device__ __forceinline__ void move_one64_t(double& x, double& v, double pb, double g, uint4 r, const SwarmDev64& s) {
-    const double cognitive = __dsub_rn(pb, x);
-    const double social = __dsub_rn(g, x);
-    double vel = W1 ? v : __dmul_rn(s.w, v);
-    vel = __fma_rn(c_times_u53(s.c1, s.c1_exp, r.x, r.y), cognitive, vel);
-    vel = __fma_rn(c_times_u53(s.c2, s.c2_exp, r.z, r.w), social, vel);
-    v = clamp64(vel, s.vlo, s.vmax, s.k_vlo, s.k_vhi, s.k_inf);
-    x = clamp64(__dadd_rn(x, v), s.lo, s.hi, s.k_lo, s.k_hi, s.k_inf);
-}
-
-// The two forms apart: as one, the product w v is formed (on the narrow FP64 pipe)
-// and then not used.
-__device__ __forceinline__ void move_one64(double& x, double& v, double pb, double g, uint4 r, const SwarmDev64& s) {
-    if (s.w_one) move_one64_t<true>(x, v, pb, g, r, s);
-    else move_one64_t<false>(x, v, pb, g, r, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -534,43 +408,6 @@ __global__ void __launch_bounds__(kPaperBlock) pbest_min64_kernel(const __grid_c
 }
 
 // ---------------------------------------------------------------------------
-// Fitness from per-dimension terms, for the kernels that spread a particle's
-// dimensions over threads: the terms are formed in parallel, then one thread
-// per particle adds them in order d = 0 .. D-1 (the same operations, in the
-// same order, as FitAcc64).
-// ---------------------------------------------------------------------------
-template <int FIT>
-struct FitTerms64 {
-    static constexpr bool kNeedsNext = (FIT == kRosenbrock);
-    // term of dimension d (x = x_d, xn = x_{d+1}); Rosenbrock: d < D - 1 only
-    __device__ static __forceinline__ double term(double x, double xn) {
-        if constexpr (FIT == kCubicMax) {
-            return __fma_rn(__fma_rn(__dsub_rn(x, 0.8), x, -1000.0), x, 8000.0);
-        } else if constexpr (FIT == kRosenbrock) {
-            const double p = __fma_rn(-x, x, xn);
-            const double q = __dsub_rn(1.0, x);
-            return __fma_rn(__dmul_rn(100.0, p), p, __dmul_rn(q, q));
-        } else {
-            return 0.0;   // sphere: the sum fuses x * x, no separate term
-        }
-    }
-    // sequential sum over d of particle column p (stride P) of X / H
-    __device__ static __forceinline__ double sum(const double* X, const double* H, int P, int p, int D) {
-        double acc = 0.0;
-        if constexpr (FIT == kSphere) {
-            for (int d = 0; d < D; ++d) {
-                const double x = X[(size_t)d * P + p];
-                acc = __fma_rn(x, x, acc);
-            }
-        } else {
-            const int n = FIT == kRosenbrock ? D - 1 : D;
-            for (int d = 0; d < n; ++d) acc = __dadd_rn(acc, H[(size_t)d * P + p]);
-        }
-        return FIT == kCubicMax ? -acc : acc;
-    }
-};
-
-// ---------------------------------------------------------------------------
 // On-chip FP64 swarm: a cluster of C CTAs (1 <= C <= 16). CTA r keeps the
 // particles [r P, r P + n_r) -- x, v, pbest_pos and the fitness terms
 // ([D][P]), pbest_fit and its copy of gbest -- in shared memory for `iters`
@@ -868,301 +705,6 @@ int tile_particles(int N, int D, int num_sms) {
     return P;
 }
 
-// ---------------------------------------------------------------------------
-// Persistent FP64 swarm (a cooperative launch, so every block is resident):
-// `iters` iterations, each ending with a grid barrier instead of a kernel
-// boundary. A block's Step-5 candidate goes to its own slot of a list
-// double-buffered by parity; after the barrier every block reduces the same
-// slots in the same order, so all hold the same gbest.
-// ---------------------------------------------------------------------------
-constexpr int kPersistThreads = 128;
-
-// Bounded grid barrier: thread 0 of every block arrives on a counter; the last
-// one resets it and advances the generation the others wait on. A wait past
-// the limit sets the timeout status and returns false.
-__device__ bool grid_barrier(const PaperBufs& b, unsigned int nblocks, long long limit_ns, unsigned int* status) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        const unsigned int g = *reinterpret_cast<volatile unsigned int*>(b.bar_gen);
-        __threadfence();
-        if (atomicAdd(b.bar_count, 1u) == nblocks - 1u) {
-            *reinterpret_cast<volatile unsigned int*>(b.bar_count) = 0u;
-            __threadfence();
-            atomicAdd(b.bar_gen, 1u);
-        } else {
-            const long long deadline = global_ns() + limit_ns;
-            while (*reinterpret_cast<volatile unsigned int*>(b.bar_gen) == g) {
-                if (global_ns() > deadline) {
-                    ok = 0;
-                    atomicOr(status, kStatusTimeout);
-                    break;
-                }
-                __nanosleep(32);
-            }
-        }
-        __threadfence();
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
-template <int FIT>
-__global__ void __launch_bounds__(kPersistThreads) persist64_kernel(const __grid_constant__ SwarmDev64 s,
-                                                                   const __grid_constant__ PaperBufs b, int iters) {
-    extern __shared__ double Gsh[];   // [D] the current gbest
-    __shared__ PKey red[32];
-    const int tid = threadIdx.x;
-    const size_t Np = (size_t)s.Np;
-    const unsigned int nblk = gridDim.x;
-    const uint32_t stride = nblk * blockDim.x;
-    const uint32_t t_prev = __ldcg(s.t_dev);
-    const int cur0 = (int)(t_prev & 1u);
-    PKey K = Fp64::load_gkey(s, cur0);
-    for (int d = tid; d < s.D; d += blockDim.x) Gsh[d] = s.G[(size_t)cur0 * s.D + d];
-    __syncthreads();
-    bool nan = false;
-    int done = 0;
-    for (int k = 0; k < iters; ++k) {
-        const uint32_t t = t_prev + 1u + (uint32_t)k;
-        PKey cand = key_none();
-        for (uint32_t i = blockIdx.x * blockDim.x + tid; i < (uint32_t)s.N; i += stride) {
-            const double f = Fp64::step_particle<FIT>(s, i, t, Gsh);   // Steps 2-3
-            nan |= (f != f);
-            if (f < s.pf[i]) {                                          // Step 4
-                s.pf[i] = f;
-                for (int d = 0; d < s.D; ++d) s.pb[(size_t)d * Np + i] = s.x[(size_t)d * Np + i];
-                const PKey c = Fp64::key(f, i);
-                if (key_less(c, K) && key_less(c, cand)) cand = c;
-            }
-        }
-        const PKey mine = block_min_key(cand, red);
-        PKey* slots = b.list + (size_t)(k & 1) * nblk;
-        if (tid == 0) {
-            slots[blockIdx.x].k = mine.k;
-            slots[blockIdx.x].i = mine.i;
-        }
-        if (!grid_barrier(b, nblk, s.wait_limit_ns, s.status)) break;
-        // Step 5: the same reduction in every block
-        PKey m = K;
-        for (unsigned int j = tid; j < nblk; j += blockDim.x) {
-            PKey c;
-            c.k = __ldcg(&slots[j].k);
-            c.i = __ldcg(&slots[j].i);
-            c.pad = 0u;
-            if (key_less(c, m)) m = c;
-        }
-        const PKey nbest = block_min_key(m, red);
-        if (key_less(nbest, K)) {
-            K = nbest;
-            for (int d = tid; d < s.D; d += blockDim.x) Gsh[d] = __ldcg(s.pb + (size_t)d * Np + nbest.i);
-        }
-        __syncthreads();
-        done = k + 1;
-    }
-    if (__syncthreads_or(nan) && tid == 0) atomicOr(s.status, kStatusNaN);
-    if (blockIdx.x == 0) {
-        const uint32_t t_end = t_prev + (uint32_t)done;
-        const int out = (int)(t_end & 1u);
-        for (int d = tid; d < s.D; d += blockDim.x) s.G[(size_t)out * s.D + d] = Gsh[d];
-        if (tid == 0) {
-            Fp64::store_gkey(s, 0, K);
-            Fp64::store_gkey(s, 1, K);
-            *s.t_dev = t_end;
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Resident variant of the persistent FP64 swarm, for swarms of at most one
-// particle per thread: x, v and pbest_pos stay in shared memory ([D][TB]) and
-// pbest_fit in a register for all iterations of the launch, so an iteration
-// touches global memory only for the Step-5 exchange. A block's candidate goes
-// to its slot together with its position (index first, position after, as in
-// Sec. 4.3); after the barrier every block reduces the same slots in the same
-// order, and for D <= kResPos the position travels with the key in that one
-// pass over the slots.
-// ---------------------------------------------------------------------------
-constexpr int kResPos = 4;
-constexpr int kResMaxIters = 1 << 24;   // per launch: (k + 1) * blocks stays below 2^32
-
-__device__ __forceinline__ unsigned int add_release_gpu(unsigned int* p, unsigned int v) {
-    unsigned int old;
-    asm volatile("atom.add.release.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-    return old;
-}
-__device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Bounded grid barrier number k of a launch that started with the counter at
-// zero: thread 0 of every block adds one arrival, and barrier k is complete
-// once all blocks have arrived k + 1 times. One atomic per block, no reset and
-// no generation word to read first. The arrival releases the block's writes
-// (ordered before it by the block barrier) and the wait acquires the others'.
-// A wait past the limit sets the timeout status and returns false.
-__device__ bool grid_barrier_k(const PaperBufs& b, unsigned int nblocks, int k, long long limit_ns,
-                               unsigned int* status) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        const unsigned int target = (unsigned int)(k + 1) * nblocks;
-        if (add_release_gpu(b.bar_count, 1u) + 1u < target) {
-            const long long deadline = global_ns() + limit_ns;
-            while (ld_acquire_gpu(b.bar_count) < target) {
-                if (global_ns() > deadline) {
-                    ok = 0;
-                    atomicOr(status, kStatusTimeout);
-                    break;
-                }
-            }
-        } else {
-            (void)ld_acquire_gpu(b.bar_count);   // the last arrival acquires too
-        }
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
-__host__ __device__ inline size_t res_slot_bytes(int D) { return (sizeof(PKey) + sizeof(double) * (size_t)D + 15) / 16 * 16; }
-
-template <int FIT>
-__global__ void __launch_bounds__(512) persist64r_kernel(const __grid_constant__ SwarmDev64 s,
-                                                          const __grid_constant__ PaperBufs b, int iters) {
-    extern __shared__ double sm64[];
-    __shared__ PKey red[32];
-    const int TB = (int)blockDim.x, D = s.D, tid = threadIdx.x;
-    double* X = sm64;                       // [D][TB]
-    double* V = X + (size_t)D * TB;
-    double* PB = V + (size_t)D * TB;
-    double* Gsh = PB + (size_t)D * TB;      // [D] the current gbest
-    const unsigned int nblk = gridDim.x;
-    const uint32_t i = blockIdx.x * (uint32_t)TB + (uint32_t)tid;
-    const bool own = i < (uint32_t)s.N;
-    const size_t Np = (size_t)s.Np;
-    const size_t rec = res_slot_bytes(D);
-    unsigned char* slots = reinterpret_cast<unsigned char*>(b.list);
-    const uint32_t t_prev = __ldcg(s.t_dev);
-    const int cur0 = (int)(t_prev & 1u);
-    PKey K = Fp64::load_gkey(s, cur0);
-    for (int d = tid; d < D; d += TB) Gsh[d] = s.G[(size_t)cur0 * D + d];
-    double pf = 0.0;
-    if (own) {
-        pf = s.pf[i];
-        for (int d = 0; d < D; ++d) {
-            const size_t g = (size_t)d * Np + i;
-            X[d * TB + tid] = s.x[g];
-            V[d * TB + tid] = s.v[g];
-            PB[d * TB + tid] = s.pb[g];
-        }
-    }
-    __syncthreads();
-    bool nan = false;
-    int done = 0;
-    for (int k = 0; k < iters; ++k) {
-        const uint32_t t = t_prev + 1u + (uint32_t)k;
-        PKey cand = key_none();
-        if (own) {   // Steps 2-4 of this thread's particle
-            FitAcc64<FIT> acc;
-            for (int d = 0; d < D; ++d) {
-                const uint4 r = philox4x32_10(make_uint4((uint32_t)d, i, t, s.swarm), s.key0, s.key1);
-                const int j = d * TB + tid;
-                double x = X[j], v = V[j];
-                move_one64(x, v, PB[j], Gsh[d], r, s);
-                X[j] = x;
-                V[j] = v;
-                acc.add(d, x);
-            }
-            const double f = acc.finish();
-            nan |= (f != f);
-            if (f < pf) {
-                pf = f;
-                for (int d = 0; d < D; ++d) PB[d * TB + tid] = X[d * TB + tid];
-                const PKey c = Fp64::key(f, i);
-                if (key_less(c, K)) cand = c;
-            }
-        }
-        const PKey best = block_min_key(cand, red);
-        unsigned char* mine = slots + ((size_t)(k & 1) * nblk + blockIdx.x) * rec;
-        if (best.i == kNoIdx) {
-            if (tid == 0) *reinterpret_cast<PKey*>(mine) = key_none();
-        } else if (best.i == i) {   // the candidate's own thread fills the slot
-            double* pos = reinterpret_cast<double*>(mine + sizeof(PKey));
-            for (int d = 0; d < D; ++d) pos[d] = PB[d * TB + tid];
-            *reinterpret_cast<PKey*>(mine) = best;
-        }
-        if (!grid_barrier_k(b, nblk, k, s.wait_limit_ns, s.status)) break;
-        // Step 5: the same reduction over the slots in every block
-        PKey m = K;
-        int mj = -1;
-        double mpos[kResPos];
-        for (unsigned int j = tid; j < nblk; j += TB) {
-            const unsigned char* sl = slots + ((size_t)(k & 1) * nblk + j) * rec;
-            const PKey* pk = reinterpret_cast<const PKey*>(sl);
-            PKey c;
-            c.k = __ldcg(&pk->k);
-            c.i = __ldcg(&pk->i);
-            c.pad = 0u;
-            double q[kResPos];
-            if (D <= kResPos) {
-#pragma unroll
-                for (int d = 0; d < kResPos; ++d)
-                    q[d] = d < D ? __ldcg(reinterpret_cast<const double*>(sl + sizeof(PKey)) + d) : 0.0;
-            }
-            if (key_less(c, m)) {
-                m = c;
-                mj = (int)j;
-#pragma unroll
-                for (int d = 0; d < kResPos; ++d) mpos[d] = D <= kResPos ? q[d] : 0.0;
-            }
-        }
-        const PKey nbest = block_min_key(m, red);
-        if (key_less(nbest, K)) {
-            // the thread that read the winning slot brings its position
-            if (mj >= 0 && m.i == nbest.i && m.k == nbest.k) {
-                if (D <= kResPos) {
-#pragma unroll
-                    for (int d = 0; d < kResPos; ++d)
-                        if (d < D) Gsh[d] = mpos[d];
-                } else {
-                    const double* pos =
-                        reinterpret_cast<const double*>(slots + ((size_t)(k & 1) * nblk + mj) * rec + sizeof(PKey));
-                    for (int d = 0; d < D; ++d) Gsh[d] = __ldcg(pos + d);
-                }
-            }
-            K = nbest;
-        }
-        __syncthreads();
-        done = k + 1;
-    }
-    if (own) {
-        s.pf[i] = pf;
-        for (int d = 0; d < D; ++d) {
-            const size_t g = (size_t)d * Np + i;
-            s.x[g] = X[d * TB + tid];
-            s.v[g] = V[d * TB + tid];
-            s.pb[g] = PB[d * TB + tid];
-        }
-    }
-    if (__syncthreads_or(nan) && tid == 0) atomicOr(s.status, kStatusNaN);
-    if (blockIdx.x == 0) {
-        const uint32_t t_end = t_prev + (uint32_t)done;
-        const int out = (int)(t_end & 1u);
-        for (int d = tid; d < D; d += TB) s.G[(size_t)out * D + d] = Gsh[d];
-        if (tid == 0) {
-            Fp64::store_gkey(s, 0, K);
-            Fp64::store_gkey(s, 1, K);
-            *s.t_dev = t_end;
-        }
-    }
-}
-
 #define CUPSO_DISPATCH_FIT32(fid, CALL)            \
     switch (fid) {                                 \
         case kSphere: { constexpr int F = kSphere; CALL; break; }         \
@@ -1203,8 +745,6 @@ PaperBufs paper_bufs_at(void* base, int Np, int list_cap) {
     b.lock = w;
     b.ticket = w + 1;
     b.list_n = w + 2;
-    b.bar_count = w + 3;
-    b.bar_gen = w + 4;
     return b;
 }
 
@@ -1270,104 +810,6 @@ cudaError_t launch_step64(const SwarmDev64& s, const PaperBufs& b, int fid, int 
             CUPSO_DISPATCH_FIT64(fid, return launch_pdl(paper_step_kernel<Fp64, F, kAggQueueLock>, g1, b1, 0, st, s, b));
         case kAggSyncList:
             CUPSO_DISPATCH_FIT64(fid, return launch_pdl(paper_step_kernel<Fp64, F, kAggSyncList>, g1, b1, 0, st, s, b));
-        default:
-            return cudaErrorInvalidValue;
-    }
-}
-
-int persist64_grid(int fid, int N, int D, int num_sms) {
-    int per_sm = 0;
-    const size_t smem = sizeof(double) * (size_t)D;
-    cudaError_t e = cudaErrorInvalidValue;
-    switch (fid) {
-        case kSphere: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persist64_kernel<kSphere>, kPersistThreads, smem); break;
-        case kRosenbrock: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persist64_kernel<kRosenbrock>, kPersistThreads, smem); break;
-        case kCubicMax: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persist64_kernel<kCubicMax>, kPersistThreads, smem); break;
-        default: break;
-    }
-    if (e != cudaSuccess || per_sm < 1) {
-        cudaGetLastError();
-        per_sm = 1;
-    }
-    const long long want = ((long long)N + kPersistThreads - 1) / kPersistThreads;
-    const long long cap = (long long)per_sm * num_sms;
-    return (int)(want < cap ? want : cap);
-}
-
-namespace {
-
-const void* persist64r_fn(int fid) {
-    switch (fid) {
-        case kSphere: return (const void*)persist64r_kernel<kSphere>;
-        case kRosenbrock: return (const void*)persist64r_kernel<kRosenbrock>;
-        case kCubicMax: return (const void*)persist64r_kernel<kCubicMax>;
-        default: return nullptr;
-    }
-}
-
-// Threads per block of the resident variant (one particle each, at most one
-// block per SM, block size from 128 doubling to 512), or 0 where it does not
-// apply: too many particles, state over 48 KB per block, slots beyond the
-// candidate list, or blocks that cannot all be resident.
-int persist64r_block(int fid, int N, int D, int num_sms, unsigned int list_cap) {
-    int tb = 128;
-    while ((N + tb - 1) / tb > num_sms && tb < 512) tb *= 2;
-    const int nblk = (N + tb - 1) / tb;
-    if (nblk > num_sms) return 0;
-    const size_t smem = sizeof(double) * (3 * (size_t)D * tb + (size_t)D);
-    if (smem > 48 * 1024) return 0;
-    if (2 * (size_t)nblk * res_slot_bytes(D) > sizeof(PKey) * (size_t)list_cap) return 0;
-    const void* fn = persist64r_fn(fid);
-    int per_sm = 0;
-    if (!fn || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, tb, smem) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
-    return (long long)per_sm * num_sms >= nblk ? tb : 0;
-}
-
-}  // namespace
-
-cudaError_t launch_persist64(const SwarmDev64& s, const PaperBufs& b, int fid, int iters, int num_sms,
-                             cudaStream_t st) {
-    if (s.D > 4096) return cudaErrorInvalidValue;
-    if (const int tb = persist64r_block(fid, s.N, s.D, num_sms, b.list_cap)) {
-        const int nblk = (s.N + tb - 1) / tb;
-        const size_t smem = sizeof(double) * (3 * (size_t)s.D * tb + (size_t)s.D);
-        for (int left = iters; left > 0;) {
-            // the barrier counter starts every launch at zero
-            cudaError_t me = cudaMemsetAsync(b.bar_count, 0, sizeof(unsigned int), st);
-            if (me != cudaSuccess) return me;
-            int iters_arg = left < kResMaxIters ? left : kResMaxIters;
-            left -= iters_arg;
-            SwarmDev64 s_arg = s;
-            PaperBufs b_arg = b;
-            void* args[] = {&s_arg, &b_arg, &iters_arg};
-            cudaError_t e = cudaLaunchCooperativeKernel(persist64r_fn(fid), dim3(nblk), dim3(tb), args, smem, st);
-            if (e != cudaSuccess) return e;
-        }
-        return cudaSuccess;
-    }
-    const int grid = persist64_grid(fid, s.N, s.D, num_sms);
-    if (2u * (unsigned)grid > b.list_cap) return cudaErrorInvalidConfiguration;
-    // a barrier abandoned by a timed-out launch must not leave arrivals behind
-    cudaError_t me = cudaMemsetAsync(b.bar_count, 0, sizeof(unsigned int), st);
-    if (me != cudaSuccess) return me;
-    const size_t smem = sizeof(double) * (size_t)s.D;
-    int iters_arg = iters;
-    SwarmDev64 s_arg = s;
-    PaperBufs b_arg = b;
-    void* args[] = {&s_arg, &b_arg, &iters_arg};
-    switch (fid) {
-        case kSphere:
-            return cudaLaunchCooperativeKernel((const void*)persist64_kernel<kSphere>, dim3(grid), dim3(kPersistThreads),
-                                               args, smem, st);
-        case kRosenbrock:
-            return cudaLaunchCooperativeKernel((const void*)persist64_kernel<kRosenbrock>, dim3(grid),
-                                               dim3(kPersistThreads), args, smem, st);
-        case kCubicMax:
-            return cudaLaunchCooperativeKernel((const void*)persist64_kernel<kCubicMax>, dim3(grid),
-                                               dim3(kPersistThreads), args, smem, st);
         default:
             return cudaErrorInvalidValue;
     }

@@ -123,9 +123,6 @@ __device__ __forceinline__ float row_fitness(const float* X, const float* H, int
     return a.finish(D);
 }
 
-__device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
-__device__ __forceinline__ void bar_arrive(int id, int threads) { asm volatile("barrier.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
-
 }  // namespace
 
 // P particles per CTA, blockDim.x >= P * rows in whole warps, ITEMS * rows >=

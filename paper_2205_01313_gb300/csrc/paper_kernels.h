@@ -32,8 +32,6 @@ struct PaperBufs {
     unsigned int* ticket;  // last-block counter of the one-kernel variants
     unsigned int* list_n;  // entries in `list`
     unsigned int list_cap; // capacity of `list`: no launch may have more blocks
-    unsigned int* bar_count;  // grid barrier of the persistent kernel: arrivals
-    unsigned int* bar_gen;    // and generation
 };
 
 // Device state of a double-precision swarm. Same layouts as SwarmDev:
@@ -99,13 +97,17 @@ cudaError_t launch_init64(const SwarmDev64& s, const PaperBufs& b, int fid, cuda
 // particle's dimensions over threads; num_sms sizes its tiles.
 cudaError_t launch_step64(const SwarmDev64& s, const PaperBufs& b, int fid, int agg, int num_sms, cudaStream_t st);
 cudaError_t launch_recompute64(const SwarmDev64& s, const PaperBufs& b, cudaStream_t st);
-// Persistent FP64 swarm: one cooperative launch runs `iters` synchronous
-// iterations, one particle per thread (looping when N exceeds the resident
-// threads), with a bounded grid barrier per iteration in place of the kernel
-// boundary.
-cudaError_t launch_persist64(const SwarmDev64& s, const PaperBufs& b, int fid, int iters, int num_sms,
-                             cudaStream_t st);
-int persist64_grid(int fid, int N, int D, int num_sms);
+// `iters` synchronous iterations in one cooperative launch (kernels_sync64.cu): the
+// swarm in registers where it fits, else in memory. Any N; D up to what one
+// particle's terms take of an SM's shared memory (sync64_bytes is 0 beyond).
+struct Sync64Bufs {
+    unsigned long long* bar = nullptr;   // arrivals and candidate counts
+    unsigned char* slots = nullptr;      // [2][grid] candidates: key, position
+};
+__host__ __device__ inline size_t sync64_slot_bytes(int D) { return (sizeof(PKey) + sizeof(double) * (size_t)D + 15) / 16 * 16; }
+size_t sync64_bytes(int fid, int N, int D, int num_sms);
+Sync64Bufs sync64_bufs_at(void* base);
+cudaError_t launch_sync64(const SwarmDev64& s, const Sync64Bufs& rb, int fid, int iters, int num_sms, cudaStream_t st);
 
 // On-chip FP64 swarm: the whole swarm in the shared memory of one CTA cluster
 // (1 to 16 CTAs, chosen from (N, D) by onchip64_cluster), `iters` iterations
