@@ -35,7 +35,8 @@ DEFAULT_WORKLOAD = "rosenbrock_1048576x64"
 FALLBACK_HBM_GBS = 6800.0
 # Every file compiled into the benchmark's kernel (sync_panel_kernel): a
 # stored traffic figure is only used while their hash is unchanged.
-KERNEL_SOURCES = ["paper_2205_01313_gb300/csrc/kernels_panel.cu", "paper_2205_01313_gb300/csrc/stream_common.cuh",
+KERNEL_SOURCES = ["paper_2205_01313_gb300/csrc/kernels_panel.cu", "paper_2205_01313_gb300/csrc/panel_common.cuh",
+                  "paper_2205_01313_gb300/csrc/stream_common.cuh",
                   "paper_2205_01313_gb300/csrc/cupso_device.cuh", "paper_2205_01313_gb300/csrc/cupso_internal.h"]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic_sync_panel_kernel.json")
 

@@ -1,10 +1,12 @@
 // cupso_batch.cu -- cupso_solve_batch: many independent swarms at once.
 //
-// All swarms of a batch live in one device arena. One launch runs Step 1 of
-// every swarm (batch_init_kernel), then every iteration is ONE launch of
-// batch_step_kernel covering the units of all swarms (kernels_batch.cu); the
+// All swarms of a batch live in one device arena. Swarms of kBatchPanelMinD
+// dimensions or more are kept in panels and advance together, one launch per
+// iteration (kernels_batch_panel.cu). The others have a launch of their own: one
+// runs Step 1 of every swarm (batch_init_kernel), then every iteration is ONE launch
+// of batch_step_kernel covering the units of all of them (kernels_batch.cu). The
 // `iters` launches are replayed from captured CUDA graphs. Two kernels can
-// run the step: the streaming one (kernels_batch.cu: 128-particle units per
+// run the step of the swarms that are not in panels: the streaming one (kernels_batch.cu: 128-particle units per
 // warp, rows staged through a cp.async ring) and the tiled one
 // (kernels_tiled.cu: tiles of P particles with all their dimensions per CTA,
 // P chosen per swarm so that tiles cost about the same). The launch shape
@@ -40,15 +42,29 @@ namespace {
 size_t up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Shape {
-    int stages;          // ring depth of the streaming kernel; 0: the tiled kernel
+    int stages;          // ring depth of the streaming kernel; 0: the tiled kernel; -1: the panels'
     int minb;            // register budget: CTAs per SM
-    int blocks_per_sm;   // CTAs per SM launched
+    int blocks_per_sm;   // CTAs per SM launched (the panels' kernel: CTAs in all)
 };
 
 // Launch shapes remembered per batch signature.
 std::mutex g_tune_mutex;
 std::map<std::tuple<int, long long, int, int>, Shape> g_tuned;
 
+// BatchSwarm::cst from the other fields.
+void set_constants(BatchSwarm& w) {
+    uint32_t rk0[10], rk1[10];
+    philox_round_keys(w.key0, w.key1, rk0, rk1);
+    for (int k = 0; k < 5; ++k) w.cst[k] = make_uint4(rk0[2 * k], rk1[2 * k], rk0[2 * k + 1], rk1[2 * k + 1]);
+    const float m[6] = {w.w, w.fast ? w.c1s : w.c1, w.fast ? w.c2s : w.c2, w.vmax, w.lo, w.hi};
+    uint32_t u[6];
+    std::memcpy(u, m, sizeof u);
+    w.cst[5] = make_uint4(u[0], u[1], u[2], u[3]);
+    w.cst[6] = make_uint4(u[4], u[5], w.swarm, 0u);
+    w.cst[7] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// The swarms that advance in one launch.
 struct BatchRun {
     cudaStream_t st = nullptr;
     BatchDev dev{};
@@ -65,6 +81,7 @@ struct BatchRun {
     cudaError_t launch(const Shape& sh) { return launch_on(sh, st); }
 
     cudaError_t launch_on(const Shape& sh, cudaStream_t s) {
+        if (sh.stages < 0) return launch_batch_panel(dev, sh.blocks_per_sm, s);
         if (sh.stages == 0) return launch_batch_tiled(dev, tiles, num_sms * sh.blocks_per_sm, s);
         return launch_batch_step(dev, sh.stages, sh.minb, num_sms * sh.blocks_per_sm, s);
     }
@@ -148,8 +165,9 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
     }
     if (n_swarms == 0) return CUPSO_OK;
 
-    BatchRun run;
-    cudaStream_t own = nullptr;
+    BatchRun run, prun;   // the swarms with a launch of their own, those in panels
+    cudaStream_t own = nullptr, side = nullptr;
+    cudaEvent_t handover = nullptr;
     if (cuda_stream) {
         run.st = static_cast<cudaStream_t>(cuda_stream);
     } else {
@@ -179,10 +197,38 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&run.num_sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess) e = prepare_batch();
+        if (e == cudaSuccess) e = prepare_batch_panel();
         if (e != cudaSuccess) { set_cuda_error(e, "batch setup"); rc = CUPSO_ERR_CUDA; break; }
 
         // Arena: per-swarm planes, then gbest positions, keys, words, flags, descriptors, units, counters.
+        // CUPSO_BATCH_KERNEL=tiled|streaming keeps every swarm out of the panels and fixes
+        // the kernel (for tests and measurements; all kernels give the same bits).
+        const char* force = std::getenv("CUPSO_BATCH_KERNEL");
+        const bool want_tiled = force && std::strcmp(force, "tiled") == 0;
+        const bool want_stream = force && std::strcmp(force, "streaming") == 0;
         const size_t A = 256;
+        // Panels from kBatchPanelMinD dimensions (the ring's look-ahead) to 65,536
+        // particles: 16 swarms of 50,000 x 128 take 378 us an iteration there and 413 out of
+        // them, 8 of 100,000 x 96 317 and 311 (with the limit on D
+        // it also keeps offsets of 16 bytes in 32 bits). And not where particles are too few to fill the chip and the dimensions
+        // many: a particle's panels follow one another, about 0.9 us each, where the tiled
+        // kernel spreads them over a CTA -- 256 dimensions, 4,000 particles in all: 26.5 us
+        // and 20.9; 8,000: 28.3 and 34.4; 64 dimensions: 11.4 and 17.7.
+        std::vector<char> panel(nb);
+        long long panel_pd = 0;
+        int panel_maxD = 0;
+        for (int j = 0; j < nb; ++j) {
+            const cupso_problem& p = problems[batched[j]];
+            panel[j] = !want_tiled && !want_stream && p.D >= kBatchPanelMinD && p.D <= 65536 &&
+                       p.N <= 65536;
+            if (!panel[j]) continue;
+            panel_pd += (long long)p.N * p.D;
+            panel_maxD = std::max(panel_maxD, p.D);
+        }
+        if (panel_maxD > 64 && panel_pd < 6144ll * panel_maxD) panel.assign(nb, 0);
+        std::vector<int> rows(nb);   // dimensions the state has room for
+        size_t panel_units = 0;
+        int nlegacy = 0;
         std::vector<size_t> o_state(nb), o_G(nb), o_flag(nb);
         std::vector<int> Np(nb);
         size_t off = 0, total_units = 0, sumG = 0, sumFlag = 0, total_tiles = 0;
@@ -193,12 +239,18 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
         for (int j = 0; j < nb; ++j) {
             const cupso_problem& p = problems[batched[j]];
             Np[j] = (p.N + kPad - 1) / kPad * kPad;
+            rows[j] = panel[j] ? (p.D + 7) / 8 * 8 : p.D;
             o_state[j] = off;
-            off = up(off + sizeof(float) * ((size_t)3 * p.D * Np[j] + Np[j]), A);
-            o_G[j] = sumG;
-            sumG += 2 * (size_t)p.D;
+            off = up(off + sizeof(float) * ((size_t)3 * rows[j] * Np[j] + Np[j]), A);
+            o_G[j] = sumG = up(sumG, 4);   // 16-byte rows
+            sumG += 2 * (size_t)rows[j];
             o_flag[j] = sumFlag;
             sumFlag += (size_t)Np[j];
+            if (panel[j]) {
+                panel_units += (size_t)Np[j] / 16;
+                continue;
+            }
+            ++nlegacy;
             total_units += (size_t)Np[j] / 128;
             tileP[j] = batch_tile_particles(p.D);
             ntiles[j] = tileP[j] > 0 ? (unsigned)((p.N + tileP[j] - 1) / tileP[j]) : 0u;
@@ -213,10 +265,11 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
         const size_t o_flags = off; off = up(off + sumFlag, A);
         const size_t o_desc = off; off = up(off + sizeof(BatchSwarm) * nb, A);
         const size_t o_units = off; off = up(off + sizeof(uint2) * total_units, A);
+        const size_t o_punits = off; off = up(off + sizeof(uint2) * panel_units, A);
         const size_t o_tunits = off; off = up(off + sizeof(uint2) * std::max<size_t>(total_tiles, 1), A);
         const size_t o_tileP = off; off = up(off + sizeof(int) * nb, A);
         const size_t o_ntiles = off; off = up(off + sizeof(unsigned) * nb, A);
-        const size_t o_ctr = off; off = up(off + 64, A);
+        const size_t o_ctr = off; off = up(off + 128, A);
         e = cudaMalloc(&arena, off);
         if (e != cudaSuccess) { set_cuda_error(e, "cudaMalloc (batch arena)"); rc = e == cudaErrorMemoryAllocation ? CUPSO_ERR_OOM : CUPSO_ERR_CUDA; break; }
         char* base = static_cast<char*>(arena);
@@ -224,10 +277,11 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
         unsigned long long* keys = reinterpret_cast<unsigned long long*>(base + o_keys);
         unsigned int* words = reinterpret_cast<unsigned int*>(base + o_words);   // done, status, 2 spare
         unsigned char* flags = reinterpret_cast<unsigned char*>(base + o_flags);
-        unsigned int* ctr = reinterpret_cast<unsigned int*>(base + o_ctr);       // work[2], ticket, t
+        unsigned int* ctr = reinterpret_cast<unsigned int*>(base + o_ctr);       // work[2], ticket, t; the panels' from 16
         e = cudaMemsetAsync(keys, 0xFF, sizeof(unsigned long long) * 2 * nb, run.st);
         if (e == cudaSuccess) e = cudaMemsetAsync(base + o_words, 0, o_desc - o_words, run.st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(ctr, 0, 64, run.st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(ctr, 0, 128, run.st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(Gall, 0, sizeof(float) * sumG, run.st);
         if (e != cudaSuccess) { set_cuda_error(e, "cudaMemsetAsync"); rc = CUPSO_ERR_CUDA; break; }
 
         // The descriptor of every swarm.
@@ -235,7 +289,7 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
         for (int j = 0; j < nb; ++j) {
             const cupso_problem& p = problems[batched[j]];
             float* st = reinterpret_cast<float*>(base + o_state[j]);
-            const size_t plane = (size_t)p.D * Np[j];
+            const size_t plane = (size_t)rows[j] * Np[j];
             BatchSwarm& w = desc[j];
             w.x = st;
             w.v = st + plane;
@@ -243,11 +297,13 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
             w.pf = st + 3 * plane;
             w.pflag = flags + o_flag[j];
             w.G = Gall + o_G[j];
+            w.g16 = (uint32_t)(o_G[j] / 4);
             w.gkey = keys + 2 * j;
             w.done = words + 4 * j + 0;
             w.status = words + 4 * j + 1;
             w.N = p.N; w.D = p.D; w.Np = Np[j]; w.fid = p.fitness_id;
-            w.nunits = (unsigned)(Np[j] / 128);
+            w.Gs = rows[j];
+            w.nunits = (unsigned)(Np[j] / (panel[j] ? 16 : 128));
             w.lo = p.bounds.min_pos; w.hi = p.bounds.max_pos; w.vmax = p.bounds.max_v;
             w.w = p.w; w.c1 = p.c1; w.c2 = p.c2;
             w.c1s = std::ldexp(p.c1, -24);
@@ -255,10 +311,13 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
             const bool fast_cr = std::ldexp(w.c1s, 24) == p.c1 && std::ldexp(w.c2s, 24) == p.c2 &&
                                  (p.c1 == 0.0f || std::fabs(w.c1s) >= FLT_MIN) &&
                                  (p.c2 == 0.0f || std::fabs(w.c2s) >= FLT_MIN);
-            w.fast = fast_cr && p.bounds.min_pos != 0.0f && p.bounds.max_pos != 0.0f;
+            const bool has_cos = p.fitness_id == CUPSO_RASTRIGIN || p.fitness_id == CUPSO_ACKLEY;
+            const bool small = std::fabs(p.bounds.min_pos) <= kSmallX && std::fabs(p.bounds.max_pos) <= kSmallX;
+            w.fast = (!panel[j] || !has_cos || small) && fast_cr && p.bounds.min_pos != 0.0f && p.bounds.max_pos != 0.0f;
             w.key0 = (uint32_t)(p.seed & 0xFFFFFFFFull);
             w.key1 = (uint32_t)(p.seed >> 32);
             w.swarm = p.swarm_id;
+            set_constants(w);
         }
         if (rc != CUPSO_OK) break;
 
@@ -267,31 +326,47 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
         // instructions; within such a class the units with the most dimensions
         // first, swarms of equal D interleaved. The smallest units come last
         // and fill the tail.
-        std::vector<uint2> units;
-        units.reserve(total_units);
         std::vector<int> order(nb);
         for (int j = 0; j < nb; ++j) order[j] = j;
         auto code_of = [&](int j) { return desc[j].fid * 2 + desc[j].fast; };
-        auto same_group = [&](int a, int b) { return code_of(a) == code_of(b) && desc[a].D == desc[b].D; };
         std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+            if (panel[a] != panel[b]) return panel[a] > panel[b];
             if (code_of(a) != code_of(b)) return code_of(a) < code_of(b);
             return desc[a].D > desc[b].D;
         });
-        for (size_t pos = 0; pos < (size_t)nb;) {
-            size_t endg = pos;
-            while (endg < (size_t)nb && same_group(order[endg], order[pos])) ++endg;
-            unsigned most = 0;
-            for (size_t q = pos; q < endg; ++q) most = std::max(most, desc[order[q]].nunits);
-            for (unsigned u = 0; u < most; ++u)
-                for (size_t q = pos; q < endg; ++q)
-                    if (u < desc[order[q]].nunits) units.push_back(make_uint2((unsigned)order[q], u));
-            pos = endg;
-        }
+        auto same_group = [&](int a, int b) {
+            return panel[a] == panel[b] && code_of(a) == code_of(b) && desc[a].D == desc[b].D;
+        };
+        // (swarm, unit) pairs of the swarms in panels or of the others, `count(j)` of each
+        auto hand_out = [&](bool panels, size_t total, auto count) {
+            std::vector<uint2> out;
+            out.reserve(total);
+            for (size_t pos = 0; pos < (size_t)nb;) {
+                size_t endg = pos;
+                while (endg < (size_t)nb && same_group(order[endg], order[pos])) ++endg;
+                if ((panel[order[pos]] != 0) == panels) {
+                    unsigned most = 0;
+                    for (size_t q = pos; q < endg; ++q) most = std::max(most, count(order[q]));
+                    for (unsigned u = 0; u < most; ++u)
+                        for (size_t q = pos; q < endg; ++q)
+                            if (u < count(order[q])) out.push_back(make_uint2((unsigned)order[q], u));
+                }
+                pos = endg;
+            }
+            return out;
+        };
+        auto units_of = [&](int j) { return desc[j].nunits; };
+        const std::vector<uint2> units = hand_out(false, total_units, units_of);
+        const std::vector<uint2> punits = hand_out(true, panel_units, units_of);
         e = cudaMemcpyAsync(base + o_desc, desc.data(), sizeof(BatchSwarm) * nb, cudaMemcpyHostToDevice, run.st);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(base + o_units, units.data(), sizeof(uint2) * units.size(), cudaMemcpyHostToDevice,
                                 run.st);
+        if (e == cudaSuccess && !punits.empty())
+            e = cudaMemcpyAsync(base + o_punits, punits.data(), sizeof(uint2) * punits.size(), cudaMemcpyHostToDevice,
+                                run.st);
         if (e != cudaSuccess) { set_cuda_error(e, "cudaMemcpyAsync"); rc = CUPSO_ERR_CUDA; break; }
+        run.dev.G = Gall;
         run.dev.swarms = reinterpret_cast<const BatchSwarm*>(base + o_desc);
         run.dev.units = reinterpret_cast<const uint2*>(base + o_units);
         run.dev.nunits = (unsigned)units.size();
@@ -299,25 +374,26 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
         run.dev.ticket = ctr + 2;
         run.dev.t_dev = ctr + 3;
 
-        // Step 1 of every swarm, one launch.
-        e = launch_batch_init(run.dev, run.num_sms * 4, run.st);
+        prun.num_sms = run.num_sms;
+        prun.dev = run.dev;
+        prun.dev.units = reinterpret_cast<const uint2*>(base + o_punits);
+        prun.dev.nunits = (unsigned)punits.size();
+        prun.dev.work = ctr + 16;
+        prun.dev.ticket = ctr + 18;
+        prun.dev.t_dev = ctr + 19;
+        const Shape pshape{-1, 0, prun.dev.nunits ? batch_panel_grid(prun.dev.nunits, run.num_sms) : 0};
+
+        // Step 1 of every swarm, one launch for each kind.
+        e = cudaSuccess;
+        if (prun.dev.nunits) e = launch_batch_panel_init(prun.dev, run.num_sms, run.st);
+        if (e == cudaSuccess && run.dev.nunits) e = launch_batch_init(run.dev, run.num_sms * 4, run.st);
         if (e != cudaSuccess) { set_cuda_error(e, "batch init launch"); rc = CUPSO_ERR_CUDA; break; }
 
         // The tiled kernel's units in the same order.
-        const bool tiled_ok = maxD <= kTiledItems;
+        const bool tiled_ok = nlegacy > 0 && maxD <= kTiledItems;
+        std::vector<uint2> tunits;
         if (tiled_ok) {
-            std::vector<uint2> tunits;
-            tunits.reserve(total_tiles);
-            for (size_t pos = 0; pos < (size_t)nb;) {
-                size_t endg = pos;
-                while (endg < (size_t)nb && same_group(order[endg], order[pos])) ++endg;
-                unsigned most = 0;
-                for (size_t q = pos; q < endg; ++q) most = std::max(most, ntiles[order[q]]);
-                for (unsigned u = 0; u < most; ++u)
-                    for (size_t q = pos; q < endg; ++q)
-                        if (u < ntiles[order[q]]) tunits.push_back(make_uint2((unsigned)order[q], u));
-                pos = endg;
-            }
+            tunits = hand_out(false, total_tiles, [&](int j) { return ntiles[j]; });
             e = cudaMemcpyAsync(base + o_tunits, tunits.data(), sizeof(uint2) * tunits.size(), cudaMemcpyHostToDevice,
                                 run.st);
             if (e == cudaSuccess)
@@ -338,25 +414,19 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
         cand.push_back(Shape{3, 2, batch_blocks_per_sm(3, 2)});
         cand.push_back(Shape{3, 3, batch_blocks_per_sm(3, 3)});
         if (tiled_ok) cand.push_back(Shape{0, 0, batch_tiled_blocks_per_sm()});
-        const auto key = std::make_tuple(nb, total_pd, minD, maxD);
+        const auto key = std::make_tuple(nlegacy, total_pd, minD, maxD);
         Shape best = cand[0];
-        bool known = false;
-        {
+        bool known = nlegacy == 0;
+        if (!known) {
             std::lock_guard<std::mutex> lk(g_tune_mutex);
             auto it = g_tuned.find(key);
             if (it != g_tuned.end()) { best = it->second; known = true; }
         }
-        // CUPSO_BATCH_KERNEL=tiled|streaming fixes the kernel instead of tuning
-        // (for tests and measurements; both kernels give the same bits).
-        if (const char* force = std::getenv("CUPSO_BATCH_KERNEL")) {
-            const bool want_tiled = std::strcmp(force, "tiled") == 0;
-            const bool want_stream = std::strcmp(force, "streaming") == 0;
-            if (want_tiled && !tiled_ok) { set_last_error("CUPSO_BATCH_KERNEL=tiled: D too large"); rc = CUPSO_ERR_UNSUPPORTED; break; }
-            if (want_tiled || want_stream) {
-                for (const Shape& sh : cand)
-                    if ((sh.stages == 0) == want_tiled) { best = sh; break; }
-                known = true;
-            }
+        if (want_tiled && !tiled_ok) { set_last_error("CUPSO_BATCH_KERNEL=tiled: D too large"); rc = CUPSO_ERR_UNSUPPORTED; break; }
+        if (want_tiled || want_stream) {
+            for (const Shape& sh : cand)
+                if ((sh.stages == 0) == want_tiled) { best = sh; break; }
+            known = true;
         }
         int done_iters = 0;
         const int probe = 2;
@@ -386,8 +456,25 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
             }
         }
         if (rc != CUPSO_OK) break;
-        rc = run.run(best, iters - done_iters);
+        // Neither kind waits for the other: with both, the panels advance on a stream
+        // of their own, from here until the results are read.
+        prun.st = run.st;
+        if (prun.dev.nunits && run.dev.nunits) {
+            e = cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking);
+            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&handover, cudaEventDisableTiming);
+            if (e == cudaSuccess) e = cudaEventRecord(handover, run.st);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(side, handover, 0);
+            if (e != cudaSuccess) { set_cuda_error(e, "batch streams"); rc = CUPSO_ERR_CUDA; break; }
+            prun.st = side;
+        }
+        if (prun.dev.nunits) rc = prun.run(pshape, iters);
+        if (rc == CUPSO_OK && run.dev.nunits) rc = run.run(best, iters - done_iters);
         if (rc != CUPSO_OK) break;
+        if (side) {
+            e = cudaEventRecord(handover, side);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(run.st, handover, 0);
+            if (e != cudaSuccess) { set_cuda_error(e, "batch streams"); rc = CUPSO_ERR_CUDA; break; }
+        }
 
         // Results: gbest key, position and status of every swarm.
         std::vector<unsigned long long> hkeys(2 * (size_t)nb);
@@ -404,7 +491,7 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
             const unsigned long long k = hkeys[2 * j + cur];
             r.fit = key_fit(k);
             r.idx = (int64_t)(k & 0xFFFFFFFFull);
-            if (r.pos) std::memcpy(r.pos, hG.data() + o_G[j] + (size_t)cur * desc[j].D, sizeof(float) * desc[j].D);
+            if (r.pos) std::memcpy(r.pos, hG.data() + o_G[j] + (size_t)cur * desc[j].Gs, sizeof(float) * desc[j].D);
             r.status = (hw[4 * j + 1] & kStatusTimeout) ? CUPSO_ERR_DEVICE_TIMEOUT
                        : (hw[4 * j + 1] & kStatusNaN)   ? CUPSO_ERR_NAN
                                                         : CUPSO_OK;
@@ -415,10 +502,13 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
         for (int j = 0; j < nb; ++j) results[batched[j]].status = rc;
         note(rc);
     }
+    if (side) cudaStreamSynchronize(side);
     if (arena) {
         cudaStreamSynchronize(run.st);
         cudaFree(arena);
     }
+    if (handover) cudaEventDestroy(handover);
+    if (side) cudaStreamDestroy(side);
     if (own) cudaStreamDestroy(own);
     return first;
 }

@@ -55,25 +55,31 @@ struct SwarmDev {
     uint32_t rk0[10], rk1[10];
 };
 
-// One swarm of a batch (kernels_batch.cu): its state in the batch arena and
-// its parameters. Same layouts as SwarmDev.
+// One swarm of a batch (kernels_batch.cu, kernels_batch_panel.cu): its state in the
+// batch arena and its parameters. Same layouts as SwarmDev.
 struct BatchSwarm {
     float *x, *v, *pb, *pf;
     unsigned char* pflag;
-    float* G;                   // [2][D]
+    float* G;                   // [2][Gs]
     unsigned long long* gkey;   // [2]
     unsigned int* done;         // units of this swarm finished in the current iteration
     unsigned int* status;
     int N, D, Np, fid;
-    unsigned int nunits;        // Np / 128
+    int Gs;                     // D, or D rounded up to whole panels where the state is in panels
+    unsigned int nunits;        // units of 128 particles, or of 16 where the state is in panels
     float lo, hi, vmax, w, c1, c2, c1s, c2s;
     uint32_t key0, key1, swarm;
     int fast;                   // fast_cr && fast_clamp
+    uint32_t g16;               // states in panels: G is 16 g16 bytes into BatchDev::G
+    // What every move needs, in vectors: five of Philox round keys (rk0 and rk1 of rounds
+    // 2 k and 2 k + 1), (w, c1, c2, vmax) with c1s, c2s where fast, (lo, hi, swarm, 0)
+    uint4 cst[8];
 };
 
 struct BatchDev {
     const BatchSwarm* swarms;
     const uint2* units;         // (swarm, unit) in hand-out order
+    const float* G;             // every swarm's G is in here
     unsigned int nunits;
     unsigned int* work;         // [2] unit counters, alternating by iteration parity
     unsigned int* ticket;

@@ -58,6 +58,16 @@ cudaError_t launch_batch_step(const BatchDev& b, int stages, int minb, int grid,
 // pflag zero.
 cudaError_t launch_batch_init(const BatchDev& b, int grid, cudaStream_t st);
 
+// The same on states in panels of 8 dimensions (kernels_batch_panel.cu), units of 16
+// particles, swarms of at least kBatchPanelMinD dimensions (any number of them: the
+// last panel may be partly used). Panel (d / 8), particle i: 8 floats at
+// (d / 8 * Np + i) * 8; gbest_pos rows 16-byte aligned, zero past D.
+constexpr int kBatchPanelMinD = 25;
+cudaError_t prepare_batch_panel();
+int batch_panel_grid(unsigned int nunits, int num_sms);
+cudaError_t launch_batch_panel(const BatchDev& b, int grid, cudaStream_t st);
+cudaError_t launch_batch_panel_init(const BatchDev& b, int num_sms, cudaStream_t st);
+
 // Fused SYNC step on the panel layout (kernels_panel.cu): element (d, i) of
 // x, v, pb at ((d / W) * Np + i) * W + d % W, panel width W = 8 or 16, ring
 // depth 3 or 5 panels.

@@ -192,11 +192,12 @@ __device__ __forceinline__ void run_unit_t(const BatchDev& b, unsigned* work, fl
     const bool lane_cand = best < K;
     best = warp_min_u64(best);
     const bool any_nan = __any_sync(0xFFFFFFFFu, nan);
-    // Publish, then count the unit; the warp that completes the swarm gathers
-    // its gbest. The gather reads only the winner's row and improvement flag,
-    // and the winner was a candidate below K in its unit, so only a lane that
-    // holds such a candidate makes its stores visible before lane 0 counts
-    // (a fence per unit in every lane stalled each warp on its own stores).
+    // Publish, then count the unit; the warp that completes the swarm sets its
+    // gbest_pos: from the winner's pos (its pbest_pos, pending, as it improved in
+    // this iteration), or from the other parity's where no key below K came. So
+    // only a lane that holds a candidate below K makes its stores visible before
+    // lane 0 counts (a fence per unit in every lane stalled each warp on its own
+    // stores), and no other particle's row is read here.
     if (lane_cand) __threadfence();
     __syncwarp();
     int last = 0;
@@ -213,12 +214,8 @@ __device__ __forceinline__ void run_unit_t(const BatchDev& b, unsigned* work, fl
     if (last) {
         const unsigned long long knew = __ldcg(w.gkey + nxt);
         const uint32_t gi = (uint32_t)(knew & 0xFFFFFFFFull);
-        if (gi < (uint32_t)w.N) {
-            const bool lazy = (__ldcg(reinterpret_cast<const unsigned int*>(w.pflag) + (gi >> 2)) >>
-                               (8u * (gi & 3u))) & 0xFFu;
-            const float* src = lazy ? w.x : w.pb;
-            for (int d = lane_id; d < D; d += 32) w.G[(size_t)nxt * D + d] = __ldcg(src + (size_t)d * Np + gi);
-        }
+        for (int d = lane_id; d < D; d += 32)
+            w.G[(size_t)nxt * D + d] = knew < K ? __ldcg(w.x + (size_t)d * Np + gi) : __ldcg(G + d);
         __syncwarp();
         if (lane_id == 0) {
             w.gkey[cur] = knew;
