@@ -177,6 +177,60 @@ __device__ __forceinline__ float cos2pi_small(float x) {
     return __uint_as_float(__float_as_uint(cos2pi_poly(r)) ^ (__float_as_uint(m) << 31));
 }
 
+// Two floats per 64-bit register: one instruction for two IEEE operations, each the
+// scalar one's bits.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 both(float a) { return pack2(a, a); }
+__device__ __forceinline__ void unpack2(f32x2 p, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// cos2pi_small of two values.
+__device__ __forceinline__ void cos2pi_small2(float x0, float x1, float& c0, float& c1) {
+    const f32x2 x = pack2(x0, x1);
+    const f32x2 m = fma2(both(2.0f), x, both(0x1.8p23f));
+    const f32x2 r = fma2(both(-0.5f), sub2(m, both(0x1.8p23f)), x);
+    const f32x2 z = mul2(r, r);
+    f32x2 q = both(-0x1.b6e25p+0f);
+    q = fma2(q, z, both(0x1.f9d38ap+2f));
+    q = fma2(q, z, both(-0x1.a6d1f2p+4f));
+    q = fma2(q, z, both(0x1.e1f506p+5f));
+    q = fma2(q, z, both(-0x1.55d3c8p+6f));
+    q = fma2(q, z, both(0x1.03c1fp+6f));
+    q = fma2(q, z, both(-0x1.3bd3ccp+4f));
+    q = fma2(q, z, both(0x1p+0f));
+    float m0, m1;
+    unpack2(m, m0, m1);
+    unpack2(q, c0, c1);
+    c0 = __uint_as_float(__float_as_uint(c0) ^ (__float_as_uint(m0) << 31));
+    c1 = __uint_as_float(__float_as_uint(c1) ^ (__float_as_uint(m1) << 31));
+}
+
 // SMALL: every x lies within kSmallX.
 template <bool SMALL>
 __device__ __forceinline__ float cosine2pi(float x) {

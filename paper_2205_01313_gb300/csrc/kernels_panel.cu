@@ -39,6 +39,8 @@
 // (two at a time when the swarm has many per warp).
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "cupso_device.cuh"
 #include "cupso_internal.h"
 #include "panel_common.cuh"
@@ -183,14 +185,23 @@ __device__ __forceinline__ unsigned long long panel_units(const SwarmDev& s, flo
 #pragma unroll
             for (int g = 0; g < 2; ++g) {
                 const uint4 r = philox4x32_10_rk(make_uint4((uint32_t)((d0 >> 1) + g), i, t, s.swarm), s.rk0, s.rk1);
+                if constexpr (FAST) {
+                    const int k = 2 * g;
+                    float x0 = lane(X, k), x1 = lane(X, k + 1), v0 = lane(V, k), v1 = lane(V, k + 1);
+                    move_two_fast(x0, x1, v0, v1, pack2(lane(Pb, k), lane(Pb, k + 1)),
+                                  *reinterpret_cast<const f32x2*>(Gs + d0 + k), pack2(hi24(r.x), hi24(r.z)),
+                                  pack2(hi24(r.y), hi24(r.w)), s);
+                    set_lane(X, k, x0);
+                    set_lane(X, k + 1, x1);
+                    set_lane(V, k, v0);
+                    set_lane(V, k + 1, v1);
+                    continue;
+                }
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
                     const int k = 2 * g + hh;
                     float xj = lane(X, k), vj = lane(V, k);
-                    if constexpr (FAST)
-                        move_one_fast(xj, vj, lane(Pb, k), Gs[d0 + k], hi24(word(r, 2 * hh)),
-                                      hi24(word(r, 2 * hh + 1)), s);
-                    else
+                    if constexpr (!FAST)
                         move_one(xj, vj, lane(Pb, k), Gs[d0 + k], u01(word(r, 2 * hh)), u01(word(r, 2 * hh + 1)),
                                  s);
                     set_lane(X, k, xj);
@@ -199,7 +210,7 @@ __device__ __forceinline__ unsigned long long panel_units(const SwarmDev& s, flo
             }
             st4(s.x + off, X);
             st4(s.v + off, V);
-            panel_sum<FIT, L, false>(acc, X, d0, D, j, lane_id, carry);
+            panel_sum<FIT, L, false, FAST>(acc, X, d0, D, j, lane_id, carry);
             if (++stage == STAGES) stage = 0;
         }
         // Step 4 (strict improvement; the new pbest_pos is pos, flagged) and
@@ -231,7 +242,10 @@ __device__ __forceinline__ unsigned long long panel_units(const SwarmDev& s, flo
 
 // `iters` synchronous iterations. Requires D % W == 0, D / W >= STAGES - 1,
 // Np a multiple of 128, s.pflag, s.work and s.bar set, work and bar zero at
-// launch. FAST selects move_one_fast (requires s.fast_cr and s.fast_clamp).
+// launch. FAST: panel_fast(s, FIT); moves and cosines of two dimensions per instruction
+// (fma.rn.f32x2): the kernel's issue slots were 61 % taken, and an iteration of
+// Rastrigin's 65536 x 128 took 33.6 us with scalar ones and the rounding instruction,
+// now 31.7 (Ackley 34.3 and 32.4, sphere 29.0 and 28.2).
 //
 // Each warp takes unit (its warp index) first in every iteration, then units
 // from the counter. With more than one iteration, every CTA must be resident
@@ -397,6 +411,12 @@ const void* panel_kernel(int width, int stages, bool fast, int fid) {
 
 }  // namespace
 
+// The fast form's cosines are cos2pi_small.
+bool panel_fast(const SwarmDev& s, int fid) {
+    const bool has_cos = fid == kRastrigin || fid == kAckley;
+    return s.fast_cr && s.fast_clamp && (!has_cos || (std::fabs(s.lo) <= kSmallX && std::fabs(s.hi) <= kSmallX));
+}
+
 bool panel_supported(int width, int stages, int D) {
     return (width == 8 || width == 16) && (stages == 3 || stages == 5) && D % width == 0 &&
            D / width >= stages - 1 && D <= kPanelMaxD;
@@ -430,7 +450,7 @@ cudaError_t launch_sync_panel(const SwarmDev& s, int fid, int width, int stages,
     if (!panel_supported(width, stages, s.D) || !s.pflag || !s.work || !s.bar || s.Np % 128 != 0 || iters < 1 ||
         iters > kPanelMaxIters || grid < 1 || (unsigned long long)iters * ((unsigned long long)grid + 2ull) >= (1ull << 32))
         return cudaErrorInvalidValue;
-    const void* k = panel_kernel(width, stages, s.fast_cr && s.fast_clamp, fid);
+    const void* k = panel_kernel(width, stages, panel_fast(s, fid), fid);
     if (!k) return cudaErrorInvalidValue;
     unsigned int expect = (unsigned int)grid + (stall_barrier ? 1u : 0u);
     void* args[] = {const_cast<SwarmDev*>(&s), &iters, &expect};

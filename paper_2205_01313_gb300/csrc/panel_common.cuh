@@ -26,6 +26,18 @@ __device__ __forceinline__ void pull(FitAcc<FIT>& a, int src) {
     if constexpr (FIT == kAckley) a.acc2 = __shfl_sync(0xFFFFFFFFu, a.acc2, src);
 }
 
+// cos(2 pi x) of four values.
+template <bool SMALL>
+__device__ __forceinline__ void cosines(const float (&x)[4], float (&c)[4]) {
+    if constexpr (SMALL) {
+        cos2pi_small2(x[0], x[1], c[0], c[1]);
+        cos2pi_small2(x[2], x[3], c[2], c[3]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) c[k] = cos2pi(x[k]);
+    }
+}
+
 // Adds the fitness terms of this lane's four dimensions (d0 .. d0 + 3) in the
 // oracle's order. The terms themselves do not depend on the running sum
 // (Rastrigin's x^2 - 10 cos 2 pi x + 10, Rosenbrock's 100 (x_{d+1} - x_d^2)^2 +
@@ -46,11 +58,14 @@ __device__ __forceinline__ void panel_sum(FitAcc<FIT>& a, const float4& X, int d
     float t[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     const int base = lane_id - j;
     if constexpr (FIT == kRastrigin) {
+        cosines<SMALL>(x, t);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) t[k] = __fmaf_rn(x[k], x[k], __fmaf_rn(-10.0f, cosine2pi<SMALL>(x[k]), 10.0f));
+        for (int k = 0; k < 4; k += 2) {
+            const f32x2 xx = pack2(x[k], x[k + 1]);
+            unpack2(fma2(xx, xx, fma2(both(-10.0f), pack2(t[k], t[k + 1]), both(10.0f))), t[k], t[k + 1]);
+        }
     } else if constexpr (FIT == kAckley) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) t[k] = cosine2pi<SMALL>(x[k]);
+        cosines<SMALL>(x, t);
     } else if constexpr (FIT == kCubicMax) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)

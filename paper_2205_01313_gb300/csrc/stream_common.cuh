@@ -47,6 +47,22 @@ __device__ __forceinline__ void move_one_fast(float& x, float& v, float pb, floa
     x = clampf_minmax(__fadd_rn(x, v), s.lo, s.hi);
 }
 
+// Two dimensions at once, the same bits.
+__device__ __forceinline__ void move_two_fast(float& x0, float& x1, float& v0, float& v1, f32x2 pb, f32x2 g, f32x2 k1,
+                                              f32x2 k2, const SwarmDev& s) {
+    const f32x2 x = pack2(x0, x1);
+    const f32x2 c1s = both(s.c1s), c2s = both(s.c2s);
+    f32x2 vel = mul2(both(s.w), pack2(v0, v1));
+    vel = fma2(fma2(c1s, k1, c1s), sub2(pb, x), vel);
+    vel = fma2(fma2(c2s, k2, c2s), sub2(g, x), vel);
+    unpack2(vel, v0, v1);
+    v0 = clampf_minmax(v0, -s.vmax, s.vmax);
+    v1 = clampf_minmax(v1, -s.vmax, s.vmax);
+    unpack2(add2(x, pack2(v0, v1)), x0, x1);
+    x0 = clampf_minmax(x0, s.lo, s.hi);
+    x1 = clampf_minmax(x1, s.lo, s.hi);
+}
+
 __device__ __forceinline__ float hi24(uint32_t w) { return __uint2float_rn(w >> 8); }
 
 // Steps 2-3 for the particles i0..i0+3 at iteration t: reads x, v, pb, writes
