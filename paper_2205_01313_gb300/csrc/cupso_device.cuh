@@ -356,12 +356,10 @@ __device__ __forceinline__ float clampf_minmax(float a, float lo, float hi) {
 }
 
 __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long k) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long other = __shfl_xor_sync(0xFFFFFFFFu, k, o);
-        k = other < k ? other : k;
-    }
-    return k;
+    const unsigned int hi = (unsigned int)(k >> 32);
+    const unsigned int mh = __reduce_min_sync(0xFFFFFFFFu, hi);
+    const unsigned int ml = __reduce_min_sync(0xFFFFFFFFu, hi == mh ? (unsigned int)k : 0xFFFFFFFFu);
+    return ((unsigned long long)mh << 32) | ml;
 }
 
 // Named barriers of a block: wait with, or count towards, `threads` threads.

@@ -88,7 +88,9 @@ __global__ void __launch_bounds__(kBlock) lsq_move_kernel(const __grid_constant_
 // tile, three 2-D tensor copies (pos, v, pbest_pos; rows past D read as zeros)
 // and one bulk copy of the tile's 64 improvement flags, all completing on the
 // stage's mbarrier; a stage is refilled as soon as every thread is done with
-// it. Thread q takes 4 particles x one dimension pair of the tile; new pos and
+// it. FAST (s.fast_cr and s.fast_clamp): two particles per instruction
+// (fma.rn.f32x2), 33.7 us at 8192 x 1024 against 34.8; 28 at the copy's rate.
+// Thread q takes 4 particles x one dimension pair of the tile; new pos and
 // v go straight back to global memory; the operand's transposition goes
 // through shared memory, so its rows are written in whole segments.
 // Lazy pbest: a particle flagged in s.pflag improved in the previous
@@ -104,7 +106,7 @@ constexpr int kMoveBox = 64 * 64 * 4;   // one array's tile
 constexpr int kMoveStageBytes = (3 * kMoveBox + 64 + 127) / 128 * 128;
 constexpr uint32_t kMoveTx = 3 * kMoveBox + 64;
 
-template <bool FP8>
+template <bool FP8, bool FAST>
 __global__ void __launch_bounds__(kMoveThreads, 1) lsq_move_q_kernel(const __grid_constant__ SwarmDev s,
                                                                      const __grid_constant__ MoveMaps maps,
                                                                      void* __restrict__ Xq, int Kp, float sx) {
@@ -184,13 +186,28 @@ __global__ void __launch_bounds__(kMoveThreads, 1) lsq_move_q_kernel(const __gri
                     st4(s.pb + off, Ph);
                 }
                 const float gd = __ldg(G + d);
+                if constexpr (FAST) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    float xj = lane(Xh, j), vj = lane(Vh, j);
-                    move_one(xj, vj, lane(Ph, j), gd, u01(word(r[j], 2 * h)), u01(word(r[j], 2 * h + 1)), s);
-                    set_lane(Xh, j, xj);
-                    set_lane(Vh, j, vj);
-                    xn[h][j] = __fsub_rn(xj, gd);
+                    for (int j = 0; j < 4; j += 2) {
+                        float x0 = lane(Xh, j), x1 = lane(Xh, j + 1), v0 = lane(Vh, j), v1 = lane(Vh, j + 1);
+                        move_two_fast(x0, x1, v0, v1, pack2(lane(Ph, j), lane(Ph, j + 1)), both(gd),
+                                      pack2(hi24(word(r[j], 2 * h)), hi24(word(r[j + 1], 2 * h))),
+                                      pack2(hi24(word(r[j], 2 * h + 1)), hi24(word(r[j + 1], 2 * h + 1))), s);
+                        set_lane(Xh, j, x0);
+                        set_lane(Xh, j + 1, x1);
+                        set_lane(Vh, j, v0);
+                        set_lane(Vh, j + 1, v1);
+                        unpack2(sub2(pack2(x0, x1), both(gd)), xn[h][j], xn[h][j + 1]);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        float xj = lane(Xh, j), vj = lane(Vh, j);
+                        move_one(xj, vj, lane(Ph, j), gd, u01(word(r[j], 2 * h)), u01(word(r[j], 2 * h + 1)), s);
+                        set_lane(Xh, j, xj);
+                        set_lane(Vh, j, vj);
+                        xn[h][j] = __fsub_rn(xj, gd);
+                    }
                 }
                 st4(s.x + off, Xh);
                 st4(s.v + off, Vh);
@@ -325,118 +342,85 @@ __global__ void lsq_gather_kernel(const __grid_constant__ SwarmDev s) {
     }
 }
 
-// The 16 smallest keys a warp holds, ascending, into out[0..15] (lane 0
-// writes): round r takes the smallest key above round r-1's (keys are unique:
-// the particle index is in the low bits; kKeyNone fills the rounds past the
-// last key). item(q) is the lane's q-th key, q < n (N > 0: n = N, unrolled).
-template <int N, typename Item>
-__device__ __forceinline__ void warp_top(Item item, int n, unsigned long long* out) {
-    unsigned long long last = 0;
-    for (int r = 0; r < kCand; ++r) {
-        unsigned long long lm = kKeyNone;
-        if constexpr (N > 0) {
-#pragma unroll
-            for (int q = 0; q < N; ++q) {
-                const unsigned long long k = item(q);
-                if ((r == 0 || k > last) && k < lm) lm = k;
-            }
-        } else {
-            for (int q = 0; q < n; ++q) {
-                const unsigned long long k = item(q);
-                if ((r == 0 || k > last) && k < lm) lm = k;
-            }
-        }
-        const unsigned long long m = warp_min_u64(lm);
-        if ((threadIdx.x & 31) == 0) out[r] = m;
-        last = m;
-    }
-}
-
 // Step 4 with an approximate fitness, and the 16 lowest keys among the
 // particles that improved (all particles when `all` is set: the first gbest).
 // One particle per thread, blocks of kSel threads (small, so that even a swarm
 // of a few thousand particles spreads over most SMs). Each thread loads all
 // its partial sums at once (with its pbest_fit) and adds them in k order; each
-// warp sorts its 32 keys with a bitonic network of lane exchanges and writes
-// its 16 lowest as one ascending list (cand[list][16], list = 2 block + warp).
-// The last block to finish merges all lists into top[16], ascending (kKeyNone
-// where fewer): for up to 32 * kMergeLists lists, a k-way merge (the first
-// kStageDepth keys of every list staged in shared memory in one round, then
-// merged by warp 0 alone: each lane holds the heads of kMergeLists lists, a
-// warp minimum per round, no block barrier between rounds; a list's deeper
-// keys, needed only when it gives up more than kStageDepth of the 16, come
-// from global memory), else a selection over all their keys. The fitness
-// comes from `fit`, or, with `part`, as the sum of the product's nparts
-// partial sums in their order.
+// warp sorts its 32 keys with a bitonic network of lane exchanges, the first one
+// merges the two lists, and the block writes its 16 lowest keys as one ascending
+// list (cand[block][16]). top[16], ascending (kKeyNone where fewer), are the 16
+// lowest of all lists: merged by every block of the float-float rescoring for
+// itself (`merge` false) up to kMaxMerge lists, else here by the last block to
+// finish. The fitness comes from `fit`, or, with `part`, as the sum of the
+// product's nparts partial sums in their order.
+// Bound by its chain of loads and exchanges: at 8192 particles 5.1 us, where a last
+// block that took a k-way merge of 256 lists one key at a time made it 11.8; at 12000,
+// where it searched all keys 16 times, an iteration went from 121 to 39 us.
 constexpr int kSel = 64;
 constexpr int kSelWarps = kSel / 32;
-constexpr int kMergeLists = 8;     // lists per lane of the last block's k-way merge
-constexpr int kStageDepth = 4;     // keys of each list staged for the merge
-// top[16] = the 16 lowest keys of the nl ascending lists cand[list][16]
-// (kKeyNone where fewer), by one block of kSel threads.
-__device__ __forceinline__ void merge_lists(const unsigned long long* __restrict__ cand, int nl,
-                                         unsigned long long* __restrict__ top) {
-    __shared__ unsigned long long stage[32 * kMergeLists * kStageDepth];
-    __shared__ unsigned long long wtop[kSelWarps][kCand];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n = nl * kCand;
-    const int tid = (int)threadIdx.x;
-    if (nl <= 32 * kMergeLists) {
-        // k-way merge of the ascending lists: lane l of warp 0 owns lists l,
-        // l + 32, ...; each round the smallest head over the warp is taken and
-        // its list advances (keys are unique, so one owner moves)
-        constexpr int kPer = 32 * kMergeLists * kStageDepth / kSel;
-        unsigned long long v[kPer];
+constexpr int kRound = 128;        // lists a block merges at once, in registers
+constexpr int kMaxMerge = 256;     // lists that every block of the float-float rescoring merges for itself
+
+// Lanes 0 .. 15 and 16 .. 31 each hold an ascending list in a and one in b, a key per
+// lane: a becomes the 16 lowest of both, ascending. The lower of key l of one and 15 - l
+// of the other are those 16, and a bitonic sequence.
+__device__ __forceinline__ unsigned long long merge_half(unsigned long long a, unsigned long long b, int lane) {
+    const unsigned long long o = __shfl_xor_sync(0xFFFFFFFFu, b, kCand - 1);
+    a = o < a ? o : a;
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const int e = tid + kSel * j, l = e / kStageDepth;
-            v[j] = l < nl ? __ldcg(cand + (size_t)l * kCand + e % kStageDepth) : kKeyNone;
-        }
+    for (int j = kCand / 2; j > 0; j >>= 1) {
+        const unsigned long long p = __shfl_xor_sync(0xFFFFFFFFu, a, j);
+        a = ((lane & j) == 0) == (p < a) ? p : a;
+    }
+    return a;
+}
+
+// The 16 lowest keys of n ascending lists (n <= 2 K): half h of the warp folds lists
+// h, 2 + h, 4 + h, .. (list(l) gives this lane's key of list l) and the halves' results
+// are folded into one, which both halves return.
+template <int K, typename List>
+__device__ __forceinline__ unsigned long long merge_warp(List list, int lane) {
+    const int h = lane / kCand;
+    unsigned long long v[K];
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) stage[tid + kSel * j] = v[j];
-        __syncthreads();
-        if (warp == 0) {
-            int head[kMergeLists];
-            unsigned long long hv[kMergeLists];
+    for (int k = 0; k < K; ++k) v[k] = list(2 * k + h);
 #pragma unroll
-            for (int q = 0; q < kMergeLists; ++q) {
-                head[q] = 0;
-                hv[q] = stage[(lane + 32 * q) * kStageDepth];
-            }
-            for (int r = 0; r < kCand; ++r) {
-                unsigned long long lm = kKeyNone;
+    for (int w = K / 2; w > 0; w >>= 1)
 #pragma unroll
-                for (int q = 0; q < kMergeLists; ++q) lm = hv[q] < lm ? hv[q] : lm;
-                const unsigned long long m = warp_min_u64(lm);
-                if (lane == 0) top[r] = m;
-                if (m != kKeyNone) {
-#pragma unroll
-                    for (int q = 0; q < kMergeLists; ++q)
-                        if (hv[q] == m) {
-                            const int b = lane + 32 * q, h = ++head[q];
-                            hv[q] = h < kStageDepth ? stage[b * kStageDepth + h]
-                                    : h < kCand   ? __ldcg(cand + (size_t)b * kCand + h)
-                                                  : kKeyNone;
-                        }
-                }
-            }
-        }
-    } else {
-        // many lists: a selection over all their keys, per warp then over the
-        // warps' lists
-        const int per = tid < n ? (n - tid + kSel - 1) / kSel : 0;   // this thread's entries: tid + kSel q
-        warp_top<0>([&](int q) { return __ldcg(cand + (size_t)tid + (size_t)kSel * q); }, per, wtop[warp]);
-        __syncthreads();
-        constexpr int kPerLane = kSelWarps * kCand / 32;
-        const unsigned long long* flat = &wtop[0][0];
-        if (warp == 0) warp_top<kPerLane>([&](int q) { return flat[lane + 32 * q]; }, kPerLane, top);
+        for (int k = 0; k < w; ++k) v[k] = merge_half(v[k], v[k + w], lane);
+    return merge_half(v[0], __shfl_xor_sync(0xFFFFFFFFu, v[0], kCand), lane);
+}
+
+// The 16 lowest keys of nl lists by WARPS warps (a power of two up to 8),
+// into top (shared memory): a warp for each share of the lists, then one for theirs.
+template <int WARPS>
+__device__ __forceinline__ void merge_block(const unsigned long long* __restrict__ cand, int nl,
+                                            unsigned long long (*part)[kCand], unsigned long long* top) {
+    const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+    constexpr int K = kRound / WARPS / 2;
+    unsigned long long m = kKeyNone;
+    for (int l0 = 0; l0 < nl; l0 += kRound) {
+        const unsigned long long v = merge_warp<K>(
+            [&](int l) {
+                const int g = l0 + l * WARPS + warp;
+                return g < nl ? __ldcg(cand + (size_t)g * kCand + lane % kCand) : kKeyNone;
+            },
+            lane);
+        m = l0 == 0 ? v : merge_half(m, v, lane);
+    }
+    if (lane < kCand) part[warp][lane] = m;
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned long long r = merge_warp<WARPS / 2>([&](int l) { return part[l][lane % kCand]; }, lane);
+        if (lane < kCand) top[lane] = r;
     }
 }
 
 __global__ void __launch_bounds__(kSel) lsq_select_cand_kernel(const __grid_constant__ SwarmDev s,
                                                                const float* __restrict__ fit,
                                                                const float* __restrict__ part, int nparts,
-                                                               int all,
+                                                               int all, bool merge,
                                                                unsigned long long* __restrict__ cand,
                                                                unsigned int* __restrict__ flags,
                                                                unsigned long long* __restrict__ top,
@@ -487,7 +471,16 @@ __global__ void __launch_bounds__(kSel) lsq_select_cand_kernel(const __grid_cons
             key = (lower == asc) ? (o < key ? o : key) : (o > key ? o : key);
         }
     }
-    if (lane < kCand) cand[((size_t)blockIdx.x * kSelWarps + warp) * kCand + lane] = key;
+    // the two warps' 16 lowest into one list
+    static_assert(kSelWarps == 2 && kCand == 16, "two lists of half a warp");
+    __shared__ unsigned long long second[kCand];
+    if (warp == 1 && lane < kCand) second[lane] = key;
+    __syncthreads();
+    if (warp == 0) {
+        key = merge_half(key, second[lane % kCand], lane);
+        if (lane < kCand) cand[(size_t)blockIdx.x * kCand + lane] = key;
+    }
+    if (!merge) return;
     // the last block merges: the lists are written (barrier), thread 0 releases
     // them with its ticket and, in the last block, acquires all the others
     __syncthreads();
@@ -498,8 +491,18 @@ __global__ void __launch_bounds__(kSel) lsq_select_cand_kernel(const __grid_cons
     }
     __syncthreads();
     if (!s_last) return;
-    merge_lists(cand, (int)gridDim.x * kSelWarps, top);
+    __shared__ unsigned long long wtop[kSelWarps][kCand];
+    merge_block<kSelWarps>(cand, (int)gridDim.x, wtop, top);
     if (threadIdx.x == 0) *ticket = 0u;
+}
+
+// An integer that orders as the (not NaN) double does, -0 as +0; NaN as kKeyNone, which
+// no number has.
+__device__ __forceinline__ unsigned long long order64(double f) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(f), mag = u & 0x7FFFFFFFFFFFFFFFull;
+    if (mag > 0x7FF0000000000000ull) return kKeyNone;
+    if (mag == 0ull) return 0x8000000000000000ull;
+    return u >> 63 ? ~u : u | 0x8000000000000000ull;
 }
 
 // Accepts the best rescored candidate if its rescored value beats gbest's; rolls t.
@@ -538,6 +541,7 @@ __device__ void accept_best(const SwarmDev& s, const float* __restrict__ src, co
             }
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
+                if (32 * k >= chunks) break;
                 f0 += v0[k];
                 f1 += v1[k];
             }
@@ -547,31 +551,31 @@ __device__ void accept_best(const SwarmDev& s, const float* __restrict__ src, co
                 if (c1 >= 0) f1 += __ldcg(partial + (size_t)c1 * chunks + h);
             }
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            f0 += __shfl_xor_sync(0xFFFFFFFFu, f0, o);
-            f1 += __shfl_xor_sync(0xFFFFFFFFu, f1, o);
-        }
-        if (lane == 0) {
-            fsum[c0] = f0;
-            if (c1 >= 0) fsum[c1] = f1;
-        }
+        // one butterfly for both: after its first level every value is held twice, so the
+        // lower half of the lanes goes on with the first candidate's, the upper with the
+        // second's
+        const bool up = lane >= 16;
+        const double o0 = __shfl_xor_sync(0xFFFFFFFFu, up ? f0 : f1, 16);
+        double f = (up ? f1 : f0) + o0;
+        for (int o = 8; o > 0; o >>= 1) f += __shfl_xor_sync(0xFFFFFFFFu, f, o);
+        if (lane == 0) fsum[c0] = f;
+        if (lane == 16 && c1 >= 0) fsum[c1] = f;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int best = -1;
-        double bf = 0.0;
-        for (int c = 0; c < kCand; ++c) {
-            const unsigned long long k = skey[c];
-            if (k == kKeyNone) break;
-            const double f = fsum[c];
-            const int i = (int)(k & 0xFFFFFFFFull);
-            if (f == f && (best < 0 || f < bf || (f == bf && i < best))) {
-                best = i;
-                bf = f;
-            }
-        }
-        s_best = (best >= 0 && bf < s_g64) ? best : -1;
-        s_f = bf;
+    // the lowest sum, NaN passed over, ties to the lower index: a lane per candidate,
+    // on integers that order as the doubles do (a comparison of doubles takes the FP64
+    // pipe, 64 cycles each, three a candidate in one thread before)
+    if (warp == 0) {
+        const unsigned long long k = lane < kCand ? skey[lane] : kKeyNone;
+        const double f = lane < kCand ? fsum[lane] : 0.0;
+        const unsigned long long o = k != kKeyNone ? order64(f) : kKeyNone;
+        const unsigned long long om = warp_min_u64(o);
+        const unsigned int i = o == om ? (unsigned int)(k & 0xFFFFFFFFull) : 0xFFFFFFFFu;
+        const unsigned int im = __reduce_min_sync(0xFFFFFFFFu, i);
+        const unsigned long long og = order64(s_g64);
+        const bool won = om != kKeyNone && og != kKeyNone && om < og;
+        if (lane == 0) s_best = won ? (int)im : -1;
+        if (won && o == om && i == im) s_f = f;
     }
     __syncthreads();
     const int best = s_best;
@@ -603,7 +607,8 @@ struct AcceptArgs {
     int* stale;
 };
 
-__device__ __forceinline__ void last_block_accepts(const SwarmDev& s, const AcceptArgs& a) {
+__device__ __forceinline__ void last_block_accepts(const SwarmDev& s, const AcceptArgs& a,
+                                                   const unsigned long long* top) {
     if (!a.ticket) return;
     __shared__ int s_last;
     // the block's partial sums are written (barrier); thread 0 releases them
@@ -616,8 +621,19 @@ __device__ __forceinline__ void last_block_accepts(const SwarmDev& s, const Acce
     }
     __syncthreads();
     if (!s_last) return;
-    accept_best(s, a.src, a.top, a.partial, a.chunks, a.g64, a.stale);
+    accept_best(s, a.src, top, a.partial, a.chunks, a.g64, a.stale);
     if (threadIdx.x == 0) *a.ticket = 0u;
+}
+
+// (double)f on the integer pipes: the conversion instruction runs on the FP64 pipe, which
+// is what the rescoring is bound by (16 candidates of 512 x 1024: 92 us an iteration with it, 73
+// now).
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t u = __float_as_uint(f);
+    if ((u & 0x7F800000u) - 0x00800000u < 0x7F000000u)   // neither 0, subnormal, infinite nor NaN
+        return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+    if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
+    return (double)f;
 }
 
 // FP64 rescoring: partial[c][chunk] = sum over rows m of the chunk of
@@ -638,7 +654,7 @@ __global__ void __launch_bounds__(256) lsq_rescore_kernel(const __grid_constant_
     double* out = partial + ((size_t)c * gridDim.y + chunk);
     if (key == kKeyNone) {
         if (threadIdx.x == 0) *out = __longlong_as_double(0x7FF8000000000000ll);   // no candidate
-        last_block_accepts(s, acc_args);
+        last_block_accepts(s, acc_args, acc_args.top);
         return;
     }
     const uint32_t i = (uint32_t)(key & 0xFFFFFFFFull);
@@ -647,22 +663,42 @@ __global__ void __launch_bounds__(256) lsq_rescore_kernel(const __grid_constant_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = chunk * rows_per_chunk, m1 = min(M, m0 + rows_per_chunk);
     double acc = 0.0;   // this warp's rows, in order
-    for (int m = m0 + warp; m < m1; m += 8) {
-        const float* row = A + (size_t)m * s.D;
-        // four independent chains per lane (d = lane + 32 (4k + j)), summed in a fixed order
-        double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0;
+    // two rows at a time: a coordinate is read once for both, and one butterfly sums both
+    for (int m = m0 + warp; m < m1; m += 16) {
+        const bool two = m + 8 < m1;
+        const float* ra = A + (size_t)m * s.D;
+        const float* rb = two ? ra + (size_t)8 * s.D : ra;
+        // four independent chains per lane and row (d = lane + 32 (4k + j)), summed in a fixed order
+        double p[4] = {0.0, 0.0, 0.0, 0.0}, u[4] = {0.0, 0.0, 0.0, 0.0};
         int d = lane;
         for (; d + 96 < s.D; d += 128) {
-            p0 = fma((double)row[d], xc[d], p0);
-            p1 = fma((double)row[d + 32], xc[d + 32], p1);
-            p2 = fma((double)row[d + 64], xc[d + 64], p2);
-            p3 = fma((double)row[d + 96], xc[d + 96], p3);
+            float fa[4], fb[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                fa[j] = __ldg(ra + d + 32 * j);
+                fb[j] = __ldg(rb + d + 32 * j);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const double x = xc[d + 32 * j];
+                p[j] = fma(widen(fa[j]), x, p[j]);
+                if (two) u[j] = fma(widen(fb[j]), x, u[j]);
+            }
         }
-        for (; d < s.D; d += 32) p0 = fma((double)row[d], xc[d], p0);
-        double p = (p0 + p1) + (p2 + p3);
-        for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xFFFFFFFFu, p, o);
-        const double r = p - (double)b[m];
-        acc = fma(r, r, acc);
+        for (; d < s.D; d += 32) {
+            p[0] = fma(widen(__ldg(ra + d)), xc[d], p[0]);
+            if (two) u[0] = fma(widen(__ldg(rb + d)), xc[d], u[0]);
+        }
+        const double pa = (p[0] + p[1]) + (p[2] + p[3]), pb = (u[0] + u[1]) + (u[2] + u[3]);
+        // after the first level every value is held twice: the lower half of the lanes goes
+        // on with the first row's, the upper with the second's
+        const bool up = lane >= 16;
+        double q = (up ? pb : pa) + __shfl_xor_sync(0xFFFFFFFFu, up ? pa : pb, 16);
+        for (int o = 8; o > 0; o >>= 1) q += __shfl_xor_sync(0xFFFFFFFFu, q, o);
+        const double r = q - widen(__ldg(b + (up && two ? m + 8 : m)));
+        const double ro = __shfl_xor_sync(0xFFFFFFFFu, r, 16);
+        acc = fma(up ? ro : r, up ? ro : r, acc);
+        if (two) acc = fma(up ? r : ro, up ? r : ro, acc);
     }
     if (lane == 0) wsum[warp] = acc;
     __syncthreads();
@@ -671,7 +707,7 @@ __global__ void __launch_bounds__(256) lsq_rescore_kernel(const __grid_constant_
         for (int w = 0; w < 8; ++w) tot += wsum[w];
         *out = tot;
     }
-    last_block_accepts(s, acc_args);
+    last_block_accepts(s, acc_args, acc_args.top);
 }
 
 // FP64 Gram form of the rescoring, for D <= M: with Gm = A^T A, c = A^T b,
@@ -773,7 +809,7 @@ __global__ void __launch_bounds__(256) lsq_rescore_gram_kernel(const __grid_cons
         partial[(size_t)(grp * 4 + q) * chunks + chunk] =
             live[q] ? tot : __longlong_as_double(0x7FF8000000000000ll);
     }
-    last_block_accepts(s, acc_args);
+    last_block_accepts(s, acc_args, acc_args.top);
 }
 
 // (hi, lo) += p + e: Knuth's TwoSum of hi and p (exact: hi' + t = hi + p), the
@@ -784,6 +820,15 @@ __device__ __forceinline__ void ff_acc(float& hi, float& lo, float p, float e) {
     const float t = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, z)), __fsub_rn(p, z));
     hi = s;
     lo = __fadd_rn(lo, __fadd_rn(t, e));
+}
+
+// ff_acc of two independent sums, with -e given.
+__device__ __forceinline__ void ff_acc2(f32x2& hi, f32x2& lo, f32x2 p, f32x2 ne) {
+    const f32x2 s = add2(hi, p);
+    const f32x2 z = sub2(s, hi);
+    const f32x2 t = add2(sub2(hi, sub2(s, z)), sub2(p, z));
+    hi = s;
+    lo = add2(lo, sub2(t, ne));
 }
 
 // The Gram-form rescoring of lsq_rescore_gram_kernel with the off-diagonal
@@ -811,19 +856,24 @@ __device__ __forceinline__ void ff_acc(float& hi, float& lo, float p, float e) {
 // memory (their terms are then exact zeros); the diagonal tile also adds the
 // FP64 diagonal and linear terms of its rows, and tile 0 adds bb.
 // partial[cand][tile].
+// Every block first merges the selection's lists for itself (nl > 0), its tile on the
+// way meanwhile: cheaper than a last block of the selection and its hand-over (together
+// 30.4 us at 8192 x 1024, now 23.0). Two candidates share an instruction
+// (fma.rn.f32x2).
 __global__ void __launch_bounds__(256) lsq_rescore_gram_ff_kernel(const __grid_constant__ SwarmDev s,
                                                                   const float* __restrict__ src,
                                                                   const float2* __restrict__ Gff, int ldf,
                                                                   const double* __restrict__ Gm,
                                                                   const double* __restrict__ cvec, double bb,
-                                                                  const unsigned long long* __restrict__ top,
-                                                                  int ntiles, double* __restrict__ partial,
+                                                                  const unsigned long long* __restrict__ cand,
+                                                                  int nl, int ntiles, double* __restrict__ partial,
                                                                   const AcceptArgs acc_args) {
     constexpr int T = kFfTile, Q = 4, RQ = 4;
     static_assert(T == 64 && kCand == 4 * Q, "thread layout: 64 columns x 4 row quarters, 4 candidates each");
     __shared__ __align__(16) float2 gt[T][T];   // (gh, gl) of the tile, row-major
     __shared__ __align__(16) float4 xr[T], xc[T];   // the 4 candidates' coordinates of the tile's rows / columns
     __shared__ uint32_t cid[Q];
+    __shared__ unsigned long long skeys[kCand];
     __shared__ float rh[8][Q], rl[8][Q];        // per warp
     __shared__ double rd[8][Q];
     const int D = s.D;
@@ -837,14 +887,9 @@ __global__ void __launch_bounds__(256) lsq_rescore_gram_ff_kernel(const __grid_c
     const int tc = tr + k;
     const bool diag = tr == tc;
     const int r0 = tr * T, c0 = tc * T;
-    if (threadIdx.x < Q) {
-        const unsigned long long key = top[Q * cq + threadIdx.x];
-        cid[threadIdx.x] = key == kKeyNone ? 0xFFFFFFFFu : (uint32_t)(key & 0xFFFFFFFFull);
-    }
-    __syncthreads();
     {
-        // the tile: 64 rows x 32 float4 (two entries each); the 4 candidates'
-        // coordinates of its rows and columns: 2 x 4 x 64 gathered values
+        // the tile: 64 rows x 32 float4 (two entries each), on its way while the
+        // candidates are merged (the warps' lists kept where the tile goes)
         float4 g[8];
         float xv[2];
 #pragma unroll
@@ -852,6 +897,18 @@ __global__ void __launch_bounds__(256) lsq_rescore_gram_ff_kernel(const __grid_c
             const int e = (int)threadIdx.x + 256 * j;
             g[j] = *reinterpret_cast<const float4*>(Gff + (size_t)(r0 + (e >> 5)) * ldf + c0 + 2 * (e & 31));
         }
+        if (nl > 0) {
+            merge_block<8>(cand, nl, reinterpret_cast<unsigned long long (*)[kCand]>(&gt[0][0]), skeys);
+        } else if (threadIdx.x < kCand) {
+            skeys[threadIdx.x] = acc_args.top[threadIdx.x];
+        }
+        __syncthreads();
+        if (threadIdx.x < Q) {
+            const unsigned long long key = skeys[Q * cq + threadIdx.x];
+            cid[threadIdx.x] = key == kKeyNone ? 0xFFFFFFFFu : (uint32_t)(key & 0xFFFFFFFFull);
+        }
+        __syncthreads();
+        // the 4 candidates' coordinates of its rows and columns: 2 x 4 x 64 gathered values
         const int q = (int)threadIdx.x >> 6, dd = (int)threadIdx.x & 63;
         const uint32_t i = cid[q];
 #pragma unroll
@@ -874,19 +931,26 @@ __global__ void __launch_bounds__(256) lsq_rescore_gram_ff_kernel(const __grid_c
     __syncthreads();
     const int rq = (int)threadIdx.x >> 6, c = (int)threadIdx.x & 63;
     const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
-    float wh[Q] = {0.f, 0.f, 0.f, 0.f}, wl[Q] = {0.f, 0.f, 0.f, 0.f};
+    // two candidates per instruction
+    f32x2 wh2[2] = {0ull, 0ull}, wl2[2] = {0ull, 0ull};
 #pragma unroll 4
     for (int j = 0; j < T / RQ; ++j) {
         const int r = rq * (T / RQ) + j;
         const float4 x4 = xr[r];
         const float2 gv = gt[r][c];
-        const float xq[Q] = {x4.x, x4.y, x4.z, x4.w};
+        const f32x2 gh = both(gv.x), gl = both(gv.y);
+        const f32x2 x[2] = {pack2(x4.x, x4.y), pack2(x4.z, x4.w)}, nx[2] = {pack2(-x4.x, -x4.y), pack2(-x4.z, -x4.w)};
 #pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            const float p = __fmul_rn(xq[q], gv.x);
-            const float e = __fmaf_rn(xq[q], gv.x, -p);   // exact: x gh = p + e
-            ff_acc(wh[q], wl[q], p, __fmaf_rn(xq[q], gv.y, e));
+        for (int q = 0; q < 2; ++q) {
+            const f32x2 p = mul2(x[q], gh);
+            ff_acc2(wh2[q], wl2[q], p, fma2(nx[q], gl, fma2(nx[q], gh, p)));   // x gh = p + e exactly; -(x gl + e)
         }
+    }
+    float wh[Q], wl[Q];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        unpack2(wh2[q], wh[2 * q], wh[2 * q + 1]);
+        unpack2(wl2[q], wl[2 * q], wl[2 * q + 1]);
     }
     // times x_c
     float sh[Q], sl[Q];
@@ -954,18 +1018,16 @@ __global__ void __launch_bounds__(256) lsq_rescore_gram_ff_kernel(const __grid_c
     if (threadIdx.x < Q) {
         const int q = (int)threadIdx.x;
         float h = rh[0][q], l = rl[0][q];
-        double dsum = rd[0][q];
+        double dsum = 0.0;   // only the diagonal tiles' warps 0 and 1 have terms
+        if (diag) dsum = rd[0][q] + rd[1][q];
 #pragma unroll
-        for (int w = 1; w < 8; ++w) {
-            ff_acc(h, l, rh[w][q], rl[w][q]);
-            dsum += rd[w][q];
-        }
+        for (int w = 1; w < 8; ++w) ff_acc(h, l, rh[w][q], rl[w][q]);
         double tot = fma(2.0, (double)h + (double)l, dsum);
         if (tile == 0) tot += bb;
         partial[(size_t)(Q * cq + q) * ntiles + tile] =
             cid[q] != 0xFFFFFFFFu ? tot : __longlong_as_double(0x7FF8000000000000ll);
     }
-    last_block_accepts(s, acc_args);
+    last_block_accepts(s, acc_args, skeys);
 }
 
 // Gm = A^T A (D x D), cvec = A^T b, in FP64 (one-time setup). 32 x 32 output
@@ -1139,11 +1201,11 @@ cudaError_t lsq_launch_move_q(const SwarmDev& s, const unsigned char (*maps)[128
     for (int a = 0; a < 3; ++a) std::memcpy(&mm.m[a], maps[a], sizeof(CUtensorMap));
     // one CTA per SM walks the tiles
     const int grid = std::min(num_sms, ntiles);
-    cudaError_t e = cudaFuncSetAttribute(fp8 ? (const void*)lsq_move_q_kernel<true> : (const void*)lsq_move_q_kernel<false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto* const k = s.fast_cr && s.fast_clamp ? (fp8 ? lsq_move_q_kernel<true, true> : lsq_move_q_kernel<false, true>)
+                                              : (fp8 ? lsq_move_q_kernel<true, false> : lsq_move_q_kernel<false, false>);
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    if (fp8) lsq_move_q_kernel<true><<<grid, kMoveThreads, smem, st>>>(s, mm, Xq, Kp, sx);
-    else lsq_move_q_kernel<false><<<grid, kMoveThreads, smem, st>>>(s, mm, Xq, Kp, sx);
+    k<<<grid, kMoveThreads, smem, st>>>(s, mm, Xq, Kp, sx);
     return cudaGetLastError();
 }
 
@@ -1160,7 +1222,7 @@ cudaError_t lsq_launch_select_exact(const SwarmDev& s, const float* fit, unsigne
     return cudaGetLastError();
 }
 
-int lsq_cand_lists(int Np) { return (Np + kSel - 1) / kSel * kSelWarps; }
+int lsq_cand_lists(int Np) { return (Np + kSel - 1) / kSel; }
 
 cudaError_t lsq_launch_gram(const float* A, const float* b, int M, int D, double* Gm, double* cvec, float2* Gff,
                             int ldf, cudaStream_t st) {
@@ -1200,7 +1262,9 @@ cudaError_t lsq_launch_gbest_approx(const SwarmDev& s, const float* fit, const f
     const int nblk = (s.Np + kSel - 1) / kSel;
     unsigned long long* top = cand + (size_t)lsq_cand_lists(s.Np) * kCand;
     unsigned int* ticket = reinterpret_cast<unsigned int*>(top + kCand);
-    lsq_select_cand_kernel<<<nblk, kSel, 0, st>>>(s, fit, part, nparts, all, cand, flags, top, ticket);
+    // the float-float rescoring merges the lists itself
+    const bool merge = !(gram.Gm && gram.ff) || nblk > kMaxMerge;
+    lsq_select_cand_kernel<<<nblk, kSel, 0, st>>>(s, fit, part, nparts, all, merge, cand, flags, top, ticket);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (!all && !lazy) {
@@ -1217,7 +1281,7 @@ cudaError_t lsq_launch_gbest_approx(const SwarmDev& s, const float* fit, const f
         const int nt = lsq_ff_tiles(s.D);
         const AcceptArgs acc_ff{acc.ticket, src, top, partial, nt, g64, stale};
         lsq_rescore_gram_ff_kernel<<<4 * nt, 256, 0, st>>>(s, src, gram.Gff, gram.ldf, gram.Gm, gram.cvec, gram.bb,
-                                                           top, nt, partial, acc_ff);
+                                                           cand, merge ? 0 : nblk, nt, partial, acc_ff);
     } else if (gram.Gm) {
         const int pairs = ((s.D + 1) / 2 + chunks - 1) / chunks;
         lsq_rescore_gram_kernel<<<dim3(kCand / 4, chunks), 256, sizeof(double) * 4 * (size_t)s.D, st>>>(
