@@ -18,13 +18,15 @@
 //
 // Measured on one GB300 (one evaluation; before: a block kept 64 particles x
 // all M, 32 blocks for 2048 particles on 152 SMs): FP32 2048 x 500 x 2000
-// 1.9 ms -> 117 us (the product 41 TFLOP/s), 8192 x 1024 x 4096 7.88 -> 1.53 ms
-// (46 TFLOP/s of about 80 at 128 lanes per SM and clock); FP64 8192 x 1024 x
+// 1.9 ms -> 101 us (the product 46 TFLOP/s), 8192 x 1024 x 4096 7.88 -> 1.23 ms
+// (60 TFLOP/s of about 80 at 128 lanes per SM and clock; the shared-memory reads and
+// the doubling of A's values beside the multiplications are the rest); FP64 8192 x 1024 x
 // 4096 127 -> 64 ms (1.08 TFLOP/s, the FP64 pipe: A and x are converted once
 // per stage, not in every thread's inner loop).
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "cupso_device.cuh"
 #include "cupso_internal.h"
@@ -38,9 +40,10 @@ constexpr size_t kExactWsBytes = 64u << 20;   // residual workspace at most
 constexpr int kResidThreads = 128;            // 16 x 8 threads of TM x TN residuals
 constexpr int kBk = 16;                       // dimensions per shared-memory stage
 constexpr int kRowTile = 128;                 // chunk sizes are multiples of this
-constexpr int kSumThreads = 128;
+constexpr int kSumCopiers = 128;              // the threads after the summing warp
+constexpr int kSumThreads = 32 + kSumCopiers;
 constexpr int kSumStageBytes = 8192;
-constexpr int kSumStages = 4;
+constexpr int kSumStages = 6;
 
 // TM x TN residuals of one thread: r[a][c] += av[a] * xv[c], one rounding each.
 template <typename T, int TM, int TN>
@@ -57,10 +60,8 @@ struct Acc<float, TM, TN> {
 #pragma unroll
         for (int c = 0; c < TN / 2; ++c) r[a][c] = p;
     }
-    __device__ __forceinline__ void step(const float (&av)[TM], const float (&xv)[TN]) {
-        unsigned long long x2[TN / 2];
-#pragma unroll
-        for (int c = 0; c < TN / 2; ++c) asm("mov.b64 %0, {%1, %2};" : "=l"(x2[c]) : "f"(xv[2 * c]), "f"(xv[2 * c + 1]));
+    // av: rows, x2: particles in pairs
+    __device__ __forceinline__ void step(const float (&av)[TM], const unsigned long long (&x2)[TN / 2]) {
 #pragma unroll
         for (int a = 0; a < TM; ++a) {
             unsigned long long a2;
@@ -92,7 +93,11 @@ struct Acc<double, TM, TN> {
     __device__ __forceinline__ double get(int a, int c) const { return r[a][c]; }
 };
 
-// 4 consecutive T from shared memory (16-byte aligned).
+// 4 consecutive T from shared memory (16-byte aligned), floats in pairs.
+__device__ __forceinline__ void ld4s(const float* p, unsigned long long* v) {
+    const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(p);
+    v[0] = q.x; v[1] = q.y;
+}
 __device__ __forceinline__ void ld4s(const float* p, float* v) {
     const float4 q = *reinterpret_cast<const float4*>(p);
     v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
@@ -118,16 +123,16 @@ __device__ __forceinline__ void st4g(double* p, const double* v) {
 // summed). vecA: A's rows may be read as float4 (D % 4 == 0, A 16-byte aligned).
 //
 // Block tile 16 TM rows x 8 TN particles, K in slices of kBk through two shared
-// stages: the next slice's A and x are loaded to registers while the current
-// one is multiplied, so one barrier per slice. A's slice is transposed on its
-// way ([k][row], padded), both operands are then read as 16-byte vectors that a
-// warp shares (4 row groups x 8 particle groups: one wavefront each). Zeros
-// past D leave a residual's square unchanged.
+// stages: the next slice's A is loaded to registers, its x copied to the other
+// stage (FP64: to registers, converted), while the current one is multiplied, so one
+// barrier per slice. A's slice is transposed on its way ([k][row], padded), both
+// operands are then read as 16-byte vectors that a warp shares (4 row groups x 8
+// particle groups). Zeros past D leave a residual's square unchanged.
 // FUSED: all rows fit one tile, so the block adds its particles' squares itself and
-// writes f; no workspace, no second launch (M = 40: 12.0 -> XX us per iteration of
+// writes f; no workspace, no second launch (M = 40: 12.0 -> 10.1 us per iteration of
 // a 256 x 16 swarm).
 template <typename T, int TM, int TN, bool FUSED>
-__global__ void __launch_bounds__(kResidThreads) lsq_resid_kernel(const float* __restrict__ x, int ldx, int D,
+__global__ void __launch_bounds__(kResidThreads, TM * TN == 128 ? 2 : TM * TN == 64 ? 3 : 1) lsq_resid_kernel(const float* __restrict__ x, int ldx, int D,
                                                                   const float* __restrict__ A,
                                                                   const float* __restrict__ b, int m0, int m1,
                                                                   T* __restrict__ R, int ldr, int vecA, int N,
@@ -135,16 +140,20 @@ __global__ void __launch_bounds__(kResidThreads) lsq_resid_kernel(const float* _
     constexpr int BM = 16 * TM, BN = 8 * TN;
     constexpr int AK = kBk * BM / kResidThreads;   // A elements per thread and slice: consecutive k of one row
     constexpr int XV = kBk * BN / 4 / kResidThreads;   // float4 of x per thread and slice
+    constexpr bool kF32 = sizeof(T) == 4;
     __shared__ __align__(16) T As[2][kBk][BM + 4];
     __shared__ __align__(16) T Xs[2][kBk][BN];
     const int tid = threadIdx.x;
-    const int tx = tid & 7, ty = tid >> 3;
+    // a warp's 4 row groups x 8 particle groups, neighbouring lanes in different rows: a
+    // quarter of the warp then reads 2 rows' and 4 particles' vectors (8192 x 1024 x 4096:
+    // 1572 us an iteration with 1 and 8, 1469 so)
+    const int tx = (tid >> 1) & 7, ty = ((tid >> 4) << 1) | (tid & 1);
     const int i0 = blockIdx.x * BN, mt = m0 + blockIdx.y * BM;
     const int arow = tid % BM, ak = (tid / BM) * AK;
     const float* aptr = A + (size_t)min(mt + arow, m1 - 1) * (size_t)D;   // rows past m1 are computed, not stored
     float ar[AK];
     float4 xr[XV];
-    auto fetch = [&](int k0) {
+    auto fetch = [&](int k0, int st) {
         const int ka = k0 + ak;
         if (vecA) {
 #pragma unroll
@@ -159,42 +168,51 @@ __global__ void __launch_bounds__(kResidThreads) lsq_resid_kernel(const float* _
 #pragma unroll
         for (int q = 0; q < XV; ++q) {
             const int e = tid + q * kResidThreads, k = k0 + e / (BN / 4);
-            xr[q] = k < D ? *reinterpret_cast<const float4*>(x + (size_t)k * ldx + i0 + 4 * (e % (BN / 4)))
-                          : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float* from = x + (size_t)k * ldx + i0 + 4 * (e % (BN / 4));
+            if constexpr (kF32) {   // straight to the stage
+                const unsigned to = (unsigned)__cvta_generic_to_shared(&Xs[st][e / (BN / 4)][4 * (e % (BN / 4))]);
+                const unsigned n = k < D ? 16u : 0u;   // zeros past D
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(k < D ? from : x), "r"(n)
+                             : "memory");
+            } else {
+                xr[q] = k < D ? *reinterpret_cast<const float4*>(from) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
         }
     };
     auto stage = [&](int st) {
 #pragma unroll
         for (int j = 0; j < AK; ++j) As[st][ak + j][arow] = (T)ar[j];
+        if constexpr (kF32) asm volatile("cp.async.wait_all;" ::: "memory");
 #pragma unroll
-        for (int q = 0; q < XV; ++q) {
+        for (int q = 0; q < (kF32 ? 0 : XV); ++q) {
             const int e = tid + q * kResidThreads;
             const T v[4] = {(T)xr[q].x, (T)xr[q].y, (T)xr[q].z, (T)xr[q].w};
             st4g(&Xs[st][e / (BN / 4)][4 * (e % (BN / 4))], v);
         }
     };
-    // the thread's rows ty * 4 + j (+ BM / 2) and particles tx * 4 + j (+ BN / 2)
-    auto row_of = [&](int a) { return (a / 4) * (BM / 2) + ty * 4 + a % 4; };
+    // the thread's rows ty * 4 + j (+ 64) and particles tx * 4 + j (+ 32, 64, 96)
+    auto row_of = [&](int a) { return (a / 4) * (BM * 4 / TM) + ty * 4 + a % 4; };
     Acc<T, TM, TN> acc;
 #pragma unroll
     for (int a = 0; a < TM; ++a) {
         const int m = mt + row_of(a);
         acc.set(a, m < m1 ? -(T)b[m] : (T)0);
     }
-    fetch(0);
+    fetch(0, 0);
     stage(0);
     __syncthreads();
     const int slices = (D + kBk - 1) / kBk;
     for (int s = 0; s < slices; ++s) {
         const int st = s & 1;
-        if (s + 1 < slices) fetch((s + 1) * kBk);
+        if (s + 1 < slices) fetch((s + 1) * kBk, st ^ 1);
 #pragma unroll
         for (int k = 0; k < kBk; ++k) {
-            T av[TM], xv[TN];
+            T av[TM];
+            std::conditional_t<kF32, unsigned long long, T> xv[kF32 ? TN / 2 : TN];
 #pragma unroll
-            for (int a = 0; a < TM; a += 4) ld4s(&As[st][k][(a / 4) * (BM / 2) + ty * 4], av + a);
+            for (int a = 0; a < TM; a += 4) ld4s(&As[st][k][(a / 4) * (BM * 4 / TM) + ty * 4], av + a);
 #pragma unroll
-            for (int c = 0; c < TN; c += 4) ld4s(&Xs[st][k][(c / 4) * (BN / 2) + tx * 4], xv + c);
+            for (int c = 0; c < TN; c += 4) ld4s(&Xs[st][k][(c / 4) * (BN * 4 / TN) + tx * 4], xv + (kF32 ? c / 2 : c));
             acc.step(av, xv);
         }
         if (s + 1 < slices) stage(st ^ 1);   // the other stage: read last before the previous barrier
@@ -205,7 +223,7 @@ __global__ void __launch_bounds__(kResidThreads) lsq_resid_kernel(const float* _
 #pragma unroll
         for (int a = 0; a < TM; ++a)
 #pragma unroll
-            for (int c = 0; c < TN; ++c) Rs[row_of(a)][(c / 4) * (BN / 2) + tx * 4 + c % 4] = acc.get(a, c);
+            for (int c = 0; c < TN; ++c) Rs[row_of(a)][(c / 4) * (BN * 4 / TN) + tx * 4 + c % 4] = acc.get(a, c);
         __syncthreads();
         if (tid < BN && i0 + tid < N) {
             T sum = (T)0;
@@ -232,13 +250,13 @@ __global__ void __launch_bounds__(kResidThreads) lsq_resid_kernel(const float* _
 #pragma unroll
                 for (int e = 0; e < 4; ++e) v[e] = __dmul_rn(v[e], v[e]);
             }
-            st4g(row + (c / 4) * (BN / 2) + tx * 4, v);
+            st4g(row + (c / 4) * (BN * 4 / TN) + tx * 4, v);
         }
     }
 }
 
 // carry[i] (+)= the squares of R[0 .. rows - 1][i] (FP64: R itself) in row order; the last chunk
-// rounds the sum into f[i]. A block takes 32 particles: all its threads copy the
+// rounds the sum into f[i]. A block takes 32 particles: four warps copy the
 // rows into a ring of kSumStages shared stages ahead of warp 0, which adds one
 // particle per lane -- a dependent chain of `rows` operations that no split can
 // shorten, so only the loads are taken off it.
@@ -248,15 +266,17 @@ __global__ void __launch_bounds__(kSumThreads) lsq_sumsq_kernel(const T* __restr
                                                                 float* __restrict__ f) {
     constexpr int kRows = kSumStageBytes / (32 * (int)sizeof(T));   // rows per stage
     constexpr int kVec = 16 / (int)sizeof(T);
-    constexpr int kCopies = kSumStageBytes / 16 / kSumThreads;
+    constexpr int kCopies = kSumStageBytes / 16 / kSumCopiers;
+    constexpr int kAhead = 16;
+    static_assert(kRows % kAhead == 0 && kSumStageBytes % (16 * kSumCopiers) == 0, "whole groups");
     __shared__ __align__(16) T ring[kSumStages][kRows][32];
     const int tid = threadIdx.x, i0 = blockIdx.x * 32, i = i0 + tid;
     const int stages = (rows + kRows - 1) / kRows;
     auto issue = [&](int st) {
-        if (st < stages) {
+        if (st < stages && tid >= 32) {
 #pragma unroll
             for (int q = 0; q < kCopies; ++q) {
-                const int e = tid + q * kSumThreads, rr = e / (32 / kVec), col = (e % (32 / kVec)) * kVec;
+                const int e = tid - 32 + q * kSumCopiers, rr = e / (32 / kVec), col = (e % (32 / kVec)) * kVec;
                 const int row = st * kRows + rr;
                 if (row < rows) {
                     const unsigned sa = (unsigned)__cvta_generic_to_shared(&ring[st % kSumStages][rr][col]);
@@ -279,11 +299,27 @@ __global__ void __launch_bounds__(kSumThreads) lsq_sumsq_kernel(const T* __restr
         if (tid < 32) {
             const int n = min(kRows, rows - st * kRows);
             const T(*row)[32] = ring[st % kSumStages];
-#pragma unroll 16
-            for (int rr = 0; rr < n; ++rr) {
-                const T v = row[rr][tid];
+            auto add = [&](T v) {
                 if constexpr (sizeof(T) == 8) acc = __dadd_rn(acc, v);
                 else acc = __fmaf_rn(v, v, acc);
+            };
+            if (n == kRows) {   // the next kAhead rows' values are read while these are added
+                T v[kAhead], w[kAhead];
+#pragma unroll
+                for (int e = 0; e < kAhead; ++e) v[e] = row[e][tid];
+#pragma unroll
+                for (int rr = kAhead; rr <= kRows; rr += kAhead) {
+                    if (rr < kRows) {
+#pragma unroll
+                        for (int e = 0; e < kAhead; ++e) w[e] = row[rr + e][tid];
+                    }
+#pragma unroll
+                    for (int e = 0; e < kAhead; ++e) add(v[e]);
+#pragma unroll
+                    for (int e = 0; e < kAhead; ++e) v[e] = w[e];
+                }
+            } else {
+                for (int rr = 0; rr < n; ++rr) add(row[rr][tid]);
             }
         }
     }
@@ -341,9 +377,18 @@ cudaError_t exact_launch(const float* x, int ldx, int N, int D, const float* A, 
             } else {
                 // 128 x 64 tiles once they cover half the SMs (1024 x 1024 x 1024, 128 of them:
                 // 70 us against 97 with 64 x 32 tiles), the small ones below (1024 x 64 x 512,
-                // 64 large tiles: 6.3 us against 8.3)
-                const long long big = (long long)(np / 64) * ((m1 - m0 + 127) / 128);
-                if (2 * big >= num_sms) launch_resid<T, 8, 8>(x + p0, ldx, np, D, A, b, m0, m1, R, st);
+                // 64 large tiles: 6.3 us against 8.3). 128 x 128 tiles take a fifth less time for
+                // the same residuals (half the shared-memory reads per product), so they run
+                // where the tiles of the fullest SM come to less at that rate: an iteration of
+                // 8192 x 1024 x 4096 1279 us against 1471, 2048 x 500 x 2000 136 against 142;
+                // 4000 x 300 x 1200, 3 tiles against 5, 112 against 105
+                // and the SMs mostly get two (8000 x 16 x 130, 126 tiles: 16.9 against 15.7)
+                const long long rows = (m1 - m0 + 127) / 128, big = (long long)(np / 64) * rows;
+                const long long wide = (long long)(np / 128) * rows;
+                const long long of128 = (wide + num_sms - 1) / num_sms, of64 = (big + num_sms - 1) / num_sms;
+                if (5 * of128 < 3 * of64 && 2 * wide >= 3 * num_sms)
+                    launch_resid<T, 8, 16>(x + p0, ldx, np, D, A, b, m0, m1, R, st);
+                else if (2 * big >= num_sms) launch_resid<T, 8, 8>(x + p0, ldx, np, D, A, b, m0, m1, R, st);
                 else launch_resid<T, 4, 4>(x + p0, ldx, np, D, A, b, m0, m1, R, st);
             }
             lsq_sumsq_kernel<T><<<(n + 31) / 32, kSumThreads, 0, st>>>(R, np, m1 - m0, n, carry, m0 == 0, m1 == M, f + p0);
