@@ -32,6 +32,19 @@ struct FitTerms {
             return 0.0f;
         }
     }
+    // two dimensions' terms, |x| <= kSmallX (not Rosenbrock's)
+    __device__ static __forceinline__ float2 two(float x0, float x1) {
+        if constexpr (FIT == kRastrigin || FIT == kAckley) {
+            float c0, c1;
+            cos2pi_small2(x0, x1, c0, c1);
+            if constexpr (FIT == kAckley) return make_float2(c0, c1);
+            const f32x2 x = pack2(x0, x1);
+            unpack2(fma2(x, x, fma2(both(-10.0f), pack2(c0, c1), both(10.0f))), c0, c1);
+            return make_float2(c0, c1);
+        } else {
+            return make_float2(term<true>(x0, 0.0f), term<true>(x1, 0.0f));
+        }
+    }
     // particle column p (stride P) of X and H
     __device__ static __forceinline__ float sum(const float* X, const float* H, int P, int p, int D) {
         FitAcc<FIT> a;
