@@ -72,7 +72,8 @@ cudaError_t launch_batch_panel_init(const BatchDev& b, int num_sms, cudaStream_t
 // x, v, pb at ((d / W) * Np + i) * W + d % W, panel width W = 8 or 16, ring
 // depth 3 or 5 panels.
 bool panel_supported(int width, int stages, int D);
-bool panel_fast(const SwarmDev& s, int fid);   // whether the fast form runs
+// Whether the fast forms of the panel and pipelined kernels run (move_two_fast, cos2pi_small2).
+bool fast_form(const SwarmDev& s, int fid);
 cudaError_t prepare_panel(int fid, bool fast);
 int panel_blocks_per_sm(int width, int stages, int fid, int D);
 // Iterations of one panel launch; more than one is a cooperative launch with a

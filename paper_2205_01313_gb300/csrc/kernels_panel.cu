@@ -242,7 +242,7 @@ __device__ __forceinline__ unsigned long long panel_units(const SwarmDev& s, flo
 
 // `iters` synchronous iterations. Requires D % W == 0, D / W >= STAGES - 1,
 // Np a multiple of 128, s.pflag, s.work and s.bar set, work and bar zero at
-// launch. FAST: panel_fast(s, FIT); moves and cosines of two dimensions per instruction
+// launch. FAST: fast_form(s, FIT); moves and cosines of two dimensions per instruction
 // (fma.rn.f32x2): the kernel's issue slots were 61 % taken, and an iteration of
 // Rastrigin's 65536 x 128 took 33.6 us with scalar ones and the rounding instruction,
 // now 31.7 (Ackley 34.3 and 32.4, sphere 29.0 and 28.2).
@@ -412,7 +412,7 @@ const void* panel_kernel(int width, int stages, bool fast, int fid) {
 }  // namespace
 
 // The fast form's cosines are cos2pi_small.
-bool panel_fast(const SwarmDev& s, int fid) {
+bool fast_form(const SwarmDev& s, int fid) {
     const bool has_cos = fid == kRastrigin || fid == kAckley;
     return s.fast_cr && s.fast_clamp && (!has_cos || (std::fabs(s.lo) <= kSmallX && std::fabs(s.hi) <= kSmallX));
 }
@@ -450,7 +450,7 @@ cudaError_t launch_sync_panel(const SwarmDev& s, int fid, int width, int stages,
     if (!panel_supported(width, stages, s.D) || !s.pflag || !s.work || !s.bar || s.Np % 128 != 0 || iters < 1 ||
         iters > kPanelMaxIters || grid < 1 || (unsigned long long)iters * ((unsigned long long)grid + 2ull) >= (1ull << 32))
         return cudaErrorInvalidValue;
-    const void* k = panel_kernel(width, stages, panel_fast(s, fid), fid);
+    const void* k = panel_kernel(width, stages, fast_form(s, fid), fid);
     if (!k) return cudaErrorInvalidValue;
     unsigned int expect = (unsigned int)grid + (stall_barrier ? 1u : 0u);
     void* args[] = {const_cast<SwarmDev*>(&s), &iters, &expect};

@@ -194,17 +194,36 @@ __global__ void __launch_bounds__(kBlock, (P == 4 ? 3 : (P == 2 ? 4 : 5)))
                     stv<P>(s.pb + off, Pb);
                 }
                 const float gd = Gs[d];
+                if constexpr (FAST && P >= 2) {
 #pragma unroll
-                for (int j = 0; j < P; ++j) {
-                    float xj = vget(X, j), vj = vget(V, j);
-                    if constexpr (FAST)
-                        move_one_fast(xj, vj, vget(Pb, j), gd, hi24(word(rr[j], 2 * h)), hi24(word(rr[j], 2 * h + 1)),
-                                      s);
-                    else
-                        move_one(xj, vj, vget(Pb, j), gd, u01(word(rr[j], 2 * h)), u01(word(rr[j], 2 * h + 1)), s);
-                    vset(X, j, xj);
-                    vset(V, j, vj);
-                    acc[j].add(d, xj);
+                    for (int j = 0; j < P; j += 2) {
+                        float x0 = vget(X, j), x1 = vget(X, j + 1), v0 = vget(V, j), v1 = vget(V, j + 1);
+                        move_two_fast(x0, x1, v0, v1, pack2(vget(Pb, j), vget(Pb, j + 1)), both(gd),
+                                      pack2(hi24(word(rr[j], 2 * h)), hi24(word(rr[j + 1], 2 * h))),
+                                      pack2(hi24(word(rr[j], 2 * h + 1)), hi24(word(rr[j + 1], 2 * h + 1))), s);
+                        vset(X, j, x0);
+                        vset(X, j + 1, x1);
+                        vset(V, j, v0);
+                        vset(V, j + 1, v1);
+                        float c0 = 0.0f, c1 = 0.0f;
+                        if constexpr (FitAcc<FIT>::kNeedsCos) cos2pi_small2(x0, x1, c0, c1);
+                        acc[j].add_c(d, x0, c0);
+                        acc[j + 1].add_c(d, x1, c1);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < P; ++j) {
+                        float xj = vget(X, j), vj = vget(V, j);
+                        if constexpr (FAST)
+                            move_one_fast(xj, vj, vget(Pb, j), gd, hi24(word(rr[j], 2 * h)),
+                                          hi24(word(rr[j], 2 * h + 1)), s);
+                        else
+                            move_one(xj, vj, vget(Pb, j), gd, u01(word(rr[j], 2 * h)), u01(word(rr[j], 2 * h + 1)), s);
+                        vset(X, j, xj);
+                        vset(V, j, vj);
+                        if constexpr (FAST && FitAcc<FIT>::kNeedsCos) acc[j].add_c(d, xj, cos2pi_small(xj));
+                        else acc[j].add(d, xj);
+                    }
                 }
                 stv<P>(s.x + off, X);
                 stv<P>(s.v + off, V);
@@ -338,7 +357,7 @@ cudaError_t launch_materialize(const SwarmDev& s, int grid, cudaStream_t st) {
 cudaError_t launch_sync_pipelined(const SwarmDev& s, int fid, int stages, int ppt, int grid, cudaStream_t st) {
     if (!pipelined_supported(stages, s.D) || !s.pflag || (ppt != 1 && ppt != 2 && ppt != 4))
         return cudaErrorInvalidValue;
-    const void* k = kernel_of(stages, s.fast_cr && s.fast_clamp, fid, ppt);
+    const void* k = kernel_of(stages, fast_form(s, fid), fid, ppt);
     if (!k) return cudaErrorInvalidValue;
     void* args[] = {const_cast<SwarmDev*>(&s)};
     return cudaLaunchKernel(k, dim3(grid), dim3(kBlock), args, smem_of(stages, ppt, s.D), st);
