@@ -138,14 +138,15 @@ int resolved_mode(const cupso_swarm* h) {
 // Particles per tile when the tiled SYNC kernel runs, else 0. AUTO takes it
 // for D >= 8 up to the crossover measured on a GB300 against the pipelined
 // kernel (which runs over d inside each thread and needs many particles per
-// SM to hide its row latency): about 896 particles per SM, or 224 when the
-// tiles are narrow (D > 64, so at most 32 particles per tile) and the fitness
-// is cheap (no cos(2 pi x) to spread over the threads).
+// SM to hide its row latency), tiled and pipelined in us per iteration: sphere 50000 x
+// 63 19.3 and 23.3, 100000 x 15 12.1 and 11.9, 60000 x 99 30.5 and 33.7, 80000 x 99 42.4 and
+// 42.2, 50000 x 150 46.4 and 48.0, 60000 x 201 76 and 64; Rosenbrock, whose terms need the
+// next dimension's value too, 50000 x 33 14.5 and 15.4, 60000 x 65 28.9 and 25.2, 35000 x
+// 201 54 and 53.
 int sync_tile(const cupso_swarm* h) {
     if (h->fp64) return 0;
     if (h->sync_kernel == CUPSO_SYNC_KERNEL_TILED) return tiled_particles(h->N, h->D, h->num_sms);
     if (h->sync_kernel != CUPSO_SYNC_KERNEL_AUTO || h->D < 8) return 0;
-    const bool has_cos = h->fid == CUPSO_RASTRIGIN || h->fid == CUPSO_ACKLEY;
     if (h->panel_ok && h->D % 8 == 0) {
         // against the panel kernel running each cupso_step call in one cooperative
         // launch (sweep on one GB300, N = 4096 .. 262144, D = 16 .. 256, Rosenbrock and
@@ -154,7 +155,7 @@ int sync_tile(const cupso_swarm* h) {
         const long long pd = (long long)h->N * h->D;
         return pd < (1ll << 17) ? tiled_particles(h->N, h->D, h->num_sms) : 0;
     }
-    const long long per_sm = (has_cos || h->D <= 64) ? 896 : 224;
+    const long long per_sm = h->fid == CUPSO_ROSENBROCK ? (h->D <= 64 ? 330 : 224) : (h->D <= 128 ? 400 : 330);
     if ((long long)h->N > per_sm * h->num_sms) return 0;
     return tiled_particles(h->N, h->D, h->num_sms);
 }
@@ -219,15 +220,26 @@ PanelCfg panel_cfg(const cupso_swarm* h) {
     return c;
 }
 
-// Particles per thread of the pipelined kernel: 4 when the swarm has enough
-// 128-particle units to keep every resident warp busy twice over, else fewer
-// (more, smaller units).
+// Particles per thread of the pipelined kernel: fewer make more and shorter units, more
+// share the Philox calls' latency and their copies' instructions. Sweep on one GB300 (us
+// per iteration with 1, 2 and 4): 2000 x 7 6.9, 7.1, 7.8; 35000 x 65 22.8, 20.2, 24.5; 80000
+// x 127 66, 53, 56; 100000 x 127 74, 65, 57; 300000 x 63 93, 87, 83; 10^6 x 7 46, 32, 28.
 int sync_ppt(const cupso_swarm* h) {
     if (h->ppt_option) return h->ppt_option;
-    const long long resident_warps = (long long)h->num_sms * 16;
-    if ((long long)h->Np >= 128ll * 2 * resident_warps) return 4;
-    if ((long long)h->Np >= 64ll * resident_warps) return 2;
+    if ((long long)h->Np >= 640ll * h->num_sms) return 4;
+    if ((long long)h->Np >= 128ll * h->num_sms) return 2;
     return 1;
+}
+
+// CTAs of a kernel whose warps take units, the first ones CTA by CTA: the same number on
+// every SM, at most `per_sm`, as few as hold a warp per unit. (With the units' own number
+// of CTAs some SMs had two and most one: 40000 x 32 in panels 11.1 us an iteration, now
+// 8.5; 20000 x 128 15.2 and 12.9.)
+int even_grid(const cupso_swarm* h, int units, int per_sm) {
+    const int warps = kBlock / 32;
+    if (h->grid_override > 0) return std::min(h->grid_override, (units + warps - 1) / warps);
+    const int want = (int)(((long long)units + (long long)warps * h->num_sms - 1) / ((long long)warps * h->num_sms));
+    return std::min(h->num_sms * std::min(per_sm, want), units);
 }
 
 int sync_grid(const cupso_swarm* h) {
@@ -235,20 +247,14 @@ int sync_grid(const cupso_swarm* h) {
     if (pc.width) {
         // persistent: warps pull units of 128 / width particles from a counter
         const int units = h->Np / (128 / pc.width);
-        int g = h->grid_override > 0 ? h->grid_override
-                                     : h->num_sms * panel_blocks_per_sm(pc.width, pc.stages, h->fid, h->D);
-        const int useful = (units + kBlock / 32 - 1) / (kBlock / 32);
-        return g < useful ? g : useful;
+        return even_grid(h, units, panel_blocks_per_sm(pc.width, pc.stages, h->fid, h->D));
     }
     const int stages = sync_stages(h);
     if (stages) {
         // persistent: warps pull units of 32 * ppt particles from a counter
         const int ppt = sync_ppt(h);
         const int units = h->Np / (32 * ppt);
-        const int per_sm = pipelined_blocks_per_sm(stages, h->fid, h->D, ppt);
-        int g = h->grid_override > 0 ? h->grid_override : h->num_sms * per_sm;
-        const int useful = (units + kBlock / 32 - 1) / (kBlock / 32);
-        return g < useful ? g : useful;
+        return even_grid(h, units, pipelined_blocks_per_sm(stages, h->fid, h->D, ppt));
     }
     const int ntiles = tiles_of(h->Np);
     int g = h->grid_override > 0 ? h->grid_override : h->num_sms * sync_blocks_per_sm(h->fid, h->D);
@@ -312,8 +318,8 @@ int async_block(const cupso_swarm* h) {
 }
 
 // Particles per tile of the tiled asynchronous kernel (0: the streaming one),
-// by the crossover of the synchronous kernels: tiles where the tiled SYNC
-// kernel is the faster one, else the streaming layout, which large swarms fill.
+// tiles up to about 896 particles per SM (224 with narrow tiles and a cheap fitness),
+// else the streaming layout, which large swarms fill.
 int async_tile(const cupso_swarm* h) {
     if (h->fp64 || h->D < 2) return 0;
     const bool has_cos = h->fid == CUPSO_RASTRIGIN || h->fid == CUPSO_ACKLEY;

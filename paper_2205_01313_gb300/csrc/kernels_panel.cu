@@ -66,7 +66,9 @@ struct UnitFeed {
     uint32_t spare = 0xFFFFFFFFu;   // the second unit of the last fetch, if not yet taken
     uint32_t base;
     uint32_t npairs;                // fetches 0 .. npairs - 1 hand out two units
-    __device__ __forceinline__ UnitFeed(uint32_t nunits, uint32_t nwarps) : base(nwarps), npairs(0u) {
+    bool more;                      // there are units after the warps' own
+    __device__ __forceinline__ UnitFeed(uint32_t nunits, uint32_t nwarps)
+        : base(nwarps), npairs(0u), more(nunits > nwarps) {
         if (nunits >= 8u * nwarps) {
             const uint32_t dyn = nunits - nwarps, tail = 2u * nwarps;
             npairs = (dyn - tail) / 2u;
@@ -78,6 +80,7 @@ struct UnitFeed {
             spare = 0xFFFFFFFFu;
             return u;
         }
+        if (!more) return base;
         uint32_t k = 0;
         if (lane_id == 0) k = atomicAdd(s.work, 1u);
         k = __shfl_sync(0xFFFFFFFFu, k, 0);
@@ -247,7 +250,7 @@ __device__ __forceinline__ unsigned long long panel_units(const SwarmDev& s, flo
 // Rastrigin's 65536 x 128 took 33.6 us with scalar ones and the rounding instruction,
 // now 31.7 (Ackley 34.3 and 32.4, sphere 29.0 and 28.2).
 //
-// Each warp takes unit (its warp index) first in every iteration, then units
+// Each warp takes unit (its warp in the CTA) x gridDim.x + blockIdx.x first in every iteration, then units
 // from the counter. With more than one iteration, every CTA must be resident
 // (a cooperative launch): an iteration ends in a grid barrier on s.bar -- each
 // CTA arrives once; the last to arrive gathers gbest_pos and releases the
@@ -269,7 +272,8 @@ __global__ void __launch_bounds__(kBlock, 3) sync_panel_kernel(const __grid_cons
     const uint32_t pl = (uint32_t)(lane_id / L);
     const uint32_t nunits = (uint32_t)s.Np / PU;
     const uint32_t nwarps = gridDim.x * (kBlock / 32);
-    const uint32_t u0 = blockIdx.x * (kBlock / 32) + (uint32_t)(threadIdx.x >> 5);
+    // CTA by CTA, so that every SM gets the same number when there are few
+    const uint32_t u0 = (uint32_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     float4* my = ring + threadIdx.x;
     const uint32_t t_prev = __ldcg(s.t_dev);
 

@@ -4,13 +4,13 @@
 // Same arithmetic and the same aggregation as sync_step_kernel (Steps 2-5 in
 // one launch; conditional warp argmin + one 64-bit atomicMin; last CTA gathers
 // gbest_pos), organised for bandwidth:
-//  * each thread copies its own float4 of pos, v and pbest_pos rows into a
+//  * each warp copies its own stretch of pos, v and pbest_pos rows into a
 //    private slot ring in shared memory with cp.async, STAGES-1 dimension
 //    pairs ahead of the pair it computes on, so the bytes in flight per SM no
 //    longer depend on how many registers hold loaded values (the structure-of-
 //    arrays rows of Sec. 4.1 stay fully coalesced: a warp copies 512 B of one
 //    row per instruction);
-//  * no thread reads another thread's slots, so the ring needs no barrier;
+//  * no warp reads another warp's slots, so the ring needs no barrier of the block;
 //  * warps take units of 32 x PPT particles from a counter, so work is
 //    balanced across SMs to within one unit instead of one 1024-particle
 //    tile; PPT (particles per thread: 4, 2 or 1, loaded as float4, float2 or
@@ -49,15 +49,9 @@ __device__ __forceinline__ void stv(float* p, const typename VT<P>::T& v) {
     *reinterpret_cast<typename VT<P>::T*>(p) = v;
 }
 
-template <int P>
-__device__ __forceinline__ void cp_async_v(typename VT<P>::T* smem, const float* gmem) {
+__device__ __forceinline__ void cp16(void* smem, const float* gmem) {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    if constexpr (P == 4)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-    else if constexpr (P == 2)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -65,28 +59,51 @@ __device__ __forceinline__ void cp_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-__device__ __forceinline__ uint32_t fetch_unit(const SwarmDev& s, int lane_id) {
+// The units after the warps' first ones, from the counter; none is drawn where every unit
+// has its warp.
+__device__ __forceinline__ uint32_t fetch_unit(const SwarmDev& s, uint32_t nunits, int lane_id) {
+    const uint32_t warps = gridDim.x * (kBlock / 32);
+    if (nunits <= warps) return nunits;
     uint32_t u = 0;
-    if (lane_id == 0) u = atomicAdd(s.work, 1u);
+    if (lane_id == 0) u = warps + atomicAdd(s.work, 1u);
     return __shfl_sync(0xFFFFFFFFu, u, 0);
 }
 
 // Copies of one step (unit u, dimension pair g) into ring stage `stage`:
 // rows 2g and 2g+1 of pos, v and pbest_pos, P floats per lane per row.
-// Slot (stage, a, r) of this thread is my[(stage * 6 + 2 * a + r) * kBlock].
+// Slot (stage, a, r) of a thread is my[(stage * 6 + 2 * a + r) * kBlock]; the 32 slots of
+// a warp are contiguous, and the warp copies them in pieces of 16 bytes past L1 whatever
+// P is, so with P < 4 a lane copies other lanes' values: a __syncwarp comes between the
+// wait and the reads, and between the reads and the next copies into a stage. (With each
+// lane copying its own 4 or 8 bytes through L1, 130000 x 201 took 169 us an iteration at P = 1
+// and 129 at P = 2, so 143 and 120.)
 template <int P>
 __device__ __forceinline__ void issue_step(const SwarmDev& s, typename VT<P>::T* my, uint32_t u, int g, int stage,
                                            uint32_t nunits, int lane_id) {
+    constexpr int kPieces = 8 * P;   // of a row
     if (u < nunits) {
-        const size_t col = (size_t)u * (32 * P) + (size_t)lane_id * P;
+        const float* const from[3] = {s.x, s.v, s.pb};
+        float* to = reinterpret_cast<float*>(my - lane_id + stage * 6 * kBlock);
+        if constexpr (P == 4) {
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int d = 2 * g + r;
-            if (d < s.D) {
-                const size_t off = (size_t)d * (size_t)s.Np + col;
-                cp_async_v<P>(my + (stage * 6 + 0 + r) * kBlock, s.x + off);
-                cp_async_v<P>(my + (stage * 6 + 2 + r) * kBlock, s.v + off);
-                cp_async_v<P>(my + (stage * 6 + 4 + r) * kBlock, s.pb + off);
+            for (int r = 0; r < 2; ++r) {
+                const int d = 2 * g + r;
+                if (d < s.D) {
+                    const size_t off = (size_t)d * (size_t)s.Np + (size_t)u * 128 + (size_t)lane_id * 4;
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) cp16(to + (2 * a + r) * kBlock * 4 + 4 * lane_id, from[a] + off);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < (6 * kPieces + 31) / 32; ++k) {
+                const int c = lane_id + 32 * k, slot = c / kPieces, piece = c % kPieces;
+                const int d = 2 * g + (slot & 1);
+                if (slot < 6 && d < s.D) {
+                    const float* f = slot < 2 ? s.x : slot < 4 ? s.v : s.pb;
+                    cp16(to + slot * kBlock * P + 4 * piece,
+                         f + (size_t)d * (size_t)s.Np + (size_t)u * (32 * P) + 4 * piece);
+                }
             }
         }
     }
@@ -142,7 +159,8 @@ __global__ void __launch_bounds__(kBlock, (P == 4 ? 3 : (P == 2 ? 4 : 5)))
     const size_t Np = (size_t)s.Np;
     T* my = ring + threadIdx.x;
 
-    uint32_t u_cur = fetch_unit(s, lane_id);
+    // first units CTA by CTA, so that every SM gets the same number when there are few
+    uint32_t u_cur = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     uint32_t fl_cur = u_cur < nunits ? load_flags<P>(s, u_cur * kUnit + (uint32_t)lane_id * P) : 0u;
     uint32_t u_nxt = 0xFFFFFFFFu, fl_nxt = 0u;
 #pragma unroll
@@ -159,13 +177,14 @@ __global__ void __launch_bounds__(kBlock, (P == 4 ? 3 : (P == 2 ? 4 : 5)))
         for (int g = 0; g < npairs; ++g) {
             // keep STAGES-1 pairs in flight: issue the pair STAGES-1 ahead
             {
+                if constexpr (P < 4) __syncwarp();
                 int ws = stage + STAGES - 1;
                 if (ws >= STAGES) ws -= STAGES;
                 if (ig < npairs) {
                     issue_step<P>(s, my, u_cur, ig, ws, nunits, lane_id);
                 } else {
                     if (u_nxt == 0xFFFFFFFFu) {
-                        u_nxt = fetch_unit(s, lane_id);
+                        u_nxt = fetch_unit(s, nunits, lane_id);
                         if (u_nxt < nunits) fl_nxt = load_flags<P>(s, u_nxt * kUnit + (uint32_t)lane_id * P);
                     }
                     issue_step<P>(s, my, u_nxt, ig - npairs, ws, nunits, lane_id);
@@ -174,6 +193,7 @@ __global__ void __launch_bounds__(kBlock, (P == 4 ? 3 : (P == 2 ? 4 : 5)))
             }
             if (g == npairs - 1) PF = ldv<P>(s.pf + i0);  // needed after the last pair
             cp_wait<STAGES - 1>();  // this thread's copies of the current pair have landed
+            if constexpr (P < 4) __syncwarp();
             uint4 rr[P];
 #pragma unroll
             for (int j = 0; j < P; ++j)
