@@ -13,8 +13,8 @@
 // dimensions, and a batch of a few dozen swarms is over when its last 256-dimensional
 // unit is -- 64 uneven swarms (N 64 .. 8192, D 8 .. 256) have 2100 such units for 2432
 // resident warps. Units of 16 particles are an eighth of that: 258 us an iteration
-// before and 150 now; 16 swarms of 8192 x 256 298 and 139, 512 uneven swarms, which fill
-// the chip either way, 1077 and 1048. What bounds it at 512 is memory (20 bytes per
+// before and 150 now; 8 uneven swarms 53 and 31, 16 swarms of 8192 x 256 298 and 139, 512 uneven ones, which fill
+// the chip either way, 1077 and 1041. What bounds it at 512 is memory (20 bytes per
 // particle and dimension: 0.82 ms at the copy's rate) with the issue slots half taken.
 // Swarms of fewer than kBatchPanelMinD dimensions have too few panels for the ring's
 // look-ahead and stay there.
@@ -92,14 +92,14 @@ struct PPipe {
     int stage;      // ring stage of the panel being computed
 };
 
-// The first unit of a warp is that of its own number, the others come from the counter:
-// nothing is drawn where every unit has its warp.
+// The first units go out CTA by CTA, so that every SM gets as many, and as long ones; the
+// others come from the counter: nothing is drawn where every unit has its warp.
 __device__ __forceinline__ void next_unit(const BatchDev& b, unsigned* work, PPipe& pp, bool first, int cur,
                                           int lane_id) {
     const uint32_t warps = gridDim.x * (kBlock / 32);
     uint32_t k = b.nunits;
     if (first) {
-        k = blockIdx.x * (kBlock / 32) + (threadIdx.x >> 5);
+        k = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     } else if (b.nunits > warps) {
         if (lane_id == 0) k = warps + atomicAdd(work, 1u);
         k = __shfl_sync(0xFFFFFFFFu, k, 0);
@@ -417,9 +417,9 @@ int batch_panel_grid(unsigned int nunits, int num_sms) {
         cudaGetLastError();
         n = 1;
     }
-    // four warps of eight with work: units that do not fill the chip spread over more SMs
-    const long long useful = ((long long)nunits + 3) / 4;
-    return (int)std::max<long long>(1, std::min<long long>((long long)std::max(n, 1) * num_sms, useful));
+    const long long warps = (long long)num_sms * (kBlock / 32);
+    const long long want = ((long long)nunits + warps - 1) / warps;   // CTAs per SM for a warp per unit
+    return (int)std::min<long long>(num_sms * std::min<long long>(std::max(n, 1), want), nunits);
 }
 
 cudaError_t launch_batch_panel(const BatchDev& b, int grid, cudaStream_t st) {
