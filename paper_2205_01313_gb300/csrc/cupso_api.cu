@@ -626,7 +626,8 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
     s.lock = w32 + 3;
     s.seq = w32 + 4;
     s.work = w32 + 5;
-    s.bar = w32 + 6;
+    s.bar = reinterpret_cast<unsigned long long*>(w32 + 6);
+    s.phase = w32 + 10;
     s.N = N;
     s.D = D;
     s.Np = h->Np;
@@ -1011,7 +1012,7 @@ int cupso_set_option(cupso_handle h, int key, long long value) {
             // with the status, the counters a wait that expired may have left behind
             CUPSO_CUDA(cudaMemsetAsync(h->dev.status, 0, sizeof(unsigned), h->stream), "cudaMemsetAsync");
             CUPSO_CUDA(cudaMemsetAsync(h->dev.ticket, 0, sizeof(unsigned), h->stream), "cudaMemsetAsync");
-            CUPSO_CUDA(cudaMemsetAsync(h->dev.work, 0, 2 * sizeof(unsigned), h->stream), "cudaMemsetAsync");
+            CUPSO_CUDA(cudaMemsetAsync(h->dev.work, 0, 6 * sizeof(unsigned), h->stream), "cudaMemsetAsync");
             return CUPSO_OK;
         case CUPSO_OPT_GRID:
             if (value < 0 || value > (1 << 20)) return fail(CUPSO_ERR_INVALID_ARG, "grid out of range%s");
@@ -1143,7 +1144,7 @@ int cupso_step(cupso_handle h, int iters) {
             const int grid = panel_persist_grid(h, pc);
             while (left > 1) {
                 const int n = std::min(left, P);
-                e = cudaMemsetAsync(h->dev.work, 0, 2 * sizeof(unsigned), h->stream);
+                e = cudaMemsetAsync(h->dev.work, 0, 6 * sizeof(unsigned), h->stream);
                 if (e == cudaSuccess)
                     e = launch_sync_panel(h->dev, h->fid, pc.width, pc.stages, grid, n, h->stall_barrier != 0,
                                           h->stream);

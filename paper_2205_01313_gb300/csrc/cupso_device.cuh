@@ -29,7 +29,9 @@ struct SwarmDev {
     unsigned int* status;       // sticky error bits (kStatus*)
     unsigned long long* aux;    // tree baseline: one key per block of the first kernel
     unsigned int* work;         // pipelined step: next 128-particle unit to hand out
-    unsigned int* bar;          // panel step over several iterations: grid-barrier counter
+    unsigned long long* bar;    // [2], panel step over several iterations, by parity: arrivals in the low
+                                // half, those with a candidate in the high one
+    unsigned int* phase;        // the last of its iterations whose new gbest_pos is out (bar, phase follow work)
     // Lazy pbest (pipelined step): byte i is 1 when particle i improved in the
     // last iteration and its pbest_pos row has not been written yet; its
     // pbest_pos is then its pos. NULL or all-zero means pb is complete.

@@ -67,12 +67,16 @@ struct UnitFeed {
     uint32_t base;
     uint32_t npairs;                // fetches 0 .. npairs - 1 hand out two units
     bool more;                      // there are units after the warps' own
-    __device__ __forceinline__ UnitFeed(uint32_t nunits, uint32_t nwarps)
+    uint32_t drawn;                 // what the counter stood at when the iteration began
+    // The counter runs on from iteration to iteration: in each, the fetches that find units
+    // (npairs and then the single ones) and one of every warp that finds none.
+    __device__ __forceinline__ UnitFeed(uint32_t nunits, uint32_t nwarps, uint32_t it)
         : base(nwarps), npairs(0u), more(nunits > nwarps) {
         if (nunits >= 8u * nwarps) {
             const uint32_t dyn = nunits - nwarps, tail = 2u * nwarps;
             npairs = (dyn - tail) / 2u;
         }
+        drawn = it * (nunits - npairs);   // (nunits - nwarps - npairs) + nwarps
     }
     __device__ __forceinline__ uint32_t next(const SwarmDev& s, int lane_id) {
         if (spare != 0xFFFFFFFFu) {
@@ -82,7 +86,7 @@ struct UnitFeed {
         }
         if (!more) return base;
         uint32_t k = 0;
-        if (lane_id == 0) k = atomicAdd(s.work, 1u);
+        if (lane_id == 0) k = atomicAdd(s.work, 1u) - drawn;
         k = __shfl_sync(0xFFFFFFFFu, k, 0);
         if (k >= npairs) return base + npairs + k;   // single units after the pairs: 2 npairs + (k - npairs)
         spare = base + 2u * k + 1u;
@@ -109,26 +113,44 @@ __device__ __forceinline__ void issue_panel(const SwarmDev& s, float4* my, uint3
     cp_commit();  // an empty group when there is nothing left to copy
 }
 
-// gbest_pos of iteration parity nxt from the winner's pbest_pos, or from pos
-// when its row is still pending -- exactly when the key improved in this
-// iteration (K: the key it started from): the winner then improved its own
-// pbest, and a gbest particle that did not improve has had its row written
-// in this iteration. Run by the last CTA of an iteration.
+// Puts the winner's position of an iteration that improved gbest into gbest_pos of parity
+// nxt and into Gs: its pos, as it improved its pbest in that iteration.
 template <int W>
-__device__ __forceinline__ void gather_gbest_panel(const SwarmDev& s, int nxt, unsigned long long K) {
-    const unsigned long long knew = __ldcg(s.gkey + nxt);
+__device__ __forceinline__ void gather_gbest_panel(const SwarmDev& s, int nxt, unsigned long long knew, float* Gs) {
     const uint32_t g = (uint32_t)(knew & 0xFFFFFFFFull);
-    if (g < (uint32_t)s.N) {
-        const float* src = knew < K ? s.x : s.pb;
-        for (int d = threadIdx.x; d < s.D; d += blockDim.x)
-            s.G[(size_t)nxt * s.D + d] = __ldcg(src + panel_off<W>(s, d / W, g) + (d % W));
+    for (int d = threadIdx.x; d < s.D; d += blockDim.x) {
+        const float x = __ldcg(s.x + panel_off<W>(s, d / W, g) + d % W);
+        s.G[(size_t)nxt * s.D + d] = x;
+        Gs[d] = x;
     }
 }
 
-__device__ __forceinline__ unsigned int ld_acquire_gpu_u32(const unsigned int* p) {
+__device__ __forceinline__ unsigned int ld_acquire(const unsigned int* p) {
     unsigned int v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
+}
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Polls *p until reached(value), at most s.wait_limit_ns (then the timeout status is set
+// and the result is false).
+template <typename T, typename Reached>
+__device__ __forceinline__ bool wait_for(const SwarmDev& s, const T* p, T& v, Reached reached) {
+    v = ld_acquire(p);
+    if (reached(v)) return true;
+    const long long deadline = global_ns() + s.wait_limit_ns;
+    while (!reached(v = ld_acquire(p))) {
+        if (global_ns() > deadline) {
+            atomicOr(s.status, kStatusTimeout);
+            return false;
+        }
+        __nanosleep(32);
+    }
+    return true;
 }
 
 // One iteration of a warp's units: first u_cur, whose first STAGES - 1 panels
@@ -198,17 +220,15 @@ __device__ __forceinline__ unsigned long long panel_units(const SwarmDev& s, flo
                     set_lane(X, k + 1, x1);
                     set_lane(V, k, v0);
                     set_lane(V, k + 1, v1);
-                    continue;
-                }
+                } else {
 #pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                    const int k = 2 * g + hh;
-                    float xj = lane(X, k), vj = lane(V, k);
-                    if constexpr (!FAST)
-                        move_one(xj, vj, lane(Pb, k), Gs[d0 + k], u01(word(r, 2 * hh)), u01(word(r, 2 * hh + 1)),
-                                 s);
-                    set_lane(X, k, xj);
-                    set_lane(V, k, vj);
+                    for (int hh = 0; hh < 2; ++hh) {
+                        const int k = 2 * g + hh;
+                        float xj = lane(X, k), vj = lane(V, k);
+                        move_one(xj, vj, lane(Pb, k), Gs[d0 + k], u01(word(r, 2 * hh)), u01(word(r, 2 * hh + 1)), s);
+                        set_lane(X, k, xj);
+                        set_lane(V, k, vj);
+                    }
                 }
             }
             st4(s.x + off, X);
@@ -252,14 +272,20 @@ __device__ __forceinline__ unsigned long long panel_units(const SwarmDev& s, flo
 //
 // Each warp takes unit (its warp in the CTA) x gridDim.x + blockIdx.x first in every iteration, then units
 // from the counter. With more than one iteration, every CTA must be resident
-// (a cooperative launch): an iteration ends in a grid barrier on s.bar -- each
-// CTA arrives once; the last to arrive gathers gbest_pos and releases the
-// others -- and while a CTA waits, its warps already load the first panels of
-// their own unit for the next iteration (rows they wrote themselves, so they
-// need nothing from the barrier). The wait is bounded by s.wait_limit_ns: on
-// expiry the timeout status is set and the CTA stops. `expect` is the number
-// of arrivals that completes a barrier: gridDim.x (one more only to test that
-// bound).
+// (a cooperative launch): an iteration ends in a grid barrier on s.bar[its parity] --
+// each CTA arrives once, and while it waits, its warps already load the first panels of
+// their own unit for the next iteration (rows they wrote themselves, so they need
+// nothing from the barrier). Without a candidate among the arrivals gbest stands and the
+// next iteration begins at once; with one, the CTA that arrived last gathers the new
+// gbest_pos and releases the others a second time, by s.phase. (With the last CTA
+// gathering in every iteration and the others reading it back, Rastrigin 40000 x 32 took
+// 9.0 us an iteration and 65536 x 128 31.9, now 6.9 and 29.9. The pause between looks
+// matters: without it 456 CTAs held up the line that the gathering CTA reads, 7.0 and
+// 31.1.) Every wait is bounded by s.wait_limit_ns: on expiry the timeout status is set and
+// the CTA stops. `expect` is the number of arrivals that completes a barrier: gridDim.x
+// (one more only to test that bound). During the launch the keys of the two parities
+// may be behind gbest's, which every CTA holds in K; they only ever take candidates
+// below it.
 template <int FIT, int W, int STAGES, bool FAST>
 __global__ void __launch_bounds__(kBlock, 3) sync_panel_kernel(const __grid_constant__ SwarmDev s, int iters,
                                                                unsigned int expect) {
@@ -267,7 +293,7 @@ __global__ void __launch_bounds__(kBlock, 3) sync_panel_kernel(const __grid_cons
     constexpr uint32_t PU = 32 / L;
     extern __shared__ float4 ring[];      // [STAGES][3][kBlock], then gbest_pos [D]
     float* Gs = reinterpret_cast<float*>(ring + STAGES * 3 * kBlock);
-    __shared__ int s_last, s_ok;
+    __shared__ int s_step;   // 0: on to the next iteration, 1: when gbest_pos is out, 2: gather it, -1: timeout
     const int lane_id = threadIdx.x & 31;
     const uint32_t pl = (uint32_t)(lane_id / L);
     const uint32_t nunits = (uint32_t)s.Np / PU;
@@ -281,58 +307,86 @@ __global__ void __launch_bounds__(kBlock, 3) sync_panel_kernel(const __grid_cons
 #pragma unroll
     for (int k = 0; k < STAGES - 1; ++k) issue_panel<W>(s, my, u0, k, k, nunits, lane_id, fl0);
     bool nan = false;
+    unsigned long long K = __ldcg(s.gkey + (t_prev & 1u));   // gbest's key, the same in every thread
+    for (int d = threadIdx.x; d < s.D; d += blockDim.x) Gs[d] = __ldcg(s.G + (size_t)(t_prev & 1u) * s.D + d);
+    __syncthreads();
+    uint32_t seen[2] = {0u, 0u};           // thread 0: the candidates' arrivals by parity so far
     for (int it = 0; it < iters; ++it) {
         const uint32_t t = t_prev + 1u + (uint32_t)it;
-        const int cur = (int)((t - 1u) & 1u), nxt = cur ^ 1;
-        const unsigned long long K = __ldcg(s.gkey + cur);  // gbest at the end of t-1
-        for (int d = threadIdx.x; d < s.D; d += blockDim.x) Gs[d] = __ldcg(s.G + (size_t)cur * s.D + d);
-        __syncthreads();
-        UnitFeed feed(nunits, nwarps);
+        const int cur = (int)((t - 1u) & 1u), nxt = cur ^ 1, par = it & 1;
+        UnitFeed feed(nunits, nwarps, (uint32_t)it);
         unsigned long long best = panel_units<FIT, W, STAGES, FAST>(s, my, Gs, feed, u0, fl0, nunits, t, K, nan);
         best = warp_min_u64(best);
         if (lane_id == 0 && best < K) atomicMin(s.gkey + nxt, best);
 
-        // arrival; the last CTA completes Step 5 and releases the barrier
+        // arrival: releases this CTA's rows, flags and candidates
         __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) s_last = atomicAdd(s.bar, 1u) == (uint32_t)(it + 1) * (expect + 1u) - 2u;
-        __syncthreads();
-        const bool final_it = it + 1 == iters;
-        if (s_last) {
-            __threadfence();
-            gather_gbest_panel<W>(s, nxt, K);
-            __syncthreads();
+        const bool cand = __syncthreads_or(best < K);
+        const uint32_t target = (uint32_t)(it / 2 + 1) * expect;
+        unsigned long long arrived = 0ull;
+        if (threadIdx.x == 0) arrived = atomicAdd(s.bar + par, 1ull + (cand ? 1ull << 32 : 0ull));
+        if (it + 1 == iters) {
+            // the last CTA leaves the state of iteration t: gbest_pos, the key in both parities
             if (threadIdx.x == 0) {
-                s.gkey[cur] = __ldcg(s.gkey + nxt);
-                *s.t_dev = t;
-                *s.work = 0u;
-                if (final_it) *s.bar = 0u;
-                __threadfence();
-                if (!final_it) atomicAdd(s.bar, 1u);
+                const bool improved = (uint32_t)(arrived >> 32) + (cand ? 1u : 0u) != seen[par];
+                s_step = (uint32_t)arrived != target - 1u ? 0 : improved ? 2 : 1;
             }
+            __syncthreads();
+            if (s_step) {
+                __threadfence();
+                const unsigned long long knew = s_step == 2 ? __ldcg(s.gkey + nxt) : K;
+                if (s_step == 2) {
+                    gather_gbest_panel<W>(s, nxt, knew, Gs);
+                } else {
+                    for (int d = threadIdx.x; d < s.D; d += blockDim.x) s.G[(size_t)nxt * s.D + d] = Gs[d];
+                }
+                __syncthreads();   // every thread has read the key
+                if (threadIdx.x == 0) {
+                    s.gkey[0] = knew;
+                    s.gkey[1] = knew;
+                    *s.t_dev = t;
+                    *s.work = 0u;
+                    s.bar[0] = 0ull;
+                    s.bar[1] = 0ull;
+                    *s.phase = 0u;
+                }
+            }
+            break;
         }
-        if (final_it) break;
 
         // the first panels of this warp's own unit for the next iteration
         fl0 = u0 < nunits ? (uint32_t)__ldcg(s.pflag + u0 * PU + pl) : 0u;
 #pragma unroll
         for (int k = 0; k < STAGES - 1; ++k) issue_panel<W>(s, my, u0, k, k, nunits, lane_id, fl0);
         if (threadIdx.x == 0) {
-            const uint32_t target = (uint32_t)(it + 1) * (expect + 1u);
-            const long long deadline = global_ns() + s.wait_limit_ns;
-            int ok = 1;
-            while (ld_acquire_gpu_u32(s.bar) < target) {
-                if (global_ns() > deadline) {
-                    ok = 0;
-                    atomicOr(s.status, kStatusTimeout);
-                    break;
-                }
-                __nanosleep(32);
+            unsigned long long w = arrived + (cand ? 1ull << 32 : 0ull) + 1ull;
+            const bool last = (uint32_t)w == target;   // it need not look again
+            const bool ok = last || wait_for(s, s.bar + par, w, [&](unsigned long long v) { return (uint32_t)v >= target; });
+            const uint32_t now = (uint32_t)(w >> 32);   // final: nobody is two iterations ahead
+            s_step = !ok ? -1 : now == seen[par] ? 0 : last ? 2 : 1;
+            seen[par] = now;
+            if (s_step == 1) {
+                // the gathering CTA needs two round trips to memory and a fence; looking before
+                // then only takes its line's time
+                __nanosleep(500);
+                uint32_t v;
+                if (!wait_for(s, s.phase, v, [&](uint32_t p) { return p >= (uint32_t)(it + 1); })) s_step = -1;
             }
-            s_ok = ok;
         }
         __syncthreads();
-        if (!s_ok) {
+        if (s_step == 2) {
+            __threadfence();
+            K = __ldcg(s.gkey + nxt);
+            gather_gbest_panel<W>(s, nxt, K, Gs);
+            __threadfence();
+            __syncthreads();
+            if (threadIdx.x == 0) atomicExch(s.phase, (uint32_t)(it + 1));
+        } else if (s_step == 1) {
+            K = __ldcg(s.gkey + nxt);
+            for (int d = threadIdx.x; d < s.D; d += blockDim.x) Gs[d] = __ldcg(s.G + (size_t)nxt * s.D + d);
+            __syncthreads();
+        }
+        if (s_step < 0) {
             cp_wait<0>();
             break;
         }
