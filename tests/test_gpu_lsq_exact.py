@@ -19,7 +19,8 @@ def P():
 # M, D, N, floats by which A is shifted off its allocation
 @pytest.mark.parametrize("M,D,N,shift", [
     (1, 1, 1, 0), (520, 36, 1300, 0), (520, 36, 1300, 1), (521, 33, 1281, 0), (129, 16, 5000, 0), (127, 17, 63, 0),
-    (4000, 4, 4500, 0), (3, 2, 140000, 0), (66, 2, 140000, 0), (64, 17, 257, 0), (65, 17, 257, 0),
+    (4000, 4, 4500, 0), (3, 2, 140000, 0), (66, 2, 140000, 0), (64, 17, 257, 0), (65, 17, 257, 0), (128, 128, 300, 0), (128, 129, 300, 0),
+    (101, 33, 40, 1),
     (2501, 21, 2490, 0),   # 128 x 128 tiles, ragged on every side
 ])
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
