@@ -542,7 +542,7 @@ def batch_report(P, a, stream, plain_every=1):
                          % max(1, plain_every)},
         "batched_over_plain": plain_s / batched_s,
         "alone_vs_batched_mismatches": mism,
-        "roofline": {"bound": "hbm", "kernel": "batch_step_kernel", "achieved": achieved, "peak": peak,
+        "roofline": {"bound": "hbm", "kernel": "batch_panel_kernel", "achieved": achieved, "peak": peak,
                      "unit": "GB/s", "frac": achieved / peak, "traffic": None,
                      "algorithmic_bytes_per_iteration": alg, "peak_source": src},
         "clocks": clk,
