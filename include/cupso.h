@@ -155,16 +155,17 @@ typedef enum {
 
 /* The implementations of the SYNC step; all compute the same bits. */
 typedef enum {
-    CUPSO_SYNC_KERNEL_AUTO = 0,       /* tiled for small swarms, else the panel kernel where D
-                                         allows, else the deepest pipelined ring supported, else
-                                         register                                           */
+    CUPSO_SYNC_KERNEL_AUTO = 0,       /* for several iterations per call, a swarm that registers hold
+                                         stays there; else tiled for small swarms, else the panel
+                                         kernel where D allows, else the deepest pipelined ring
+                                         supported, else register                           */
     CUPSO_SYNC_KERNEL_REGISTER = 1,   /* loads straight into registers, 1024-particle tiles */
     CUPSO_SYNC_KERNEL_PIPELINED3 = 2, /* rows staged through shared memory, 2 pairs ahead   */
     CUPSO_SYNC_KERNEL_PIPELINED4 = 3, /* the same, 3 pairs ahead                            */
     CUPSO_SYNC_KERNEL_TILED = 4,      /* a tile of particles with all their dimensions per block,
                                          the (dimension pair, particle) items spread over threads;
-                                         AUTO uses it for D >= 8 up to about 896 particles per SM
-                                         (224 for D > 64 without cos(2 pi x) in the fitness)     */
+                                         AUTO uses it for D >= 8, D % 8 != 0 up to 400 particles per SM
+                                         (330 for D > 128; Rosenbrock 330, and 224 for D > 64)   */
     CUPSO_SYNC_KERNEL_PANEL8 = 5,     /* the state in panels of 8 dimensions (each particle's 8 values
                                          of a panel contiguous), two threads per particle, rows staged
                                          through shared memory; D % 8 == 0, D >= 16. A particle whose
