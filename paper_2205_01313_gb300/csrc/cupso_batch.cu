@@ -43,7 +43,7 @@ size_t up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct Shape {
     int stages;          // ring depth of the streaming kernel; 0: the tiled kernel; -1: the panels'
-    int minb;            // register budget: CTAs per SM
+    int minb;            // register budget: CTAs per SM (the panels' kernel: its deep ring)
     int blocks_per_sm;   // CTAs per SM launched (the panels' kernel: CTAs in all)
 };
 
@@ -81,7 +81,7 @@ struct BatchRun {
     cudaError_t launch(const Shape& sh) { return launch_on(sh, st); }
 
     cudaError_t launch_on(const Shape& sh, cudaStream_t s) {
-        if (sh.stages < 0) return launch_batch_panel(dev, sh.blocks_per_sm, s);
+        if (sh.stages < 0) return launch_batch_panel(dev, sh.minb != 0, sh.blocks_per_sm, s);
         if (sh.stages == 0) return launch_batch_tiled(dev, tiles, num_sms * sh.blocks_per_sm, s);
         return launch_batch_step(dev, sh.stages, sh.minb, num_sms * sh.blocks_per_sm, s);
     }
@@ -215,7 +215,7 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
         // kernel spreads them over a CTA -- 256 dimensions, 4,000 particles in all: 26.5 us
         // and 20.9; 8,000: 28.3 and 34.4; 64 dimensions: 11.4 and 17.7.
         std::vector<char> panel(nb);
-        long long panel_pd = 0;
+        long long panel_pd = 0, shallow_pd = 0;
         int panel_maxD = 0;
         for (int j = 0; j < nb; ++j) {
             const cupso_problem& p = problems[batched[j]];
@@ -223,8 +223,14 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
                        p.N <= 65536;
             if (!panel[j]) continue;
             panel_pd += (long long)p.N * p.D;
+            if (p.D < kBatchPanelDeepD) shallow_pd += (long long)p.N * p.D;
             panel_maxD = std::max(panel_maxD, p.D);
         }
+        // the deep ring from about 300 swarms of 4000 x 130 on, where few are too narrow for it
+        const bool deep = panel_pd >= (160ll << 20) && shallow_pd * 16 <= panel_pd;
+        if (deep)
+            for (int j = 0; j < nb; ++j)
+                if (problems[batched[j]].D < kBatchPanelDeepD) panel[j] = 0;
         if (panel_maxD > 64 && panel_pd < 6144ll * panel_maxD) panel.assign(nb, 0);
         std::vector<int> rows(nb);   // dimensions the state has room for
         size_t panel_units = 0;
@@ -381,7 +387,8 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
         prun.dev.work = ctr + 16;
         prun.dev.ticket = ctr + 18;
         prun.dev.t_dev = ctr + 19;
-        const Shape pshape{-1, 0, prun.dev.nunits ? batch_panel_grid(prun.dev.nunits, run.num_sms) : 0};
+        const Shape pshape{-1, deep ? 1 : 0,
+                           prun.dev.nunits ? batch_panel_grid(prun.dev.nunits, deep, run.num_sms) : 0};
 
         // Step 1 of every swarm, one launch for each kind.
         e = cudaSuccess;

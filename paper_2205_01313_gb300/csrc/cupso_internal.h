@@ -62,10 +62,11 @@ cudaError_t launch_batch_init(const BatchDev& b, int grid, cudaStream_t st);
 // particles, swarms of at least kBatchPanelMinD dimensions (any number of them: the
 // last panel may be partly used). Panel (d / 8), particle i: 8 floats at
 // (d / 8 * Np + i) * 8; gbest_pos rows 16-byte aligned, zero past D.
-constexpr int kBatchPanelMinD = 25;
+constexpr int kBatchPanelMinD = 25;    // with the ring of 5 stages
+constexpr int kBatchPanelDeepD = 33;   // with the ring of 6 (deep)
 cudaError_t prepare_batch_panel();
-int batch_panel_grid(unsigned int nunits, int num_sms);
-cudaError_t launch_batch_panel(const BatchDev& b, int grid, cudaStream_t st);
+int batch_panel_grid(unsigned int nunits, bool deep, int num_sms);
+cudaError_t launch_batch_panel(const BatchDev& b, bool deep, int grid, cudaStream_t st);
 cudaError_t launch_batch_panel_init(const BatchDev& b, int num_sms, cudaStream_t st);
 
 // Fused SYNC step on the panel layout (kernels_panel.cu): element (d, i) of

@@ -13,11 +13,14 @@
 // dimensions, and a batch of a few dozen swarms is over when its last 256-dimensional
 // unit is -- 64 uneven swarms (N 64 .. 8192, D 8 .. 256) have 2100 such units for 2432
 // resident warps. Units of 16 particles are an eighth of that: 258 us an iteration
-// before and 150 now; 8 uneven swarms 53 and 31, 16 swarms of 8192 x 256 298 and 139, 512 uneven ones, which fill
-// the chip either way, 1077 and 1041. What bounds it at 512 is memory (20 bytes per
-// particle and dimension: 0.82 ms at the copy's rate) with the issue slots half taken.
+// before and 150 now; 8 uneven swarms 53 and 31, 16 swarms of 8192 x 256 298 and 139, 512
+// uneven ones, which fill the chip either way, 1077 and 1009. What bounds it at 512 is
+// memory (20 bytes per particle and dimension: 0.82 ms at the copy's rate) with the issue
+// slots half taken.
 // Swarms of fewer than kBatchPanelMinD dimensions have too few panels for the ring's
-// look-ahead and stay there.
+// look-ahead and stay there. In batches of hundreds of swarms a ring of 6 stages (`deep`) is
+// the faster one, 1046 and 1009 us at 512, and those of fewer than kBatchPanelDeepD dimensions
+// stay there too; with 128 it is 276 and 282.
 //
 // Three CTAs of 256 threads an SM leave 80 registers a thread, and two of 128 were
 // slower where the chip is full (1.29 against 1.13 ms). What a swarm's move needs
@@ -39,7 +42,6 @@ namespace {
 
 constexpr int kW = 8, kL = kW / 4;          // panel width, lanes per particle
 constexpr uint32_t kPU = 32 / kL;           // particles per unit
-constexpr int kStages = 5;
 
 struct PUnit {
     uint32_t sw, u;                         // swarm (0xFFFFFFFF: none), unit within it
@@ -83,7 +85,7 @@ __device__ __forceinline__ void issue_panel(const BatchDev& b, const Feed& f, fl
     if (lane_id < kL) cp16(gring + stage * kL + lane_id, b.G + 4ull * (f.g + (uint32_t)(kL * q + lane_id)));
 }
 
-// The copies run kStages - 1 panels ahead of the arithmetic, into the next unit.
+// The copies run STAGES - 1 panels ahead of the arithmetic, into the next unit.
 struct PPipe {
     PUnit nxt;      // the unit that is being copied
     Feed feed;
@@ -196,9 +198,9 @@ __device__ __forceinline__ void close_unit(const BatchSwarm& w, unsigned long lo
     }
 }
 
-// One unit at iteration t: its first kStages - 1 panels are in the ring (feed: its
+// One unit at iteration t: its first STAGES - 1 panels are in the ring (feed: its
 // flags); keeps that many in flight, of the next unit once its own are issued.
-template <int FIT, bool FAST>
+template <int FIT, bool FAST, int STAGES>
 __device__ __forceinline__ void run_unit(const BatchDev& b, unsigned* work, float4* my, float4* gring, uint32_t cst, PUnit cu,
                                          const Feed me, PPipe& pp, uint32_t t, int lane_id) {
     const BatchSwarm& w = b.swarms[cu.sw];
@@ -218,14 +220,14 @@ __device__ __forceinline__ void run_unit(const BatchDev& b, unsigned* work, floa
     for (int q = 0; q < Dq; ++q) {
         {
             __syncwarp();   // every lane has read the stage that is copied into
-            int ws = pp.stage + kStages - 1;
-            if (ws >= kStages) ws -= kStages;
-            // every unit has at least kStages - 1 panels, so the look-ahead ends within the next one
+            int ws = pp.stage + STAGES - 1;
+            if (ws >= STAGES) ws -= STAGES;
+            // every unit has at least STAGES - 1 panels, so the look-ahead ends within the next one
             if (pp.left == 0) next_unit(b, work, pp, false, cur, lane_id);
             issue_next(b, pp, my, gring, ws, lane_id);
         }
         const int d0 = kW * q + 4 * j;
-        cp_wait<kStages - 1>();
+        cp_wait<STAGES - 1>();
         __syncwarp();   // lanes 0 and 1 copied gbest_pos
         const float4 g4 = gring[pp.stage * kL + j];
         const float4* slot = my + (size_t)pp.stage * 3 * kBlock;
@@ -266,7 +268,7 @@ __device__ __forceinline__ void run_unit(const BatchDev& b, unsigned* work, floa
         st4(reinterpret_cast<float*>(to + plane), V);
         if (q + 1 < Dq) panel_sum<FIT, kL, false, FAST>(acc, X, d0, D, j, lane_id, carry);
         else panel_sum<FIT, kL, true, FAST>(acc, X, d0, D, j, lane_id, carry);
-        if (++pp.stage == kStages) pp.stage = 0;
+        if (++pp.stage == STAGES) pp.stage = 0;
     }
     // Steps 4-5 in the particle's last lane, which holds the whole sum
     unsigned long long best = kKeyNone;
@@ -335,7 +337,8 @@ __device__ __forceinline__ void init_unit(const BatchSwarm& wg, uint32_t u, int 
 
 }  // namespace
 
-// Requires D >= kBatchPanelMinD for every swarm of the batch and states of whole panels.
+// Requires at least STAGES - 1 panels of every swarm of the batch and states of whole panels.
+template <int STAGES>
 __global__ void __launch_bounds__(kBlock, 3) batch_panel_kernel(const __grid_constant__ BatchDev b) {
     extern __shared__ float4 ring_p[];
     const uint32_t t = __ldcg(b.t_dev) + 1u;
@@ -343,7 +346,7 @@ __global__ void __launch_bounds__(kBlock, 3) batch_panel_kernel(const __grid_con
     const int lane_id = threadIdx.x & 31;
     float4* my = ring_p + threadIdx.x;
     __shared__ uint4 s_cst[kBlock / 32][8];
-    __shared__ float4 s_g[kBlock / 32][kStages * kL];
+    __shared__ float4 s_g[kBlock / 32][STAGES * kL];
     float4* gring = s_g[threadIdx.x >> 5];
     const uint32_t cst = (uint32_t)__cvta_generic_to_shared(s_cst[threadIdx.x >> 5]);
 
@@ -352,22 +355,22 @@ __global__ void __launch_bounds__(kBlock, 3) batch_panel_kernel(const __grid_con
     pp.feed = Feed{};
     next_unit(b, work, pp, true, (int)((t - 1u) & 1u), lane_id);
 #pragma unroll
-    for (int k = 0; k < kStages - 1; ++k) issue_next(b, pp, my, gring, k, lane_id);
+    for (int k = 0; k < STAGES - 1; ++k) issue_next(b, pp, my, gring, k, lane_id);
     PUnit cu = pp.nxt;
     Feed me = pp.feed;
     while (cu.sw != 0xFFFFFFFFu) {
         const bool fast = b.swarms[cu.sw].fast != 0;
         switch (b.swarms[cu.sw].fid * 2 + (fast ? 1 : 0)) {
-            case kSphere * 2 + 1: run_unit<kSphere, true>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
-            case kSphere * 2: run_unit<kSphere, false>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
-            case kRastrigin * 2 + 1: run_unit<kRastrigin, true>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
-            case kRastrigin * 2: run_unit<kRastrigin, false>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
-            case kAckley * 2 + 1: run_unit<kAckley, true>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
-            case kAckley * 2: run_unit<kAckley, false>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
-            case kRosenbrock * 2 + 1: run_unit<kRosenbrock, true>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
-            case kRosenbrock * 2: run_unit<kRosenbrock, false>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
-            case kCubicMax * 2 + 1: run_unit<kCubicMax, true>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
-            default: run_unit<kCubicMax, false>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;   // nothing else is admitted
+            case kSphere * 2 + 1: run_unit<kSphere, true, STAGES>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
+            case kSphere * 2: run_unit<kSphere, false, STAGES>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
+            case kRastrigin * 2 + 1: run_unit<kRastrigin, true, STAGES>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
+            case kRastrigin * 2: run_unit<kRastrigin, false, STAGES>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
+            case kAckley * 2 + 1: run_unit<kAckley, true, STAGES>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
+            case kAckley * 2: run_unit<kAckley, false, STAGES>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
+            case kRosenbrock * 2 + 1: run_unit<kRosenbrock, true, STAGES>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
+            case kRosenbrock * 2: run_unit<kRosenbrock, false, STAGES>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
+            case kCubicMax * 2 + 1: run_unit<kCubicMax, true, STAGES>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;
+            default: run_unit<kCubicMax, false, STAGES>(b, work, my, gring, cst, cu, me, pp, t, lane_id); break;   // nothing else is admitted
         }
         cu = pp.nxt;        // every unit ends with the next one fetched
         me = pp.feed;
@@ -403,17 +406,22 @@ __global__ void __launch_bounds__(kBlock) batch_panel_init_kernel(const __grid_c
 }
 
 namespace {
-constexpr size_t kPanelRing = sizeof(float4) * (size_t)kStages * 3 * kBlock;
-static_assert(kBatchPanelMinD > kW * (kStages - 2), "the ring's look-ahead spans at most two units");
+static_assert(kBatchPanelMinD > kW * 3 && kBatchPanelDeepD > kW * 4, "rings of 5 and 6 stages: 4 and 5 panels");
+constexpr size_t ring_bytes(int stages) { return sizeof(float4) * (size_t)stages * 3 * kBlock; }
 }  // namespace
 
 cudaError_t prepare_batch_panel() {
-    return cudaFuncSetAttribute(batch_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPanelRing);
+    cudaError_t e = cudaFuncSetAttribute(batch_panel_kernel<5>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)ring_bytes(5));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(batch_panel_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_bytes(6));
+    return e;
 }
 
-int batch_panel_grid(unsigned int nunits, int num_sms) {
+int batch_panel_grid(unsigned int nunits, bool deep, int num_sms) {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_panel_kernel, kBlock, kPanelRing) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, deep ? batch_panel_kernel<6> : batch_panel_kernel<5>, kBlock,
+                                                      ring_bytes(deep ? 6 : 5)) != cudaSuccess) {
         cudaGetLastError();
         n = 1;
     }
@@ -422,8 +430,9 @@ int batch_panel_grid(unsigned int nunits, int num_sms) {
     return (int)std::min<long long>(num_sms * std::min<long long>(std::max(n, 1), want), nunits);
 }
 
-cudaError_t launch_batch_panel(const BatchDev& b, int grid, cudaStream_t st) {
-    batch_panel_kernel<<<grid, kBlock, kPanelRing, st>>>(b);
+cudaError_t launch_batch_panel(const BatchDev& b, bool deep, int grid, cudaStream_t st) {
+    if (deep) batch_panel_kernel<6><<<grid, kBlock, ring_bytes(6), st>>>(b);
+    else batch_panel_kernel<5><<<grid, kBlock, ring_bytes(5), st>>>(b);
     return cudaGetLastError();
 }
 

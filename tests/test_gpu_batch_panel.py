@@ -67,3 +67,19 @@ def test_iteration_counts_match_oracle(P, iters, monkeypatch):
     probs = [problem(k % 5, 3000 if k == 3 else 100 + 50 * k, 25 + 9 * k, k) for k in range(8)]
     probs.append(problem(0, 6500, 88, 60))
     assert check(P, probs, iters) == P.CUPSO_OK
+
+
+def test_large_batch_edges_match_oracle(P, monkeypatch):
+    """A batch large enough for the deeper ring: the smallest widths it takes, edges of the
+    panels and units, and narrower swarms, which then run outside the panels; the three
+    that make it large are not compared."""
+    monkeypatch.delenv("CUPSO_BATCH_KERNEL", raising=False)
+    probs = [problem(k % 5, SIZES[(3 * k) % len(SIZES)], D, k)
+             for k, D in enumerate((33, 34, 39, 40, 41, 48, 255, 256, 25, 32, 24, 8, 33, 40, 41))]
+    large = [problem(k, 65536, 900, 70 + k) for k in (0, 1, 3)]
+    rc, res = P.cupso_solve_batch(probs + large, 7)
+    assert rc == P.CUPSO_OK
+    for k, p in enumerate(probs):
+        ref = oracle_swarm(p["fitness_id"], p["N"], p["D"], p["seed"], swarm=p["swarm_id"]).init().step_sync(7)
+        assert res[k]["idx"] == ref.gbest_idx, (k, p)
+        assert same_bits(res[k]["fit"], ref.gbest_fit) and same_bits(res[k]["pos"], ref.gbest_pos), (k, p)
