@@ -644,7 +644,8 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
     s.wait_limit_ns = 2000000000ll;
     h->pbufs = paper_bufs_at(base + o_paper, h->Np, list_cap);
     set_fast_paths(&s);
-    if (res_bytes && resident_fits(s, fid, h->num_sms)) h->rbufs = resident_bufs_at(base + o_res);
+    if (res_bytes && resident_fits(s, fid, h->num_sms) && prepare_resident(s, fid, h->num_sms) == cudaSuccess)
+        h->rbufs = resident_bufs_at(base + o_res);
 
     int cl = 0, per = 0;
     h->onchip_cluster = (fid != CUPSO_LSQ && onchip_fits(N, D, &cl, &per)) ? cl : 0;
@@ -739,7 +740,6 @@ int create_swarm64(int D, int N, const cupso_bounds_f64* b, double w, double c1,
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
     char* base = static_cast<char*>(h->arena);
     h->rec_now = base + o_rec;
-    if (s64_bytes) h->s64bufs = sync64_bufs_at(base + o_s64);
     SwarmDev64& s = h->dev64;
     s.x = reinterpret_cast<double*>(base + o_x);
     s.v = reinterpret_cast<double*>(base + o_v);
@@ -775,6 +775,7 @@ int create_swarm64(int D, int N, const cupso_bounds_f64* b, double w, double c1,
     h->dev.wait_limit_ns = s.wait_limit_ns;
     h->dev.status = s.status;
     h->pbufs = paper_bufs_at(base + o_paper, h->Np, list_cap);
+    if (s64_bytes && prepare_sync64(s, fid, h->num_sms) == cudaSuccess) h->s64bufs = sync64_bufs_at(base + o_s64);
     h->onchip_cluster = onchip64_cluster(N, D);
     h->onchip64 = h->onchip_cluster > 0;
     cudaGetLastError();

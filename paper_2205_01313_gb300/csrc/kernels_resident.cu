@@ -62,6 +62,7 @@ constexpr int max_threads(int items) {
     return items <= 1 ? 1024 : (items <= 3 ? 768 : (items <= 4 ? 640 : (items <= 8 ? 512 : (items <= 12 ? 384 : 256))));
 }
 constexpr int kResItems[] = {1, 2, 3, 4, 5, 6, 8, 12, 16};   // instantiated
+constexpr size_t kResSmem = 200u * 1024u;   // dynamic shared memory of a CTA at most
 
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
     unsigned long long v;
@@ -376,7 +377,7 @@ bool res_plan(int N, int D, int num_sms, ResPlan* r) {
         const int q = (2 * items * rows + 3) / 4;   // quarter of the row stride, made odd
         r->S = 4 * (q | 1);
         r->smem = sizeof(float) * (2 * (size_t)P * r->S + 2 * (size_t)items * rows) + (size_t)P;
-        return r->smem <= 200u * 1024u;
+        return r->smem <= kResSmem;
     }
     return false;
 }
@@ -429,6 +430,17 @@ ResidentBufs resident_bufs_at(void* base) {
                         reinterpret_cast<float*>(p + 64)};
 }
 
+// Raises the shared-memory limit of this swarm's kernel. The limit belongs to the kernel,
+// which other swarms run too, from other host threads as well: every swarm sets the same one,
+// when it is created. (With each swarm's own before each of its launches, two threads with 77824 x 16
+// and 20000 x 48 took it from one another and the larger one's launch was refused.)
+cudaError_t prepare_resident(const SwarmDev& s, int fid, int num_sms) {
+    ResPlan r;
+    const void* k = res_plan(s.N, s.D, num_sms, &r) ? res_kernel(r.items, fid) : nullptr;
+    if (!k) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem);
+}
+
 cudaError_t launch_resident(const SwarmDev& s, const ResidentBufs& rb, int fid, int panel, int iters, bool stall_barrier,
                             int num_sms, cudaStream_t st) {
     ResPlan r;
@@ -437,8 +449,7 @@ cudaError_t launch_resident(const SwarmDev& s, const ResidentBufs& rb, int fid, 
         return cudaErrorInvalidValue;
     const void* k = res_kernel(r.items, fid);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)r.smem);
-    if (e == cudaSuccess) e = cudaMemsetAsync(rb.key, 0xFF, 2 * sizeof(unsigned long long), st);
+    cudaError_t e = cudaMemsetAsync(rb.key, 0xFF, 2 * sizeof(unsigned long long), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(rb.bar, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     unsigned int expect = (unsigned int)r.grid + (stall_barrier ? 1u : 0u);

@@ -44,7 +44,7 @@ namespace cupso {
 
 namespace {
 
-constexpr size_t kSync64Smem = 200u * 1024u;
+constexpr size_t kSync64Smem = 200u * 1024u;   // dynamic shared memory of a CTA at most
 constexpr int kMemThreads = 512;
 constexpr int kMemChunk = 4;   // items whose loads a thread issues together
 
@@ -515,12 +515,21 @@ Sync64Bufs sync64_bufs_at(void* base) {
     return Sync64Bufs{static_cast<unsigned long long*>(base), static_cast<unsigned char*>(base) + 64};
 }
 
+// Raises the shared-memory limit of this swarm's kernel, to the same value for every swarm (it
+// belongs to the kernel, which swarms of other sizes run from other host threads).
+cudaError_t prepare_sync64(const SwarmDev64& s, int fid, int num_sms) {
+    Plan64 r;
+    const void* k = plan64(fid, s.N, s.D, num_sms, &r) ? kernel64(fid, s.w_one != 0, r.items) : nullptr;
+    if (!k) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSync64Smem);
+}
+
 cudaError_t launch_sync64(const SwarmDev64& s, const Sync64Bufs& rb, int fid, int iters, int num_sms, cudaStream_t st) {
     Plan64 r;
     if (!rb.slots || iters < 1 || !plan64(fid, s.N, s.D, num_sms, &r)) return cudaErrorInvalidValue;
     const void* k = kernel64(fid, s.w_one != 0, r.items);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)r.smem);
+    cudaError_t e = cudaSuccess;
     for (int left = iters; e == cudaSuccess && left > 0;) {
         int n = std::min(left, 1 << 22);   // n x SMs arrivals stay below 2^32
         left -= n;

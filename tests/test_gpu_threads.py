@@ -1,0 +1,55 @@
+"""Handles of different host threads: two swarms that run the same kernel at different sizes, each
+stepped by a thread of its own, take no launch limit from one another and get the bits that
+they get alone."""
+import threading
+
+import numpy as np
+import pytest
+
+from tests.gpu_common import BOUNDS, C12, W, load_cupso
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    return load_cupso()
+
+
+def _run(P, fid, N, D, mode, dtype, rounds, iters, start=None):
+    with P.Swarm(D, N, BOUNDS[fid], W, C12, C12, fid, N, mode=mode, dtype=dtype) as s:
+        if start:
+            start.wait()
+        for _ in range(rounds):
+            s.step(iters)
+        return s.gbest(), s.state()
+
+
+# the larger swarm's kernel takes more shared memory than the smaller one's: 82 and 55 KB in
+# registers (8 pairs a thread), 105 and 25 KB in double precision, and on a cluster
+@pytest.mark.parametrize("mode,dtype,fid,large,small", [
+    ("sync", "f32", 1, (77824, 16), (20000, 48)),
+    ("sync", "f64", 0, (16384, 120), (200000, 7))])
+def test_two_threads_step_two_sizes(P, mode, dtype, fid, large, small):
+    rounds, iters = 300, 5
+    got, errors, start = {}, [], threading.Barrier(2)
+
+    def work(size):
+        try:
+            got[size] = _run(P, fid, *size, mode, dtype, rounds, iters, start)
+        except Exception as e:
+            errors.append((size, e))
+
+    threads = [threading.Thread(target=work, args=(size,)) for size in (large, small)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for size in (large, small):
+        (rc, fit, idx, pos), st = got[size]
+        (rc1, fit1, idx1, pos1), st1 = _run(P, fid, *size, mode, dtype, rounds, iters)
+        assert (rc, fit, idx) == (rc1, fit1, idx1) == (P.CUPSO_OK, fit, idx)
+        np.testing.assert_array_equal(pos, pos1)
+        for name in ("pos", "v", "pbest_pos", "pbest_fit"):
+            assert st[name].tobytes() == st1[name].tobytes(), name
