@@ -232,20 +232,29 @@ __global__ void __launch_bounds__(kOnchipThreads) onchip_kernel(const __grid_con
     cluster.sync();
 }
 
-int max_optin_smem() {
+// Dynamic shared memory that a CTA may take: the device's limit less room for the static
+// shared arrays.
+int max_onchip_smem() {
     int dev = 0, v = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
-    return v;
+    return v - 2048;
+}
+
+// A kernel's limits belong to all swarms that run it, from whichever host thread: always
+// raised to the same values (with a swarm's own size, another thread's swarm lowered
+// it between here and the launch).
+template <typename K>
+cudaError_t raise_limits(K kernel, int C) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_onchip_smem());
+    if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
 }
 
 // The cluster can be scheduled: the device reports room for at least one.
 bool cluster_schedulable(int C, size_t smem) {
     auto kernel = onchip_kernel<kSphere, false>;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return false;
-    if (C > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-        return false;
+    if (raise_limits(kernel, C) != cudaSuccess) return false;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)C, 1, 1);
     cfg.blockDim = dim3(kOnchipThreads, 1, 1);
@@ -269,7 +278,7 @@ bool cluster_schedulable(int C, size_t smem) {
 
 bool onchip_fits(int N, int D, int* cluster_out, int* per_cta_out) {
     const int Np = (N + kPad - 1) / kPad * kPad;
-    const int limit = max_optin_smem() - 2048;   // room for the static shared arrays
+    const int limit = max_onchip_smem();
     if (limit <= 0) return false;
     // Smallest cluster that fits, then grow towards ~64 particles per CTA for
     // parallelism; shrink again if the device cannot schedule that cluster.
@@ -295,12 +304,8 @@ cudaError_t launch_onchip_t(const SwarmDev& s, int iters, cudaStream_t st) {
     if (!onchip_fits(s.N, s.D, &C, &P)) return cudaErrorInvalidConfiguration;
     const OnchipLayout L = onchip_layout(s.Np, s.D, C);
     auto kernel = onchip_kernel<FIT, FAST>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.bytes);
+    const cudaError_t e = raise_limits(kernel, C);
     if (e != cudaSuccess) return e;
-    if (C > 8) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)C, 1, 1);
     cfg.blockDim = dim3(kOnchipThreads, 1, 1);

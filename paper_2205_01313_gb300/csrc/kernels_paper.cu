@@ -817,11 +817,13 @@ cudaError_t launch_step64(const SwarmDev64& s, const PaperBufs& b, int fid, int 
 
 namespace {
 
-int max_optin_smem64() {
+// Dynamic shared memory that a CTA of the on-chip kernel may take: the device's limit less
+// room for the static shared arrays.
+int max_onchip64_smem() {
     int dev = 0, v = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
-    return v;
+    return v - 1024;
 }
 
 int threads_for(int P, int D) {
@@ -830,9 +832,11 @@ int threads_for(int P, int D) {
     return th < 32 ? 32 : (th > kOnchip64Threads ? kOnchip64Threads : th);
 }
 
+// The same limits whatever the swarm: they belong to the kernel, which swarms of other sizes
+// run from other host threads.
 template <int FIT>
-cudaError_t set_onchip64_attrs(size_t smem, int C) {
-    cudaError_t e = cudaFuncSetAttribute(onchip64_kernel<FIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t set_onchip64_attrs(int C) {
+    cudaError_t e = cudaFuncSetAttribute(onchip64_kernel<FIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_onchip64_smem());
     if (e == cudaSuccess && C > 8)
         e = cudaFuncSetAttribute(onchip64_kernel<FIT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
@@ -855,7 +859,7 @@ cudaLaunchConfig_t onchip64_config(int C, int threads, size_t smem, cudaStream_t
 
 bool cluster64_schedulable(int N, int D, int C) {
     const Onchip64Layout L = onchip64_layout(N, D, C);
-    if (set_onchip64_attrs<kSphere>(L.bytes, C) != cudaSuccess) {
+    if (set_onchip64_attrs<kSphere>(C) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -876,7 +880,7 @@ bool cluster64_schedulable(int N, int D, int C) {
 // the FP64 work of an iteration spreads over that many SMs), at least the
 // smallest count whose shared memory fits, at most 16.
 int onchip64_cluster(int N, int D) {
-    const int limit = max_optin_smem64() - 1024;   // room for the static shared arrays
+    const int limit = max_onchip64_smem();
     if (limit <= 0) return 0;
     const long long pd = (long long)N * D;
     int C = 1;
@@ -901,15 +905,15 @@ cudaError_t launch_onchip64(const SwarmDev64& s, int fid, int iters, cudaStream_
     cudaLaunchConfig_t cfg = onchip64_config(C, threads, L.bytes, st, attr);
     switch (fid) {
         case kSphere: {
-            cudaError_t e = set_onchip64_attrs<kSphere>(L.bytes, C);
+            cudaError_t e = set_onchip64_attrs<kSphere>(C);
             return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, onchip64_kernel<kSphere>, s, iters);
         }
         case kRosenbrock: {
-            cudaError_t e = set_onchip64_attrs<kRosenbrock>(L.bytes, C);
+            cudaError_t e = set_onchip64_attrs<kRosenbrock>(C);
             return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, onchip64_kernel<kRosenbrock>, s, iters);
         }
         case kCubicMax: {
-            cudaError_t e = set_onchip64_attrs<kCubicMax>(L.bytes, C);
+            cudaError_t e = set_onchip64_attrs<kCubicMax>(C);
             return e != cudaSuccess ? e : cudaLaunchKernelEx(&cfg, onchip64_kernel<kCubicMax>, s, iters);
         }
         default:

@@ -29,7 +29,9 @@ def _run(P, fid, N, D, mode, dtype, rounds, iters, start=None):
 # registers (8 pairs a thread), 105 and 25 KB in double precision, and on a cluster
 @pytest.mark.parametrize("mode,dtype,fid,large,small", [
     ("sync", "f32", 1, (77824, 16), (20000, 48)),
-    ("sync", "f64", 0, (16384, 120), (200000, 7))])
+    ("sync", "f64", 0, (16384, 120), (200000, 7)),
+    ("onchip", "f32", 1, (3072, 48), (512, 8)),
+    ("onchip", "f64", 0, (4096, 16), (512, 16))])
 def test_two_threads_step_two_sizes(P, mode, dtype, fid, large, small):
     rounds, iters = 300, 5
     got, errors, start = {}, [], threading.Barrier(2)
@@ -39,6 +41,7 @@ def test_two_threads_step_two_sizes(P, mode, dtype, fid, large, small):
             got[size] = _run(P, fid, *size, mode, dtype, rounds, iters, start)
         except Exception as e:
             errors.append((size, e))
+            start.abort()   # the other thread may be waiting for this one
 
     threads = [threading.Thread(target=work, args=(size,)) for size in (large, small)]
     for t in threads:
