@@ -1232,10 +1232,11 @@ cudaError_t lsq_launch_gram(const float* A, const float* b, int M, int D, double
     lsq_gram_kernel<<<dim3((D + 31) / 32, (D + 31) / 32), 256, 0, st>>>(A, b, M, D, Gm, cvec, Gff, ldf);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    // the rescoring keeps 4 candidates x D doubles in shared memory: past the
-    // default 48 KB from D = 1537 on
+    // the rescoring keeps 4 candidates x D doubles in shared memory: past the default 48 KB
+    // from D = 1537 on. The limit belongs to the kernel, so it is the same for every
+    // swarm (with each swarm's own, 64 dimensions took it from an earlier swarm of 1600).
     return cudaFuncSetAttribute(lsq_rescore_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(sizeof(double) * 4 * (size_t)D));
+                                (int)(sizeof(double) * 4 * (size_t)kGramMaxD));
 }
 
 // cand: [lists * 16] + [16] + ticket; partial: [16 * chunks]; flags: [Np / 4].
@@ -1245,10 +1246,11 @@ cudaError_t lsq_launch_offsets(const SwarmDev& s, const float* A, const float* b
                                int num_sms, cudaStream_t st) {
     const int grid = std::max(1, std::min(num_sms * 4, (M + 7) / 8));
     const size_t smem = sizeof(float) * (size_t)s.D;   // gbest_pos in shared memory
+    constexpr size_t kMost = 227 * 1024;   // what a CTA can have; the kernel's limit is set to it for every swarm
     if (smem > 48 * 1024) {
-        if (smem > 227 * 1024) return cudaErrorInvalidValue;
+        if (smem > kMost) return cudaErrorInvalidValue;
         const cudaError_t e = cudaFuncSetAttribute(lsq_offset_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)smem);
+                                                   (int)kMost);
         if (e != cudaSuccess) return e;
     }
     lsq_offset_kernel<<<grid, 256, smem, st>>>(s, A, b, M, off, stale);

@@ -1,6 +1,6 @@
-"""Handles of different host threads: two swarms that run the same kernel at different sizes, each
-stepped by a thread of its own, take no launch limit from one another and get the bits that
-they get alone."""
+"""Several handles: two swarms that run the same kernel at different sizes, each stepped by a host
+thread of its own or one after the other, take no launch limit from one another and get the
+bits that they get alone."""
 import threading
 
 import numpy as np
@@ -56,3 +56,25 @@ def test_two_threads_step_two_sizes(P, mode, dtype, fid, large, small):
         np.testing.assert_array_equal(pos, pos1)
         for name in ("pos", "v", "pbest_pos", "pbest_fit"):
             assert st[name].tobytes() == st1[name].tobytes(), name
+
+
+def test_lsq_rescoring_keeps_its_limit_beside_a_smaller_swarm(P):
+    """The FP64 Gram rescoring of 1600 dimensions (51 KB of shared memory) after a swarm of 64 was set up."""
+    import torch
+
+    torch.manual_seed(1)
+
+    def swarm(D, N=256):
+        A, b = torch.randn(D, D, device="cuda"), torch.randn(D, device="cuda")
+        s = P.Swarm(D, N, (-5.0, 5.0, 1.0), W, C12, C12, "lsq", 3)
+        s.set_option(P.CUPSO_OPT_LSQ_RESCORE, 1)
+        s.set_lsq(A.data_ptr(), b.data_ptr(), D, "bf16")
+        return s, A, b
+
+    large, A, b = swarm(1600)
+    small, A2, b2 = swarm(64)
+    for s in (large, small):
+        before = s.gbest_f64()
+        s.step(5)
+        assert s.gbest()[0] == P.CUPSO_OK and s.gbest_f64() <= before
+        s.close()
