@@ -1011,7 +1011,9 @@ int cupso_set_option(cupso_handle h, int key, long long value) {
             return CUPSO_OK;
         case CUPSO_OPT_CLEAR_STATUS:
             // with the status, the counters a wait that expired may have left behind
+            // (a double-precision swarm has none: each launch clears its own barrier)
             CUPSO_CUDA(cudaMemsetAsync(h->dev.status, 0, sizeof(unsigned), h->stream), "cudaMemsetAsync");
+            if (h->fp64) return CUPSO_OK;
             CUPSO_CUDA(cudaMemsetAsync(h->dev.ticket, 0, sizeof(unsigned), h->stream), "cudaMemsetAsync");
             CUPSO_CUDA(cudaMemsetAsync(h->dev.work, 0, 6 * sizeof(unsigned), h->stream), "cudaMemsetAsync");
             return CUPSO_OK;
