@@ -147,9 +147,10 @@ typedef enum {
                                      terms are binary64 either way. */
     CUPSO_OPT_FAULT_HOLD_LOCK = 100, /* test hook: ASYNC starts with the gbest lock held, so every
                                         lock wait must expire and report CUPSO_ERR_DEVICE_TIMEOUT */
-    CUPSO_OPT_FAULT_STALL_BARRIER = 101 /* test hook: a multi-iteration panel launch waits for one CTA
-                                           more than it has, so its first barrier wait expires and
-                                           reports CUPSO_ERR_DEVICE_TIMEOUT; the swarm's state is then
+    CUPSO_OPT_FAULT_STALL_BARRIER = 101 /* test hook: a cooperative launch of several iterations (panels,
+                                           registers, double precision) waits for one CTA more than it
+                                           has, so its first barrier wait expires and reports
+                                           CUPSO_ERR_DEVICE_TIMEOUT; the swarm's state is then
                                            undefined (CUPSO_OPT_CLEAR_STATUS resets the counters) */
 } cupso_option;
 

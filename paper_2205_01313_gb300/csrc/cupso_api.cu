@@ -73,7 +73,7 @@ struct cupso_swarm {
     int graph_mode = -1, graph_len = 0;
     uint32_t t_host = 0;
     int hold_lock = 0;
-    int stall_barrier = 0;          // test hook: the multi-iteration panel launch waits for one CTA more
+    int stall_barrier = 0;          // test hook: the cooperative multi-iteration launches wait for one CTA more
     int iters_per_launch = 0;       // panel SYNC step: iterations per launch, 0 = automatic
     int lsq_rescore = 0;            // CUPSO_OPT_LSQ_RESCORE: 0 float-float, 1 FP64
     int grid_override = 0;
@@ -1091,7 +1091,7 @@ int cupso_step(cupso_handle h, int iters) {
     }
     const int mode = resolved_mode(h);
     if (h->fp64 && use_sync64(h, mode, iters)) {
-        cudaError_t e = launch_sync64(h->dev64, h->s64bufs, h->fid, iters, h->num_sms, h->stream);
+        cudaError_t e = launch_sync64(h->dev64, h->s64bufs, h->fid, iters, h->stall_barrier != 0, h->num_sms, h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "one-launch step");
         h->t_host += (uint32_t)iters;
         return CUPSO_OK;

@@ -136,11 +136,12 @@ __device__ __forceinline__ void store_gbest64(const SwarmDev64& s, uint32_t t_en
 
 // P particles per CTA, blockDim.x >= P * rows in whole warps, ITEMS * rows >= D; S:
 // doubles per particle's row of X and H (odd, >= ITEMS * rows). rb zero (bar) and all
-// ones (slots) at launch. W1: s.w is 1.
+// ones (slots) at launch. W1: s.w is 1. `expect`: arrivals that complete a barrier
+// (gridDim.x; one more only to test that its bound works).
 template <int FIT, bool W1, int ITEMS>
 __global__ void __launch_bounds__(max_threads64(ITEMS), 1) sync64_reg_kernel(const __grid_constant__ SwarmDev64 s,
                                                                             const __grid_constant__ Sync64Bufs rb, int P,
-                                                                            int rows, int S, int iters) {
+                                                                            int rows, int S, int iters, unsigned int expect) {
     constexpr bool kNext = FitTerms64<FIT>::kNeedsNext;
     constexpr bool kH = FIT != kSphere;
     extern __shared__ __align__(16) double sm_s64[];
@@ -282,7 +283,7 @@ __global__ void __launch_bounds__(max_threads64(ITEMS), 1) sync64_reg_kernel(con
         if (more) words(t_prev + 2u + (uint32_t)k);
         if (!sums) bar_sync(2, T);
         if (more) begin(imp[p] != 0);
-        if (tid == poller) s_state = poll64(s, rb, (unsigned int)(k + 1) * gridDim.x, par, seen);
+        if (tid == poller) s_state = poll64(s, rb, (unsigned int)(k + 1) * expect, par, seen);
         __syncthreads();
         const int state = s_state;
         if (!state) break;
@@ -312,7 +313,7 @@ __global__ void __launch_bounds__(max_threads64(ITEMS), 1) sync64_reg_kernel(con
 template <int FIT, bool W1>
 __global__ void __launch_bounds__(kMemThreads, 1) sync64_mem_kernel(const __grid_constant__ SwarmDev64 s,
                                                                    const __grid_constant__ Sync64Bufs rb, int PC, int P,
-                                                                   int iters) {
+                                                                   int iters, unsigned int expect) {
     constexpr bool kNext = FitTerms64<FIT>::kNeedsNext;
     extern __shared__ __align__(16) double sm_s64[];
     const int D = s.D, T = (int)blockDim.x, tid = (int)threadIdx.x;
@@ -435,7 +436,7 @@ __global__ void __launch_bounds__(kMemThreads, 1) sync64_mem_kernel(const __grid
         }
         if (tid == 0) {
             arrive64(rb, par, has);
-            s_state = poll64(s, rb, (unsigned int)(k + 1) * gridDim.x, par, seen);
+            s_state = poll64(s, rb, (unsigned int)(k + 1) * expect, par, seen);
         }
         __syncthreads();
         const int state = s_state;
@@ -524,22 +525,24 @@ cudaError_t prepare_sync64(const SwarmDev64& s, int fid, int num_sms) {
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSync64Smem);
 }
 
-cudaError_t launch_sync64(const SwarmDev64& s, const Sync64Bufs& rb, int fid, int iters, int num_sms, cudaStream_t st) {
+cudaError_t launch_sync64(const SwarmDev64& s, const Sync64Bufs& rb, int fid, int iters, bool stall_barrier, int num_sms,
+                          cudaStream_t st) {
     Plan64 r;
     if (!rb.slots || iters < 1 || !plan64(fid, s.N, s.D, num_sms, &r)) return cudaErrorInvalidValue;
     const void* k = kernel64(fid, s.w_one != 0, r.items);
     if (!k) return cudaErrorInvalidValue;
+    unsigned int expect = (unsigned int)r.grid + (stall_barrier ? 1u : 0u);
     cudaError_t e = cudaSuccess;
     for (int left = iters; e == cudaSuccess && left > 0;) {
-        int n = std::min(left, 1 << 22);   // n x SMs arrivals stay below 2^32
+        int n = std::min(left, 1 << 22);   // n x (SMs + 1) arrivals stay below 2^32
         left -= n;
         e = cudaMemsetAsync(rb.bar, 0, sizeof(unsigned long long), st);
         if (e == cudaSuccess) e = cudaMemsetAsync(rb.slots, 0xFF, 2 * (size_t)r.grid * sync64_slot_bytes(s.D), st);
         if (e != cudaSuccess) break;
         SwarmDev64 sa = s;
         Sync64Bufs ba = rb;
-        void* reg_args[] = {&sa, &ba, &r.P, &r.rows, &r.S, &n};
-        void* mem_args[] = {&sa, &ba, &r.PC, &r.P, &n};
+        void* reg_args[] = {&sa, &ba, &r.P, &r.rows, &r.S, &n, &expect};
+        void* mem_args[] = {&sa, &ba, &r.PC, &r.P, &n, &expect};
         e = cudaLaunchCooperativeKernel(k, dim3(r.grid), dim3(r.threads), r.items ? reg_args : mem_args, r.smem, st);
     }
     return e;

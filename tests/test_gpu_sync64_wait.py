@@ -20,3 +20,19 @@ def test_status_of_a_double_precision_swarm_can_be_cleared(P, mode):
         s.set_option(P.CUPSO_OPT_CLEAR_STATUS, 1)
         s.step(6)
         assert s.gbest()[0] == P.CUPSO_OK
+
+
+# in registers; in memory, Rosenbrock with its second term array
+@pytest.mark.parametrize("mode,fid,N,D", [("sync", 0, 500, 7), ("persistent", 4, 2000, 1), ("sync", 3, 20000, 120)])
+def test_barrier_wait_expires_and_reports(P, mode, fid, N, D):
+    """A barrier that waits for one CTA more than there are: the wait ends at its limit, the status is
+    reported, and the swarm steps again once it is cleared."""
+    with P.Swarm(D, N, BOX, 1.0, 2.0, 2.0, fid, 7, mode=mode, dtype="f64") as s:
+        s.set_option(P.CUPSO_OPT_WAIT_LIMIT_NS, 50_000_000)
+        s.set_option(P.CUPSO_OPT_FAULT_STALL_BARRIER, 1)
+        s.step(6)
+        assert s.gbest()[0] == P.CUPSO_ERR_DEVICE_TIMEOUT
+        s.set_option(P.CUPSO_OPT_FAULT_STALL_BARRIER, 0)
+        s.set_option(P.CUPSO_OPT_CLEAR_STATUS, 1)
+        s.step(6)
+        assert s.gbest()[0] == P.CUPSO_OK
