@@ -132,13 +132,13 @@ typedef enum {
                                      BF16/FP8: the tensor-core product alone (the move kernel
                                      before it writes the operand; the selection after it adds the
                                      product's partial sums) */
-    CUPSO_OPT_ITERS_PER_LAUNCH = 9, /* SYNC step on the panel layout or in registers: iterations per
-                                       launch of a cupso_step call. 1: one kernel per iteration
-                                       (graphs per CUPSO_OPT_GRAPH_CHUNK); n > 1: up to n per
+    CUPSO_OPT_ITERS_PER_LAUNCH = 9, /* SYNC step on the panel layout, in registers or in double precision:
+                                       iterations per launch of a cupso_step call. 1: one kernel per
+                                       iteration (graphs per CUPSO_OPT_GRAPH_CHUNK); n > 1: up to n per
                                        cooperative launch, all CTAs resident, a grid barrier between
                                        iterations (each wait bounded by CUPSO_OPT_WAIT_LIMIT_NS);
-                                       0 (default): up to 4096 (registers: 2^22). Same results either
-                                       way. */
+                                       0 (default): up to 4096 (registers, double precision: 2^22).
+                                       Same results either way. PERSISTENT takes all of a call. */
     CUPSO_OPT_LSQ_RESCORE = 10,   /* BF16 / FP8 least-squares swarm with D <= M: arithmetic of
                                      the Gram-form rescoring of its gbest candidates. 0 (default):
                                      the off-diagonal part of x^T (A^T A) x in float-float (pairs

@@ -1091,7 +1091,10 @@ int cupso_step(cupso_handle h, int iters) {
     }
     const int mode = resolved_mode(h);
     if (h->fp64 && use_sync64(h, mode, iters)) {
-        cudaError_t e = launch_sync64(h->dev64, h->s64bufs, h->fid, iters, h->stall_barrier != 0, h->num_sms, h->stream);
+        // PERSISTENT: one launch by definition
+        const int most = mode != CUPSO_MODE_PERSISTENT && h->iters_per_launch > 0 ? h->iters_per_launch : kSync64MaxIters;
+        const cudaError_t e = launch_sync64(h->dev64, h->s64bufs, h->fid, iters, most, h->stall_barrier != 0, h->num_sms,
+                                            h->stream);
         if (e != cudaSuccess) return cuda_fail(e, "one-launch step");
         h->t_host += (uint32_t)iters;
         return CUPSO_OK;

@@ -525,16 +525,16 @@ cudaError_t prepare_sync64(const SwarmDev64& s, int fid, int num_sms) {
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSync64Smem);
 }
 
-cudaError_t launch_sync64(const SwarmDev64& s, const Sync64Bufs& rb, int fid, int iters, bool stall_barrier, int num_sms,
-                          cudaStream_t st) {
+cudaError_t launch_sync64(const SwarmDev64& s, const Sync64Bufs& rb, int fid, int iters, int per_launch, bool stall_barrier,
+                          int num_sms, cudaStream_t st) {
     Plan64 r;
-    if (!rb.slots || iters < 1 || !plan64(fid, s.N, s.D, num_sms, &r)) return cudaErrorInvalidValue;
+    if (!rb.slots || iters < 1 || per_launch < 1 || per_launch > kSync64MaxIters || !plan64(fid, s.N, s.D, num_sms, &r)) return cudaErrorInvalidValue;
     const void* k = kernel64(fid, s.w_one != 0, r.items);
     if (!k) return cudaErrorInvalidValue;
     unsigned int expect = (unsigned int)r.grid + (stall_barrier ? 1u : 0u);
     cudaError_t e = cudaSuccess;
     for (int left = iters; e == cudaSuccess && left > 0;) {
-        int n = std::min(left, 1 << 22);   // n x (SMs + 1) arrivals stay below 2^32
+        int n = std::min(left, per_launch);
         left -= n;
         e = cudaMemsetAsync(rb.bar, 0, sizeof(unsigned long long), st);
         if (e == cudaSuccess) e = cudaMemsetAsync(rb.slots, 0xFF, 2 * (size_t)r.grid * sync64_slot_bytes(s.D), st);

@@ -108,8 +108,10 @@ __host__ __device__ inline size_t sync64_slot_bytes(int D) { return (sizeof(PKey
 size_t sync64_bytes(int fid, int N, int D, int num_sms);
 Sync64Bufs sync64_bufs_at(void* base);
 cudaError_t prepare_sync64(const SwarmDev64& s, int fid, int num_sms);   // once, before the first launch
-cudaError_t launch_sync64(const SwarmDev64& s, const Sync64Bufs& rb, int fid, int iters, bool stall_barrier, int num_sms,
-                          cudaStream_t st);
+constexpr int kSync64MaxIters = 1 << 22;   // per launch: iterations x (SMs + 1) stays below 2^32
+// `iters` iterations in launches of up to `per_launch`.
+cudaError_t launch_sync64(const SwarmDev64& s, const Sync64Bufs& rb, int fid, int iters, int per_launch, bool stall_barrier,
+                          int num_sms, cudaStream_t st);
 
 // On-chip FP64 swarm: the whole swarm in the shared memory of one CTA cluster
 // (1 to 16 CTAs, chosen from (N, D) by onchip64_cluster), `iters` iterations
