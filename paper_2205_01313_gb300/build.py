@@ -19,7 +19,7 @@ SOURCES = ["cupso_api.cu", "cupso_batch.cu", "cupso_lsq.cu", "kernels_state.cu",
            "kernels_batch.cu", "kernels_batch_panel.cu", "kernels_lsq.cu", "kernels_lsq_exact.cu", "kernels_lsq_swarm.cu", "kernels_onchip.cu",
            "kernels_paper.cu", "kernels_sync64.cu", "kernels_tiled.cu", "kernels_panel.cu", "kernels_resident.cu", "cupso_noalloc.cu"]
 HEADERS = ["cupso_device.cuh", "cupso_internal.h", "stream_common.cuh", "paper_kernels.h", "tiled_kernels.h",
-           "async_common.cuh", "pdl.cuh", "lsq_internal.h", "tma_common.cuh", "fit_terms.cuh", "fp64_common.cuh", "panel_common.cuh"]
+           "async_common.cuh", "pdl.cuh", "lsq_internal.h", "tma_common.cuh", "fit_terms.cuh", "fp64_common.cuh", "panel_common.cuh", "resident.h"]
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVFLAGS = ARCH + [

@@ -20,6 +20,7 @@
 #include "cupso_internal.h"
 #include "lsq_internal.h"
 #include "paper_kernels.h"
+#include "resident.h"
 #include "tiled_kernels.h"
 
 using namespace cupso;

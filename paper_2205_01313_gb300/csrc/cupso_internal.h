@@ -100,7 +100,6 @@ constexpr int kResidentMaxIters = 1 << 22;   // per launch: iterations x (SMs + 
 bool resident_fits(const SwarmDev& s, int fid, int num_sms);
 size_t resident_bytes(int N, int D, int num_sms);   // 0: does not fit
 ResidentBufs resident_bufs_at(void* base);
-cudaError_t prepare_resident(const SwarmDev& s, int fid, int num_sms);   // once, before the first launch
 cudaError_t launch_resident(const SwarmDev& s, const ResidentBufs& rb, int fid, int panel, int iters, bool stall_barrier,
                             int num_sms, cudaStream_t st);
 

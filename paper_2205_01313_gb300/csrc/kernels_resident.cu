@@ -50,6 +50,7 @@
 #include "cupso_device.cuh"
 #include "cupso_internal.h"
 #include "fit_terms.cuh"
+#include "resident.h"
 #include "stream_common.cuh"
 
 namespace cupso {
