@@ -203,7 +203,14 @@ def workload_config(name, cfg, world):
             "parallelism": "replicas" if world > 1 else "single GPU"}
 
 
-def kernel_name(info):
+def in_registers(info, iters):
+    """Whether a call of `iters` iterations runs them in one launch with the swarm in registers."""
+    return 0 < info["one_launch_iters"] <= iters
+
+
+def kernel_name(info, iters):
+    if in_registers(info, iters):
+        return "resident_kernel"
     if info["sync_tile"]:
         return "sync_tiled_kernel"
     if info.get("sync_panel"):
@@ -277,7 +284,10 @@ def run_ours(a):
     sw.set_option(P.CUPSO_OPT_SYNC_KERNEL, P.SYNC_KERNELS[a.sync_kernel])
     info = sw.info()
     mode_used = {v: k for k, v in P.MODES.items()}[info["mode"]]
-    if mode_used == "sync":
+    resident = in_registers(info, a.steps)
+    if resident:
+        mode_used += " (the swarm in registers)"
+    elif mode_used == "sync":
         if info["sync_tile"]:
             mode_used = "sync (tiled kernel, %d particles per tile)" % info["sync_tile"]
         else:
@@ -293,11 +303,11 @@ def run_ours(a):
     sw.step(1)
     torch.cuda.synchronize()
 
-    # The K timed iterations in one cupso_step call: on the panel layout one
-    # cooperative launch runs them with a grid barrier between iterations (up
+    # The K timed iterations in one cupso_step call: in registers one cooperative
+    # launch, on the panel layout one with a grid barrier between iterations (up
     # to sync_iters_per_launch per launch), otherwise one launch per iteration.
     K = a.steps
-    ipl = min(K, info["sync_iters_per_launch"]) if mode_used.startswith("sync (panels") else 1
+    ipl = K if resident else min(K, info["sync_iters_per_launch"]) if mode_used.startswith("sync (panels") else 1
     launches = -(-K // ipl)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     clocks = ClockSampler(local)
@@ -350,7 +360,7 @@ def run_ours(a):
         "ms_per_step": total_ms / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": "f32", "data": "synthetic",
         "config": workload_config(a.workload, cfg, world),
-        "run": {"mode": mode_used, "grid": info["sync_grid"],
+        "run": {"mode": mode_used, "grid": None if resident else info["sync_grid"],
                 "timed": "the %d iterations in one cupso_step call: %d launch(es) of %d iteration(s)"
                          % (K, launches, ipl)},
         "e2e": {"value": work / e2e_s, "unit": UNIT, "h2d_bytes_per_step": 0,
@@ -361,7 +371,7 @@ def run_ours(a):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak,
                      "traffic": measured_traffic(a.workload, a.warmup + 1, ipl) if launches == 1 else None,
-                     "kernel": kernel_name(info),
+                     "kernel": kernel_name(info, K),
                      "algorithmic_bytes_per_launch": bpl,
                      "improved_fraction_timed": p_timed,
                      "improved_fraction_range": [min(fr[a.warmup:]), max(fr[a.warmup:])],
@@ -373,6 +383,10 @@ def run_ours(a):
         "clocks": clk,
         "result": {"gbest_fit": float(fit), "gbest_idx": idx, "status": rc},
     }
+    if resident:   # its iterations move nothing through memory
+        out["roofline"] = {"bound": "grid barrier", "achieved": None, "peak": peak, "unit": "GB/s", "frac": None,
+                           "traffic": None, "kernel": kernel_name(info, K), "iterations_per_launch": ipl,
+                           "launch_ms": per_launch_ms, "peak_source": peak_src}
     if rank == 0 and world == 1 and not a.no_cpu_baseline:
         out["cpu_baseline"] = cpu_baseline(cfg, a.cpu_iters)
     if rank == 0 and world == 1 and not a.no_extras and a.workload == DEFAULT_WORKLOAD:
@@ -542,7 +556,8 @@ def batch_report(P, a, stream, plain_every=1):
                          % max(1, plain_every)},
         "batched_over_plain": plain_s / batched_s,
         "alone_vs_batched_mismatches": mism,
-        "roofline": {"bound": "hbm", "kernel": "batch_panel_kernel", "achieved": achieved, "peak": peak,
+        "roofline": {"bound": "hbm", "kernel": "batch_panel_kernel, and batch_step_kernel or batch_tiled_kernel beside it for "
+                     "the swarms that are not in panels", "achieved": achieved, "peak": peak,
                      "unit": "GB/s", "frac": achieved / peak, "traffic": None,
                      "algorithmic_bytes_per_iteration": alg, "peak_source": src},
         "clocks": clk,

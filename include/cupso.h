@@ -193,6 +193,10 @@ typedef struct {
     int sync_tile;        /* particles per tile of the tiled SYNC kernel (0: not in use) */
     float fitness_ms;     /* mean fitness-phase time of the timed LSQ iterations, 0 if none */
     int fitness_timed;    /* how many iterations that mean covers */
+    int one_launch_iters; /* a cupso_step call of at least this many iterations runs them in one
+                             cooperative launch of its own kernel (the swarm in registers; double
+                             precision: or in memory), whatever the sync_ fields and onchip_cluster
+                             say, which describe shorter calls; 0: no call does */
     uint64_t device_bytes;/* device memory held by the handle        */
     int sync_panel;       /* panel width (8 or 16) when the SYNC step runs the panel kernel, else 0 */
     int sync_iters_per_launch; /* most iterations one SYNC launch runs (CUPSO_OPT_ITERS_PER_LAUNCH) */

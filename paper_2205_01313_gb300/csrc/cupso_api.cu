@@ -268,9 +268,9 @@ int panel_iters_per_launch(const cupso_swarm* h) {
     return h->iters_per_launch > 0 ? h->iters_per_launch : kPanelMaxIters;
 }
 
-// Whether `iters` iterations run in the resident kernel (kernels_resident.cu):
-// synchronous swarm, AUTO kernel choice, default grid, several iterations per
-// launch allowed.
+// The iterations of a call from which they run in the resident kernel
+// (kernels_resident.cu), 0: never. Synchronous swarm, AUTO kernel choice, default grid,
+// several iterations per launch allowed.
 //  * SYNC: loading and storing the registers costs as much as one or two iterations
 //    of the kernels that keep the state in memory; measured per iteration against
 //    them at 2, 3 and 4 iterations: 1024 x 32 6.4, 4.6, 4.2 us against 5.4, 5.3, 5.2;
@@ -281,29 +281,32 @@ int panel_iters_per_launch(const cupso_swarm* h) {
 //    1) to 4.7 (2048 x 32) on the cluster, whose launch costs less: 2048 x 32 at 4
 //    iterations 4.0 against 6.7 us, 1000 x 2 3.1 against 2.8; 300 x 8 (Rosenbrock)
 //    at 100 1.95 against 1.68, at 1000 1.51 against 1.58.
-bool use_resident(const cupso_swarm* h, int mode, int iters) {
+int resident_from(const cupso_swarm* h, int mode) {
     if (!h->rbufs.slots || h->sync_kernel != CUPSO_SYNC_KERNEL_AUTO || h->grid_override != 0 || h->iters_per_launch == 1)
-        return false;
-    if (mode == CUPSO_MODE_SYNC) return iters >= (h->panel ? 4 : 3);
-    if (mode != CUPSO_MODE_ONCHIP || h->mode != CUPSO_MODE_AUTO) return false;
-    return h->N >= 1000 ? iters >= 5 : ((long long)h->N * h->D >= 1000 && iters >= 300);
+        return 0;
+    if (mode == CUPSO_MODE_SYNC) return h->panel ? 4 : 3;
+    if (mode != CUPSO_MODE_ONCHIP || h->mode != CUPSO_MODE_AUTO) return 0;
+    return h->N >= 1000 ? 5 : (long long)h->N * h->D >= 1000 ? 300 : 0;
 }
 
-// Whether `iters` iterations of an FP64 swarm run in one cooperative launch
-// (kernels_sync64.cu). Its start and end cost as much as two to five iterations of the
+// The iterations of a call from which those of an FP64 swarm run in one cooperative
+// launch (kernels_sync64.cu), 0: never. Its start and end cost as much as two to five iterations of the
 // kernels with a launch per iteration (SYNC; us per iteration at 2 and 10: 32 x 1 5.6
 // and 2.3 against 4.6 and 4.5, 131072 x 1 10.7 and 6.3 against 9.2, 30000 x 10 at 10
 // 11.9 against 15.8), and more than those of the cluster (AUTO where the swarm
 // fits one: 512 x 1 at 10 and 200 2.4 and 1.55 against 2.3 and 1.8, 8192 x 1 2.6 and
 // 1.6 against 4.7 and 4.2).
-bool use_sync64(const cupso_swarm* h, int mode, int iters) {
-    if (!h->s64bufs.slots) return false;
-    if (mode == CUPSO_MODE_PERSISTENT) return true;
-    if (h->iters_per_launch == 1) return false;
+int sync64_from(const cupso_swarm* h, int mode) {
+    if (!h->s64bufs.slots) return 0;
+    if (mode == CUPSO_MODE_PERSISTENT) return 1;
+    if (h->iters_per_launch == 1) return 0;
     const long long pd = (long long)h->N * h->D;
-    if (mode == CUPSO_MODE_SYNC) return iters >= (pd >= (1 << 18) ? 5 : 3);
-    return mode == CUPSO_MODE_ONCHIP && h->mode == CUPSO_MODE_AUTO && iters >= (pd >= 2000 ? 10 : 50);
+    if (mode == CUPSO_MODE_SYNC) return pd >= (1 << 18) ? 5 : 3;
+    return mode == CUPSO_MODE_ONCHIP && h->mode == CUPSO_MODE_AUTO ? (pd >= 2000 ? 10 : 50) : 0;
 }
+
+// The same for either precision.
+int one_launch_from(const cupso_swarm* h, int mode) { return h->fp64 ? sync64_from(h, mode) : resident_from(h, mode); }
 
 // CTAs of a multi-iteration panel launch: the SYNC grid, at most what the SMs
 // hold at once (a cooperative launch).
@@ -1091,7 +1094,9 @@ int cupso_step(cupso_handle h, int iters) {
         return CUPSO_OK;
     }
     const int mode = resolved_mode(h);
-    if (h->fp64 && use_sync64(h, mode, iters)) {
+    const int from = one_launch_from(h, mode);
+    const bool one_launch = from > 0 && iters >= from;
+    if (h->fp64 && one_launch) {
         // PERSISTENT: one launch by definition
         const int most = mode != CUPSO_MODE_PERSISTENT && h->iters_per_launch > 0 ? h->iters_per_launch : kSync64MaxIters;
         const cudaError_t e = launch_sync64(h->dev64, h->s64bufs, h->fid, iters, most, h->stall_barrier != 0, h->num_sms,
@@ -1106,7 +1111,7 @@ int cupso_step(cupso_handle h, int iters) {
         h->t_host += (uint32_t)iters;
         return CUPSO_OK;
     }
-    if (!h->fp64 && use_resident(h, mode, iters)) {
+    if (one_launch) {
         // any layout, pending pbest rows included; a launch's iterations as for the panel step
         const int most = h->iters_per_launch > 0 ? h->iters_per_launch : kResidentMaxIters;
         for (int left = iters; left > 0;) {
@@ -1520,6 +1525,7 @@ int cupso_get_info(cupso_handle h, cupso_info* info) {
         info->sync_panel = pc.width;
         info->sync_iters_per_launch = pc.width ? panel_iters_per_launch(h) : 1;
     }
+    info->one_launch_iters = h->fid == CUPSO_LSQ ? 0 : one_launch_from(h, info->mode);
     info->fitness_ms = 0.0f;
     info->fitness_timed = 0;
     if (h->lsq) {

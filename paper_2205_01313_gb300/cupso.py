@@ -70,7 +70,7 @@ class cupso_info(C.Structure):
     _fields_ = [("N", C.c_int), ("D", C.c_int), ("Np", C.c_int), ("mode", C.c_int), ("t", C.c_uint32),
                 ("sync_grid", C.c_int), ("async_grid", C.c_int), ("onchip_cluster", C.c_int),
                 ("sync_stages", C.c_int), ("sync_ppt", C.c_int), ("sync_tile", C.c_int), ("fitness_ms", C.c_float),
-                ("fitness_timed", C.c_int),
+                ("fitness_timed", C.c_int), ("one_launch_iters", C.c_int),
                 ("device_bytes", C.c_uint64), ("sync_panel", C.c_int), ("sync_iters_per_launch", C.c_int)]
 
 
