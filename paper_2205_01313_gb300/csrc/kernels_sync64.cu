@@ -47,6 +47,11 @@ namespace {
 constexpr size_t kSync64Smem = 200u * 1024u;   // dynamic shared memory of a CTA at most
 constexpr int kMemThreads = 512;
 constexpr int kMemChunk = 4;   // items whose loads a thread issues together
+// Particles of a tile at most: one per thread, and with few dimensions enough for two
+// chunks of items per thread. With 512 whatever D, a one-dimensional tile was one item per thread
+// between four barriers: 4 10^6 x 1 (sphere) 169 us an iteration, and 142 in a launch per iteration;
+// now 128. 10^6 x 2 61 and 59, now 52; 4 10^6 x 3 330 and 313, now 299.
+constexpr int mem_tile(int D) { return std::max(kMemThreads, 2 * kMemChunk * kMemThreads / D); }
 
 // Threads per CTA at most for ITEMS dimensions per thread: what the register file
 // holds at 10 registers per item (whole warps per quarter SM).
@@ -307,7 +312,7 @@ __global__ void __launch_bounds__(max_threads64(ITEMS), 1) sync64_reg_kernel(con
     if (blockIdx.x == 0) store_gbest64(s, t_prev + (uint32_t)done, K, Gs);
 }
 
-// The state in memory: PC particles per CTA, taken in tiles of P (at most blockDim.x
+// The state in memory: PC particles per CTA, taken in tiles of P (at most mem_tile(D)
 // and what fits shared memory). A thread keeps its (dimension, particle) items of a
 // tile in every iteration, issuing the loads of kMemChunk of them together.
 template <int FIT, bool W1>
@@ -398,12 +403,12 @@ __global__ void __launch_bounds__(kMemThreads, 1) sync64_mem_kernel(const __grid
                 }
                 __syncthreads();
             }
-            if (tid < n) {
-                const uint32_t i = base + (uint32_t)tid;
-                const double f = FitTerms64<FIT>::sum(Y, Y, P, tid, D);
+            for (int q = tid; q < n; q += T) {   // more than one each only where D < 2 kMemChunk
+                const uint32_t i = base + (uint32_t)q;
+                const double f = FitTerms64<FIT>::sum(Y, Y, P, q, D);
                 nan |= (f != f);
                 const bool better = f < s.pf[i];
-                imp[tid] = better ? 1 : 0;
+                imp[q] = better ? 1 : 0;
                 if (better) {
                     s.pf[i] = f;
                     const PKey c{fit_key64(f), i, 0u};
@@ -473,7 +478,7 @@ bool plan64(int fid, int N, int D, int num_sms, Plan64* r) {
     // tiles of equal size, as few as fit shared memory
     const size_t per = sizeof(double) * (size_t)D * (fid == kRosenbrock ? 2 : 1) + 1;
     const size_t room = kSync64Smem - std::min(kSync64Smem, sizeof(double) * (size_t)D);
-    const int most = (int)std::min<size_t>(kMemThreads, room / per);
+    const int most = (int)std::min<size_t>(mem_tile(D), room / per);
     if (most < 1) return false;
     const int tiles = (PC + most - 1) / most;
     r->items = 0;
