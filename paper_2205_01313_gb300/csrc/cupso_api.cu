@@ -661,7 +661,9 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
     e = cudaMemsetAsync(base + o_words, 0, 128, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s.pflag, 0, (size_t)h->Np, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s.gkey, 0xFF, 2 * sizeof(unsigned long long), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + o_paper, 0, paper_bufs_bytes(h->Np, list_cap), h->stream);
+    // the queue designs' storage and the words of the resident kernel's exchange behind it
+    const size_t res_words = std::min<size_t>(res_bytes, 64);
+    if (e == cudaSuccess) e = cudaMemsetAsync(base + o_paper, 0, o_res + res_words - o_paper, h->stream);
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMemsetAsync"));
     const int grid = std::min(tiles_of(h->Np), h->num_sms * 4);
     e = launch_init(s, fid, grid, h->stream);
@@ -736,9 +738,9 @@ int create_swarm64(int D, int N, const cupso_bounds_f64* b, double w, double c1,
     const size_t o_words = off; off = align_up(off + 64, A);
     const int list_cap = h->Np;   // the tiled step may run up to one block per particle
     const size_t o_paper = off; off = align_up(off + paper_bufs_bytes(h->Np, list_cap), A);
-    const size_t o_rec = off; off = align_up(off + rec_bytes(D, true), A);
     const size_t s64_bytes = sync64_bytes(fid, N, D, h->num_sms);
     const size_t o_s64 = off; off = align_up(off + s64_bytes, A);
+    const size_t o_rec = off; off = align_up(off + rec_bytes(D, true), A);
     h->arena_bytes = off;
     e = cudaMalloc(&h->arena, h->arena_bytes);
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
@@ -786,7 +788,9 @@ int create_swarm64(int D, int N, const cupso_bounds_f64* b, double w, double c1,
 
     e = cudaMemsetAsync(base + o_words, 0, 64, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s.gkey, 0xFF, 2 * sizeof(PKey), h->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(base + o_paper, 0, paper_bufs_bytes(h->Np, list_cap), h->stream);
+    // the queue designs' storage and the words of the one-launch steps' exchange behind it
+    const size_t s64_words = std::min<size_t>(s64_bytes, 64);
+    if (e == cudaSuccess) e = cudaMemsetAsync(base + o_paper, 0, o_s64 + s64_words - o_paper, h->stream);
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMemsetAsync"));
     e = launch_init64(s, h->pbufs, fid, h->stream);
     if (e != cudaSuccess) return bail(cuda_fail(e, "init launch"));

@@ -142,7 +142,10 @@ __device__ __forceinline__ float row_fitness(const float* X, const float* H, int
 // quarter is odd, so that the summing threads' 16-byte reads spread over the
 // banks; >= 2 ITEMS rows). State in `panel` layout (0: dimension-major), pending
 // pbest rows (s.pflag) taken over and cleared. Requires s.fast_cr and s.fast_clamp (and, for a fitness with cos, bounds
-// within kSmallX), a cooperative launch, *rb.bar zero and rb.key all ones at launch.
+// within kSmallX), a cooperative launch, *rb.bar, the word behind it and rb.key zero at launch: the CTA
+// that leaves last clears them, so that a launch needs nothing before it (two memsets before
+// each took 1.3 of the 3.5 us of host time of a call).
+// rb.key holds complements, so that zero is "none".
 // `expect`: arrivals that complete a barrier (gridDim.x; one more only to test that
 // its bound works).
 // *rb.bar: arrivals in bits 0..31, the candidates of even and odd iterations in
@@ -270,7 +273,7 @@ __global__ void __launch_bounds__(max_threads(ITEMS), 1) resident_kernel(const _
                 // done before the barriers of this iteration: nothing to order, and a release would
                 // wait about 0.3 us.
                 if (cand != kKeyNone) {
-                    atomicMin(rb.key + par, cand);
+                    atomicMax(rb.key + par, ~cand);
                     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(rb.bar),
                                  "l"(1ull + (1ull << (32 + 16 * par)))
                                  : "memory");
@@ -303,7 +306,7 @@ __global__ void __launch_bounds__(max_threads(ITEMS), 1) resident_kernel(const _
             unsigned long long key = kKeyNone;
             if (now != (seen & mask)) {   // acquire what the candidates' arrivals released
                 asm volatile("fence.acq_rel.gpu;" ::: "memory");
-                key = __ldcg(rb.key + par);
+                key = ~__ldcg(rb.key + par);
             }
             s_key = key;
             seen = (seen & ~mask) | now;
@@ -343,6 +346,16 @@ __global__ void __launch_bounds__(max_threads(ITEMS), 1) resident_kernel(const _
         s.pflag[base + tid] = 0;
     }
     if (__syncthreads_or(nan) && tid == 0) atomicOr(s.status, kStatusNaN);
+    if (tid == 0) {   // every thread of the CTA is done with the exchange
+        unsigned int* gone = reinterpret_cast<unsigned int*>(rb.bar + 1);
+        __threadfence();   // this CTA's arrivals and candidates before its leaving
+        if (atomicAdd(gone, 1u) == gridDim.x - 1) {
+            __threadfence();
+            rb.key[0] = rb.key[1] = 0ull;
+            *rb.bar = 0ull;
+            *gone = 0u;
+        }
+    }
     if (blockIdx.x == 0) {
         const uint32_t t_end = t_prev + (uint32_t)done;
         const int out = (int)(t_end & 1u);
@@ -450,9 +463,6 @@ cudaError_t launch_resident(const SwarmDev& s, const ResidentBufs& rb, int fid, 
         return cudaErrorInvalidValue;
     const void* k = res_kernel(r.items, fid);
     if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(rb.key, 0xFF, 2 * sizeof(unsigned long long), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(rb.bar, 0, sizeof(unsigned long long), st);
-    if (e != cudaSuccess) return e;
     unsigned int expect = (unsigned int)r.grid + (stall_barrier ? 1u : 0u);
     ResidentBufs b = rb;
     void* args[] = {const_cast<SwarmDev*>(&s), &b, &r.P, &r.rows, &r.S, &panel, &iters, &expect};

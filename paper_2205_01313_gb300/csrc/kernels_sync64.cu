@@ -78,10 +78,13 @@ __device__ __forceinline__ PKey* slot_of(const Sync64Bufs& rb, int par, uint32_t
 }
 
 // One arrival; `cand`: it carries a candidate of this parity, whose slot was written
-// by threads that have passed a barrier with the caller since.
-__device__ __forceinline__ void arrive64(const Sync64Bufs& rb, int par, bool cand) {
-    if (cand)
-        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(rb.bar), "l"(1ull + (1ull << (32 + 16 * par))) : "memory");
+// by threads that have passed a barrier with the caller since. `first`: the launch's first, which
+// releases the cleared slots.
+__device__ __forceinline__ void arrive64(const Sync64Bufs& rb, int par, bool cand, bool first) {
+    if (cand || first)
+        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(rb.bar),
+                     "l"(1ull + (cand ? 1ull << (32 + 16 * par) : 0ull))
+                     : "memory");
     else
         asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(rb.bar), "l"(1ull) : "memory");
 }
@@ -126,6 +129,28 @@ __device__ __forceinline__ void take_gbest64(const Sync64Bufs& rb, int par, int 
     }
 }
 
+// No candidate in this CTA's slots yet (thread 0, whose first arrival releases it).
+__device__ __forceinline__ void clear_slots64(const Sync64Bufs& rb, int D) {
+    for (int par = 0; par < 2; ++par) {
+        PKey* slot = slot_of(rb, par, blockIdx.x, D);
+        __stcg(&slot->k, ~0ull);
+        __stcg(&slot->i, kNoIdx);
+    }
+}
+
+// Thread 0, after a barrier of the CTA: it is done with the exchange. The CTA that leaves last
+// clears the counters, so that a launch needs nothing before it (with two memsets before each, a
+// PERSISTENT call of one iteration took 11.2 us, with the kernel it had before 10.3; now 8.4).
+__device__ __forceinline__ void leave64(const Sync64Bufs& rb) {
+    unsigned int* gone = reinterpret_cast<unsigned int*>(rb.bar + 1);
+    __threadfence();   // this CTA's arrivals before its leaving
+    if (atomicAdd(gone, 1u) == gridDim.x - 1) {
+        __threadfence();
+        *rb.bar = 0ull;
+        *gone = 0u;
+    }
+}
+
 // The end of a launch: gbest and the iteration counter (one CTA).
 __device__ __forceinline__ void store_gbest64(const SwarmDev64& s, uint32_t t_end, const PKey& K, const double* Gs) {
     const int out = (int)(t_end & 1u);
@@ -140,8 +165,8 @@ __device__ __forceinline__ void store_gbest64(const SwarmDev64& s, uint32_t t_en
 }  // namespace
 
 // P particles per CTA, blockDim.x >= P * rows in whole warps, ITEMS * rows >= D; S:
-// doubles per particle's row of X and H (odd, >= ITEMS * rows). rb zero (bar) and all
-// ones (slots) at launch. W1: s.w is 1. `expect`: arrivals that complete a barrier
+// doubles per particle's row of X and H (odd, >= ITEMS * rows). rb.bar and the word behind
+// it zero at launch. W1: s.w is 1. `expect`: arrivals that complete a barrier
 // (gridDim.x; one more only to test that its bound works).
 template <int FIT, bool W1, int ITEMS>
 __global__ void __launch_bounds__(max_threads64(ITEMS), 1) sync64_reg_kernel(const __grid_constant__ SwarmDev64 s,
@@ -171,6 +196,7 @@ __global__ void __launch_bounds__(max_threads64(ITEMS), 1) sync64_reg_kernel(con
     const size_t Np = (size_t)s.Np;
     const uint32_t t_prev = __ldcg(s.t_dev);
     const int cur0 = (int)(t_prev & 1u);
+    if (tid == 0) clear_slots64(rb, D);
 
     double x[ITEMS], v[ITEMS], pb[ITEMS], cr1[ITEMS], cr2[ITEMS];
     // dimensions past D are skipped: an FP64 instruction costs more than the test
@@ -281,7 +307,7 @@ __global__ void __launch_bounds__(max_threads64(ITEMS), 1) sync64_reg_kernel(con
                 }
                 bar_sync(1, sum_threads);
             }
-            if (tid == 0) arrive64(rb, par, has);
+            if (tid == 0) arrive64(rb, par, has, k == 0);
             if (T > sum_threads) bar_arrive(2, T);   // the flags are written
         }
         const bool more = k + 1 < iters && active;
@@ -309,6 +335,7 @@ __global__ void __launch_bounds__(max_threads64(ITEMS), 1) sync64_reg_kernel(con
     }
     if (tid < n) s.pf[base + tid] = pf;
     if (__syncthreads_or(nan) && tid == 0) atomicOr(s.status, kStatusNaN);
+    if (tid == 0) leave64(rb);
     if (blockIdx.x == 0) store_gbest64(s, t_prev + (uint32_t)done, K, Gs);
 }
 
@@ -334,6 +361,7 @@ __global__ void __launch_bounds__(kMemThreads, 1) sync64_mem_kernel(const __grid
     const size_t Np = (size_t)s.Np;
     const uint32_t t_prev = __ldcg(s.t_dev);
     const int cur0 = (int)(t_prev & 1u);
+    if (tid == 0) clear_slots64(rb, D);
     for (int d = tid; d < D; d += T) Gs[d] = s.G[(size_t)cur0 * D + d];
     PKey K = load_gkey64(s, cur0);
     uint32_t seen = 0u;
@@ -440,7 +468,7 @@ __global__ void __launch_bounds__(kMemThreads, 1) sync64_mem_kernel(const __grid
             __syncthreads();
         }
         if (tid == 0) {
-            arrive64(rb, par, has);
+            arrive64(rb, par, has, k == 0);
             s_state = poll64(s, rb, (unsigned int)(k + 1) * expect, par, seen);
         }
         __syncthreads();
@@ -450,6 +478,7 @@ __global__ void __launch_bounds__(kMemThreads, 1) sync64_mem_kernel(const __grid
         done = k + 1;
     }
     if (__syncthreads_or(nan) && tid == 0) atomicOr(s.status, kStatusNaN);
+    if (tid == 0) leave64(rb);
     if (blockIdx.x == 0) store_gbest64(s, t_prev + (uint32_t)done, K, Gs);
 }
 
@@ -541,9 +570,6 @@ cudaError_t launch_sync64(const SwarmDev64& s, const Sync64Bufs& rb, int fid, in
     for (int left = iters; e == cudaSuccess && left > 0;) {
         int n = std::min(left, per_launch);
         left -= n;
-        e = cudaMemsetAsync(rb.bar, 0, sizeof(unsigned long long), st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(rb.slots, 0xFF, 2 * (size_t)r.grid * sync64_slot_bytes(s.D), st);
-        if (e != cudaSuccess) break;
         SwarmDev64 sa = s;
         Sync64Bufs ba = rb;
         void* reg_args[] = {&sa, &ba, &r.P, &r.rows, &r.S, &n, &expect};

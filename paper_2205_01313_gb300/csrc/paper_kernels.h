@@ -101,7 +101,8 @@ cudaError_t launch_recompute64(const SwarmDev64& s, const PaperBufs& b, cudaStre
 // swarm in registers where it fits, else in memory. Any N; D up to what one
 // particle's terms take of an SM's shared memory (sync64_bytes is 0 beyond).
 struct Sync64Bufs {
-    unsigned long long* bar = nullptr;   // arrivals and candidate counts
+    unsigned long long* bar = nullptr;   // arrivals and candidate counts; behind it the CTAs that have left.
+                                         // Zero before the first launch, and again after each
     unsigned char* slots = nullptr;      // [2][grid] candidates: key, position
 };
 __host__ __device__ inline size_t sync64_slot_bytes(int D) { return (sizeof(PKey) + sizeof(double) * (size_t)D + 15) / 16 * 16; }
