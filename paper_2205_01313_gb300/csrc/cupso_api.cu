@@ -115,8 +115,7 @@ struct cupso_swarm {
     // kStageBytes unless one particle's row is larger)
     void* stage = nullptr;
     size_t stage_bytes = 0;
-    char* rec_now = nullptr;        // device record of a gbest read, in the arena
-    std::vector<char> rec_copy;     // its host copy
+    std::vector<char> head_copy;    // host copy of a gbest read: the arena's head and gbest_pos
     // result slots of cupso_gbest_post / _wait (allocated on first use): a
     // device record and a pinned host copy per slot, the copy stream, and per
     // slot the events of the snapshot and of its copy
@@ -543,7 +542,10 @@ int cupso::check_problem_args(int D, int N, const cupso_bounds* b, float w, floa
 }
 
 namespace {
-size_t rec_bytes(int D, bool fp64);   // of a gbest read's record, below
+// What a gbest read needs stands together in the arena, so that one copy brings it: the
+// keys of both parities, the counters and words with the sticky status, and from kHeadBytes
+// gbest_pos of both parities.
+constexpr size_t kHeadBytes = 128, kHeadStatus = 40, kHeadStatus64 = 36;
 }
 
 // The fast arithmetic path's constants and whether it gives the same bits:
@@ -586,7 +588,7 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaStreamCreate"));
     h->stream = user_stream ? user_stream : h->own;
 
-    // One arena: x, v, pb [D][Np]; pf [Np]; G [2][D]; Grec [D]; aux; words.
+    // One arena: x, v, pb [D][Np]; pf [Np]; words, G [2][D]; Grec [D]; aux; ...
     const size_t A = 256;
     const size_t plane = sizeof(float) * (size_t)D * (size_t)h->Np;
     const size_t ntiles = (size_t)tiles_of(h->Np);
@@ -595,21 +597,19 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
     const size_t o_v = off; off = align_up(off + plane, A);
     const size_t o_pb = off; off = align_up(off + plane, A);
     const size_t o_pf = off; off = align_up(off + sizeof(float) * (size_t)h->Np, A);
+    const size_t o_words = off; off += kHeadBytes;
     const size_t o_G = off; off = align_up(off + sizeof(float) * 2 * (size_t)D, A);
     const size_t o_Grec = off; off = align_up(off + sizeof(float) * (size_t)D, A);
     const size_t o_aux = off; off = align_up(off + sizeof(unsigned long long) * ntiles, A);
     const size_t o_flag = off; off = align_up(off + (size_t)h->Np, A);
-    const size_t o_words = off; off = align_up(off + 128, A);
     const int list_cap = paper_blocks(h->Np);      // one candidate per block of the queue designs
     const size_t o_paper = off; off = align_up(off + paper_bufs_bytes(h->Np, list_cap), A);
     const size_t res_bytes = fid == CUPSO_LSQ ? 0 : resident_bytes(N, D, h->num_sms);
     const size_t o_res = off; off = align_up(off + res_bytes, A);
-    const size_t o_rec = off; off = align_up(off + rec_bytes(D, false), A);
     h->arena_bytes = off;
     e = cudaMalloc(&h->arena, h->arena_bytes);
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
     char* base = static_cast<char*>(h->arena);
-    h->rec_now = base + o_rec;
     SwarmDev& s = h->dev;
     s.x = reinterpret_cast<float*>(base + o_x);
     s.v = reinterpret_cast<float*>(base + o_v);
@@ -626,7 +626,7 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
     unsigned int* w32 = reinterpret_cast<unsigned int*>(w64 + 4);
     s.ticket = w32 + 0;
     s.t_dev = w32 + 1;
-    s.status = w32 + 2;
+    s.status = w32 + 2;   // kHeadStatus
     s.lock = w32 + 3;
     s.seq = w32 + 4;
     s.work = w32 + 5;
@@ -658,7 +658,7 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
     h->panel_ok = fid != CUPSO_LSQ && panel_supported(8, 3, D) && prepare_panel(fid, fast_form(s, fid)) == cudaSuccess;
     cudaGetLastError();
 
-    e = cudaMemsetAsync(base + o_words, 0, 128, h->stream);
+    e = cudaMemsetAsync(base + o_words, 0, kHeadBytes, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s.pflag, 0, (size_t)h->Np, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(s.gkey, 0xFF, 2 * sizeof(unsigned long long), h->stream);
     // the queue designs' storage and the words of the resident kernel's exchange behind it
@@ -686,7 +686,7 @@ int pow2_exponent(double c) {
 }
 
 // A double-precision swarm: arena x, v, pb [D][Np], pf [Np], G [2][D]
-// (binary64), gbest keys, counters, and the working storage of the
+// (binary64) behind the gbest keys and counters, and the working storage of the
 // one-particle-per-thread kernels.
 int create_swarm64(int D, int N, const cupso_bounds_f64* b, double w, double c1, double c2, int fid, uint64_t seed,
                    cupso_handle* out) {
@@ -733,19 +733,17 @@ int create_swarm64(int D, int N, const cupso_bounds_f64* b, double w, double c1,
     const size_t o_v = off; off = align_up(off + plane, A);
     const size_t o_pb = off; off = align_up(off + plane, A);
     const size_t o_pf = off; off = align_up(off + sizeof(double) * (size_t)h->Np, A);
+    const size_t o_key = off;
+    const size_t o_words = off + 2 * sizeof(PKey); off += kHeadBytes;
     const size_t o_G = off; off = align_up(off + sizeof(double) * 2 * (size_t)D, A);
-    const size_t o_key = off; off = align_up(off + 2 * sizeof(PKey), A);
-    const size_t o_words = off; off = align_up(off + 64, A);
     const int list_cap = h->Np;   // the tiled step may run up to one block per particle
     const size_t o_paper = off; off = align_up(off + paper_bufs_bytes(h->Np, list_cap), A);
     const size_t s64_bytes = sync64_bytes(fid, N, D, h->num_sms);
     const size_t o_s64 = off; off = align_up(off + s64_bytes, A);
-    const size_t o_rec = off; off = align_up(off + rec_bytes(D, true), A);
     h->arena_bytes = off;
     e = cudaMalloc(&h->arena, h->arena_bytes);
     if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc"));
     char* base = static_cast<char*>(h->arena);
-    h->rec_now = base + o_rec;
     SwarmDev64& s = h->dev64;
     s.x = reinterpret_cast<double*>(base + o_x);
     s.v = reinterpret_cast<double*>(base + o_v);
@@ -755,7 +753,7 @@ int create_swarm64(int D, int N, const cupso_bounds_f64* b, double w, double c1,
     s.gkey = reinterpret_cast<PKey*>(base + o_key);
     unsigned int* w32 = reinterpret_cast<unsigned int*>(base + o_words);
     s.t_dev = w32 + 0;
-    s.status = w32 + 1;
+    s.status = w32 + 1;   // kHeadStatus64
     s.N = N;
     s.D = D;
     s.Np = h->Np;
@@ -913,52 +911,54 @@ void cupso::set_cuda_error(cudaError_t e, const char* where) { cuda_fail(e, wher
 
 namespace {
 
-// One result record: the gbest key at 0 (16 bytes, of which a single-precision
-// swarm uses 8), the sticky status at 16, gbest_pos from 32.
+// A posted result's record: the gbest key at 0, the sticky status at 16, gbest_pos from 32.
 constexpr size_t kRecStatus = 16, kRecPos = 32;
-size_t rec_bytes(int D, bool fp64) { return align_up(kRecPos + (fp64 ? 8 : 4) * (size_t)D, 256); }
+size_t rec_bytes(int D) { return align_up(kRecPos + sizeof(float) * (size_t)D, 256); }
 
-// The current gbest into a contiguous record, so that one copy brings it to the host.
-__global__ void gbest_record_kernel(const uint32_t* __restrict__ key, int key_words, const unsigned* __restrict__ status,
-                                    const uint32_t* __restrict__ G, int g_words, uint32_t* __restrict__ rec) {
-    for (int e = threadIdx.x; e < g_words; e += blockDim.x) rec[kRecPos / 4 + e] = __ldcg(G + e);
-    if ((int)threadIdx.x < key_words) rec[threadIdx.x] = __ldcg(key + threadIdx.x);
+// The current gbest into a contiguous record, a snapshot that later steps do not change.
+__global__ void gbest_record_kernel(const uint32_t* __restrict__ key, const unsigned* __restrict__ status,
+                                    const uint32_t* __restrict__ G, int D, uint32_t* __restrict__ rec) {
+    for (int e = threadIdx.x; e < D; e += blockDim.x) rec[kRecPos / 4 + e] = __ldcg(G + e);
+    if (threadIdx.x < 2) rec[threadIdx.x] = __ldcg(key + threadIdx.x);
     if (threadIdx.x == 32) rec[kRecStatus / 4] = __ldcg(status);
 }
 
 cudaError_t queue_record(const cupso_swarm* h, char* rec) {
     const size_t cur = h->t_host & 1u, D = (size_t)h->D;
-    uint32_t* out = reinterpret_cast<uint32_t*>(rec);
-    if (h->fp64)
-        gbest_record_kernel<<<1, 256, 0, h->stream>>>(reinterpret_cast<const uint32_t*>(h->dev64.gkey + cur), 4,
-                                                      h->dev64.status, reinterpret_cast<const uint32_t*>(h->dev64.G + cur * D),
-                                                      (int)(2 * D), out);
-    else
-        gbest_record_kernel<<<1, 256, 0, h->stream>>>(reinterpret_cast<const uint32_t*>(h->dev.gkey + cur), 2, h->dev.status,
-                                                      reinterpret_cast<const uint32_t*>(h->dev.G + cur * D), (int)D, out);
+    gbest_record_kernel<<<1, 256, 0, h->stream>>>(reinterpret_cast<const uint32_t*>(h->dev.gkey + cur), h->dev.status,
+                                                  reinterpret_cast<const uint32_t*>(h->dev.G + cur * D), (int)D,
+                                                  reinterpret_cast<uint32_t*>(rec));
     return cudaGetLastError();
 }
 
-// The current gbest in h->rec_copy (its position only if asked for): one kernel, one
-// copy into ordinary memory and one wait (24 us with the wait for an idle stream, as
-// with a copy per field into pinned memory, which took 130 us to allocate with the
-// first read and 120 to free with the handle).
-int read_record(cupso_swarm* h, bool pos) {
-    const size_t bytes = pos ? kRecPos + (h->fp64 ? 8 : 4) * (size_t)h->D : kRecPos;
+// The arena's head in h->head_copy, and *pos, unless null, at the current gbest_pos in it: one copy
+// into ordinary memory and one wait (14 us through the Python binding, as with a copy per
+// field into pinned memory, which took 130 us to allocate with the first read and 120 to free with the
+// handle; with a kernel that gathers a record first 19). It takes both parities' positions
+// along where the current one comes second, unless they are long.
+int read_head(cupso_swarm* h, const char** pos) {
+    const size_t cur = h->t_host & 1u, row = (h->fp64 ? sizeof(double) : sizeof(float)) * (size_t)h->D;
+    const bool apart = pos && cur && row > (64u << 10);
+    const size_t tail = !pos || apart ? 0 : (cur + 1) * row;
     try {
-        h->rec_copy.resize(rec_bytes(h->D, h->fp64));
+        h->head_copy.resize(kHeadBytes + (apart ? row : tail));
     } catch (...) {
         return fail(CUPSO_ERR_OOM, "host allocation failed%s");
     }
-    CUPSO_CUDA(queue_record(h, h->rec_now), "gbest record launch");
-    CUPSO_CUDA(cudaMemcpyAsync(h->rec_copy.data(), h->rec_now, bytes, cudaMemcpyDeviceToHost, h->stream), "cudaMemcpyAsync");
+    char* const to = h->head_copy.data();
+    const char* const head = h->fp64 ? reinterpret_cast<const char*>(h->dev64.gkey) : reinterpret_cast<const char*>(h->dev.gkey);
+    CUPSO_CUDA(cudaMemcpyAsync(to, head, kHeadBytes + tail, cudaMemcpyDeviceToHost, h->stream), "cudaMemcpyAsync");
+    if (apart)
+        CUPSO_CUDA(cudaMemcpyAsync(to + kHeadBytes, head + kHeadBytes + row, row, cudaMemcpyDeviceToHost, h->stream),
+                   "cudaMemcpyAsync");
     CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    if (pos) *pos = to + kHeadBytes + (apart ? 0 : cur * row);
     return CUPSO_OK;
 }
 
 int ensure_records(cupso_swarm* h) {
     if (h->rec_dev) return CUPSO_OK;
-    const size_t bytes = 2 * rec_bytes(h->D, false);
+    const size_t bytes = 2 * rec_bytes(h->D);
     CUPSO_CUDA(cudaMalloc(&h->rec_dev, bytes), "cudaMalloc (gbest records)");
     CUPSO_CUDA(cudaMallocHost(&h->rec_host, bytes), "cudaMallocHost (gbest records)");
     CUPSO_CUDA(cudaStreamCreateWithFlags(&h->rec_stream, cudaStreamNonBlocking), "cudaStreamCreate");
@@ -1191,14 +1191,14 @@ int cupso_step(cupso_handle h, int iters) {
 int cupso_get_gbest(cupso_handle h, float* fit_out, float* pos_out, int64_t* idx_out) {
     if (!h) return fail(CUPSO_ERR_INVALID_ARG, "handle is NULL%s");
     if (h->fp64) return fail(CUPSO_ERR_UNSUPPORTED, "double-precision swarm: use the _fp64 functions%s");
-    int rc = read_record(h, pos_out != nullptr);
+    const char* pos = nullptr;
+    int rc = read_head(h, pos_out ? &pos : nullptr);
     if (rc) return rc;
-    const char* rec = h->rec_copy.data();
     unsigned long long key = 0;
     unsigned st = 0;
-    std::memcpy(&key, rec, 8);
-    std::memcpy(&st, rec + kRecStatus, 4);
-    if (pos_out) std::memcpy(pos_out, rec + kRecPos, sizeof(float) * (size_t)h->D);
+    std::memcpy(&key, h->head_copy.data() + sizeof(key) * (h->t_host & 1u), sizeof(key));
+    std::memcpy(&st, h->head_copy.data() + kHeadStatus, sizeof(st));
+    if (pos_out) std::memcpy(pos_out, pos, sizeof(float) * (size_t)h->D);
     if (fit_out) *fit_out = key_to_fit(key);
     if (idx_out) *idx_out = (int64_t)(key & 0xFFFFFFFFull);
     rc = status_code(st);
@@ -1213,7 +1213,7 @@ int cupso_gbest_post(cupso_handle h, int slot) {
     if (h->rec_posted[slot]) return fail(CUPSO_ERR_INVALID_ARG, "slot already holds a result; wait for it first%s");
     int rc = ensure_records(h);
     if (rc) return rc;
-    const size_t rb = rec_bytes(h->D, false);
+    const size_t rb = rec_bytes(h->D);
     char* dev = h->rec_dev + (size_t)slot * rb;
     // the snapshot follows the queued steps on the handle's stream; the next
     // step cannot change what it copies (a step rewrites these words only
@@ -1235,7 +1235,7 @@ int cupso_gbest_wait(cupso_handle h, int slot, float* fit_out, float* pos_out, i
     if (!h->rec_posted[slot]) return fail(CUPSO_ERR_INVALID_ARG, "nothing posted to this slot%s");
     CUPSO_CUDA(cudaEventSynchronize(h->rec_done[slot]), "cudaEventSynchronize");
     h->rec_posted[slot] = false;
-    const char* rec = h->rec_host + (size_t)slot * rec_bytes(h->D, false);
+    const char* rec = h->rec_host + (size_t)slot * rec_bytes(h->D);
     unsigned long long key = 0;
     unsigned st = 0;
     std::memcpy(&key, rec, 8);
@@ -1442,14 +1442,14 @@ int cupso_create_fp64(int D, int N, const cupso_bounds_f64* bounds, double w, do
 int cupso_get_gbest_fp64(cupso_handle h, double* fit_out, double* pos_out, int64_t* idx_out) {
     if (!h) return fail(CUPSO_ERR_INVALID_ARG, "handle is NULL%s");
     if (!h->fp64) return fail(CUPSO_ERR_UNSUPPORTED, "not a double-precision swarm%s");
-    int rc = read_record(h, pos_out != nullptr);
+    const char* pos = nullptr;
+    int rc = read_head(h, pos_out ? &pos : nullptr);
     if (rc) return rc;
-    const char* rec = h->rec_copy.data();
     PKey key{};
     unsigned st = 0;
-    std::memcpy(&key, rec, sizeof(PKey));
-    std::memcpy(&st, rec + kRecStatus, 4);
-    if (pos_out) std::memcpy(pos_out, rec + kRecPos, sizeof(double) * (size_t)h->D);
+    std::memcpy(&key, h->head_copy.data() + sizeof(PKey) * (h->t_host & 1u), sizeof(PKey));
+    std::memcpy(&st, h->head_copy.data() + kHeadStatus64, sizeof(st));
+    if (pos_out) std::memcpy(pos_out, pos, sizeof(double) * (size_t)h->D);
     if (fit_out) *fit_out = key_to_fit64(key.k);
     if (idx_out) *idx_out = (int64_t)key.i;
     rc = status_code(st);
