@@ -147,11 +147,14 @@ typedef enum {
                                      terms are binary64 either way. */
     CUPSO_OPT_FAULT_HOLD_LOCK = 100, /* test hook: ASYNC starts with the gbest lock held, so every
                                         lock wait must expire and report CUPSO_ERR_DEVICE_TIMEOUT */
-    CUPSO_OPT_FAULT_STALL_BARRIER = 101 /* test hook: a cooperative launch of several iterations (panels,
+    CUPSO_OPT_FAULT_STALL_BARRIER = 101, /* test hook: a cooperative launch of several iterations (panels,
                                            registers, double precision) waits for one CTA more than it
                                            has, so its first barrier wait expires and reports
                                            CUPSO_ERR_DEVICE_TIMEOUT; the swarm's state is then
                                            undefined (CUPSO_OPT_CLEAR_STATUS resets the counters) */
+    CUPSO_OPT_FAULT_NO_STAGING = 102 /* test hook: cupso_get_state and cupso_set_state (both precisions)
+                                        find no device memory for their staging buffer and go through
+                                        host memory instead; set it before their first call */
 } cupso_option;
 
 /* The implementations of the SYNC step; all compute the same bits. */

@@ -113,6 +113,7 @@ struct cupso_swarm {
     Lsq* lsq = nullptr;
     // staged rows of get_state / set_state (allocated on first use, at most
     // kStageBytes unless one particle's row is larger)
+    bool no_staging = false;        // test hook: there is no device memory for it
     void* stage = nullptr;
     size_t stage_bytes = 0;
     std::vector<char> head_copy;    // host copy of a gbest read: the arena's head and gbest_pos
@@ -799,26 +800,46 @@ int create_swarm64(int D, int N, const cupso_bounds_f64* b, double w, double c1,
 }
 
 // The staging buffer for rows of `row` bytes, N of them: all at once, or chunks
-// of up to kStageBytes; fewer when memory is short, down to one row.
+// of up to kStageBytes; fewer when memory is short, down to one row. Kept as it is once
+// there. Leaves h->stage null where not even one row fits: the rows then go through host
+// memory (host_planes), which needs none on the device.
 constexpr size_t kStageBytes = 32u << 20;
 int ensure_stage(cupso_swarm* h, size_t row, size_t N) {
-    const size_t least = row;
-    if (h->stage_bytes >= std::min(row * N, std::max(least, kStageBytes))) return CUPSO_OK;
-    if (h->stage) cudaFree(h->stage);
-    h->stage = nullptr;
-    h->stage_bytes = 0;
-    size_t want = std::min(row * N, std::max(least, kStageBytes));
+    if (h->stage || h->no_staging) return CUPSO_OK;
+    size_t want = std::min(row * N, std::max(row, kStageBytes));
     cudaError_t e;
-    while ((e = cudaMalloc(&h->stage, want)) == cudaErrorMemoryAllocation && want > least) {
+    while ((e = cudaMalloc(&h->stage, want)) == cudaErrorMemoryAllocation && want > row) {
         cudaGetLastError();
-        want = std::max(least, want / 4);
+        want = std::max(row, want / 4);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
         h->stage = nullptr;
-        return cuda_fail(e, "cudaMalloc (state staging)");
+        return e == cudaErrorMemoryAllocation ? CUPSO_OK : cuda_fail(e, "cudaMalloc (state staging)");
     }
     h->stage_bytes = want;
+    return CUPSO_OK;
+}
+
+// Element (d, i) of a plane in `panel` layout (0: dimension-major).
+size_t plane_at(size_t d, size_t i, size_t Np, size_t panel) {
+    return panel ? ((d / panel) * Np + i) * panel + d % panel : d * Np + i;
+}
+
+template <typename T>
+void unpack_plane(const cupso_swarm* h, const T* plane, int panel, T* out) {
+    const size_t N = (size_t)h->N, D = (size_t)h->D, Np = (size_t)h->Np;
+    for (size_t i = 0; i < N; ++i)
+        for (size_t d = 0; d < D; ++d) out[i * D + d] = plane[plane_at(d, i, Np, (size_t)panel)];
+}
+
+// `count` bytes of host memory for whole planes.
+int host_planes(std::vector<char>* mem, size_t count) {
+    try {
+        mem->resize(count);
+    } catch (...) {
+        return fail(CUPSO_ERR_OOM, "host allocation failed%s");
+    }
     return CUPSO_OK;
 }
 
@@ -831,8 +852,17 @@ int download_rows(cupso_swarm* h, const T* src, int panel, T* out) {
         CUPSO_CUDA(cudaMemcpyAsync(out, src, sizeof(T) * (size_t)h->N, cudaMemcpyDeviceToHost, h->stream), "cudaMemcpyAsync");
         return CUPSO_OK;
     }
-    const int rc = ensure_stage(h, row, (size_t)h->N);
+    int rc = ensure_stage(h, row, (size_t)h->N);
     if (rc) return rc;
+    if (!h->stage) {
+        std::vector<char> mem;
+        rc = host_planes(&mem, row * (size_t)h->Np);
+        if (rc) return rc;
+        CUPSO_CUDA(cudaMemcpyAsync(mem.data(), src, mem.size(), cudaMemcpyDeviceToHost, h->stream), "cudaMemcpyAsync");
+        CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+        unpack_plane(h, reinterpret_cast<const T*>(mem.data()), panel, out);
+        return CUPSO_OK;
+    }
     const int per = (int)std::min<size_t>((size_t)h->N, h->stage_bytes / row);
     for (int i0 = 0; i0 < h->N; i0 += per) {
         const int n = std::min(per, h->N - i0);
@@ -844,9 +874,26 @@ int download_rows(cupso_swarm* h, const T* src, int panel, T* out) {
     return CUPSO_OK;
 }
 
-// The reverse: a device array in `panel` layout from in[i][d], zeros in the padding.
+// The whole state to the host, waited for.
 template <typename T>
-int upload_rows(cupso_swarm* h, const T* in, int panel, T* dst) {
+int download_state(cupso_swarm* h, const T* const (&planes)[3], const T* pf, int panel, T* const (&outs)[3], T* pf_out) {
+    const size_t N = (size_t)h->N;
+    for (int a = 0; a < 3; ++a) {
+        if (!outs[a]) continue;
+        const int rc = download_rows(h, planes[a], panel, outs[a]);
+        if (rc) return rc;
+    }
+    if (pf_out)
+        CUPSO_CUDA(cudaMemcpyAsync(pf_out, pf, sizeof(T) * N, cudaMemcpyDeviceToHost, h->stream), "cudaMemcpyAsync");
+    CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    return CUPSO_OK;
+}
+
+// The reverse of download_rows: a device array in `panel` layout from in[i][d], zeros in the
+// padding. ensure_stage comes before, so that a state is not left half loaded; without a
+// stage `host` holds a plane.
+template <typename T>
+int upload_rows(cupso_swarm* h, const T* in, int panel, T* dst, std::vector<char>& host) {
     const size_t D = (size_t)h->D, row = sizeof(T) * D;
     const int pad = h->Np - h->N;
     if (D == 1) {
@@ -854,8 +901,15 @@ int upload_rows(cupso_swarm* h, const T* in, int panel, T* dst) {
         CUPSO_CUDA(cudaMemsetAsync(dst + h->N, 0, sizeof(T) * (size_t)pad, h->stream), "cudaMemsetAsync");
         return CUPSO_OK;
     }
-    const int rc = ensure_stage(h, row, (size_t)h->N);
-    if (rc) return rc;
+    if (!h->stage) {
+        T* plane = reinterpret_cast<T*>(host.data());
+        std::fill(plane, plane + D * (size_t)h->Np, T(0));
+        for (size_t i = 0; i < (size_t)h->N; ++i)
+            for (size_t d = 0; d < D; ++d) plane[plane_at(d, i, (size_t)h->Np, (size_t)panel)] = in[i * D + d];
+        CUPSO_CUDA(cudaMemcpyAsync(dst, plane, row * (size_t)h->Np, cudaMemcpyHostToDevice, h->stream), "cudaMemcpyAsync");
+        CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+        return CUPSO_OK;
+    }
     const int per = (int)std::min<size_t>((size_t)h->N, h->stage_bytes / row);
     for (int i0 = 0; i0 < h->N; i0 += per) {
         const int n = std::min(per, h->N - i0);
@@ -866,6 +920,23 @@ int upload_rows(cupso_swarm* h, const T* in, int panel, T* dst) {
                                     h->stream),
                    "pack launch");
         if (last) break;
+    }
+    return CUPSO_OK;
+}
+
+// pos, v and pbest_pos into the arena.
+template <typename T>
+int upload_state(cupso_swarm* h, const T* const (&ins)[3], int panel, T* const (&dsts)[3]) {
+    std::vector<char> host;
+    if (h->D > 1) {
+        const size_t row = sizeof(T) * (size_t)h->D;
+        int rc = ensure_stage(h, row, (size_t)h->N);
+        if (rc == CUPSO_OK && !h->stage) rc = host_planes(&host, row * (size_t)h->Np);
+        if (rc) return rc;
+    }
+    for (int a = 0; a < 3; ++a) {
+        const int rc = upload_rows(h, ins[a], panel, dsts[a], host);
+        if (rc) return rc;
     }
     return CUPSO_OK;
 }
@@ -1064,6 +1135,9 @@ int cupso_set_option(cupso_handle h, int key, long long value) {
         case CUPSO_OPT_FAULT_STALL_BARRIER:
             h->stall_barrier = value ? 1 : 0;
             return CUPSO_OK;
+        case CUPSO_OPT_FAULT_NO_STAGING:
+            h->no_staging = value != 0;
+            return CUPSO_OK;
         default:
             return fail(CUPSO_ERR_INVALID_ARG, "unknown option%s");
     }
@@ -1253,17 +1327,10 @@ int cupso_get_state(cupso_handle h, float* pos, float* v, float* pbest_pos, floa
     if (h->fp64) return fail(CUPSO_ERR_UNSUPPORTED, "double-precision swarm: use the _fp64 functions%s");
     const int mrc = ensure_materialized(h);
     if (mrc) return mrc;
-    float* outs[3] = {pos, v, pbest_pos};
-    const float* srcs[3] = {h->dev.x, h->dev.v, h->dev.pb};
-    for (int a = 0; a < 3; ++a) {
-        if (!outs[a]) continue;
-        const int rc = download_rows(h, srcs[a], h->panel, outs[a]);
-        if (rc) return rc;
-    }
-    if (pbest_fit)
-        CUPSO_CUDA(cudaMemcpyAsync(pbest_fit, h->dev.pf, sizeof(float) * (size_t)h->N, cudaMemcpyDeviceToHost, h->stream),
-                   "cudaMemcpyAsync");
-    CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    float* const outs[3] = {pos, v, pbest_pos};
+    const float* const planes[3] = {h->dev.x, h->dev.v, h->dev.pb};
+    const int rc = download_state(h, planes, static_cast<const float*>(h->dev.pf), h->panel, outs, pbest_fit);
+    if (rc) return rc;
     if (t_out) *t_out = h->t_host;
     return CUPSO_OK;
 }
@@ -1276,12 +1343,10 @@ int cupso_set_state(cupso_handle h, const float* pos, const float* v, const floa
     CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
     // straight into the layout that the next step reads
     const int panel = resolved_mode(h) == CUPSO_MODE_SYNC ? panel_cfg(h).width : 0;
-    const float* ins[3] = {pos, v, pbest_pos};
-    float* dsts[3] = {h->dev.x, h->dev.v, h->dev.pb};
-    for (int a = 0; a < 3; ++a) {
-        const int rc = upload_rows(h, ins[a], panel, dsts[a]);
-        if (rc) return rc;
-    }
+    const float* const ins[3] = {pos, v, pbest_pos};
+    float* const dsts[3] = {h->dev.x, h->dev.v, h->dev.pb};
+    const int rc = upload_state(h, ins, panel, dsts);
+    if (rc) return rc;
     CUPSO_CUDA(cudaMemcpyAsync(h->dev.pf, pbest_fit, sizeof(float) * (size_t)h->N, cudaMemcpyHostToDevice, h->stream),
                "cudaMemcpyAsync");
     CUPSO_CUDA(cudaMemsetAsync(h->dev.pflag, 0, (size_t)h->Np, h->stream), "cudaMemsetAsync");
@@ -1461,17 +1526,10 @@ int cupso_get_state_fp64(cupso_handle h, double* pos, double* v, double* pbest_p
                          uint32_t* t_out) {
     if (!h) return fail(CUPSO_ERR_INVALID_ARG, "handle is NULL%s");
     if (!h->fp64) return fail(CUPSO_ERR_UNSUPPORTED, "not a double-precision swarm%s");
-    double* outs[3] = {pos, v, pbest_pos};
-    const double* srcs[3] = {h->dev64.x, h->dev64.v, h->dev64.pb};
-    for (int a = 0; a < 3; ++a) {
-        if (!outs[a]) continue;
-        const int rc = download_rows(h, srcs[a], 0, outs[a]);
-        if (rc) return rc;
-    }
-    if (pbest_fit)
-        CUPSO_CUDA(cudaMemcpyAsync(pbest_fit, h->dev64.pf, sizeof(double) * (size_t)h->N, cudaMemcpyDeviceToHost, h->stream),
-                   "cudaMemcpyAsync");
-    CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
+    double* const outs[3] = {pos, v, pbest_pos};
+    const double* const planes[3] = {h->dev64.x, h->dev64.v, h->dev64.pb};
+    const int rc = download_state(h, planes, static_cast<const double*>(h->dev64.pf), 0, outs, pbest_fit);
+    if (rc) return rc;
     if (t_out) *t_out = h->t_host;
     return CUPSO_OK;
 }
@@ -1483,12 +1541,10 @@ int cupso_set_state_fp64(cupso_handle h, const double* pos, const double* v, con
     if (!pos || !v || !pbest_pos || !pbest_fit) return fail(CUPSO_ERR_INVALID_ARG, "state array is NULL%s");
     const size_t N = (size_t)h->N;
     CUPSO_CUDA(cudaStreamSynchronize(h->stream), "cudaStreamSynchronize");
-    const double* ins[3] = {pos, v, pbest_pos};
-    double* dsts[3] = {h->dev64.x, h->dev64.v, h->dev64.pb};
-    for (int a = 0; a < 3; ++a) {
-        const int rc = upload_rows(h, ins[a], 0, dsts[a]);
-        if (rc) return rc;
-    }
+    const double* const ins[3] = {pos, v, pbest_pos};
+    double* const dsts[3] = {h->dev64.x, h->dev64.v, h->dev64.pb};
+    const int rc = upload_state(h, ins, 0, dsts);
+    if (rc) return rc;
     static const std::vector<double> inf((size_t)kPad, (double)INFINITY);   // pbest_fit of the padding
     CUPSO_CUDA(cudaMemcpyAsync(h->dev64.pf, pbest_fit, sizeof(double) * N, cudaMemcpyHostToDevice, h->stream), "cudaMemcpyAsync");
     CUPSO_CUDA(cudaMemcpyAsync(h->dev64.pf + N, inf.data(), sizeof(double) * (size_t)(h->Np - h->N), cudaMemcpyHostToDevice,

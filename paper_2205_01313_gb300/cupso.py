@@ -42,6 +42,7 @@ CUPSO_OPT_LSQ_RESCORE = 10
 SYNC_KERNELS = {"auto": 0, "register": 1, "pipelined3": 2, "pipelined4": 3, "tiled": 4, "panel8": 5, "panel16": 6}
 CUPSO_OPT_FAULT_HOLD_LOCK = 100
 CUPSO_OPT_FAULT_STALL_BARRIER = 101
+CUPSO_OPT_FAULT_NO_STAGING = 102
 
 # The names the library must export (every function of include/cupso.h).
 ABI_FUNCTIONS = ("cupso_create", "cupso_set_stream", "cupso_set_option", "cupso_step", "cupso_get_gbest",
