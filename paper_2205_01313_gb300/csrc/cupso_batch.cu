@@ -215,12 +215,30 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
         // kernel spreads them over a CTA -- 256 dimensions, 4,000 particles in all: 26.5 us
         // and 20.9; 8,000: 28.3 and 34.4; 64 dimensions: 11.4 and 17.7.
         std::vector<char> panel(nb);
-        long long panel_pd = 0, shallow_pd = 0;
-        int panel_maxD = 0;
+        long long rest = 0, padded = 0;   // units of 128 particles out of the panels, and of swarms that padding slows
+        std::vector<char> pad(nb);
         for (int j = 0; j < nb; ++j) {
             const cupso_problem& p = problems[batched[j]];
             panel[j] = !want_tiled && !want_stream && p.D >= kBatchPanelMinD && p.D <= 65536 &&
                        p.N <= 65536;
+            const int past = (p.D + 7) / 8 * 8 - p.D;
+            pad[j] = panel[j] && past * 100ll > (p.N <= 8192 ? 5ll : 1ll) * p.D;
+            (panel[j] ? padded : rest) += !panel[j] || pad[j] ? (p.N + 127) / 128 : 0;
+        }
+        // A panel partly used moves its unused dimensions too. Where memory bounds the batch
+        // either way, swarms that it adds more than 5 % to (1 % of long rows, which the
+        // streaming kernel moves best) stay out: when with those that stay out anyway there
+        // are units of 128 particles for five quarters of the streaming kernel's warps (16 an SM). 500
+        // swarms of up to 20000 x 25 to 32: 618 us an iteration out of the panels, 700 in
+        // them; 100 of up to 60000 x 30 to 60 528 and 600. With fewer units the
+        // panels' shorter ones win all the same: 200 of up to 4000 x 3 to 256 317 and 231.
+        if (rest + padded >= 20ll * run.num_sms)
+            for (int j = 0; j < nb; ++j)
+                if (pad[j]) panel[j] = 0;
+        long long panel_pd = 0, shallow_pd = 0;
+        int panel_maxD = 0;
+        for (int j = 0; j < nb; ++j) {
+            const cupso_problem& p = problems[batched[j]];
             if (!panel[j]) continue;
             panel_pd += (long long)p.N * p.D;
             if (p.D < kBatchPanelDeepD) shallow_pd += (long long)p.N * p.D;
