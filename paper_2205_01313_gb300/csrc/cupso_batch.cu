@@ -251,50 +251,66 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
                 if (problems[batched[j]].D < kBatchPanelDeepD) panel[j] = 0;
         if (panel_maxD > 64 && panel_pd < 6144ll * panel_maxD) panel.assign(nb, 0);
         std::vector<int> rows(nb);   // dimensions the state has room for
-        size_t panel_units = 0;
-        int nlegacy = 0;
         std::vector<size_t> o_state(nb), o_G(nb), o_flag(nb);
-        std::vector<int> Np(nb);
-        size_t off = 0, total_units = 0, sumG = 0, sumFlag = 0, total_tiles = 0;
-        std::vector<int> tileP(nb);
+        std::vector<int> Np(nb), tileP(nb);
         std::vector<unsigned> ntiles(nb);
-        int minD = 1 << 30, maxD = 0;
-        long long total_pd = 0;
-        for (int j = 0; j < nb; ++j) {
-            const cupso_problem& p = problems[batched[j]];
-            Np[j] = (p.N + kPad - 1) / kPad * kPad;
-            rows[j] = panel[j] ? (p.D + 7) / 8 * 8 : p.D;
-            o_state[j] = off;
-            off = up(off + sizeof(float) * ((size_t)3 * rows[j] * Np[j] + Np[j]), A);
-            o_G[j] = sumG = up(sumG, 4);   // 16-byte rows
-            sumG += 2 * (size_t)rows[j];
-            o_flag[j] = sumFlag;
-            sumFlag += (size_t)Np[j];
-            if (panel[j]) {
-                panel_units += (size_t)Np[j] / 16;
-                continue;
+        size_t off, total_units, panel_units, sumG, sumFlag, total_tiles;
+        int nlegacy, minD, maxD;
+        long long total_pd;
+        size_t o_Gall, o_keys, o_words, o_flags, o_desc, o_units, o_punits, o_tunits, o_tileP, o_ntiles, o_ctr;
+        auto place = [&](size_t bytes) {
+            const size_t o = off;
+            off = up(off + bytes, A);
+            return o;
+        };
+        auto layout = [&] {
+            off = total_units = panel_units = sumG = sumFlag = total_tiles = 0;
+            nlegacy = maxD = 0;
+            minD = 1 << 30;
+            total_pd = 0;
+            for (int j = 0; j < nb; ++j) {
+                const cupso_problem& p = problems[batched[j]];
+                Np[j] = (p.N + kPad - 1) / kPad * kPad;
+                rows[j] = panel[j] ? (p.D + 7) / 8 * 8 : p.D;
+                o_state[j] = place(sizeof(float) * ((size_t)3 * rows[j] * Np[j] + Np[j]));
+                o_G[j] = sumG = up(sumG, 4);   // 16-byte rows
+                sumG += 2 * (size_t)rows[j];
+                o_flag[j] = sumFlag;
+                sumFlag += (size_t)Np[j];
+                if (panel[j]) {
+                    panel_units += (size_t)Np[j] / 16;
+                    continue;
+                }
+                ++nlegacy;
+                total_units += (size_t)Np[j] / 128;
+                tileP[j] = batch_tile_particles(p.D);
+                ntiles[j] = tileP[j] > 0 ? (unsigned)((p.N + tileP[j] - 1) / tileP[j]) : 0u;
+                total_tiles += ntiles[j];
+                minD = std::min(minD, p.D);
+                maxD = std::max(maxD, p.D);
+                total_pd += (long long)p.N * p.D;
             }
-            ++nlegacy;
-            total_units += (size_t)Np[j] / 128;
-            tileP[j] = batch_tile_particles(p.D);
-            ntiles[j] = tileP[j] > 0 ? (unsigned)((p.N + tileP[j] - 1) / tileP[j]) : 0u;
-            total_tiles += ntiles[j];
-            minD = std::min(minD, p.D);
-            maxD = std::max(maxD, p.D);
-            total_pd += (long long)p.N * p.D;
-        }
-        const size_t o_Gall = off; off = up(off + sizeof(float) * sumG, A);
-        const size_t o_keys = off; off = up(off + sizeof(unsigned long long) * 2 * nb, A);
-        const size_t o_words = off; off = up(off + sizeof(unsigned int) * 4 * nb, A);
-        const size_t o_flags = off; off = up(off + sumFlag, A);
-        const size_t o_desc = off; off = up(off + sizeof(BatchSwarm) * nb, A);
-        const size_t o_units = off; off = up(off + sizeof(uint2) * total_units, A);
-        const size_t o_punits = off; off = up(off + sizeof(uint2) * panel_units, A);
-        const size_t o_tunits = off; off = up(off + sizeof(uint2) * std::max<size_t>(total_tiles, 1), A);
-        const size_t o_tileP = off; off = up(off + sizeof(int) * nb, A);
-        const size_t o_ntiles = off; off = up(off + sizeof(unsigned) * nb, A);
-        const size_t o_ctr = off; off = up(off + 128, A);
+            o_Gall = place(sizeof(float) * sumG);
+            o_keys = place(sizeof(unsigned long long) * 2 * nb);
+            o_words = place(sizeof(unsigned int) * 4 * nb);
+            o_flags = place(sumFlag);
+            o_desc = place(sizeof(BatchSwarm) * nb);
+            o_units = place(sizeof(uint2) * total_units);
+            o_punits = place(sizeof(uint2) * panel_units);
+            o_tunits = place(sizeof(uint2) * std::max<size_t>(total_tiles, 1));
+            o_tileP = place(sizeof(int) * nb);
+            o_ntiles = place(sizeof(unsigned) * nb);
+            o_ctr = place(128);
+        };
+        layout();
         e = cudaMalloc(&arena, off);
+        if (e == cudaErrorMemoryAllocation && nlegacy < nb) {
+            // without the room that whole panels take
+            cudaGetLastError();
+            panel.assign(nb, 0);
+            layout();
+            e = cudaMalloc(&arena, off);
+        }
         if (e != cudaSuccess) { set_cuda_error(e, "cudaMalloc (batch arena)"); rc = e == cudaErrorMemoryAllocation ? CUPSO_ERR_OOM : CUPSO_ERR_CUDA; break; }
         char* base = static_cast<char*>(arena);
         float* Gall = reinterpret_cast<float*>(base + o_Gall);
