@@ -39,6 +39,7 @@ namespace {
 constexpr size_t kExactWsBytes = 64u << 20;   // residual workspace at most
 constexpr int kResidThreads = 128;            // 16 x 8 threads of TM x TN residuals
 constexpr int kBk = 16;                       // dimensions per shared-memory stage
+constexpr int kTrimD = 64;                    // FP32: the trimmed inner loop up to here
 constexpr int kRowTile = 128;                 // chunk sizes are multiples of this
 constexpr int kSumCopiers = 128;              // the threads after the summing warp
 constexpr int kSumThreads = 32 + kSumCopiers;
@@ -128,10 +129,14 @@ __device__ __forceinline__ void st4g(double* p, const double* v) {
 // barrier per slice. A's slice is transposed on its way ([k][row], padded), both
 // operands are then read as 16-byte vectors that a warp shares (4 row groups x 8
 // particle groups). Zeros past D leave a residual's square unchanged.
+// TRIM: no multiplications past D and, a warp at a time, past the last row. Zeros take as long: FP64
+// 30000 x 2 x 14 75 us an iteration with them, 22 without, 30000 x 2 x 300 343 and 116 (before
+// the split into tiles 26 and 183). In FP32 with more dimensions the second form of the
+// inner loop costs more than it saves (2048 x 500 x 2000 338 and 347 us for two iterations).
 // FUSED: all rows fit one tile, so the block adds its particles' squares itself and
 // writes f; no workspace, no second launch (M = 40: 12.0 -> 10.1 us per iteration of
 // a 256 x 16 swarm).
-template <typename T, int TM, int TN, bool FUSED>
+template <typename T, int TM, int TN, bool FUSED, bool TRIM>
 __global__ void __launch_bounds__(kResidThreads, TM * TN == 128 ? 2 : TM * TN == 64 ? 3 : 1) lsq_resid_kernel(const float* __restrict__ x, int ldx, int D,
                                                                   const float* __restrict__ A,
                                                                   const float* __restrict__ b, int m0, int m1,
@@ -190,6 +195,8 @@ __global__ void __launch_bounds__(kResidThreads, TM * TN == 128 ? 2 : TM * TN ==
             st4g(&Xs[st][e / (BN / 4)][4 * (e % (BN / 4))], v);
         }
     };
+    // the rows of a warp lie together, so that one past the last row need not multiply
+    const bool busy = mt + (tid >> 5) * 16 < m1;
     // the thread's rows ty * 4 + j (+ 64) and particles tx * 4 + j (+ 32, 64, 96)
     auto row_of = [&](int a) { return (a / 4) * (BM * 4 / TM) + ty * 4 + a % 4; };
     Acc<T, TM, TN> acc;
@@ -205,8 +212,7 @@ __global__ void __launch_bounds__(kResidThreads, TM * TN == 128 ? 2 : TM * TN ==
     for (int s = 0; s < slices; ++s) {
         const int st = s & 1;
         if (s + 1 < slices) fetch((s + 1) * kBk, st ^ 1);
-#pragma unroll
-        for (int k = 0; k < kBk; ++k) {
+        auto multiply = [&](int k) {
             T av[TM];
             std::conditional_t<kF32, unsigned long long, T> xv[kF32 ? TN / 2 : TN];
 #pragma unroll
@@ -214,6 +220,14 @@ __global__ void __launch_bounds__(kResidThreads, TM * TN == 128 ? 2 : TM * TN ==
 #pragma unroll
             for (int c = 0; c < TN; c += 4) ld4s(&Xs[st][k][(c / 4) * (BN * 4 / TN) + tx * 4], xv + (kF32 ? c / 2 : c));
             acc.step(av, xv);
+        };
+        const int kn = TRIM ? (busy ? min(kBk, D - s * kBk) : 0) : kBk;
+        if (kn == kBk) {
+#pragma unroll
+            for (int k = 0; k < kBk; ++k) multiply(k);
+        } else {
+#pragma unroll 2
+            for (int k = 0; k < kn; ++k) multiply(k);
         }
         if (s + 1 < slices) stage(st ^ 1);   // the other stage: read last before the previous barrier
         __syncthreads();
@@ -354,7 +368,10 @@ void launch_resid(const float* x, int ldx, int Np, int D, const float* A, const 
                   cudaStream_t st, int N = 0, float* f = nullptr) {
     const int vecA = D % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
     const dim3 grid((unsigned)(Np / (8 * TN)), (unsigned)((m1 - m0 + 16 * TM - 1) / (16 * TM)));
-    lsq_resid_kernel<T, TM, TN, FUSED><<<grid, kResidThreads, 0, st>>>(x, ldx, D, A, b, m0, m1, R, Np, vecA, N, f);
+    if (sizeof(T) == 8 || D <= kTrimD)
+        lsq_resid_kernel<T, TM, TN, FUSED, true><<<grid, kResidThreads, 0, st>>>(x, ldx, D, A, b, m0, m1, R, Np, vecA, N, f);
+    else
+        lsq_resid_kernel<T, TM, TN, FUSED, false><<<grid, kResidThreads, 0, st>>>(x, ldx, D, A, b, m0, m1, R, Np, vecA, N, f);
 }
 
 template <typename T>
