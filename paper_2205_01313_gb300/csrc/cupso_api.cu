@@ -93,6 +93,7 @@ struct cupso_swarm {
         LsqTcState tc;              // BF16 / FP8 operands and plan
         void* buf = nullptr;        // f [Np] | cand [lists*16 + 16 + ticket] | partial [16 * chunks] | g64 | exact_ws
         void* exact_ws = nullptr;   // FP32 / FP64 fitness: residual workspace
+        size_t ws_most = 0;         // and its limit
         float* f = nullptr;
         unsigned long long* cand = nullptr;
         double* partial = nullptr;
@@ -364,7 +365,7 @@ cudaError_t launch_lsq_iteration(cupso_swarm* h, cudaStream_t st) {
         cudaError_t e = lsq_launch_move(h->dev, grid, st);
         if (e == cudaSuccess)
             e = lsq_exact_launch(h->dev.x, h->Np, h->N, h->D, L.A, L.b, L.M, L.precision == CUPSO_LSQ_FP64, L.f,
-                                 L.exact_ws, h->num_sms, st);
+                                 L.exact_ws, L.ws_most, h->num_sms, st);
         if (e != cudaSuccess) return e;
         return lsq_launch_select_exact(h->dev, L.f, L.flags, grid, st);
     }
@@ -1428,8 +1429,9 @@ int cupso_set_lsq(cupso_handle h, const float* A_dev, const float* b_dev, int M,
     const size_t bytes = align_up(sizeof(float) * h->Np, 256) + align_up(sizeof(unsigned long long) * (nlists * 16 + 17), 256) +
                          align_up(sizeof(double) * 16 * npart, 256) + align_up((size_t)h->Np, 256) + 256;
     const bool fp64_fit = precision == CUPSO_LSQ_FP64;
-    const size_t ws_bytes = lsq_approx(precision) ? 0 : lsq_exact_ws_bytes(h->N, M, fp64_fit);
-    cudaError_t e = cudaMalloc(&L->buf, bytes + ws_bytes);
+    cudaError_t e = lsq_approx(precision) ? cudaMalloc(&L->buf, bytes)
+                                          : lsq_exact_alloc(&L->buf, bytes, h->N, h->D, M, fp64_fit, false, h->num_sms,
+                                                            &L->exact_ws, &L->ws_most);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc (lsq)");
     char* p = static_cast<char*>(L->buf);
     L->f = reinterpret_cast<float*>(p); p += align_up(sizeof(float) * h->Np, 256);
@@ -1437,7 +1439,6 @@ int cupso_set_lsq(cupso_handle h, const float* A_dev, const float* b_dev, int M,
     L->partial = reinterpret_cast<double*>(p); p += align_up(sizeof(double) * 16 * npart, 256);
     L->flags = reinterpret_cast<unsigned int*>(p); p += align_up((size_t)h->Np, 256);
     L->g64 = reinterpret_cast<double*>(p); p += 256;
-    if (ws_bytes) L->exact_ws = p;
     const double inf = INFINITY;
     CUPSO_CUDA(cudaMemcpyAsync(L->g64, &inf, sizeof(double), cudaMemcpyHostToDevice, h->stream), "cudaMemcpyAsync");
     CUPSO_CUDA(cudaMemsetAsync(L->f, 0, sizeof(float) * h->Np, h->stream), "cudaMemsetAsync");
@@ -1480,7 +1481,7 @@ int cupso_set_lsq(cupso_handle h, const float* A_dev, const float* b_dev, int M,
     }
     // Step 1 completes here: pbest_fit = f(pbest_pos), gbest from it.
     if (precision == CUPSO_LSQ_FP32 || precision == CUPSO_LSQ_FP64) {
-        CUPSO_CUDA(lsq_exact_launch(h->dev.pb, h->Np, h->N, h->D, A_dev, b_dev, M, fp64_fit, L->f, L->exact_ws,
+        CUPSO_CUDA(lsq_exact_launch(h->dev.pb, h->Np, h->N, h->D, A_dev, b_dev, M, fp64_fit, L->f, L->exact_ws, L->ws_most,
                                     h->num_sms, h->stream),
                    "lsq fitness");
         CUPSO_CUDA(lsq_launch_set_pf(h->dev, L->f, h->stream), "lsq pbest");

@@ -267,13 +267,15 @@ extern "C" int cupso_lsq_eval(const float* A_dev, const float* b_dev, int M, int
         float* xd = nullptr;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaMalloc(&xd, xbytes + lsq_exact_ws_bytes(N, M, f64));
+        void* ws = nullptr;
+        size_t ws_most = 0;
+        if (e == cudaSuccess)
+            e = lsq_exact_alloc(reinterpret_cast<void**>(&xd), xbytes, N, D, M, f64, true, sms, &ws, &ws_most);
         if (e != cudaSuccess) return set_cuda_error(e, "cudaMalloc"), CUPSO_ERR_OOM;
         transpose_kernel<<<dim3((D + 31) / 32, (N + 31) / 32), dim3(32, 8), 0, st>>>(X_dev, N, D, (size_t)ld, xd);
         e = cudaGetLastError();
         if (e == cudaSuccess)
-            e = lsq_exact_launch(xd, ld, N, D, A_dev, b_dev, M, f64, f_out_dev, reinterpret_cast<char*>(xd) + xbytes, sms,
-                                 st);
+            e = lsq_exact_launch(xd, ld, N, D, A_dev, b_dev, M, f64, f_out_dev, ws, ws_most, sms, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         cudaFree(xd);
         if (e != cudaSuccess) return set_cuda_error(e, "lsq fp32/fp64"), CUPSO_ERR_CUDA;

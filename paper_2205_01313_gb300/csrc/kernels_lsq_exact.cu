@@ -12,7 +12,7 @@
 // product over all (row, particle) tiles at once -- each residual one chain
 // over d in one thread, as the order demands -- and lsq_sumsq_kernel then adds
 // a particle's squares in row order. The residuals pass through a workspace
-// R[m][i] of at most kExactWsBytes (half the L2), a chunk of rows (and of
+// R[m][i] of at most kExactWsBytes (half the L2; less where memory is short), a chunk of rows (and of
 // particles, for very large swarms) at a time; the running sums carry over from
 // chunk to chunk.
 //
@@ -26,6 +26,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "cupso_device.cuh"
@@ -37,6 +38,7 @@ namespace cupso {
 namespace {
 
 constexpr size_t kExactWsBytes = 64u << 20;   // residual workspace at most
+constexpr size_t kExactWsLeast = 1u << 20;    // and where memory is short
 constexpr int kResidThreads = 128;            // 16 x 8 threads of TM x TN residuals
 constexpr int kBk = 16;                       // dimensions per shared-memory stage
 constexpr int kTrimD = 64;                    // FP32: the trimmed inner loop up to here
@@ -133,8 +135,8 @@ __device__ __forceinline__ void st4g(double* p, const double* v) {
 // 30000 x 2 x 14 75 us an iteration with them, 22 without, 30000 x 2 x 300 343 and 116 (before
 // the split into tiles 26 and 183). In FP32 with more dimensions the second form of the
 // inner loop costs more than it saves (2048 x 500 x 2000 338 and 347 us for two iterations).
-// FUSED: all rows fit one tile, so the block adds its particles' squares itself and
-// writes f; no workspace, no second launch (M = 40: 12.0 -> 10.1 us per iteration of
+// FUSED: the block goes through all rows, tile by tile, adds its particles' squares itself and
+// writes f; no workspace, no second launch (M = 40, one tile: 12.0 -> 10.1 us per iteration of
 // a 256 x 16 swarm).
 template <typename T, int TM, int TN, bool FUSED, bool TRIM>
 __global__ void __launch_bounds__(kResidThreads, TM * TN == 128 ? 2 : TM * TN == 64 ? 3 : 1) lsq_resid_kernel(const float* __restrict__ x, int ldx, int D,
@@ -153,9 +155,9 @@ __global__ void __launch_bounds__(kResidThreads, TM * TN == 128 ? 2 : TM * TN ==
     // quarter of the warp then reads 2 rows' and 4 particles' vectors (8192 x 1024 x 4096:
     // 1572 us an iteration with 1 and 8, 1469 so)
     const int tx = (tid >> 1) & 7, ty = ((tid >> 4) << 1) | (tid & 1);
-    const int i0 = blockIdx.x * BN, mt = m0 + blockIdx.y * BM;
+    const int i0 = blockIdx.x * BN;
     const int arow = tid % BM, ak = (tid / BM) * AK;
-    const float* aptr = A + (size_t)min(mt + arow, m1 - 1) * (size_t)D;   // rows past m1 are computed, not stored
+    const float* aptr = A;
     float ar[AK];
     float4 xr[XV];
     auto fetch = [&](int k0, int st) {
@@ -195,76 +197,88 @@ __global__ void __launch_bounds__(kResidThreads, TM * TN == 128 ? 2 : TM * TN ==
             st4g(&Xs[st][e / (BN / 4)][4 * (e % (BN / 4))], v);
         }
     };
-    // the rows of a warp lie together, so that one past the last row need not multiply
-    const bool busy = mt + (tid >> 5) * 16 < m1;
     // the thread's rows ty * 4 + j (+ 64) and particles tx * 4 + j (+ 32, 64, 96)
     auto row_of = [&](int a) { return (a / 4) * (BM * 4 / TM) + ty * 4 + a % 4; };
     Acc<T, TM, TN> acc;
-#pragma unroll
-    for (int a = 0; a < TM; ++a) {
-        const int m = mt + row_of(a);
-        acc.set(a, m < m1 ? -(T)b[m] : (T)0);
-    }
-    fetch(0, 0);
-    stage(0);
-    __syncthreads();
     const int slices = (D + kBk - 1) / kBk;
-    for (int s = 0; s < slices; ++s) {
-        const int st = s & 1;
-        if (s + 1 < slices) fetch((s + 1) * kBk, st ^ 1);
-        auto multiply = [&](int k) {
-            T av[TM];
-            std::conditional_t<kF32, unsigned long long, T> xv[kF32 ? TN / 2 : TN];
+    // acc = the residuals of the tile at row mt
+    auto residuals = [&](int mt) {
+        aptr = A + (size_t)min(mt + arow, m1 - 1) * (size_t)D;   // rows past m1 are computed, not stored
+        // the rows of a warp lie together, so that one past the last row need not multiply
+        const bool busy = mt + (tid >> 5) * 16 < m1;
 #pragma unroll
-            for (int a = 0; a < TM; a += 4) ld4s(&As[st][k][(a / 4) * (BM * 4 / TM) + ty * 4], av + a);
-#pragma unroll
-            for (int c = 0; c < TN; c += 4) ld4s(&Xs[st][k][(c / 4) * (BN * 4 / TN) + tx * 4], xv + (kF32 ? c / 2 : c));
-            acc.step(av, xv);
-        };
-        const int kn = TRIM ? (busy ? min(kBk, D - s * kBk) : 0) : kBk;
-        if (kn == kBk) {
-#pragma unroll
-            for (int k = 0; k < kBk; ++k) multiply(k);
-        } else {
-#pragma unroll 2
-            for (int k = 0; k < kn; ++k) multiply(k);
+        for (int a = 0; a < TM; ++a) {
+            const int m = mt + row_of(a);
+            acc.set(a, m < m1 ? -(T)b[m] : (T)0);
         }
-        if (s + 1 < slices) stage(st ^ 1);   // the other stage: read last before the previous barrier
+        fetch(0, 0);
+        stage(0);
         __syncthreads();
-    }
+        for (int s = 0; s < slices; ++s) {
+            const int st = s & 1;
+            if (s + 1 < slices) fetch((s + 1) * kBk, st ^ 1);
+            auto multiply = [&](int k) {
+                T av[TM];
+                std::conditional_t<kF32, unsigned long long, T> xv[kF32 ? TN / 2 : TN];
+#pragma unroll
+                for (int a = 0; a < TM; a += 4) ld4s(&As[st][k][(a / 4) * (BM * 4 / TM) + ty * 4], av + a);
+#pragma unroll
+                for (int c = 0; c < TN; c += 4) ld4s(&Xs[st][k][(c / 4) * (BN * 4 / TN) + tx * 4], xv + (kF32 ? c / 2 : c));
+                acc.step(av, xv);
+            };
+            const int kn = TRIM ? (busy ? min(kBk, D - s * kBk) : 0) : kBk;
+            if (kn == kBk) {
+#pragma unroll
+                for (int k = 0; k < kBk; ++k) multiply(k);
+            } else {
+#pragma unroll 2
+                for (int k = 0; k < kn; ++k) multiply(k);
+            }
+            if (s + 1 < slices) stage(st ^ 1);   // the other stage: read last before the previous barrier
+            __syncthreads();
+        }
+    };
     if constexpr (FUSED) {
         __shared__ __align__(16) T Rs[BM][BN + 4];
+        T sum = (T)0;
+        for (int mt = m0; mt < m1; mt += BM) {
+            residuals(mt);   // with barriers between the last tile's sums and the next one's Rs
 #pragma unroll
-        for (int a = 0; a < TM; ++a)
+            for (int a = 0; a < TM; ++a)
 #pragma unroll
-            for (int c = 0; c < TN; ++c) Rs[row_of(a)][(c / 4) * (BN * 4 / TN) + tx * 4 + c % 4] = acc.get(a, c);
-        __syncthreads();
-        if (tid < BN && i0 + tid < N) {
-            T sum = (T)0;
+                for (int c = 0; c < TN; ++c) Rs[row_of(a)][(c / 4) * (BN * 4 / TN) + tx * 4 + c % 4] = acc.get(a, c);
+            __syncthreads();
+            if (tid < BN) {
+                const int rows = min(BM, m1 - mt);
 #pragma unroll 8
-            for (int m = 0; m < m1; ++m) {
-                const T r = Rs[m][tid];
-                if constexpr (sizeof(T) == 8) sum = __dadd_rn(sum, __dmul_rn(r, r));
-                else sum = __fmaf_rn(r, r, sum);
+                for (int m = 0; m < rows; ++m) {
+                    const T r = Rs[m][tid];
+                    if constexpr (sizeof(T) == 8) sum = __dadd_rn(sum, __dmul_rn(r, r));
+                    else sum = __fmaf_rn(r, r, sum);
+                }
             }
+        }
+        if (tid < BN && i0 + tid < N) {
             if constexpr (sizeof(T) == 8) f[i0 + tid] = __double2float_rn(sum);
             else f[i0 + tid] = sum;
         }
-        return;
-    }
+    } else {
+        const int mt = m0 + blockIdx.y * BM;
+        residuals(mt);
 #pragma unroll
-    for (int a = 0; a < TM; ++a) {
-        const int m = mt + row_of(a);
-        if (m >= m1) continue;
-        T* row = R + (size_t)(m - m0) * (size_t)ldr + i0;
+        for (int a = 0; a < TM; ++a) {
+            const int m = mt + row_of(a);
+            if (m >= m1) continue;
+            T* row = R + (size_t)(m - m0) * (size_t)ldr + i0;
 #pragma unroll
-        for (int c = 0; c < TN; c += 4) {
-            T v[4] = {acc.get(a, c), acc.get(a, c + 1), acc.get(a, c + 2), acc.get(a, c + 3)};
-            if constexpr (sizeof(T) == 8) {
+            for (int c = 0; c < TN; c += 4) {
+                T v[4] = {acc.get(a, c), acc.get(a, c + 1), acc.get(a, c + 2), acc.get(a, c + 3)};
+                if constexpr (sizeof(T) == 8) {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) v[e] = __dmul_rn(v[e], v[e]);
+                    for (int e = 0; e < 4; ++e) v[e] = __dmul_rn(v[e], v[e]);
+                }
+                st4g(row + (c / 4) * (BN * 4 / TN) + tx * 4, v);
             }
-            st4g(row + (c / 4) * (BN * 4 / TN) + tx * 4, v);
         }
     }
 }
@@ -354,20 +368,26 @@ size_t align256(size_t n) { return (n + 255) / 256 * 256; }
 struct ExactChunk {
     int particles, rows;
 };
-ExactChunk exact_chunk(int N, int M, size_t esz) {
+ExactChunk exact_chunk(int N, int M, size_t esz, size_t ws_most) {
     const long long Np = ((long long)N + 127) / 128 * 128;
-    const long long most = (long long)(kExactWsBytes / (esz * kRowTile));   // 131072 or 65536 particles
+    const long long most = (long long)(ws_most / (esz * kRowTile)) / 128 * 128;   // 131072 or 65536 particles of 64 MB
     const long long pc = std::min(Np, most);
     const long long all = ((long long)M + kRowTile - 1) / kRowTile * kRowTile;
-    const long long fit = (long long)(kExactWsBytes / ((size_t)pc * esz)) / kRowTile * kRowTile;
+    const long long fit = (long long)(ws_most / ((size_t)pc * esz)) / kRowTile * kRowTile;
     return ExactChunk{(int)pc, (int)std::min(all, fit)};
 }
+
+// The rows that one tile takes, so that the block adds its particles' squares itself: 64 of a small
+// tile, in FP32 128 of a large one. 300 x 24 x 100 11.0 us an iteration against 13.3, 8192 x 60 x
+// 128 17.0 and 19.2; with more dimensions 128 x 64 tiles and the second launch are faster, 8192 x
+// 256 x 128 38.9 and 36.3.
+bool one_tile(int M, int D, bool fp64) { return M <= 64 || (!fp64 && M <= 128 && D <= 128); }
 
 template <typename T, int TM, int TN, bool FUSED = false>
 void launch_resid(const float* x, int ldx, int Np, int D, const float* A, const float* b, int m0, int m1, T* R,
                   cudaStream_t st, int N = 0, float* f = nullptr) {
     const int vecA = D % 4 == 0 && (reinterpret_cast<uintptr_t>(A) & 15u) == 0;
-    const dim3 grid((unsigned)(Np / (8 * TN)), (unsigned)((m1 - m0 + 16 * TM - 1) / (16 * TM)));
+    const dim3 grid((unsigned)(Np / (8 * TN)), FUSED ? 1u : (unsigned)((m1 - m0 + 16 * TM - 1) / (16 * TM)));
     if (sizeof(T) == 8 || D <= kTrimD)
         lsq_resid_kernel<T, TM, TN, FUSED, true><<<grid, kResidThreads, 0, st>>>(x, ldx, D, A, b, m0, m1, R, Np, vecA, N, f);
     else
@@ -376,22 +396,16 @@ void launch_resid(const float* x, int ldx, int Np, int D, const float* A, const 
 
 template <typename T>
 cudaError_t exact_launch(const float* x, int ldx, int N, int D, const float* A, const float* b, int M, float* f,
-                         void* ws, int num_sms, cudaStream_t st) {
-    if (ldx % 128 != 0 || ldx < N || (reinterpret_cast<uintptr_t>(x) & 15u) != 0 || !ws) return cudaErrorInvalidValue;
-    if (M <= 64) {   // the rows of one small tile
-        launch_resid<T, 4, 4, true>(x, ldx, (N + 127) / 128 * 128, D, A, b, 0, M, nullptr, st, N, f);
+                         void* ws, size_t ws_most, int num_sms, cudaStream_t st) {
+    if (ldx % 128 != 0 || ldx < N || (reinterpret_cast<uintptr_t>(x) & 15u) != 0) return cudaErrorInvalidValue;
+    const bool one = one_tile(M, D, sizeof(T) == 8);
+    if (one || !ws) {
+        if (M <= 64 || !one || sizeof(T) == 8) launch_resid<T, 4, 4, true>(x, ldx, (N + 127) / 128 * 128, D, A, b, 0, M, nullptr, st, N, f);
+        else if constexpr (sizeof(T) == 4)
+            launch_resid<T, 8, 4, true>(x, ldx, (N + 127) / 128 * 128, D, A, b, 0, M, nullptr, st, N, f);
         return cudaGetLastError();
     }
-    if constexpr (sizeof(T) == 4) {
-        // of one large one: 300 x 24 x 100 11.0 us an iteration against 13.3, 8192 x 60 x 128 17.0 and
-        // 19.2; with more dimensions 128 x 64 tiles and the second launch are faster, 8192 x 256 x
-        // 128 38.9 and 36.3
-        if (M <= 128 && D <= 128) {
-            launch_resid<T, 8, 4, true>(x, ldx, (N + 127) / 128 * 128, D, A, b, 0, M, nullptr, st, N, f);
-            return cudaGetLastError();
-        }
-    }
-    const ExactChunk ch = exact_chunk(N, M, sizeof(T));
+    const ExactChunk ch = exact_chunk(N, M, sizeof(T), ws_most);
     T* carry = static_cast<T*>(ws);
     T* R = reinterpret_cast<T*>(static_cast<char*>(ws) + align256(sizeof(T) * (size_t)ch.particles));
     for (int p0 = 0; p0 < N; p0 += ch.particles) {
@@ -426,18 +440,54 @@ cudaError_t exact_launch(const float* x, int ldx, int N, int D, const float* A, 
     return cudaSuccess;
 }
 
+// Whether the kernel that goes through all rows in the block (FUSED) is used for its own sake
+// where the rows need more than a tile.
+//  * `once` (an evaluation): it needs no workspace, and an allocation of more than a megabyte
+//    costs about 110 us, most of it once `front` is that large anyway, where small ones come out
+//    of memory the process has mapped (3000 x 8 x 500 37 us in the old kernel, 163 with a
+//    workspace, 32 so). It loses the SMs that blocks of 32 particles leave idle, and in FP32 the
+//    rate of larger tiles: estimated, in us, from 0.4 (FP32; 9.3 FP64) a slice and tile and 0.9 (6)
+//    for a tile's sums; sweep over N 64 .. 100000, D 2 .. 1000, M 65 .. 4000.
+//  * in a swarm's iterations: with few dimensions and many particles the residuals' way through
+//    memory is longer than their product (an iteration of 100000 x 30 x 300 117 us with a
+//    workspace, 110 in the old kernel, 92 so; 100000 x 2 x 4000 about 700 and 410).
+bool fused_anyway(int N, int D, int M, bool fp64, bool once, size_t front, size_t ws, int num_sms) {
+    const double share = (N + 31) / 32 / (double)num_sms;   // blocks per SM
+    if (!once) return !fp64 && (D <= 16 ? share >= 2.0 : D <= 32 && share >= 12.0);
+    const double tiles = (M + 63) / 64, slices = D / 16.0;
+    const double idle = std::ceil(share) - share, short_of = std::max(0.0, 1.0 - share);
+    const double loss = fp64 ? tiles * (9.3 * slices + 6.0) * idle
+                             : tiles * ((0.4 * slices + 0.9) * short_of + 0.15 * slices * share);
+    constexpr size_t kSmall = 1u << 20;
+    return loss <= (front > kSmall ? 40.0 : front + ws > kSmall ? 110.0 : 3.0);
+}
+
 }  // namespace
 
-size_t lsq_exact_ws_bytes(int N, int M, bool fp64) {
+cudaError_t lsq_exact_alloc(void** p, size_t front, int N, int D, int M, bool fp64, bool once, int num_sms, void** ws,
+                            size_t* ws_most) {
     const size_t esz = fp64 ? 8 : 4;
-    const ExactChunk ch = exact_chunk(N, M, esz);
-    return align256(esz * (size_t)ch.particles) + esz * (size_t)ch.particles * (size_t)ch.rows;
+    *ws = nullptr;
+    *ws_most = 0;
+    for (size_t most = one_tile(M, D, fp64) ? 0 : kExactWsBytes; most >= kExactWsLeast; most /= 4) {
+        const ExactChunk ch = exact_chunk(N, M, esz, most);
+        const size_t bytes = align256(esz * (size_t)ch.particles) + esz * (size_t)ch.particles * (size_t)ch.rows;
+        if (fused_anyway(N, D, M, fp64, once, front, bytes, num_sms)) break;
+        const cudaError_t e = cudaMalloc(p, front + bytes);
+        if (e == cudaSuccess) {
+            *ws = static_cast<char*>(*p) + front;
+            *ws_most = most;
+        }
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();
+    }
+    return cudaMalloc(p, front);
 }
 
 cudaError_t lsq_exact_launch(const float* x, int ldx, int N, int D, const float* A, const float* b, int M, bool fp64,
-                             float* f, void* ws, int num_sms, cudaStream_t st) {
-    return fp64 ? exact_launch<double>(x, ldx, N, D, A, b, M, f, ws, num_sms, st)
-                : exact_launch<float>(x, ldx, N, D, A, b, M, f, ws, num_sms, st);
+                             float* f, void* ws, size_t ws_most, int num_sms, cudaStream_t st) {
+    return fp64 ? exact_launch<double>(x, ldx, N, D, A, b, M, f, ws, ws_most, num_sms, st)
+                : exact_launch<float>(x, ldx, N, D, A, b, M, f, ws, ws_most, num_sms, st);
 }
 
 }  // namespace cupso

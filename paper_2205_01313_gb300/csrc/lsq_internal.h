@@ -69,10 +69,13 @@ int lsq_eval_tc_partials(LsqTcState* st, cudaStream_t stream);
 
 // The exact fitness (kernels_lsq_exact.cu): f[i] of X(i, d) = x[d * ldx + i],
 // i < N, in the reference order, FP32 or FP64 rounded to float. x 16-byte
-// aligned, ldx a multiple of 128; ws: lsq_exact_ws_bytes device bytes.
-size_t lsq_exact_ws_bytes(int N, int M, bool fp64);
+// aligned, ldx a multiple of 128. lsq_exact_alloc: *p = `front` device bytes and behind them the
+// residual workspace *ws, 64 MB at most (*ws_most), less where memory is short; null where the
+// rows need none, or where one evaluation (`once`) or the swarm is faster without.
+cudaError_t lsq_exact_alloc(void** p, size_t front, int N, int D, int M, bool fp64, bool once, int num_sms, void** ws,
+                            size_t* ws_most);
 cudaError_t lsq_exact_launch(const float* x, int ldx, int N, int D, const float* A, const float* b, int M, bool fp64,
-                             float* f, void* ws, int num_sms, cudaStream_t st);
+                             float* f, void* ws, size_t ws_most, int num_sms, cudaStream_t st);
 
 // Least-squares swarm iteration (kernels_lsq_swarm.cu); all read t from t_dev.
 cudaError_t lsq_launch_move(const SwarmDev& s, int grid, cudaStream_t st);
