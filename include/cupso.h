@@ -167,9 +167,11 @@ typedef enum {
     CUPSO_SYNC_KERNEL_PIPELINED3 = 2, /* rows staged through shared memory, 2 pairs ahead   */
     CUPSO_SYNC_KERNEL_PIPELINED4 = 3, /* the same, 3 pairs ahead                            */
     CUPSO_SYNC_KERNEL_TILED = 4,      /* a tile of particles with all their dimensions per block,
-                                         the (dimension pair, particle) items spread over threads;
-                                         AUTO uses it for D >= 8, D % 8 != 0 up to 400 particles per SM
-                                         (330 for D > 128; Rosenbrock 330, and 224 for D > 64)   */
+                                         the (dimension pair, particle) items spread over threads.
+                                         AUTO uses it for D >= 8: with D % 8 != 0 (or D = 8, too few
+                                         for panels) up to 780 particles per SM for D <= 16, 680 to 64,
+                                         560 to 128 and 330 above (Rosenbrock 560 to 32, 390 to 64 and
+                                         224 above), with D % 8 == 0 below 2^17 particle-dimensions */
     CUPSO_SYNC_KERNEL_PANEL8 = 5,     /* the state in panels of 8 dimensions (each particle's 8 values
                                          of a panel contiguous), two threads per particle, rows staged
                                          through shared memory; D % 8 == 0, D >= 16. A particle whose

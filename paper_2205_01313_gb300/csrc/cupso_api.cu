@@ -140,11 +140,11 @@ int resolved_mode(const cupso_swarm* h) {
 // Particles per tile when the tiled SYNC kernel runs, else 0. AUTO takes it
 // for D >= 8 up to the crossover measured on a GB300 against the pipelined
 // kernel (which runs over d inside each thread and needs many particles per
-// SM to hide its row latency), tiled and pipelined in us per iteration: sphere 50000 x
-// 63 19.3 and 23.3, 100000 x 15 12.1 and 11.9, 60000 x 99 30.5 and 33.7, 80000 x 99 42.4 and
-// 42.2, 50000 x 150 46.4 and 48.0, 60000 x 201 76 and 64; Rosenbrock, whose terms need the
-// next dimension's value too, 50000 x 33 14.5 and 15.4, 60000 x 65 28.9 and 25.2, 35000 x
-// 201 54 and 53.
+// SM to hide its row latency), tiled and pipelined in us per iteration from captured graphs and,
+// where the pipelined one costs about 2 us more and the tiled one 1, from launches one by one:
+// sphere 93703 x 30 17.4 and 17.1, 16.6 and 17.5; 110000 x 12 10.7 and 10.2, 11.0 and 12.3; 80000 x
+// 80 32.7 and 34.4, 33.1 and 36.8; 60000 x 201 75 and 64. Rosenbrock, whose terms need the next
+// dimension's value too, 80000 x 30 18.7 and 17.4, 18.0 and 18.6; 60000 x 63 26.6 and 25.5, 27 and 28.
 int sync_tile(const cupso_swarm* h) {
     if (h->fp64) return 0;
     if (h->sync_kernel == CUPSO_SYNC_KERNEL_TILED) return tiled_particles(h->N, h->D, h->num_sms);
@@ -157,7 +157,9 @@ int sync_tile(const cupso_swarm* h) {
         const long long pd = (long long)h->N * h->D;
         return pd < (1ll << 17) ? tiled_particles(h->N, h->D, h->num_sms) : 0;
     }
-    const long long per_sm = h->fid == CUPSO_ROSENBROCK ? (h->D <= 64 ? 330 : 224) : (h->D <= 128 ? 400 : 330);
+    const int D = h->D;
+    const long long per_sm = h->fid == CUPSO_ROSENBROCK ? (D <= 32 ? 560 : D <= 64 ? 390 : 224)
+                                                        : (D <= 16 ? 780 : D <= 64 ? 680 : D <= 128 ? 560 : 330);
     if ((long long)h->N > per_sm * h->num_sms) return 0;
     return tiled_particles(h->N, h->D, h->num_sms);
 }
