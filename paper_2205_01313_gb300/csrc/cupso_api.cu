@@ -258,6 +258,9 @@ int sync_grid(const cupso_swarm* h) {
         // persistent: warps pull units of 32 * ppt particles from a counter
         const int ppt = sync_ppt(h);
         const int units = h->Np / (32 * ppt);
+        // of a few dozen units the CTAs' last one waits for the fewer, the better: 846 x 5 8.2 us
+        // in 28 CTAs and 6.2 in 4
+        if (3 * units <= h->num_sms && h->grid_override == 0) return (units + kBlock / 32 - 1) / (kBlock / 32);
         return even_grid(h, units, pipelined_blocks_per_sm(stages, h->fid, h->D, ppt));
     }
     const int ntiles = tiles_of(h->Np);

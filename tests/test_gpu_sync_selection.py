@@ -31,3 +31,21 @@ def test_tiled_up_to_its_line(fid, D, per_sm):
         np.testing.assert_array_equal(g0[3], g1[3])
         for name in ("pos", "v", "pbest_pos", "pbest_fit"):
             assert s0[name].tobytes() == s1[name].tobytes(), name
+
+
+@pytest.mark.parametrize("N,ctas", [(100, 1), (846, 4), (1536, 6), (1537, 52), (3000, 96)])
+def test_few_units_in_few_ctas(N, ctas):
+    """Pipelined single steps of a few dozen units of 32 particles: whole CTAs, and the register kernel's bits."""
+    P = load_cupso()
+    runs = []
+    for kernel in ("auto", "register"):
+        with P.Swarm(5, N, BOUNDS[1], W, C12, C12, 1, 7, mode="sync") as s:
+            s.set_option(P.CUPSO_OPT_ITERS_PER_LAUNCH, 1)
+            s.set_option(P.CUPSO_OPT_SYNC_KERNEL, P.SYNC_KERNELS[kernel])
+            assert kernel != "auto" or s.info()["sync_grid"] == ctas
+            s.step(5)
+            runs.append((s.gbest(), s.state()))
+    (g0, s0), (g1, s1) = runs
+    assert g0[:3] == g1[:3]
+    for name in ("pos", "v", "pbest_pos", "pbest_fit"):
+        assert s0[name].tobytes() == s1[name].tobytes(), name
