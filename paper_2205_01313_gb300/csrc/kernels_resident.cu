@@ -375,10 +375,16 @@ struct ResPlan {
     size_t smem = 0;
 };
 
-// P = N over the SMs; the fewest pairs per thread whose threads fit, and no more
-// rows of threads than those pairs need.
+// P = N over the SMs, and of small swarms up to 128 (pair, particle) items, over at least 8 CTAs: more
+// CTAs are no faster for one swarm (an iteration of 300 x 8 1.08 us in 150 CTAs, 0.78 in 10; 1000 x 2 1.03
+// and 1.04), and cooperative launches of 150 CTAs hold up one another, so that swarms stepped on
+// streams of their own no longer ran side by side (32 of 1000 x 2: 0.33 us per swarm and
+// iteration, 0.10 on clusters, now 0.05; of 1024 x 16 0.16, 0.13 and 0.12). Then the fewest pairs
+// per thread whose threads fit, and no more rows of threads than those pairs need.
 bool res_plan(int N, int D, int num_sms, ResPlan* r) {
-    const int P = (N + num_sms - 1) / num_sms, pairs = (D + 1) / 2;
+    const int pairs = (D + 1) / 2;
+    const int small = std::min((N + 7) / 8, 128 / pairs);
+    const int P = std::max((N + num_sms - 1) / num_sms, small);
     for (int items : kResItems) {
         const int rows = (pairs + items - 1) / items;
         const long long threads = ((long long)P * rows + 31) / 32 * 32;
