@@ -121,7 +121,10 @@ typedef enum {
 typedef enum {
     CUPSO_OPT_MODE = 1,           /* value: cupso_mode                                         */
     CUPSO_OPT_GRAPH_CHUNK = 2,    /* iterations per captured CUDA graph (SYNC/TREE); 0 = none  */
-    CUPSO_OPT_WAIT_LIMIT_NS = 3,  /* bound of every device-side wait (default 2e9 ns)          */
+    CUPSO_OPT_WAIT_LIMIT_NS = 3,  /* bound of every device-side wait (default 2e9 ns). Below 1e6 ns + 1 ns
+                                     per 8 particle-dimensions, which an iteration itself might take,
+                                     SYNC and AUTO keep to kernels without waits between CTAs, panels
+                                     excepted                                                  */
     CUPSO_OPT_CLEAR_STATUS = 4,   /* any value: clear the sticky device status                 */
     CUPSO_OPT_GRID = 5,           /* CTAs of the persistent kernels (SYNC/ASYNC); 0 = automatic */
     CUPSO_OPT_SYNC_KERNEL = 6,    /* value: cupso_sync_kernel (which SYNC kernel runs)         */

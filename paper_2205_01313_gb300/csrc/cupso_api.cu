@@ -274,6 +274,13 @@ int panel_iters_per_launch(const cupso_swarm* h) {
     return h->iters_per_launch > 0 ? h->iters_per_launch : kPanelMaxIters;
 }
 
+// Whether an iteration of a swarm that waits for all CTAs ends well within the wait limit: a
+// millisecond, and 0.12 ns per particle-dimension (double precision in memory takes 0.02).
+// A shorter limit is meant for other waits; the kernels of single iterations have none.
+bool limit_ample(const cupso_swarm* h) {
+    return h->dev.wait_limit_ns >= 1000000ll + (long long)h->N * h->D / 8;
+}
+
 // The iterations of a call from which they run in the resident kernel
 // (kernels_resident.cu), 0: never. Synchronous swarm, AUTO kernel choice, default grid,
 // several iterations per launch allowed.
@@ -288,7 +295,8 @@ int panel_iters_per_launch(const cupso_swarm* h) {
 //    iterations 4.0 against 6.7 us, 1000 x 2 3.1 against 2.8; 300 x 8 (Rosenbrock)
 //    at 100 1.95 against 1.68, at 1000 1.51 against 1.58.
 int resident_from(const cupso_swarm* h, int mode) {
-    if (!h->rbufs.slots || h->sync_kernel != CUPSO_SYNC_KERNEL_AUTO || h->grid_override != 0 || h->iters_per_launch == 1)
+    if (!h->rbufs.slots || h->sync_kernel != CUPSO_SYNC_KERNEL_AUTO || h->grid_override != 0 || h->iters_per_launch == 1 ||
+        !limit_ample(h))
         return 0;
     if (mode == CUPSO_MODE_SYNC) return h->panel ? 4 : 3;
     if (mode != CUPSO_MODE_ONCHIP || h->mode != CUPSO_MODE_AUTO) return 0;
@@ -305,7 +313,7 @@ int resident_from(const cupso_swarm* h, int mode) {
 int sync64_from(const cupso_swarm* h, int mode) {
     if (!h->s64bufs.slots) return 0;
     if (mode == CUPSO_MODE_PERSISTENT) return 1;
-    if (h->iters_per_launch == 1) return 0;
+    if (h->iters_per_launch == 1 || !limit_ample(h)) return 0;
     const long long pd = (long long)h->N * h->D;
     if (mode == CUPSO_MODE_SYNC) return pd >= (1 << 18) ? 5 : 3;
     return mode == CUPSO_MODE_ONCHIP && h->mode == CUPSO_MODE_AUTO ? (pd >= 2000 ? 10 : 50) : 0;
