@@ -1206,15 +1206,25 @@ int cupso_step(cupso_handle h, int iters) {
     }
     const int mode = resolved_mode(h);
     const int from = one_launch_from(h, mode);
-    const bool one_launch = from > 0 && iters >= from;
+    bool one_launch = from > 0 && iters >= from;
+    // A stream that may use only some of the SMs (a green context's) refuses a launch whose CTAs
+    // would not all be resident: the call then runs as a shorter one would.
+    auto refused = [&](cudaError_t e) {
+        if (e != cudaErrorCooperativeLaunchTooLarge || mode == CUPSO_MODE_PERSISTENT) return false;
+        cudaGetLastError();
+        one_launch = false;
+        return true;
+    };
     if (h->fp64 && one_launch) {
         // PERSISTENT: one launch by definition
         const int most = mode != CUPSO_MODE_PERSISTENT && h->iters_per_launch > 0 ? h->iters_per_launch : kSync64MaxIters;
         const cudaError_t e = launch_sync64(h->dev64, h->s64bufs, h->fid, iters, most, h->stall_barrier != 0, h->num_sms,
                                             h->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "one-launch step");
-        h->t_host += (uint32_t)iters;
-        return CUPSO_OK;
+        if (e != cudaSuccess && !refused(e)) return cuda_fail(e, "one-launch step");
+        if (e == cudaSuccess) {
+            h->t_host += (uint32_t)iters;
+            return CUPSO_OK;
+        }
     }
     if (h->fp64 && mode == CUPSO_MODE_ONCHIP) {
         cudaError_t e = launch_onchip64(h->dev64, h->fid, iters, h->stream);
@@ -1222,19 +1232,21 @@ int cupso_step(cupso_handle h, int iters) {
         h->t_host += (uint32_t)iters;
         return CUPSO_OK;
     }
-    if (one_launch) {
+    if (!h->fp64 && one_launch) {
         // any layout, pending pbest rows included; a launch's iterations as for the panel step
         const int most = h->iters_per_launch > 0 ? h->iters_per_launch : kResidentMaxIters;
-        for (int left = iters; left > 0;) {
+        for (int left = iters; one_launch && left > 0;) {
             const int n = std::min(left, most);
             const cudaError_t e = launch_resident(h->dev, h->rbufs, h->fid, h->panel, n, h->stall_barrier != 0, h->num_sms,
                                                   h->stream);
-            if (e != cudaSuccess) return cuda_fail(e, "resident launch");
+            if (e != cudaSuccess && (left < iters || !refused(e))) return cuda_fail(e, "resident launch");
             left -= n;
         }
-        h->lazy_pending = false;
-        h->t_host += (uint32_t)iters;
-        return CUPSO_OK;
+        if (one_launch) {
+            h->lazy_pending = false;
+            h->t_host += (uint32_t)iters;
+            return CUPSO_OK;
+        }
     }
     const int panel = (!h->fp64 && mode == CUPSO_MODE_SYNC) ? panel_cfg(h).width : 0;
     {
