@@ -166,11 +166,12 @@ __device__ __forceinline__ void move_b(float& x, float& v, float pb, float g, ui
 
 // Publishes a unit's candidate (below K) and counts the unit. The warp that completes
 // the swarm sets gbest_pos of parity nxt: from the winner's pos, which is its
-// pbest_pos, as it improved in this iteration -- its lane has fenced its row before the
-// unit was counted --, or from the other parity's where no key below K came.
-__device__ __forceinline__ void close_unit(const BatchSwarm& w, unsigned long long best, bool lane_cand, bool any_nan,
+// pbest_pos, as it improved in this iteration, or from the other parity's where no key below K
+// came. The winner's row is visible then: both lanes that own it have stored it before
+// the __syncwarp, and lane 0 fences after that and before it counts the unit, as it does for
+// every unit with a candidate; the completing warp's lane 0 fences after its count.
+__device__ __forceinline__ void close_unit(const BatchSwarm& w, unsigned long long best, bool any_nan,
                                            unsigned long long K, int cur, int nxt, int lane_id) {
-    if (lane_cand) __threadfence();
     __syncwarp();
     int last = 0;
     if (lane_id == 0) {
@@ -286,9 +287,8 @@ __device__ __forceinline__ void run_unit(const BatchDev& b, unsigned* work, floa
         }
         if (fl_new != (uint32_t)me.pending) w.pflag[i] = (unsigned char)fl_new;
     }
-    const bool lane_cand = best != kKeyNone;
     best = warp_min_u64(best);
-    close_unit(w, best, lane_cand, __any_sync(0xFFFFFFFFu, nan), K, cur, nxt, lane_id);
+    close_unit(w, best, __any_sync(0xFFFFFFFFu, nan), K, cur, nxt, lane_id);
 }
 
 // Step 1 of one unit: the single-swarm init kernel's arithmetic, every key competing.
@@ -330,9 +330,8 @@ __device__ __forceinline__ void init_unit(const BatchSwarm& wg, uint32_t u, int 
         }
     }
     best = warp_min_u64(best);
-    // every particle competes, so every lane's rows may be the ones gathered; t = 0
-    // lives in slot 0, and slot 1 gets the same key
-    close_unit(w, best, true, __any_sync(0xFFFFFFFFu, nan), kKeyNone, 1, 0, lane_id);
+    // every particle competes; t = 0 lives in slot 0, and slot 1 gets the same key
+    close_unit(w, best, __any_sync(0xFFFFFFFFu, nan), kKeyNone, 1, 0, lane_id);
 }
 
 }  // namespace
