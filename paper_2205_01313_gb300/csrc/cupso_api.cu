@@ -668,7 +668,6 @@ int create_swarm(int D, int N, const cupso_bounds* b, float w, float c1, float c
 
     int cl = 0, per = 0;
     h->onchip_cluster = (fid != CUPSO_LSQ && onchip_fits(N, D, &cl, &per)) ? cl : 0;
-    const bool fast = s.fast_cr && s.fast_clamp;
     h->pipelined_ok = prepare_pipelined(fid, fast_form(s, fid)) == cudaSuccess;
     h->panel_ok = fid != CUPSO_LSQ && panel_supported(8, 3, D) && prepare_panel(fid, fast_form(s, fid)) == cudaSuccess;
     cudaGetLastError();

@@ -359,7 +359,6 @@ extern "C" int cupso_solve_batch(int n_swarms, const cupso_problem* problems, in
             w.swarm = p.swarm_id;
             set_constants(w);
         }
-        if (rc != CUPSO_OK) break;
 
         // Hand-out order: swarms that run the same code (fitness function and
         // arithmetic path) together, so that the warps of an SM share their

@@ -269,9 +269,11 @@ __global__ void __launch_bounds__(max_threads(ITEMS), 1) resident_kernel(const _
             }
             if (tid == 0) {
                 // With a candidate the arrival releases its slot and key (written before the barrier
-                // above). Without one the CTA has written nothing, and its reads of the last slots were
-                // done before the barriers of this iteration: nothing to order, and a release would
-                // wait about 0.3 us.
+                // above). Without one the CTA has written nothing that others read, and a release
+                // would wait about 0.3 us. That its reads of the last slots come before another
+                // CTA's next writes of them, two iterations on, does not follow from a relaxed
+                // arrival in the memory model; it holds because the loads have returned (their
+                // values are in Gs) before the barriers of this iteration.
                 if (cand != kKeyNone) {
                     atomicMax(rb.key + par, ~cand);
                     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(rb.bar),

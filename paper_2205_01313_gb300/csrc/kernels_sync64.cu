@@ -79,7 +79,9 @@ __device__ __forceinline__ PKey* slot_of(const Sync64Bufs& rb, int par, uint32_t
 
 // One arrival; `cand`: it carries a candidate of this parity, whose slot was written
 // by threads that have passed a barrier with the caller since. `first`: the launch's first, which
-// releases the cleared slots.
+// releases the cleared slots. A relaxed one does not order this CTA's reads of older slots
+// before other CTAs' next writes of them in the memory model; that holds because the loads
+// have returned, their values stored, before the CTA's barriers since.
 __device__ __forceinline__ void arrive64(const Sync64Bufs& rb, int par, bool cand, bool first) {
     if (cand || first)
         asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(rb.bar),
