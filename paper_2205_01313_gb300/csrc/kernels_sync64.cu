@@ -492,11 +492,15 @@ struct Plan64 {
 };
 
 bool plan64(int fid, int N, int D, int num_sms, Plan64* r) {
-    // the particles spread over the SMs, but of small swarms up to 64 (dimension, particle) items to a
-    // CTA, over at least 8 CTAs: one swarm is as fast or faster (an iteration of 300 x 2 1.97 and 1.53 us,
-    // 2000 x 1 1.62 both, 8192 x 1 1.66 and 1.57), and many on streams of their own run side by
-    // side (64 of 2000 x 1: 0.20 us per swarm and iteration, 0.09 on clusters, now 0.10)
-    const int PC = std::max((N + num_sms - 1) / num_sms, std::min((N + 7) / 8, 64 / D));
+    // The particles spread over the SMs, but of small swarms up to 64 (dimension, particle) items to a
+    // CTA, over at least 8 CTAs: one swarm is as fast or faster (an iteration of 300 x 2 1.53 and 1.09 us,
+    // 8192 x 1 1.56 and 1.49), and many on streams of their own run side by side (64 of 2000 x 1: 0.24 us
+    // per swarm and iteration, 0.09 on clusters, now 0.09). In one dimension whole warps instead, where a
+    // part of one or a second one costs more than CTAs save: 32 particles to 32 CTAs, then 64 (128 x 1
+    // 1.48 us with a CTA each, 1.52 with 16 to a CTA, 1.22-1.43 so; 1024 x 1 1.48, 1.49 with 64, 1.42; 2048 x 1
+    // 1.48, 1.50 so, and with 32 1.41 but 64 of them 0.17).
+    const int small = D == 1 ? std::min(std::max((N + 31) / 32, 32), 64) : std::min((N + 7) / 8, 64 / D);
+    const int PC = std::max((N + num_sms - 1) / num_sms, small);
     r->PC = PC;
     r->grid = (N + PC - 1) / PC;
     for (int items = 1; items <= 16; items *= 2) {

@@ -44,3 +44,23 @@ def test_small_swarms_fp64(N, D):
             assert st[name].tobytes() == np.ascontiguousarray(getattr(ref, name)).tobytes(), (fid, name)
         assert idx == ref.gbest_idx and fit == ref.gbest_fit
         np.testing.assert_array_equal(pos, ref.gbest_pos)
+
+
+@pytest.mark.parametrize("mode", ["sync", "persistent"])
+@pytest.mark.parametrize("N", [1, 31, 32, 33, 64, 1023, 1024, 1025, 1056, 2047, 2048, 2049])
+def test_one_dimension_fp64_in_whole_warps(N, mode):
+    """32 particles to a CTA up to 1024, then up to 64."""
+    P = load_cupso()
+    box = (-100.0, 100.0, 100.0)
+    with P.Swarm(1, N, box, 1.0, 2.0, 2.0, 4, 5, mode=mode, dtype="f64") as s:
+        s.step(9)
+        s.step(4)
+        st = s.state()
+        _, fit, idx, pos = s.gbest()
+    ref = O.Swarm64(N, 1, *box, 1.0, 2.0, 2.0, 4, 5)
+    ref.init()
+    ref.step_sync(13)
+    for name in ("pos", "v", "pbest_pos", "pbest_fit"):
+        assert st[name].tobytes() == np.ascontiguousarray(getattr(ref, name)).tobytes(), name
+    assert idx == ref.gbest_idx and fit == ref.gbest_fit
+    np.testing.assert_array_equal(pos, ref.gbest_pos)
