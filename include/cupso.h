@@ -105,7 +105,10 @@ typedef enum {
     CUPSO_MODE_TREE = 2,   /* parallel-reduction baseline: two kernels per iteration (Sec. 2.2) */
     CUPSO_MODE_TREE_UNROLLED = 3, /* the same with the unrolled reduction (Sec. 2.2)       */
     CUPSO_MODE_ASYNC = 4,  /* persistent CTAs, no grid barrier, lock-protected gbest (Sec. 3.2) */
-    CUPSO_MODE_ONCHIP = 5, /* whole swarm in one CTA cluster's shared memory, many iterations per launch */
+    CUPSO_MODE_ONCHIP = 5, /* whole swarm in one CTA cluster's shared memory, many iterations per launch;
+                              for many swarms stepped side by side on streams of their own (from about 32
+                              of 1024 x 32 on) faster than AUTO's one launch over all SMs, as is
+                              cupso_solve_batch                                              */
     CUPSO_MODE_QUEUE = 6,  /* the paper's queue design (Alg. 2): one particle per thread, a
                               shared-memory queue of the particles that beat gbest, a second kernel */
     CUPSO_MODE_QUEUE_LOCK = 7, /* the paper's queue-lock design (Alg. 3): the queue, then thread 0 of
@@ -256,7 +259,9 @@ CUPSO_API int cupso_gbest_wait(cupso_handle h, int slot, float* fit_out, float* 
 
 /* Wait, then copy the swarm state to host arrays in particle-major layout:
  * pos, v, pbest_pos are [N][D] (element i*D + d), pbest_fit is [N]; *t_out =
- * iterations completed. Any pointer may be NULL. */
+ * iterations completed. Any pointer may be NULL. The first call that needs one
+ * allocates a device buffer of at most 32 MB, which the handle keeps; without
+ * the memory for it the state goes through host memory, slower. */
 CUPSO_API int cupso_get_state(cupso_handle h, float* pos, float* v, float* pbest_pos, float* pbest_fit,
                     uint32_t* t_out);
 
@@ -264,7 +269,7 @@ CUPSO_API int cupso_get_state(cupso_handle h, float* pos, float* v, float* pbest
  * and set the iteration counter to t; gbest is recomputed on the device as
  * the lowest-index argmin of pbest_fit. Waits for the upload. Together with
  * cupso_get_state this is checkpoint and resume: the random draws depend only
- * on (seed, swarm, t, particle, dimension). */
+ * on (seed, swarm, t, particle, dimension). Device memory as there. */
 CUPSO_API int cupso_set_state(cupso_handle h, const float* pos, const float* v, const float* pbest_pos,
                     const float* pbest_fit, uint32_t t);
 
@@ -305,11 +310,15 @@ CUPSO_API int cupso_get_gbest_f64(cupso_handle h, double* fit_out);
  * words 0,1 give r1 (pos0 at t = 0) and words 2,3 give r2 (v0), each as
  * (m + 1) 2^-53 with m = w_hi 2^21 + (w_lo >> 11). fitness_id: CUPSO_SPHERE,
  * CUPSO_ROSENBROCK or CUPSO_CUBIC_MAX (others: CUPSO_ERR_UNSUPPORTED). Modes:
- * SYNC (one fused launch per iteration: block argmin, a candidate list, the
- * last block gathers gbest), TREE, TREE_UNROLLED, QUEUE, QUEUE_LOCK (the
- * paper's four designs, one particle per thread), ONCHIP (one CTA holds the
- * swarm in shared memory; only when it fits), PERSISTENT (one cooperative
- * launch per cupso_step call); AUTO picks ONCHIP when it fits, else SYNC.
+ * SYNC (a call of 3 iterations or more, 5 from 2^18 particle-dimensions, in
+ * one cooperative launch, the swarm in registers or dealt evenly to the SMs;
+ * a shorter one a fused launch per iteration: block argmin, a candidate list,
+ * the last block gathers gbest), TREE, TREE_UNROLLED, QUEUE, QUEUE_LOCK (the
+ * paper's four designs, one particle per thread), ONCHIP (a cluster of up to
+ * 16 CTAs holds the swarm in shared memory; only when it fits), PERSISTENT
+ * (one cooperative launch per cupso_step call of any length); AUTO picks
+ * ONCHIP when it fits (SYNC's one launch for a call of 10 iterations or more,
+ * 50 below 2000 particle-dimensions), else SYNC.
  * ASYNC is not available. Use cupso_step, cupso_set_option,
  * cupso_get_info and cupso_destroy as for any handle, and the _fp64 accessors
  * below: the float accessors return CUPSO_ERR_UNSUPPORTED on such a handle. */
@@ -351,8 +360,9 @@ typedef struct {
  * swarm's result equals what cupso_create with seed and swarm_id, then
  * cupso_step(iters), would give. Returns CUPSO_OK if every swarm succeeded,
  * else the first failing status; results[k].status holds each swarm's.
- * Every iteration of all swarms is one launch; the kernel and launch shape
- * are tuned on the first iterations (the environment variable
+ * Every iteration of all swarms is one launch, or two side by side where some
+ * of the swarms are kept in panels of 8 dimensions and others are not; the
+ * kernel and launch shape are tuned on the first iterations (the environment variable
  * CUPSO_BATCH_KERNEL=tiled or =streaming fixes the kernel instead).
  * CUPSO_ERR_INVALID_ARG (before any device work) for a bad argument in any
  * problem, and for CUPSO_LSQ, which needs the matrices of cupso_set_lsq. */
@@ -415,7 +425,8 @@ CUPSO_API int cupso_tree_step_noalloc(int D, int N, const cupso_bounds* bounds, 
  * once to float at the end; BF16 and FP8 form X A^T on the tensor cores from
  * the positions themselves (the fitness of the dense-fitness extension of the
  * method; the paper's own fitness is analytic, Sec. 5.1). Allocates temporary
- * device memory, queues on `cuda_stream` and waits. */
+ * device memory (BF16 and FP8: the operands; FP32 and FP64: where it pays, up to
+ * 64 MB for residuals), queues on `cuda_stream` and waits. */
 CUPSO_API int cupso_lsq_eval(const float* A_dev, const float* b_dev, int M, int D, const float* X_dev, int N,
                              int precision, float* f_out_dev, void* cuda_stream);
 

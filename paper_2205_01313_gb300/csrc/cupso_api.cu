@@ -293,7 +293,10 @@ bool limit_ample(const cupso_swarm* h) {
 //    1.0 to 1.5 us (2.2 while gbest improves) whatever the swarm, against 1.1 us (32 x
 //    1) to 4.7 (2048 x 32) on the cluster, whose launch costs less: 2048 x 32 at 4
 //    iterations 4.0 against 6.7 us, 1000 x 2 3.1 against 2.8; 300 x 8 (Rosenbrock)
-//    at 100 1.95 against 1.68, at 1000 1.51 against 1.58.
+//    at 100 1.95 against 1.68, at 1000 1.51 against 1.58. The cluster's time grows with D
+//    and the line by N leaves that out: below 1000 particles long ones stay on the cluster
+//    where registers would be faster (64 x 30 in calls of 100 1.2 to 2.5 against 2.3 to 3.1,
+//    512 x 16 1.1 to 1.4 against 1.7 to 2.2, but Rosenbrock there 2.2 against 2.0).
 int resident_from(const cupso_swarm* h, int mode) {
     if (!h->rbufs.slots || h->sync_kernel != CUPSO_SYNC_KERNEL_AUTO || h->grid_override != 0 || h->iters_per_launch == 1 ||
         !limit_ample(h))

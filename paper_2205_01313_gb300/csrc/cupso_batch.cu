@@ -1,7 +1,8 @@
 // cupso_batch.cu -- cupso_solve_batch: many independent swarms at once.
 //
 // All swarms of a batch live in one device arena. Swarms of kBatchPanelMinD
-// dimensions or more are kept in panels and advance together, one launch per
+// dimensions or more are kept in panels (but for those that padding to whole panels
+// would slow, or where it would not fit the device) and advance together, one launch per
 // iteration (kernels_batch_panel.cu). The others have a launch of their own: one
 // runs Step 1 of every swarm (batch_init_kernel), then every iteration is ONE launch
 // of batch_step_kernel covering the units of all of them (kernels_batch.cu). The

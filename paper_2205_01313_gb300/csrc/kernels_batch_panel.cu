@@ -18,7 +18,8 @@
 // memory (20 bytes per particle and dimension: 0.82 ms at the copy's rate) with the issue
 // slots half taken.
 // Swarms of fewer than kBatchPanelMinD dimensions have too few panels for the ring's
-// look-ahead and stay there. In batches of hundreds of swarms a ring of 6 stages (`deep`) is
+// look-ahead and stay there, and so do those whose last panel's unused dimensions would be
+// moved at a cost where memory bounds the batch (the rule stands in cupso_batch.cu). In batches of hundreds of swarms a ring of 6 stages (`deep`) is
 // the faster one, 1046 and 1009 us at 512, and those of fewer than kBatchPanelDeepD dimensions
 // stay there too; with 128 it is 276 and 282.
 //

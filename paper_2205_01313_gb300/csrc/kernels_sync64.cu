@@ -19,7 +19,7 @@
 // 120 on 152 SMs is 405 x 8 + 4 x 120 instructions per SM, 34 us of the 39.6 an
 // iteration takes. (Before: one launch per iteration of tiles of 16 particles, whose
 // sums filled half a warp and a fifth of the pipe, and 7 tiles on some SMs, 6 on
-// others: 60 us. The paper's one-dimensional swarms, 8192 particles: 1.6 us; with a
+// others: 60 us. The paper's one-dimensional swarms, 8192 particles: 1.5 us; with a
 // launch and a last-block hand-off per iteration 4.8, in a persistent kernel with one
 // particle per thread and everything between two barriers 3.3, on a cluster 4.2.)
 //
